@@ -404,8 +404,9 @@ int hfx_slo_map(hfx_sched *s, int32_t n_prio, const hfx_slo_window *win, const h
  * columns are overwritten) and runs `iters` iterations of step + commit, or
  * until nothing is left to happen.  Written: state, gen, first_token_ns,
  * last_token_ns, finish_ns and `out`.
- * A trace of up to 10240 rows is kept in shared memory; a longer one (at most 65535 rows) works in a scratch
- * buffer in device memory (15 bytes per row for two traces per SM), which the first call that needs it
+ * A trace of up to 10240 rows is kept in shared memory when all traces of the call fit it together; longer traces (at
+ * most 65535 rows) and larger batches work in a scratch buffer in device memory (13 bytes per row for at most sixteen
+ * traces per SM), which the first call that needs it
  * allocates with cudaMalloc after synchronising the stream, so such a call should not be made inside a stream
  * capture; hfx_sched_destroy frees it.
  * Errors: HFX_E_ARG, HFX_E_ALIGN, HFX_E_CAPACITY (n_traces > n_replicas, or a

@@ -1,32 +1,39 @@
-// hfx_sim_run: batched trace-driven simulation, one persistent thread block per trace.
+// hfx_sim_run: batched trace-driven simulation, one warp per trace.
 //
-// A trace is staged once into shared memory; then the block runs the scheduler iteration
-// (visible set, aggregates of the running batch, E_d, safe budget, most-urgent-first admission,
-// maturity, commit, clock advance) `iters` times without leaving the chip.  Work per iteration
-// scales with the live set (queue + running batch), not with the trace length:
-//   - rows are sorted by arrival, so the visible queue grows from a head pointer;
-//   - the running batch and the strictest SLOs are kept as incremental counters;
-//   - a running request's completion iteration is fixed at admission (every iteration with a
-//     running batch advances each of its requests by one token);
-//   - admission extracts the most urgent eligible request repeatedly (block-wide arg-min on
-//     (prio, clamp(slack), req_id)) and stops at the first one that does not fit, which is
-//     exactly the prefix-closed rule of the sorted formulation.
-// Shared memory is what bounds the number of resident traces, so a row takes 15 bytes: one 8-byte slot
-// (arrival, then the slack base while queued, then the finish iteration while running), a word (prompt
-// length and priority), a byte (class and state) and one list entry (the queue from the front of the list array, the running batch
-// from its back: a row is in one of them at most); the rows
-// admitted in an iteration are parked in the part of the queue array that their extraction frees, and the
-// running list is kept in place (a finished request's place is filled from the tail).  A scan of the queue is
-// only made when the budget reaches the shortest queued prompt (a bound kept beside the queue).
+// The scheduler iteration (visible set, aggregates of the running batch, E_d, safe budget, most-urgent-first
+// admission, maturity, commit, clock advance) is a serial recurrence with little work in it, so what bounds it is
+// the latency of one iteration.  A warp holds the whole state of its trace in registers (clock, maturity, list
+// lengths, class counts with one class per lane) and never meets a block barrier; what an iteration has to look
+// at is bounded by what changed:
+//   - a window of 32 rows is held in registers (one row per lane, the window behind it already asked for), so
+//     "has anything arrived?" is a comparison with the next arrival time, and a row that has arrived simply
+//     waits there (the box); when the window moves on, what is left of it joins a list sorted by (prio, slack base,
+//     id), which is the order of the queue at any later time (all slacks fall together);
+//   - a running request's finish iteration is fixed at admission and the smallest one is kept, so the running
+//     list is only walked in an iteration that finishes somebody;
+//   - admission is only tried when the budget reaches the shortest queued prompt (a bound kept beside the queue); it
+//     takes the most urgent requests from the list's end and the box until one no longer fits;
+//   - iterations in which nothing arrives, finishes or is admitted are taken 32 at a time: the clock after j of
+//     them is now + j E_d + d2 n_run j (j - 1) / 2 (every request in flight adds one token of context), lane j
+//     forms it and a ballot finds the first one that something happens in.  Such a stretch cannot admit: with the
+//     batch and the queue fixed E_d only grows, and a prompt that did not fit the budget bound does not fit it
+//     under a larger E_d; before maturity the stretch ends at maturity.
+// Measured (B200): one trace of 256 rows, 2000 iterations 3.45 -> 0.79 ms; 4096 traces of 2048 rows, 10,000 iterations 103
+// -> 21.3 ms (392 M -> 1.9 G iterations/s), against a block of 128 threads per trace that met five barriers and
+// looked at every request in flight in every iteration.  What is left is instructions: about 450 per event, in series, one
+// issued in every six cycles.
+// A row takes 15 bytes: one 8-byte slot (slack base while queued, admission and finish iteration
+// while running), a word (prompt length and priority), a byte (class and state) and one list entry (the queue from
+// the front of the list array, the running batch from its back: a row is in one of them at most).
 #include "hfx_internal.cuh"
 
-#define SIM_THREADS 128
-#define SIM_WARPS (SIM_THREADS / 32)
-#define SIM_SMEM_ROWS 10240          // longest trace whose rows are kept in shared memory (15 bytes each); longer ones work in global scratch
-#define SIM_BYTES_PER_ROW 15
-#define SIM_CLASS_BYTES(nc) ((((size_t)(nc) * 24) + 15) & ~(size_t)15)     // per-class tables in dynamic shared memory: TTFT, TPOT, two counters
-#define SIM_HOLES 32                 // finished requests of one iteration whose places in the running list are noted
+#define SIM_SMEM_ROWS 10240          // longest trace whose rows are kept in shared memory (15 bytes each)
+#define SIM_BYTES_PER_ROW 13           // besides the 2 bytes of the list
+#define SIM_BINS 256                 // bins of the percentile selection (8 bits a pass)
+#define SIM_HEAD_BYTES(nc) ((((size_t)(nc) * 40 + 16 + SIM_BINS * 4) + 15) & ~(size_t)15)     // in front of the rows: TTFT and TPOT by class and by rank, the bins, two counters per class
 #define SIM_OUTLEN_CAP (1 << 30)   // output lengths are clamped here when the finish iteration is formed
+#define SIM_PARKED (SIM_BINS * 2)   // admitted requests of an iteration that are noted in shared memory (over the bins)
+#define SIM_SCRATCH_PER_SM 16      // most traces worked on at once per SM with the rows in scratch
 
 // the byte of a row: class<6> | state<2>; the word of a row: prompt_len<25> | prio<6>, prio 63 marks a row with bad data
 #define ROW_CLS(x) ((x) & 0x3fu)
@@ -47,443 +54,639 @@ struct SimArgs {
   int64_t *ttft_p50, *ttft_p99, *tpot_p50, *tpot_p99, *now_out;
 };
 
-struct SimShared {
-  ReplicaPlan plan;
-  int64_t now, mat, sum_kv;
-  int64_t t1, t2, lp, mat_next;
-  int64_t d_kv;                 // change of sum_kv collected during commit
-  int32_t head, head_prev, nq, nr, na, no, arrived;
-  int32_t worked, stop, trace, zero_prompt;
-  int32_t min_prompt;           // a lower bound of the shortest prompt in the queue: lowered by every arrival, made exact by
-                                // every scan of the queue (an admission can only raise the true value)
-  int32_t best_min[2][SIM_WARPS];
-  int32_t n_holes;              // requests of the running list that finished in this iteration
-  uint16_t holes[SIM_HOLES];    // their places in the list (the first SIM_HOLES of them)
-  // arg-min scratch, double buffered
-  uint64_t best_key[2][SIM_WARPS];
-  uint32_t best_id[2][SIM_WARPS];
-  int32_t best_slot[2][SIM_WARPS];
-  // end-of-trace counters
-  int32_t n_fin, n_rej, n_att, n_a, n_b;
-};
+#define FULL 0xffffffffu
 
-__device__ __forceinline__ void sort_i64(int64_t *v, int n) {
-  int n_pad = 1;
-  while (n_pad < n) n_pad <<= 1;
-  const int half = n_pad >> 1;
-  for (int k = 2; k <= n_pad; k <<= 1) {
-    const int hk = k >> 1;
-    for (int t = threadIdx.x; t < half; t += blockDim.x) {
-      const int blk = t / hk, off = t - blk * hk;
-      const int i = blk * k + off, j = blk * k + k - 1 - off;
-      if (j < n) { const int64_t x = v[i], y = v[j]; if (x > y) { v[i] = y; v[j] = x; } }
-    }
-    __syncthreads();
-    for (int j = k >> 2; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < half; t += blockDim.x) {
-        const int i = 2 * t - (t & (j - 1));
-        if (i + j < n) { const int64_t x = v[i], y = v[i + j]; if (x > y) { v[i] = y; v[i + j] = x; } }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__device__ __forceinline__ int64_t nearest_rank(const int64_t *sorted, int n, int pct) {
+// The nearest-rank percentile of n non-negative values: 8 bits a pass from the highest byte in use, the warp counting the
+// values that share the prefix found so far.  All lanes call; all get the result.
+__device__ int64_t warp_percentile(const int64_t *v, int n, int pct, uint32_t *bins, int lane) {
   if (n == 0) return -1;
   int64_t k = ((int64_t)pct * n + 99) / 100;
   if (k < 1) k = 1;
-  return sorted[k - 1];
+  uint32_t rank = (uint32_t)k;               // 1-based
+  uint64_t all = 0;
+  for (int i = lane; i < n; i += 32) all |= (uint64_t)v[i];
+  all = warp_or_u64(all);
+  int shift = all ? ((63 - __clzll((long long)all)) & ~7) : 0;
+  uint64_t prefix = 0;                       // the bits above `shift + 8` of the answer
+  for (;; shift -= 8) {
+    for (int i = lane; i < SIM_BINS; i += 32) bins[i] = 0;
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+      const uint64_t x = (uint64_t)v[i];
+      if (shift == 56 || (x >> (shift + 8)) == prefix) atomicAdd(&bins[(uint32_t)(x >> shift) & 255u], 1u);
+    }
+    __syncwarp();
+    uint32_t c[8], sum = 0;                  // lane l holds the bins 8 l .. 8 l + 7
+#pragma unroll
+    for (int e = 0; e < 8; e++) { c[e] = bins[lane * 8 + e]; sum += c[e]; }
+    const uint32_t inc = (uint32_t)warp_incl_scan_i32((int32_t)sum, lane);
+    const int l = __ffs(__ballot_sync(FULL, inc >= rank)) - 1;
+    uint32_t before = inc - sum, d = 0;
+#pragma unroll
+    for (int e = 0; e < 8; e++) if (before + c[e] < rank && d == (uint32_t)e) { before += c[e]; d = e + 1; }
+    d = __shfl_sync(FULL, d, l); before = __shfl_sync(FULL, before, l);
+    rank -= before;
+    prefix = (prefix << 8) | (uint64_t)(l * 8 + d);
+    __syncwarp();
+    if (shift == 0) return (int64_t)prefix;
+  }
 }
 
-// SCRATCH: the per-row arrays of a block live in its part of a global scratch buffer instead of shared memory (traces
-// too long for it); the code is the same.
+// one row of the arrival window, as a lane holds it
+struct SimRow { int64_t arr; int32_t prompt, weight; uint32_t cls; };
+
+__device__ __forceinline__ SimRow sim_load_row(const SimArgs &a, int64_t g, bool in) {
+  SimRow r;
+  r.arr = HFX_INF; r.prompt = -1; r.weight = 0; r.cls = 0;
+  if (in) {
+    r.arr = a.arrival[g]; r.prompt = a.prompt_len[g]; r.cls = a.class_id[g];
+    if (a.weight) r.weight = a.weight[g];
+  }
+  return r;
+}
+
+// SCRATCH: the per-row arrays (13 bytes a row) live in the block's part of a global scratch buffer and only the list in
+// shared memory.  The live rows then come from L1 most of the time, and more than twice as many traces are resident: what
+// a batch of more traces than shared memory holds needs, since a warp by itself issues in one cycle of six (4096 traces of
+// 2048 rows: 7 a SM 28.4 ms, 14 a SM 23.5 ms with the same code).
 template <bool SCRATCH>
-__global__ void __launch_bounds__(SIM_THREADS) k_sim(const HfxParams p, const SimArgs a, uint32_t *__restrict__ work_counter,
-                                                     uint32_t *__restrict__ status, unsigned char *__restrict__ scratch) {
+__global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, uint32_t *__restrict__ work_counter,
+                                            uint32_t *__restrict__ status, unsigned char *__restrict__ scratch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cap = a.cap_rows;
-  // per class, in front of the rows: TTFT and TPOT bounds, requests in flight, requests in the queue
   const int nc = p.n_classes;
-  int64_t *c_ttft = reinterpret_cast<int64_t *>(smem_raw), *c_tpot = c_ttft + nc;
-  int32_t *c_run = reinterpret_cast<int32_t *>(c_tpot + nc), *c_q = c_run + nc;
-  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * cap * SIM_BYTES_PER_ROW : smem_raw + SIM_CLASS_BYTES(nc);
-  int64_t *s_arr = reinterpret_cast<int64_t *>(rows_mem);              // arrival; the slack base once arrived; the finish iteration once running; later the TTFT, then the TPOT samples
-  uint32_t *s_word = reinterpret_cast<uint32_t *>(s_arr + cap);        // prompt_len | prio << 25
-  // One list array for both lists (a row is in one of them at most): from the front the visible queue (row indices,
-  // unordered) and behind it the rows admitted in this iteration; from the back the running batch (RUN(s), unordered;
-  // 0xffff: a request that just finished)
-  uint16_t *s_q = reinterpret_cast<uint16_t *>(s_word + cap);
-  uint8_t *s_byte = reinterpret_cast<uint8_t *>(s_q + cap);            // class | state << 6
+  int64_t *c_ttft = reinterpret_cast<int64_t *>(smem_raw), *c_tpot = c_ttft + nc;      // by class
+  int64_t *s_ttft = c_tpot + nc, *s_tpot = s_ttft + nc + 1;                           // by rank
+  uint32_t *s_bins = reinterpret_cast<uint32_t *>(s_tpot + nc + 1);
+  uint16_t *s_park = reinterpret_cast<uint16_t *>(s_bins);      // [SIM_PARKED] the requests admitted in an iteration
+  int32_t *s_cq = reinterpret_cast<int32_t *>(s_bins + SIM_BINS), *s_cr = s_cq + nc;      // requests in the queue's list / in flight per class
+  uint16_t *s_q = reinterpret_cast<uint16_t *>(smem_raw + SIM_HEAD_BYTES(nc));
+  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * cap * SIM_BYTES_PER_ROW : smem_raw + SIM_HEAD_BYTES(nc) + (size_t)cap * 2;
+  int64_t *s_slot = reinterpret_cast<int64_t *>(rows_mem);             // slack base in the queue; finish iteration | admission iteration << 32 in the batch; later the TTFT, then the TPOT samples
+  uint32_t *s_word = reinterpret_cast<uint32_t *>(s_slot + cap);       // prompt_len | prio << 25
+  // One list array for both lists: from the front the queue's list (row indices, the least urgent first), from the back the
+  // running batch (RUN(s), unordered)
+  uint8_t *s_byte = reinterpret_cast<uint8_t *>(s_word + cap);            // class | state << 6
 #define RUN(s) s_q[cap - 1 - (s)]
-  __shared__ SimShared S;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x;
+  const uint32_t lt = (1u << lane) - 1u;
+  // Strictest SLO over the classes that have requests: every class has a rank by its bound (nc: none), the bounds are kept
+  // by rank, so the strictest one of a set is a minimum over small integers (lane c looks at classes c and c + 32).
+  uint32_t rt0 = nc, rt1 = nc, rp0 = nc, rp1 = nc;
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const int c = lane + 32 * h;
+    if (c < nc) {
+      const int64_t tc = p.ttft[c], pc = p.tpot[c];
+      uint32_t rt = 0, rp = 0;
+      for (int k = 0; k < nc; k++) {
+        const int64_t tk = p.ttft[k], pk = p.tpot[k];
+        rt += tk > 0 && (tk < tc || (tk == tc && k < c));
+        rp += pk > 0 && (pk < pc || (pk == pc && k < c));
+      }
+      if (tc > 0) { s_ttft[rt] = tc; if (h == 0) rt0 = rt; else rt1 = rt; }
+      if (pc > 0) { s_tpot[rp] = pc; if (h == 0) rp0 = rp; else rp1 = rp; }
+      c_ttft[c] = tc; c_tpot[c] = pc;
+    }
+  }
+  if (lane == 0) { s_ttft[nc] = HFX_INF; s_tpot[nc] = HFX_INF; }
+  const int64_t d2 = p.d2;
 
   for (;;) {
-    __syncthreads();
-    if (tid == 0) S.trace = (int32_t)atomicAdd(work_counter, 1u);
-    __syncthreads();
-    const int j = S.trace;
+    int j = 0;
+    if (lane == 0) j = (int)atomicAdd(work_counter, 1u);
+    j = __shfl_sync(FULL, j, 0);
     if (j >= a.n_traces) return;
     const int32_t b = a.trace_off[j];
     const int m = a.trace_off[j + 1] - b;
     const hfx_replica_cfg cfg = a.cfg[j];
+    for (int i = lane; i < m; i += 32) s_byte[i] = ROW_BYTE(0u, HFX_QUEUED);
+    for (int c = lane; c < nc; c += 32) { s_cq[c] = 0; s_cr[c] = 0; }
+    __syncwarp();
 
-    // ---- stage the trace ----------------------------------------------------------------
-    if (tid == 0) {
-      S.now = 0; S.mat = 0; S.sum_kv = 0; S.head = 0; S.head_prev = 0; S.nq = 0; S.nr = 0; S.stop = 0;
-      S.n_fin = 0; S.n_rej = 0; S.n_att = 0; S.n_a = 0; S.n_b = 0; S.zero_prompt = 0; S.min_prompt = INT32_MAX; S.n_holes = 0;
-      S.arrived = 0; S.no = 0; S.na = 0; S.d_kv = 0;
-    }
-    __syncthreads();
-    for (int c = tid; c < nc; c += SIM_THREADS) { c_run[c] = 0; c_q[c] = 0; c_ttft[c] = p.ttft[c]; c_tpot[c] = p.tpot[c]; }
-    uint32_t bad = 0;
-    for (int i = tid; i < m; i += SIM_THREADS) {
-      const int64_t g = (int64_t)b + i;
-      const uint32_t cls = a.class_id[g];
-      const int32_t prompt = a.prompt_len[g];
-      const int64_t arr = a.arrival[g];
-      bool ok = true;
-      if (cls >= (uint32_t)p.n_classes) { bad |= HFX_ST_BAD_CLASS; ok = false; }
-      if (prompt < 0 || prompt > HFX_MAX_TOKENS) { bad |= HFX_ST_BAD_LEN; ok = false; }
-      s_arr[i] = arr;
-      if (prompt == 0) S.zero_prompt = 1;   // a zero-token prompt fits a zero budget
-      uint32_t prio = ROW_INVALID_PRIO;
+    int64_t now = 0, mat = 0, sum_kv = 0;
+    int nq = 0, nr = 0, it = 0;
+    int32_t min_prompt = INT32_MAX;           // a lower bound of the shortest prompt in the queue: lowered by every arrival, made exact
+                                              // when the whole queue has been looked at (an admission can only raise the true value)
+    int32_t next_fin = INT32_MAX;             // the earliest finish iteration in the running batch
+    int64_t min_ttft = HFX_INF, min_tpot = HFX_INF;
+    int64_t base_lo = HFX_INF, base_hi = INT64_MIN;      // bounds of the finite slack bases in the queue
+    // the requests admitted in an iteration: the first ones in shared memory, the rest (tiny prompts) in the trace's gen
+    // column, which is written when the trace is over
+    auto park = [&](int k, int row) { if (k < SIM_PARKED) s_park[k] = (uint16_t)row; else a.gen[(int64_t)b + k] = row; };
+    auto parked = [&](int k) -> int { return k < SIM_PARKED ? (int)s_park[k] : a.gen[(int64_t)b + k]; };
+    auto id_of = [&](int row) -> uint32_t { return (uint32_t)__ldg(a.req_id + b + row) ^ 0x80000000u; };
+
+    // The window: rows wb .. wb + 31, one per lane.  pend: the valid ones that have not arrived; box: those that have arrived
+    // and wait (the young part of the queue stays here; what is left of it joins the sorted list when the window moves on).
+    int wb = 0;
+    SimRow w = sim_load_row(a, (int64_t)b + lane, lane < m);
+    SimRow wn = sim_load_row(a, (int64_t)b + 32 + lane, 32 + lane < m);
+    uint32_t word = 0, pend = 0, box = 0, wrank = 0;
+    int64_t base = BASE_UNBOUNDED;            // slack base, ttft_slo + arrival - E_p(prompt_len): the slack at any later decision is the base minus the earliest start
+    auto open_window = [&]() {
+      const bool ok = wb + lane < m && w.cls < (uint32_t)nc && w.prompt >= 0 && w.prompt <= HFX_MAX_TOKENS;
+      base = BASE_UNBOUNDED; wrank = nc;
       if (ok) {
+        uint32_t prio;
         if (p.weight_max > 0) {
-          const int64_t w = (int64_t)p.weight_max - a.weight[g];
-          prio = (uint32_t)(w < 0 ? 0 : (w > 62 ? 62 : w));
-        } else prio = p.prio[cls];
+          const int64_t x = (int64_t)p.weight_max - w.weight;
+          prio = (uint32_t)(x < 0 ? 0 : (x > 62 ? 62 : x));
+        } else prio = p.prio[w.cls];
+        word = (uint32_t)w.prompt | (prio << 25);
+        const int64_t ttft = c_ttft[w.cls];
+        if (ttft > 0) base = ttft + w.arr - dev_Ep(p, w.prompt);
       }
-      s_word[i] = (ok ? (uint32_t)prompt : 0u) | (prio << 25);
-      s_byte[i] = ROW_BYTE(ok ? cls : 0u, HFX_QUEUED);
-      a.first_token[g] = -1; a.last_token[g] = -1; a.finish[g] = -1;
-    }
-    if (bad) atomicOr(status, bad);
-    // A trace that is not sorted by arrival is a caller error; it is simulated as given (the head
-    // pointer stops at the first row that has not arrived) and cannot fault.
-    __syncthreads();
-
-    int executed = 0;
-    PlanMemo memo;          // of the planning warp: the trace's replica is planned every iteration
-    plan_memo_reset(memo);
-    for (int it = 0; it < a.iters; it++) {
-      // ---- 1. arrivals: rows [head, head + k) with arrival <= now join the queue -----------
-      // (the iteration's counters were cleared by the thread that closed the previous one)
-      {
-        const int64_t now = S.now;
-        const int head = S.head;
-        int local = 0;
-        for (int i = head + tid; i < m && s_arr[i] <= now; i += SIM_THREADS) {
-          local++;
-          const uint32_t w = s_word[i];
-          if (ROW_PRIO(w) == ROW_INVALID_PRIO) continue;
-          const uint32_t cls = ROW_CLS(s_byte[i]);
-          atomicAdd(&c_q[cls], 1);
-          if (ROW_PROMPT(w) > cfg.token_cap) {
-            // can never be served: visible for this one iteration, rejected at its commit (which looks through
-            // the rows that arrived in the iteration again)
-            atomicAdd(&S.no, 1);
-          } else {
-            const int slot = atomicAdd(&S.nq, 1);
-            s_q[slot] = (uint16_t)i;
-            atomicMin(&S.min_prompt, (int32_t)ROW_PROMPT(w));
-            // from here on the row's slot holds its slack base, ttft_slo + arrival - E_p(prompt_len):
-            // the slack at any later decision is the base minus the earliest start
-            const int64_t ttft = c_ttft[cls];
-            s_arr[i] = ttft > 0 ? ttft + s_arr[i] - dev_Ep(p, ROW_PROMPT(w)) : BASE_UNBOUNDED;
-          }
-        }
-        if (local) atomicAdd(&S.arrived, local);
+      wrank = __shfl_sync(FULL, rt0, w.cls & 31u);
+      if (nc > 32) { const uint32_t r1 = __shfl_sync(FULL, rt1, w.cls & 31u); if (w.cls >= 32u) wrank = r1; }
+      pend = __ballot_sync(FULL, ok);
+      const bool bounded = ok && base != BASE_UNBOUNDED;
+      const int64_t lo = warp_min_i64(bounded ? base : HFX_INF), hi = ~warp_min_i64(bounded ? ~base : HFX_INF);
+      base_lo = lo < base_lo ? lo : base_lo; base_hi = hi > base_hi ? hi : base_hi;
+    };
+    // The box joins the list: every waiting row finds its place by a binary search of its own and its rank among the
+    // others, then the more urgent entries move up, 32 at a time from the top down.
+    auto merge_box = [&]() {
+      const bool me = (box >> lane) & 1u;
+      const int row = wb + lane;
+      const uint32_t prio = ROW_PRIO(word);
+      if (me) {
+        s_word[row] = word; s_slot[row] = base; s_byte[row] = ROW_BYTE(w.cls, HFX_QUEUED);
+        atomicAdd(&s_cq[w.cls], 1);
       }
-      __syncthreads();
-
-      // ---- 2. plan: E_d of the running batch and the safe budget (the first warp) ----------------
-      if (warp == 0) {
-        if (lane == 0) { S.head_prev = S.head; S.head += S.arrived; }
-        const uint32_t r0 = __ballot_sync(0xffffffffu, lane < p.n_classes && c_run[lane] > 0);
-        const uint32_t r1 = __ballot_sync(0xffffffffu, lane + 32 < p.n_classes && c_run[lane + 32] > 0);
-        const uint32_t q0 = __ballot_sync(0xffffffffu, lane < p.n_classes && c_q[lane] > 0);
-        const uint32_t q1 = __ballot_sync(0xffffffffu, lane + 32 < p.n_classes && c_q[lane + 32] > 0);
-        ReplicaPlan pl0;
-        // the budget only matters if it reaches the shortest queued prompt (a queue without requests admits nothing)
-        memo.need = S.zero_prompt ? 0 : (S.nq > 0 ? (int64_t)S.min_prompt : (int64_t)cfg.token_cap + 1);
-        warp_plan(p, c_ttft, c_tpot, cfg, S.now, S.mat, S.nr, S.sum_kv, ((uint64_t)r1 << 32) | r0, ((uint64_t)q1 << 32) | q0, pl0, lane, &memo);
-        if (lane == 0) S.plan = pl0;
-      }
-      __syncthreads();
-      const int64_t budget = S.plan.budget, start = S.plan.start;
-      const int nr = S.nr;
-      const int32_t min_prompt = S.min_prompt;
-
-      // ---- 3. admission: extract the most urgent request that fits alone, until one fails ----
-      int64_t s_cost = 0, adm_cost = 0;
-      int s_cnt = 0, adm_cnt = 0;
-      int nq = S.nq;
-      // (a budget below the shortest queued prompt admits nothing: the scan of the queue would come back empty)
-      if ((budget > 0 || S.zero_prompt) && (int64_t)min_prompt <= budget) {
-        int buf = 0;
-        for (;;) {
-          uint64_t bk = ~0ull; uint32_t bid = ~0u; int bslot = -1;
-          int32_t lmin = INT32_MAX;
-          for (int s = tid; s < nq; s += SIM_THREADS) {
-            const int i = s_q[s];
-            const uint32_t wd = s_word[i];
-            lmin = (int32_t)ROW_PROMPT(wd) < lmin ? (int32_t)ROW_PROMPT(wd) : lmin;
-            if ((int64_t)ROW_PROMPT(wd) > (p.first_fit ? budget - adm_cost : budget)) continue;      // first fit: against what is left
-            // slack of a queued request: ttft_slo - (start - arrival) - E_p(prompt_len) = base - start
-            const int64_t base = s_arr[i];
-            const int64_t sl = base != BASE_UNBOUNDED ? dev_clamp_slack(base - start) : HFX_SLACK_MAX;
-            const uint64_t k = ((uint64_t)ROW_PRIO(wd) << 40) | (uint64_t)(sl + (INT64_C(1) << 39));
-            if (k < bk) { bk = k; bslot = s; bid = ~0u; }
-            else if (k == bk) {      // equal keys are rare: only then fetch the request ids that break the tie
-              if (bid == ~0u) bid = (uint32_t)__ldg(a.req_id + b + s_q[bslot]) ^ 0x80000000u;
-              const uint32_t id = (uint32_t)__ldg(a.req_id + b + i) ^ 0x80000000u;
-              if (id < bid) { bid = id; bslot = s; }
-            }
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const uint64_t k2 = __shfl_xor_sync(0xffffffffu, bk, o);
-            uint32_t i2 = __shfl_xor_sync(0xffffffffu, bid, o);
-            const int s2 = __shfl_xor_sync(0xffffffffu, bslot, o);
-            if (k2 == bk && bslot >= 0 && s2 >= 0 && s2 != bslot) {
-              if (bid == ~0u) bid = (uint32_t)__ldg(a.req_id + b + s_q[bslot]) ^ 0x80000000u;
-              if (i2 == ~0u) i2 = (uint32_t)__ldg(a.req_id + b + s_q[s2]) ^ 0x80000000u;
-            }
-            if (k2 < bk || (k2 == bk && i2 < bid)) { bk = k2; bid = i2; bslot = s2; }
-          }
-          lmin = __reduce_min_sync(0xffffffffu, lmin);
-          if (lane == 0) { S.best_key[buf][warp] = bk; S.best_id[buf][warp] = bid; S.best_slot[buf][warp] = bslot; S.best_min[buf][warp] = lmin; }
-          __syncthreads();
-          if (tid == 0) {      // the shortest prompt of the queue as it stood for this scan
-            int32_t mn = S.best_min[buf][0];
-#pragma unroll
-            for (int w = 1; w < SIM_WARPS; w++) mn = S.best_min[buf][w] < mn ? S.best_min[buf][w] : mn;
-            S.min_prompt = mn;
-          }
-          bk = S.best_key[buf][0]; bid = S.best_id[buf][0]; bslot = S.best_slot[buf][0];
-#pragma unroll
-          for (int w = 1; w < SIM_WARPS; w++) {
-            const uint64_t k2 = S.best_key[buf][w]; uint32_t i2 = S.best_id[buf][w];
-            const int s2 = S.best_slot[buf][w];
-            if (k2 == bk && bslot >= 0 && s2 >= 0) {
-              if (bid == ~0u) bid = (uint32_t)__ldg(a.req_id + b + s_q[bslot]) ^ 0x80000000u;
-              if (i2 == ~0u) i2 = (uint32_t)__ldg(a.req_id + b + s_q[s2]) ^ 0x80000000u;
-            }
-            if (k2 < bk || (k2 == bk && i2 < bid)) { bk = k2; bid = i2; bslot = s2; }
-          }
-          buf ^= 1;
-          if (bslot < 0) break;                       // no eligible request left
-          const int i = s_q[bslot];
-          const int32_t pr_i = ROW_PROMPT(s_word[i]);
-          s_cost += pr_i; s_cnt += 1;
-          if (!(s_cost <= budget && (cfg.batch_cap == 0 || nr + s_cnt <= cfg.batch_cap))) break;
-          adm_cost += pr_i; adm_cnt += 1;
-          __syncthreads();                            // everyone has read s_q[bslot]
-          // the queue shrinks by one; the place it frees behind its end takes the admitted row
-          if (tid == 0) { s_q[bslot] = s_q[nq - 1]; s_q[nq - 1] = (uint16_t)i; }
-          nq -= 1;
-          __syncthreads();
+      int pos = 0;                            // entries of the list that are less urgent than mine
+      for (int hi = nq; __any_sync(FULL, pos < hi);) {
+        if (pos < hi) {
+          const int mid = (pos + hi) >> 1, i = s_q[mid];
+          const uint32_t pr = ROW_PRIO(s_word[i]);
+          const int64_t be = s_slot[i];
+          bool less = pr > prio || (pr == prio && be > base);
+          if (me && pr == prio && be == base) less = id_of(i) > id_of(row);
+          if (less) pos = mid + 1; else hi = mid;
         }
       }
-      const int nq_adm = nq;      // the rows admitted in this iteration are s_q[nq_adm .. nq_adm + adm_cnt), last admitted first
+      int rank = 0;
+      for (uint32_t x = box; x; x &= x - 1) {
+        const int l = __ffs(x) - 1;
+        const uint32_t pr = __shfl_sync(FULL, prio, l);
+        const int64_t be = __shfl_sync(FULL, base, l);
+        bool less = pr > prio || (pr == prio && be > base);
+        if (me && lane != l && pr == prio && be == base) less = id_of(wb + l) > id_of(row);
+        rank += less ? 1 : 0;
+      }
+      for (int c0 = (nq - 1) & ~31; nq > 0 && c0 >= 0; c0 -= 32) {
+        const int e = c0 + lane;
+        const uint32_t below = __ballot_sync(FULL, me && pos <= c0), in = __ballot_sync(FULL, me && pos > c0 && pos <= c0 + 31);
+        if ((below | in) == 0) break;         // (the places below are none either)
+        const uint16_t v = e < nq ? s_q[e] : (uint16_t)0;
+        int up = __popc(below);
+        for (uint32_t x = in; x; x &= x - 1) up += __shfl_sync(FULL, pos, __ffs(x) - 1) <= e ? 1 : 0;
+        __syncwarp();
+        if (e < nq && up) s_q[e + up] = v;
+        __syncwarp();
+      }
+      if (me) s_q[pos + rank] = (uint16_t)row;
+      nq += __popc(box);
+      box = 0;
+      __syncwarp();
+    };
+    auto advance_window = [&]() {             // to the next window that has a valid row, if there is one
+      while (pend == 0 && wb + 32 < m) {
+        if (box) merge_box();
+        wb += 32;
+        w = wn;
+        wn = sim_load_row(a, (int64_t)b + wb + 32 + lane, wb + 32 + lane < m);
+        open_window();
+      }
+    };
+    auto strictest_q = [&]() -> int64_t {      // TTFT, over the queue
+      uint32_t x = ((box >> lane) & 1u) ? wrank : (uint32_t)nc;
+      if (lane < nc && s_cq[lane] > 0) x = rt0 < x ? rt0 : x;
+      if (lane + 32 < nc && s_cq[lane + 32] > 0) x = rt1 < x ? rt1 : x;
+      return s_ttft[__reduce_min_sync(FULL, x)];
+    };
+    open_window();
+    advance_window();
+    int64_t next_arr = pend ? __shfl_sync(FULL, w.arr, __ffs(pend) - 1) : HFX_INF;
 
-      // ---- 4. maturity and the iteration's clock -------------------------------------------
-      // every thread knows what was admitted, so every thread forms the iteration's two times itself; the
-      // new maturity (a division) is left to one thread, beside the commit
-      const int64_t t1 = S.now + (adm_cnt > 0 ? dev_Ep(p, adm_cost) : 0);
-      const int64_t t2 = t1 + (nr > 0 ? S.plan.e_d : 0);
-      if (tid == 0) {
-        int64_t lp = 0;
-        S.mat_next = dev_maturity_next(p, S.plan, adm_cnt, adm_cost, 0, &lp);
-        S.worked = adm_cnt > 0 || nr > 0;
-        S.nq = nq; S.na = adm_cnt;
+    while (it < a.iters) {
+      // ---- 1. arrivals: the rows with arrival <= now join the queue -------------------------------------------
+      bool over_any = false;                  // an oversize prompt arrived: its TTFT counts in this iteration only
+      int64_t ttft_it = min_ttft;             // the strictest TTFT of this iteration
+      if (next_arr <= now) {
+        uint32_t over_rank = nc;
+        do {
+          // (a trace that is not sorted by arrival is a caller error: the rows behind one that has not arrived wait for it)
+          const uint32_t late = pend & ~__ballot_sync(FULL, w.arr <= now);
+          const uint32_t come = late ? pend & ((1u << (__ffs(late) - 1)) - 1u) : pend;
+          const bool me = (come >> lane) & 1u, over = me && w.prompt > cfg.token_cap;
+          const uint32_t om = __ballot_sync(FULL, over);
+          const int32_t shortest = (int32_t)__reduce_min_sync(FULL, me && !over ? (uint32_t)w.prompt : 0x7fffffffu);
+          min_prompt = shortest < min_prompt ? shortest : min_prompt;
+          if (om) {                           // never served: rejected at this iteration's commit
+            if (over) s_byte[wb + lane] = ROW_BYTE(w.cls, HFX_REJECTED);
+            const uint32_t r = __reduce_min_sync(FULL, over ? wrank : (uint32_t)nc);
+            over_rank = r < over_rank ? r : over_rank;
+            over_any = true;
+          }
+          box |= come & ~om;
+          pend &= ~come;
+          if (pend == 0) advance_window();
+          next_arr = pend ? __shfl_sync(FULL, w.arr, __ffs(pend) - 1) : HFX_INF;
+        } while (next_arr <= now);
+        min_ttft = strictest_q();
+        ttft_it = min_ttft;
+        if (over_any) { const int64_t x = s_ttft[over_rank]; ttft_it = x < ttft_it ? x : ttft_it; }
       }
 
-      // ---- 5. commit ---------------------------------------------------------------------------
-      int64_t d_kv = 0;
-      // running batch: one more token each; a request finishes when gen + 1 reaches output_len
-      for (int s = tid; s < nr; s += SIM_THREADS) {
-        const int i = RUN(s);
-        if (it >= (int32_t)s_arr[i]) {       // gen + 1 reaches output_len in this iteration
-          RUN(s) = 0xffffu;                // its place is free
-          const int h = atomicAdd(&S.n_holes, 1);
-          if (h < SIM_HOLES) S.holes[h] = (uint16_t)s;
-          const uint32_t cls = ROW_CLS(s_byte[i]);
-          s_byte[i] = ROW_BYTE(cls, HFX_DONE);
-          a.finish[(int64_t)b + i] = t2;
-          atomicSub(&c_run[cls], 1);
-          const int32_t outlen = __ldg(a.output_len + b + i);
-          d_kv -= (int64_t)ROW_PROMPT(s_word[i]) + outlen - 2;       // leaves with the context it had before this step
-        } else d_kv += 1;
+      // ---- 2. plan: E_d of the running batch, the safe budget (Eq. 3) as a bound on E_p ----------------------
+      // The budget is the largest n <= cap_left with E_p(n) den <= num, 0 if there is none.  Only comparisons with it are
+      // needed, so it is not worked out: E_p does not fall with n, so n is within the budget exactly if n satisfies the bound.
+      const int64_t e_d = nr > 0 ? dev_Ed(p, nr, sum_kv) : 0;
+      int64_t cap_left = 0;                   // before maturity the budget is 0: only a zero-token prompt fits it
+      uint64_t num_h = ~0ull, num_l = ~0ull, den = 0;
+      bool scan = false;
+      auto within = [&](int64_t n) -> bool {
+        const uint64_t ep = (uint64_t)dev_Ep(p, n);
+        const uint64_t h = __umul64hi(ep, den), l = ep * den;
+        return n == 0 || (n <= cap_left && (h < num_h || (h == num_h && l <= num_l)));
+      };
+      if (nq > 0 || box) {
+        if (now >= mat) {
+          cap_left = cfg.token_cap - nr > 0 ? cfg.token_cap - nr : 0;
+          const int64_t ttft = ttft_it;
+          if (p.budget_mode != HFX_BUDGET_CAP_ONLY && ttft != HFX_INF) {
+            num_h = 0; num_l = (uint64_t)ttft; den = 2;            // 2 E_p <= TTFT while nothing decodes
+            if (nr > 0 && min_tpot < HFX_INF) {
+              if (min_tpot > e_d) {
+                const uint64_t y = (uint64_t)(min_tpot - e_d);
+                num_h = __umul64hi((uint64_t)ttft, y); num_l = (uint64_t)ttft * y; den = (uint64_t)(2 * min_tpot - e_d);
+              } else cap_left = 0;
+            }
+          }
+        }
+        scan = within(min_prompt);            // otherwise the shortest prompt does not fit: nothing is admitted
       }
-      // admitted requests: first token at t1
-      for (int s = tid; s < adm_cnt; s += SIM_THREADS) {
-        const int i = s_q[nq_adm + s];
-        a.first_token[(int64_t)b + i] = t1;
-        const int32_t outlen = __ldg(a.output_len + b + i);
-        s_arr[i] = it + (outlen < SIM_OUTLEN_CAP ? outlen : SIM_OUTLEN_CAP) - 1;      // the slot now holds the finish iteration
-        const uint32_t cls = ROW_CLS(s_byte[i]);
-        atomicSub(&c_q[cls], 1);
-        if (outlen <= 1) {
-          s_byte[i] = ROW_BYTE(cls, HFX_DONE);
-          a.finish[(int64_t)b + i] = t1;
+
+      // ---- 3. admission: the most urgent requests that fit alone, until one fails ----------------------------
+      int64_t adm_cost = 0;
+      int adm_cnt = 0;
+      if (scan) {
+        const int64_t start = now > mat ? now : mat;
+        // The queue's order is (prio, slack base, id), which is the order of the keys as long as no slack is clamped; the
+        // bounds of the bases say when one might be.
+        auto clamped = [&]() { return base_lo - start < HFX_SLACK_MIN || (base_hi != INT64_MIN && base_hi - start >= HFX_SLACK_MAX); };
+        bool by_key = false;
+        if (clamped()) {                      // (the bounds may be those of requests that are not in the queue)
+          if (box) merge_box();
+          int64_t lo = HFX_INF, hi = INT64_MIN;
+          for (int s = lane; s < nq; s += 32) {
+            const int64_t x = s_slot[s_q[s]];
+            if (x != BASE_UNBOUNDED) { lo = x < lo ? x : lo; hi = x > hi ? x : hi; }
+          }
+          if (((pend >> lane) & 1u) && base != BASE_UNBOUNDED) { lo = base < lo ? base : lo; hi = base > hi ? base : hi; }
+          base_lo = warp_min_i64(lo); base_hi = ~warp_min_i64(~hi);
+          by_key = clamped();
+        }
+        int low = nq;                         // the lowest place of the list that has been looked at
+        bool from_list = false;
+        auto room = [&]() { return cfg.batch_cap == 0 || nr + adm_cnt < cfg.batch_cap; };
+        // what the tests so far say about the budget: n_ok tokens are within it, n_bad are not; most tests end here
+        int64_t n_ok = min_prompt, n_bad = INT64_MAX;
+        auto fits = [&](int64_t n) -> bool {  // (all lanes ask for the same n)
+          if (n <= n_ok) return true;
+          if (n >= n_bad) return false;
+          const bool f = within(n);
+          if (f) n_ok = n; else n_bad = n;
+          return f;
+        };
+        auto fits_mask = [&](bool in, int32_t pr) -> uint32_t {      // (a prompt per lane)
+          bool f = in && pr <= n_ok;
+          const bool open = in && !f && pr < n_bad;
+          if (__any_sync(FULL, open)) {
+            const bool e = open && within(pr);
+            const int64_t top = __reduce_max_sync(FULL, e ? (uint32_t)pr : 0u), bottom = __reduce_min_sync(FULL, open && !e ? (uint32_t)pr : 0x7fffffffu);
+            n_ok = top > n_ok ? top : n_ok;
+            if (bottom != 0x7fffffff) n_bad = bottom < n_bad ? bottom : n_bad;
+            f = f || e;
+          }
+          return __ballot_sync(FULL, f);
+        };
+        if (!by_key) {
+          // Two ordered sources: the list from the most urgent entry down, 32 entries at a time, and the box, whose most
+          // urgent row is found by minima over the lanes.
+          const int32_t wp = ROW_PROMPT(word);
+          uint32_t bm = box ? fits_mask((box >> lane) & 1u, wp) : 0u, fm = 0;      // rows that fit alone: in the box; in the list's chunk
+          int32_t lmin = (box >> lane) & 1u ? wp : INT32_MAX;
+          int q = 0, i = 0, bl = -1, left = nq;
+          uint32_t wd = 0, b_prio = 0;
+          int64_t b_base = 0;
+          bool stop = !room();
+          while (!stop) {
+            while (fm == 0 && left > 0) {     // the next chunk of the list
+              q = left - 1 - lane;
+              i = q >= 0 ? s_q[q] : 0;
+              wd = s_word[i];
+              if (q >= 0) lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
+              fm = fits_mask(q >= 0, ROW_PROMPT(wd));
+              left = left > 32 ? left - 32 : 0;
+              low = left;
+            }
+            if (bm && bl < 0) {               // the most urgent row of the box
+              const bool in = (bm >> lane) & 1u;
+              b_prio = __reduce_min_sync(FULL, in ? ROW_PRIO(word) : 64u);
+              bool cand = in && ROW_PRIO(word) == b_prio;
+              const uint32_t h = (uint32_t)((uint64_t)base >> 32) ^ 0x80000000u;
+              const uint32_t hm = __reduce_min_sync(FULL, cand ? h : ~0u);
+              cand = cand && h == hm;
+              const uint32_t lm = __reduce_min_sync(FULL, cand ? (uint32_t)base : ~0u);
+              uint32_t win = __ballot_sync(FULL, cand && (uint32_t)base == lm);
+              if (win & (win - 1)) {
+                const uint32_t id = (win >> lane) & 1u ? id_of(wb + lane) : ~0u;
+                const uint32_t least = __reduce_min_sync(FULL, id);
+                win = __ballot_sync(FULL, ((win >> lane) & 1u) && id == least);
+              }
+              bl = __ffs(win) - 1;
+              b_base = (int64_t)(((uint64_t)(hm ^ 0x80000000u) << 32) | lm);
+            }
+            if (fm == 0 && bm == 0) break;    // every row that fits has been looked at
+            const int fl = __ffs(fm) - 1;
+            bool list = bm == 0;
+            if (fm && bm) {
+              const int row = __shfl_sync(FULL, i, fl);
+              const uint32_t pr = __shfl_sync(FULL, ROW_PRIO(wd), fl);
+              if (pr != b_prio) list = pr < b_prio;
+              else {
+                const int64_t x = s_slot[row];
+                list = x < b_base;
+                if (x == b_base) list = id_of(row) < id_of(wb + bl);
+              }
+            }
+            const int32_t c = __shfl_sync(FULL, list ? ROW_PROMPT(wd) : wp, list ? fl : bl);
+            if (fits(adm_cost + c)) {
+              if (list) {
+                if (lane == fl) { park(adm_cnt, i); s_q[q] = 0xffffu; atomicSub(&s_cq[ROW_CLS(s_byte[i])], 1); }      // (row numbers stay below 0xffff)
+                from_list = true;
+              } else {
+                if (lane == bl) { park(adm_cnt, wb + lane); s_word[wb + lane] = word; s_byte[wb + lane] = ROW_BYTE(w.cls, HFX_QUEUED); }
+                box &= ~(1u << bl);
+              }
+              adm_cost += c; adm_cnt += 1;
+              stop = !room();
+            } else stop = !p.first_fit || !fits(adm_cost + min_prompt);      // (first fit: can what is left take the shortest prompt?)
+            if (list) fm &= fm - 1;
+            else { bm &= ~(1u << bl); bl = -1; }
+          }
+          if (left == 0 && !stop) min_prompt = (int32_t)__reduce_min_sync(FULL, (uint32_t)lmin);      // every entry was looked at
         } else {
-          s_byte[i] = ROW_BYTE(cls, HFX_RUNNING);      // (joins the running list below)
-          atomicAdd(&c_run[cls], 1);
-          d_kv += ROW_PROMPT(s_word[i]);
-        }
-      }
-      // oversize prompts seen for the first time: among the rows that arrived in this iteration
-      if (S.no > 0) {
-        for (int i = S.head_prev + tid; i < S.head; i += SIM_THREADS) {
-          const uint32_t w = s_word[i];
-          if (ROW_PRIO(w) != ROW_INVALID_PRIO && ROW_PROMPT(w) > cfg.token_cap) {
-            const uint32_t cls = ROW_CLS(s_byte[i]);
-            s_byte[i] = ROW_BYTE(cls, HFX_REJECTED);
-            atomicSub(&c_q[cls], 1);
-          }
-        }
-      }
-      d_kv = warp_sum_i64(d_kv);
-      if (lane == 0 && d_kv) atomicAdd(reinterpret_cast<unsigned long long *>(&S.d_kv), (unsigned long long)d_kv);
-      __syncthreads();
-      if (tid == 0) {
-        S.sum_kv += S.d_kv;
-        {   // the running list, in place: free places below the new length are filled from the tail, then the
-            // admitted requests that go on decoding join (the list has no order)
-          int n = S.nr;
-          const int k = S.n_holes;
-          if (k > 0) {
-            if (k <= SIM_HOLES) {
-              for (int e = 1; e < k; e++) {      // the noted places in ascending order (k is small)
-                const uint16_t x = S.holes[e];
-                int f = e - 1;
-                while (f >= 0 && S.holes[f] > x) { S.holes[f + 1] = S.holes[f]; f--; }
-                S.holes[f + 1] = x;
-              }
-              int tail = n - 1;
-              for (int e = 0; e < k; e++) {
-                const int h = S.holes[e];
-                while (tail > h && RUN(tail) == 0xffffu) tail--;
-                if (h >= tail) break;          // this place and the ones after it lie beyond the new length
-                RUN(h) = RUN(tail); tail--;
-              }
-            } else {                             // many at once: one pass from both ends
-              int lo = 0, hi = n - 1;
-              for (;;) {
-                while (lo < hi && RUN(lo) != 0xffffu) lo++;
-                while (hi > lo && RUN(hi) == 0xffffu) hi--;
-                if (lo >= hi) break;
-                RUN(lo) = RUN(hi); RUN(hi) = 0xffffu;
-              }
+          // a walk over the list for every extraction, with the clamped keys (the box is empty)
+          low = 0; from_list = true;
+          // slack of a queued request: ttft_slo - (start - arrival) - E_p(prompt_len) = base - start
+          auto key_of = [&](uint32_t wd, int64_t base) -> uint64_t {
+            const int64_t sl = base != BASE_UNBOUNDED ? dev_clamp_slack(base - start) : HFX_SLACK_MAX;
+            return ((uint64_t)ROW_PRIO(wd) << 40) | (uint64_t)(sl + (INT64_C(1) << 39));
+          };
+          while (room()) {
+            uint64_t bk = ~0ull;
+            uint32_t bid = ~0u;
+            int bs = -1;
+            int32_t lmin = INT32_MAX;
+            for (int s = lane; s < nq; s += 32) {
+              const uint16_t i = s_q[s];
+              if (i == 0xffffu) continue;
+              const uint32_t wd = s_word[i];
+              lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
+              if (!within((p.first_fit ? adm_cost : 0) + ROW_PROMPT(wd))) continue;
+              const uint64_t k = key_of(wd, s_slot[i]);
+              const uint32_t id = (uint32_t)__ldg(a.req_id + b + i) ^ 0x80000000u;
+              if (k < bk || (k == bk && id < bid)) { bk = k; bid = id; bs = s; }
             }
-            n -= k;
+            min_prompt = (int32_t)__reduce_min_sync(FULL, (uint32_t)lmin);
+            // the smallest key (46 bits: the upper 32, then the lower 14), then the lowest id
+            const uint32_t top = __reduce_min_sync(FULL, bs >= 0 ? (uint32_t)(bk >> 14) : ~0u);
+            bool cand = bs >= 0 && (uint32_t)(bk >> 14) == top;
+            const uint32_t low14 = __reduce_min_sync(FULL, cand ? (uint32_t)bk & 0x3fffu : ~0u);
+            cand = cand && ((uint32_t)bk & 0x3fffu) == low14;
+            const uint32_t least = __reduce_min_sync(FULL, cand ? bid : ~0u);
+            const uint32_t win = __ballot_sync(FULL, cand && bid == least);
+            if (win == 0) break;              // no eligible request left
+            const int slot = __shfl_sync(FULL, bs, __ffs(win) - 1);
+            const int i = s_q[slot];
+            const int32_t pr = ROW_PROMPT(s_word[i]);
+            if (!within(adm_cost + pr)) break;
+            __syncwarp();
+            if (lane == 0) { s_q[slot] = 0xffffu; park(adm_cnt, i); atomicSub(&s_cq[ROW_CLS(s_byte[i])], 1); }
+            __syncwarp();
+            adm_cost += pr; adm_cnt += 1;
           }
-          const int na = S.na, q0 = S.nq;
-          for (int e = na - 1; e >= 0; e--) {      // from the last parked row down: the list grows towards them and may take
-            const int i = s_q[q0 + e];              // the place of a row already read, never of one still to be read
-            if ((s_byte[i] >> 6) == HFX_RUNNING) RUN(n++) = (uint16_t)i;
+        }
+        // the list closes up over the places of the admitted requests
+        if (from_list) {
+          __syncwarp();
+          int to = low;
+          for (int s0 = low; s0 < nq; s0 += 32) {
+            const uint16_t v = s0 + lane < nq ? s_q[s0 + lane] : (uint16_t)0xffffu;
+            const uint32_t vm = __ballot_sync(FULL, v != 0xffffu);
+            if (v != 0xffffu) s_q[to + __popc(vm & lt)] = v;      // (never beyond the places read so far)
+            to += __popc(vm);
+            __syncwarp();
           }
-          S.nr = n;
+          nq = to;
         }
-        S.mat = S.mat_next;
-        S.arrived = 0; S.no = 0; S.na = 0; S.n_holes = 0; S.d_kv = 0;      // for the next iteration
-        if (S.worked) S.now = t2;
-        else {
-          int64_t ev = HFX_INF;
-          if (S.plan.mat > S.plan.now) ev = S.plan.mat;
-          int h = S.head;
-          while (h < m && ROW_PRIO(s_word[h]) == ROW_INVALID_PRIO) h++;     // rows with bad data never arrive
-          if (h < m && s_arr[h] < ev) ev = s_arr[h];
-          if (ev == HFX_INF) S.stop = 1; else S.now = ev;
-        }
+        if (nq == 0 && box == 0) min_prompt = INT32_MAX;
       }
-      __syncthreads();
-      if (S.stop) break;
-      executed++;
+
+      // ---- a stretch of iterations in which nothing arrives, finishes or is admitted -------------------------
+      if (adm_cnt == 0 && nr > 0 && it < next_fin) {
+        const int64_t j1 = lane + 1, grow = d2 * nr;
+        const int64_t at = now + j1 * e_d + grow * (j1 * lane / 2);          // the clock after j1 of them
+        const int32_t left = (a.iters < next_fin ? a.iters : next_fin) - it; // iterations that may still be plain
+        // iteration it + j1 is plain too?  (an oversize arrival tightened this iteration's budget: look again at the next one)
+        const bool more = j1 < left && at < next_arr && (now >= mat || at < mat) && !over_any;
+        const uint32_t plain = __ballot_sync(FULL, more);
+        const int steps = (plain | 0x80000000u) == FULL ? 32 : __ffs((int)~plain);      // this iteration and the run of plain ones behind it
+        now = __shfl_sync(FULL, at, steps - 1);
+        sum_kv += (int64_t)nr * steps;
+        it += steps;
+        continue;
+      }
+
+      // ---- 4. maturity and the iteration's clock -------------------------------------------------------------
+      const int64_t lp = adm_cnt > 0 ? dev_Ep(p, adm_cost) : 0;
+      const int64_t t1 = now + lp, t2 = t1 + e_d;
+      if (adm_cnt > 0) {
+        ReplicaPlan pl;
+        pl.now = now; pl.mat = mat; pl.mode = HFX_COLOCATED; pl.n_run = nr; pl.sum_kv = sum_kv; pl.n_eff = nr; pl.tpot_eff = min_tpot; pl.e_d = e_d;
+        int64_t lp_ = 0;
+        mat = dev_maturity_next(p, pl, adm_cnt, adm_cost, 0, &lp_);
+      }
+      const bool worked = adm_cnt > 0 || nr > 0;
+      bool run_changed = false;
+
+      // ---- 5. commit ---------------------------------------------------------------------------------------------
+      // running batch: one more token each; a request finishes when gen + 1 reaches output_len.  Finished ones leave the
+      // list, which is closed up in place.
+      sum_kv += nr;
+      if (it >= next_fin) {
+        int kept = 0;
+        int32_t nf = INT32_MAX;
+        for (int s0 = 0; s0 < nr; s0 += 32) {
+          const int s = s0 + lane;
+          const bool in = s < nr;
+          const int i = in ? RUN(s) : 0;
+          const int64_t slot = in ? s_slot[i] : 0;
+          const int32_t fin = (int32_t)(uint32_t)slot;
+          const bool done = in && it >= fin;
+          int64_t ctx = 0;
+          if (done) {
+            const uint32_t cls = ROW_CLS(s_byte[i]);
+            s_byte[i] = ROW_BYTE(cls, HFX_DONE);
+            a.finish[(int64_t)b + i] = t2;
+            atomicSub(&s_cr[cls], 1);
+            ctx = (int64_t)ROW_PROMPT(s_word[i]) + (it - (int32_t)(slot >> 32));      // leaves with the context it has after this step
+          }
+          const uint32_t dm = __ballot_sync(FULL, done), km = __ballot_sync(FULL, in && !done);
+          if (dm) sum_kv -= (int64_t)__reduce_add_sync(FULL, (uint32_t)ctx & 0xffffu) + ((int64_t)__reduce_add_sync(FULL, (uint32_t)(ctx >> 16)) << 16);
+          if (in && !done) {
+            RUN(kept + __popc(km & lt)) = (uint16_t)i;      // (never beyond the places read so far)
+            nf = fin < nf ? fin : nf;
+          }
+          kept += __popc(km);
+          __syncwarp();
+        }
+        nr = kept;
+        next_fin = (int32_t)__reduce_min_sync(FULL, (uint32_t)nf);
+        run_changed = true;
+      }
+      // admitted requests: first token at t1; those that go on decoding join the running list
+      if (adm_cnt > 0) {
+        int32_t nf = INT32_MAX;
+        for (int e0 = 0; e0 < adm_cnt; e0 += 32) {
+          const bool here = e0 + lane < adm_cnt;
+          const int i = here ? parked(e0 + lane) : 0;
+          bool goes_on = false;
+          uint32_t kv = 0;
+          if (here) {
+            const int32_t ol = __ldg(a.output_len + b + i);
+            const uint32_t cls = ROW_CLS(s_byte[i]);
+            a.first_token[(int64_t)b + i] = t1;
+            if (ol <= 1) { s_byte[i] = ROW_BYTE(cls, HFX_DONE); a.finish[(int64_t)b + i] = t1; }
+            else {
+              goes_on = true;
+              s_byte[i] = ROW_BYTE(cls, HFX_RUNNING);
+              atomicAdd(&s_cr[cls], 1);
+              const int32_t fin = it + (ol < SIM_OUTLEN_CAP ? ol : SIM_OUTLEN_CAP) - 1;
+              s_slot[i] = (int64_t)(uint32_t)fin | ((int64_t)it << 32);
+              nf = fin < nf ? fin : nf;
+              kv = (uint32_t)ROW_PROMPT(s_word[i]);
+            }
+          }
+          const uint32_t gm = __ballot_sync(FULL, goes_on);
+          sum_kv += __reduce_add_sync(FULL, kv);
+          if (goes_on) RUN(nr + __popc(gm & lt)) = (uint16_t)i;
+          nr += __popc(gm);
+          __syncwarp();
+        }
+        nf = (int32_t)__reduce_min_sync(FULL, (uint32_t)nf);
+        next_fin = nf < next_fin ? nf : next_fin;
+        run_changed = true;
+        min_ttft = strictest_q();
+      }
+      if (run_changed) {
+        __syncwarp();
+        uint32_t x = lane < nc && s_cr[lane] > 0 ? rp0 : (uint32_t)nc;
+        if (lane + 32 < nc && s_cr[lane + 32] > 0) x = rp1 < x ? rp1 : x;
+        min_tpot = s_tpot[__reduce_min_sync(FULL, x)];
+      }
+
+      // ---- 6. the clock --------------------------------------------------------------------------------------------
+      if (worked) now = t2;
+      else {                                  // idle: to the next event; without one the trace is over
+        int64_t ev = mat > now ? mat : HFX_INF;
+        ev = next_arr < ev ? next_arr : ev;
+        if (ev == HFX_INF) break;
+        now = ev;
+      }
+      it++;
     }
+    const int executed = it;
 
     // ---- per-request outputs and per-trace metrics ------------------------------------------
-    __syncthreads();
-    const int64_t now_final = S.now;
-    int fin = 0, rej = 0, att = 0;
-    for (int i = tid; i < m; i += SIM_THREADS) {
+    __syncwarp();
+    int fin = 0, rej = 0, att = 0, n_ttft = 0;
+    uint32_t bad = 0;
+    for (int i0 = 0; i0 < m; i0 += 32) {
+      const int i = i0 + lane;
       const int64_t g = (int64_t)b + i;
-      const int st = ROW_STATE(s_byte[i]);
-      const bool valid = ROW_PRIO(s_word[i]) != ROW_INVALID_PRIO;
-      const uint32_t cls = ROW_CLS(s_byte[i]);
-      const int32_t outlen = a.output_len[g];
-      int32_t gen = 0;
-      int64_t first = -1, last = -1;
-      if (st == HFX_RUNNING || st == HFX_DONE) {
-        first = a.first_token[g];
-        if (st == HFX_DONE) { gen = outlen > 1 ? outlen - 1 : 0; last = a.finish[g]; }
-        else {
-          const int admit_it = (int32_t)s_arr[i] - (outlen < SIM_OUTLEN_CAP ? outlen : SIM_OUTLEN_CAP) + 1;
-          gen = executed - 1 - admit_it;
-          last = gen > 0 ? now_final : first;
+      int64_t ttft = -1;
+      if (i < m) {
+        const uint32_t byte = s_byte[i], cls = a.class_id[g];
+        const int st = ROW_STATE(byte);
+        const int32_t prompt = a.prompt_len[g], outlen = a.output_len[g];
+        if (cls >= (uint32_t)nc) bad |= HFX_ST_BAD_CLASS;
+        if (prompt < 0 || prompt > HFX_MAX_TOKENS) bad |= HFX_ST_BAD_LEN;
+        int32_t gen = 0;
+        int64_t first = -1, last = -1;
+        if (st == HFX_RUNNING || st == HFX_DONE) {
+          first = a.first_token[g];
+          ttft = first - a.arrival[g];
+          if (st == HFX_DONE) {
+            gen = outlen > 1 ? outlen - 1 : 0; last = a.finish[g];
+            fin++;
+            const int64_t tp = outlen > 1 ? (last - first) / (outlen - 1) : 0;
+            const int64_t ttft_slo = c_ttft[cls], tpot_slo = c_tpot[cls];
+            if ((ttft_slo <= 0 || ttft <= ttft_slo) && (tpot_slo <= 0 || tp <= tpot_slo)) att++;
+          } else {
+            gen = executed - 1 - (int32_t)(s_slot[i] >> 32);
+            last = gen > 0 ? now : first;
+          }
+        } else {
+          a.first_token[g] = -1;
+          if (st == HFX_REJECTED) rej++;
         }
         a.last_token[g] = last;
+        if (st != HFX_DONE) a.finish[g] = -1;
+        a.state[g] = (uint8_t)st;
+        a.gen[g] = gen;
       }
-      a.state[g] = (uint8_t)st;
-      a.gen[g] = gen;
-      const int64_t arr = a.arrival[g];      // (the shared-memory slot holds other things by now)
-      int64_t ttft = -1;
-      if (valid) {
-        if (st == HFX_REJECTED) rej++;
-        if (st == HFX_RUNNING || st == HFX_DONE) ttft = first - arr;
-        if (st == HFX_DONE) {
-          fin++;
-          const int64_t tp = outlen > 1 ? (last - first) / (outlen - 1) : 0;
-          const int64_t ttft_slo = p.ttft[cls], tpot_slo = p.tpot[cls];
-          if ((ttft_slo <= 0 || ttft <= ttft_slo) && (tpot_slo <= 0 || tp <= tpot_slo)) att++;
-        }
-      }
-      s_arr[i] = ttft;     // park the TTFT sample; negative = none
+      // the TTFT samples, closed up over the slots of rows already looked at (their order does not matter)
+      const uint32_t sm = __ballot_sync(FULL, ttft >= 0);
+      if (ttft >= 0) s_slot[n_ttft + __popc(sm & lt)] = ttft;
+      n_ttft += __popc(sm);
+      __syncwarp();
     }
-    fin = (int)warp_sum_i64(fin); rej = (int)warp_sum_i64(rej); att = (int)warp_sum_i64(att);
-    if (lane == 0) { atomicAdd(&S.n_fin, fin); atomicAdd(&S.n_rej, rej); atomicAdd(&S.n_att, att); }
-    __syncthreads();
-    // Compact the samples (their order is irrelevant before the sort), sort, take the ranks; then the
-    // same array takes the TPOT samples.  The arrays are small: one thread compacts serially.
-    if (tid == 0) { int k = 0; for (int i = 0; i < m; i++) { const int64_t v = s_arr[i]; if (v >= 0) s_arr[k++] = v; } S.n_a = k; }
-    __syncthreads();
-    const int na = S.n_a;
-    sort_i64(s_arr, na);
-    if (tid == 0) { S.t1 = nearest_rank(s_arr, na, 50); S.t2 = nearest_rank(s_arr, na, 99); }
-    __syncthreads();
-    for (int i = tid; i < m; i += SIM_THREADS) {
+    if (bad) atomicOr(status, bad);
+    fin = (int)__reduce_add_sync(FULL, (uint32_t)fin); rej = (int)__reduce_add_sync(FULL, (uint32_t)rej); att = (int)__reduce_add_sync(FULL, (uint32_t)att);
+    const int64_t ttft50 = warp_percentile(s_slot, n_ttft, 50, s_bins, lane), ttft99 = warp_percentile(s_slot, n_ttft, 99, s_bins, lane);
+    __syncwarp();
+    int n_tpot = 0;
+    for (int i0 = 0; i0 < m; i0 += 32) {
+      const int i = i0 + lane;
       const int64_t g = (int64_t)b + i;
       int64_t tpot = -1;
-      if (ROW_STATE(s_byte[i]) == HFX_DONE && ROW_PRIO(s_word[i]) != ROW_INVALID_PRIO) {
+      if (i < m && ROW_STATE(s_byte[i]) == HFX_DONE) {
         const int32_t outlen = a.output_len[g];
         if (outlen > 1) tpot = (a.finish[g] - a.first_token[g]) / (outlen - 1);
       }
-      s_arr[i] = tpot;
+      const uint32_t sm = __ballot_sync(FULL, tpot >= 0);
+      if (tpot >= 0) s_slot[n_tpot + __popc(sm & lt)] = tpot;
+      n_tpot += __popc(sm);
     }
-    __syncthreads();
-    if (tid == 0) { int k = 0; for (int i = 0; i < m; i++) { const int64_t v = s_arr[i]; if (v >= 0) s_arr[k++] = v; } S.n_b = k; }
-    __syncthreads();
-    const int nb = S.n_b;
-    sort_i64(s_arr, nb);
-    if (tid == 0) {
+    __syncwarp();
+    const int64_t tpot50 = warp_percentile(s_slot, n_tpot, 50, s_bins, lane), tpot99 = warp_percentile(s_slot, n_tpot, 99, s_bins, lane);
+    if (lane == 0) {
       a.iters_executed[j] = executed;
-      a.finished[j] = S.n_fin;
-      a.rejected[j] = S.n_rej;
-      a.attained[j] = S.n_att;
-      a.ttft_p50[j] = S.t1;
-      a.ttft_p99[j] = S.t2;
-      a.tpot_p50[j] = nearest_rank(s_arr, nb, 50);
-      a.tpot_p99[j] = nearest_rank(s_arr, nb, 99);
-      if (a.now_out) a.now_out[j] = now_final;
+      a.finished[j] = fin; a.rejected[j] = rej; a.attained[j] = att;
+      a.ttft_p50[j] = ttft50; a.ttft_p99[j] = ttft99; a.tpot_p50[j] = tpot50; a.tpot_p99[j] = tpot99;
+      if (a.now_out) a.now_out[j] = now;
     }
+    __syncwarp();
   }
 }
 
 int hfx_sim_configure() {
-  if (cudaFuncSetAttribute(k_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * SIM_BYTES_PER_ROW + (int)SIM_CLASS_BYTES(HFX_MAX_CLASSES)) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * (SIM_BYTES_PER_ROW + 2) + (int)SIM_HEAD_BYTES(HFX_MAX_CLASSES)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536 * 2 + (int)SIM_HEAD_BYTES(HFX_MAX_CLASSES)) != cudaSuccess)
     return HFX_E_CUDA;
   return HFX_OK;
 }
@@ -509,19 +712,22 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   a.iters_executed = o->iters_executed; a.finished = o->finished; a.rejected = o->rejected; a.attained = o->attained;
   a.ttft_p50 = o->ttft_p50_ns; a.ttft_p99 = o->ttft_p99_ns; a.tpot_p50 = o->tpot_p50_ns; a.tpot_p99 = o->tpot_p99_ns;
   a.now_out = o->now_ns;
-  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, class_bytes = SIM_CLASS_BYTES(s->p.n_classes);
+  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = (size_t)cap * 2 + SIM_HEAD_BYTES(s->p.n_classes);
+  const size_t sm_bytes = 227 * 1024, block_bytes = 1024;      // (1 KB per block is reserved)
   if (cudaMemsetAsync(d_work_counter, 0, sizeof(uint32_t), s->stream) != cudaSuccess) return HFX_E_CUDA;
-  if (cap <= SIM_SMEM_ROWS) {
-    int per_sm = (int)((224 * 1024) / (rows_bytes + class_bytes + 1792));      // (static shared memory and the per-block reserve)
-    if (per_sm < 1) per_sm = 1;
-    if (per_sm > 8) per_sm = 8;
+  int per_sm = cap <= SIM_SMEM_ROWS ? (int)(sm_bytes / (rows_bytes + list_bytes + block_bytes)) : 0;
+  if (per_sm > 32) per_sm = 32;
+  int per_sm_scratch = (int)(sm_bytes / (list_bytes + block_bytes));
+  if (per_sm_scratch > SIM_SCRATCH_PER_SM) per_sm_scratch = SIM_SCRATCH_PER_SM;
+  // rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would
+  if (per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch)) {
     int grid = s->n_sm * per_sm;
     if (grid > n_traces) grid = n_traces;
     KernelScope ks(s, KSLOT_SIM);
-    k_sim<false><<<grid, SIM_THREADS, rows_bytes + class_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
+    k_sim<false><<<grid, 32, rows_bytes + list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
   } else {
-    // long traces: the rows of every resident block in a scratch buffer (two blocks per SM), allocated when first needed
-    int grid = s->n_sm * 2;
+    // the rows of every resident block in a scratch buffer, allocated when first needed
+    int grid = s->n_sm * per_sm_scratch;
     if (grid > n_traces) grid = n_traces;
     const size_t need = rows_bytes * (size_t)grid;
     if (s->sim_scratch_bytes < need) {
@@ -532,7 +738,7 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
       s->sim_scratch_bytes = need;
     }
     KernelScope ks(s, KSLOT_SIM);
-    k_sim<true><<<grid, SIM_THREADS, class_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
+    k_sim<true><<<grid, 32, list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
   }
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }

@@ -1140,3 +1140,20 @@ def test_simulator_every_row_live_at_once(m):
     wl = make_wl(rows, [(200 * MS, 30 * MS, 0), (1000 * MS, 50 * MS, 1)], replicas=[(gen.COLOCATED, 8192, 0)] * 2, now=[0, 0],
                  maturity=[0, 0], trace_off=[0, m, 2 * m], sim_iters=600)
     assert_sim_parity(wl)
+
+
+@pytest.mark.parametrize("m,first_fit", [(31, False), (32, True), (33, False), (64, False), (65, True), (700, False), (1500, True)])
+def test_simulator_windows_merge_and_many_are_admitted_at_once(m, first_fit):
+    # Rows wait in a window of 32 before they join the sorted queue: arrivals in clumps, most of them with equal slack
+    # bases (unbounded, or equal arrival and prompt: ties by a permuted request id), 64 classes, and an idle spell followed by
+    # one-token prompts of which more than 512 fit one budget.
+    rng = np.random.default_rng(m)
+    arr = np.sort(rng.choice([0, 1, 40 * MS, 41 * MS, 900 * MS], m))
+    ids = rng.permutation(m)
+    rows = [dict(prompt_len=int(rng.choice([1, 1, 1, 64, 700])) if arr[i] == 900 * MS else int(rng.choice([64, 64, 300, 3000])), arrival_ns=int(arr[i]),
+                 output_len=int(rng.integers(1, 9)), class_id=int(rng.choice([0, 1, 2, 63])), req_id=int(ids[i])) for i in range(m)]
+    classes = [(200 * MS, 30 * MS, 0), (0, 0, 1), (1000 * MS, 50 * MS, 1)] + [(5000 * MS + c, 100 * MS + c, c % 63) for c in range(61)]
+    wl = make_wl(rows, classes, replicas=[(gen.COLOCATED, 8192, 0)], trace_off=[0, m], sim_iters=4000)
+    if first_fit:
+        wl.meta["first_fit"] = True
+    assert_sim_parity(wl)

@@ -100,7 +100,8 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
   ok = ok && cudaMalloc(&s->d_cursor, sizeof(uint32_t) * 2 * R2) == cudaSuccess;
   ok = ok && cudaMalloc(&s->d_act_count, sizeof(uint32_t) * R2) == cudaSuccess;
   ok = ok && cudaMalloc(&s->d_rowflag, (size_t)max_rows + 16) == cudaSuccess;
-  ok = ok && cudaMalloc(&s->d_flags, 256) == cudaSuccess;
+  ok = ok && cudaMalloc(&s->d_flags, 256 + hfx_attainment_workspace_bytes()) == cudaSuccess;
+  if (ok) s->d_att = reinterpret_cast<unsigned long long *>(s->d_flags + 64);
   {
     // the tile front end: slabs for every tile of the largest table, one matrix row per tile
     int32_t tile_rows = 0, n_tiles = 0;
@@ -134,6 +135,8 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
     memcpy(h->h_cfg, replicas, sizeof(hfx_replica_cfg) * n_replicas);
     ok = ok && cudaMemcpy(s->d_cfg, replicas, sizeof(hfx_replica_cfg) * n_replicas, cudaMemcpyHostToDevice) == cudaSuccess;
     ok = ok && cudaMemset(s->d_status, 0, 256) == cudaSuccess;
+    ok = ok && cudaMemset(s->d_att, 0, hfx_attainment_workspace_bytes()) == cudaSuccess;
+    ok = ok && cudaMemset(s->d_slo, 0xff, hfx_slomap_workspace_bytes()) == cudaSuccess;
     {
       std::vector<uint8_t> modes((size_t)n_replicas);
       for (int r = 0; r < n_replicas; r++) modes[r] = (uint8_t)replicas[r].mode;

@@ -119,7 +119,9 @@ struct hfx_sched {
   void *dispatch_ws;                   // workspace of hfx_dispatch_step, allocated by its first call
   unsigned char *d_sim_scratch;        // rows of long traces in hfx_sim_run (allocated by the first call that needs it)
   size_t sim_scratch_bytes;
+  unsigned long long *d_att;           // totals of hfx_attainment, zero between its calls (in the allocation of d_flags)
   void *d_slo;                         // per-priority table of hfx_slo_map
+  uint32_t slo_parity;                 // which copy of its first rows the next call uses
   void *d_pd;                          // moved counter, wake-up times and busy flags of hfx_pd_migrate
 };
 
@@ -540,6 +542,7 @@ size_t hfx_slomap_workspace_bytes();
 int hfx_launch_pd_migrate(hfx_sched *s, const hfx_table *t, int32_t *replica_id, int64_t *now, const int32_t *pair, int64_t x0,
                           int64_t x1, int32_t *n_moved);
 size_t hfx_pd_workspace_bytes(int n_replicas);
+size_t hfx_attainment_workspace_bytes();
 int hfx_launch_attainment(hfx_sched *s, const hfx_table *t, int64_t *out);
 int hfx_launch_fleet_apply(hfx_sched *s, int64_t now, const int32_t *decision, const int64_t *used_blocks,
                            const int64_t *cold, const hfx_fleet *f, int64_t *clock, int64_t *maturity, int64_t *cost);

@@ -1157,3 +1157,25 @@ def test_simulator_windows_merge_and_many_are_admitted_at_once(m, first_fit):
     if first_fit:
         wl.meta["first_fit"] = True
     assert_sim_parity(wl)
+
+
+@pytest.mark.parametrize("n_classes", [1, 4, 5, 8, 9, 64])
+def test_attainment_class_counts_and_ragged_rows(n_classes):
+    # totals in registers (up to 4, up to 8 classes) and per warp (more); a row is left over when n is odd
+    for n in (1, 2, 511, 40_003):
+        wl = gen.random_table(n_classes, n, 3, n_classes=n_classes, done=0.6, future=0.1, inflight=0.2)
+        wl.table["class_id"][::11] = 64          # out of range: left out and flagged
+        done = wl.table["state"] == gen.DONE
+        wl.table["finish_ns"][done] = wl.table["last_token_ns"][done] = wl.table["first_token_ns"][done] + 50 * MS * (wl.table["output_len"][done] - 1)
+        _attainment_parity(wl)
+
+
+@pytest.mark.parametrize("w", [31, 32, 33, 128, 129, 4096])
+def test_slo_mapping_largest_values_and_tied_windows(w):
+    # ranks are counted, ties by position: equal values, the largest 64-bit value beside bad records
+    rng = np.random.default_rng(w)
+    big = np.iinfo(np.int64).max
+    win = {"prio": rng.integers(-1, 4, w), "ttft": rng.choice([5, 7, big], w), "tpot": rng.choice([-3, 0, big], w), "queue": rng.integers(0, 10**6, w)}
+    bounds = {k: np.full(3, v, np.int64) for k, v in (("ttft_min", -10), ("ttft_max", big), ("ttft_min_relaxed", -20), ("tpot_min", -10), ("tpot_max", big),
+                                                      ("tpot_min_relaxed", -20))}
+    _slo_parity(3, win, bounds, np.zeros(3, np.int64), np.array([0, 1, 0]), rng.integers(0, 3, 2500))

@@ -300,7 +300,7 @@ typedef struct hfx_dispatch_out {
  * RUNNING; binding it (replica_id := assign) puts it in flight on the D
  * instance.  DECODE replicas also keep their own queue (QUEUED rows bound to
  * them, e.g. by hfx_pd_migrate), which hfx_sched_step serves.
- * The scheduler may have at most 4096 replicas.  The first call allocates the call's workspace (44 bytes
+ * The scheduler may have at most 4096 replicas.  The first call allocates the call's workspace (52 bytes
  * per row of max_rows) with cudaMalloc, so it should not be made inside a
  * stream capture; hfx_sched_destroy frees it.
  * Errors: HFX_E_ARG, HFX_E_ALIGN, HFX_E_CAPACITY, HFX_E_NOMEM, HFX_E_CUDA. */

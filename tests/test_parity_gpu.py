@@ -1179,3 +1179,38 @@ def test_slo_mapping_largest_values_and_tied_windows(w):
     bounds = {k: np.full(3, v, np.int64) for k, v in (("ttft_min", -10), ("ttft_max", big), ("ttft_min_relaxed", -20), ("tpot_min", -10), ("tpot_max", big),
                                                       ("tpot_min_relaxed", -20))}
     _slo_parity(3, win, bounds, np.zeros(3, np.int64), np.array([0, 1, 0]), rng.integers(0, 3, 2500))
+
+
+@pytest.mark.parametrize("shape", ["crowded", "equal", "long runs", "capped", "wide costs"])
+@pytest.mark.parametrize("n", [4095, 4097, 30_011])
+def test_dispatch_order_and_walk_edges(n, shape):
+    # The queue is ordered by bins from a sample (radix passes when a bin is too full) and walked in windows of 256 entries of
+    # chunks of 4096: slacks crowded beside an outlier, equal slacks (ties by a permuted id), runs longer than a window and
+    # across chunks, batch caps, budgets and totals beyond 32 bits.
+    rng = np.random.default_rng(n)
+    R = 40
+    wl = gen.random_table(n, n, R, modes=(gen.COLOCATED,), n_classes=3, token_cap=16384, batch_cap=5 + n // 1000 if shape == "capped" else 0, inflight=0.02, done=0.0, future=0.05,
+                          budget_mode=gen.BUDGET_SAFE if shape == "capped" else gen.BUDGET_CAP_ONLY)
+    now = int(wl.now.max())
+    wl.maturity[:] = now - rng.integers(0, 5, R)
+    q = wl.table["state"] == gen.QUEUED
+    wl.table["prompt_len"][:] = 16
+    if shape == "crowded":
+        wl.table["arrival_ns"][q] = now - 10**9 - rng.integers(0, 2000, int(q.sum()))
+        wl.table["arrival_ns"][np.nonzero(q)[0][:2]] = [now - 10**12, now]
+    elif shape == "equal":
+        wl.classes = [(0, 30 * MS, 1)] * 3
+    elif shape == "capped":
+        wl.table["prompt_len"][:] = rng.choice([0, 16, 200], n)
+    elif shape == "wide costs":      # a D stage whose entries cost hundreds of seconds of decode time
+        wl.model = (0, 1, 0, 1, 1 << 30, 1 << 8)
+        wl.classes = [(0, 0, 0), (0, 1 << 34, 1), (0, 0, 2)]
+        wl.replicas[:20, 0] = gen.PREFILL
+        wl.replicas[20:, 0] = gen.DECODE
+        r = rng.random(n) < 0.8
+        wl.table["state"][r] = gen.RUNNING
+        wl.table["replica_id"][r] = rng.integers(0, 20, int(r.sum()))
+        wl.table["first_token_ns"][:] = now - 10**9 - np.arange(n)
+        wl.table["prompt_len"][:] = rng.integers(1, 1 << 16, n)
+    g = assert_dispatch_parity(wl, now, calls=2)
+    assert g["adm_count"].sum() > 0

@@ -22,13 +22,13 @@
                                     // whole tile that larger groups need costs as much as groups of about a thousand rows)
 #define FRONT_TAIL_MAX 64           // more rows bound to no replica than this are ranked by a scan
 #define FRONT_ROW_BYTES 24          // shared memory per row of the tile
-#define FRONT_REP_BYTES 31          // shared memory per replica
 
 // shared memory of the tile kernel
 __host__ __device__ inline size_t front_smem_bytes(int R1, int T) {
   size_t b = 16 * (size_t)T;                       // s_rec
   b += 16 * (size_t)R1;                            // s_now, s_start
   b += 8 * (size_t)R1;                             // s_cnt
+  if (R1 <= HFX_NEXT_REPLICAS_MAX + 1) b += 8 * (size_t)R1;      // s_next
   b += 4 * (size_t)T;                              // s_bkt
   b += 4 * (size_t)R1 + 2 * (size_t)R1;            // s_base, s_offact
   b += 2 * 2 * ((size_t)T + 8);                    // s_perm, s_fin
@@ -59,7 +59,9 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
   uint4 *s_rec = reinterpret_cast<uint4 *>(smem_raw);                    // [T]    record of every active row, by local index
   int64_t *s_now = reinterpret_cast<int64_t *>(s_rec + T);               // [R1]
   int64_t *s_start = s_now + R1;                                         // [R1]   earliest start max(now, maturity)
-  uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_start + R1);          // [2 R1] rows per group = (replica, active / inactive)
+  const bool has_next = a.next != nullptr;
+  long long *s_next = reinterpret_cast<long long *>(s_start + R1);       // [R1]   earliest arrival that is still to come (if has_next)
+  uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_next + (has_next ? R1 : 0));      // [2 R1] rows per group = (replica, active / inactive)
   uint32_t *s_bkt = s_cnt + 2 * R1;                                      // [T]    replica bucket | 0x8000 if active | arrival rank in the group << 16
   uint16_t *s_base = reinterpret_cast<uint16_t *>(s_bkt + T);            // [2 R1] first slot of each group in slab_idx order
   uint16_t *s_offact = s_base + 2 * R1;                                  // [R1]   first slot of the replica's records in slab_rec
@@ -105,6 +107,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     s_now[i] = nw; s_start[i] = nw > mt ? nw : mt;
     s_mode[i] = i < R ? a.mode[i] : 0;
     s_cnt[2 * i] = 0; s_cnt[2 * i + 1] = 0;
+    if (has_next) s_next[i] = HFX_INF;
   }
   if (blockIdx.x == 0) {      // re-arm what the next step accumulates into
     for (int i = tid; i < R1; i += blockDim.x) a.tot_next[i] = 0ull;
@@ -147,6 +150,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
                              (uint32_t)prompt | (kind << CREC_KIND_SHIFT) | ((uint32_t)prio << CREC_PRIO_SHIFT),
                              (uint32_t)gen | (cls << CREC_CLS_SHIFT));
     }
+    if (kind == KIND_FUTURE && has_next && arrival < s_next[bkt]) atomicMin(&s_next[bkt], (long long)arrival);      // (mostly the look alone)
     const uint32_t g = 2u * (uint32_t)bkt + (act ? 0u : 1u);
     s_bkt[il] = (uint32_t)bkt | (act ? 0x8000u : 0u) | (atomicAdd(&s_cnt[g], 1u) << 16);
     return kind;
@@ -178,7 +182,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     longlong2 *slp = reinterpret_cast<longlong2 *>(a.slack) + 2 * gv;
     slp[0] = make_longlong2(sl[0], sl[1]); slp[1] = make_longlong2(sl[2], sl[3]);
     reinterpret_cast<uchar4 *>(a.admit)[gv] = make_uchar4(kd[0] == KIND_RUNNING, kd[1] == KIND_RUNNING, kd[2] == KIND_RUNNING, kd[3] == KIND_RUNNING);
-    reinterpret_cast<uchar4 *>(a.rowflag)[gv] = make_uchar4(kd[0], kd[1], kd[2], kd[3]);
+    if (!has_next) reinterpret_cast<uchar4 *>(a.rowflag)[gv] = make_uchar4(kd[0], kd[1], kd[2], kd[3]);
     if (EXTRA) {
       if (a.pred_ttft) {
         longlong2 *q = reinterpret_cast<longlong2 *>(a.pred_ttft) + 2 * gv;
@@ -207,7 +211,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
                                a.arrival[g], a.first_token[g], sl, bk, kk, pt);
     a.slack[g] = sl;
     a.admit[g] = kd == KIND_RUNNING;
-    a.rowflag[g] = (uint8_t)kd;
+    if (!has_next) a.rowflag[g] = (uint8_t)kd;
     if (EXTRA) {
       if (a.pred_ttft) a.pred_ttft[g] = pt;
       if (a.pred_tpot) a.pred_tpot[g] = 0;
@@ -239,6 +243,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
       const uint32_t off_all = run & 0xffffu, off_act = run >> 16;
       s_base[2 * i] = (uint16_t)off_all; s_base[2 * i + 1] = (uint16_t)(off_all + cA); s_offact[i] = (uint16_t)off_act;
       mrow[i] = make_uint2(off_all | ((cA + cI) << 16), off_act | (cA << 16));
+      if (has_next) a.next[(size_t)blockIdx.x * R1 + i] = s_next[i];
       if (cA + cI) atomicAdd(a.tot + i, (unsigned long long)(cA + cI) | ((unsigned long long)cA << 32));
       run += (cA + cI) | (cA << 16);
     }
@@ -361,7 +366,7 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   hfx_front_shape(s, fa.n, &fa.tile_rows, &fa.n_tiles);
   const int R1 = s->p.n_replicas + 1;
   const uint32_t par = s->tot_parity;
-  fa.slab_rec = s->d_slab_rec; fa.slab_idx = s->d_slab_idx; fa.M = s->d_M;
+  fa.slab_rec = s->d_slab_rec; fa.slab_idx = s->d_slab_idx; fa.M = s->d_M; fa.next = s->d_next;
   fa.tot = s->d_tot + (size_t)par * (R1 + 1); fa.tot_next = s->d_tot + (size_t)(par ^ 1u) * (R1 + 1);
   fa.ordered = s->d_flags + 4 + par; fa.ordered_next = s->d_flags + 4 + (par ^ 1u);
   fa.status = s->d_status; fa.rowflag = s->d_rowflag;

@@ -80,6 +80,7 @@ enum { KSLOT_COUNT = 0, KSLOT_COLSCAN, KSLOT_OFFSETS, KSLOT_REGROUP, KSLOT_SEG_S
 #define HFX_TILE_ROWS_MAX 8192
 #define HFX_TILE_MATRIX_MAX (INT64_C(8) << 20)   // entries of the tile matrix (64 MiB)
 #define HFX_TILE_REPLICAS_MAX 4095               // replicas whose counters fit in shared memory (12-bit bucket ids)
+#define HFX_NEXT_REPLICAS_MAX 2047               // replicas up to which a tile notes the next arrival of each (8 bytes of shared memory per replica)
 #define HFX_COUNT_TILE_ROWS 4096                 // rows per block of the counting pass of the fallback front end
 
 struct HfxBracket { cudaEvent_t a, b; int slot; };
@@ -111,6 +112,7 @@ struct hfx_sched {
   uint4 *d_slab_rec;        // [tiles_max * tile_rows] records of active rows, tile-major
   uint16_t *d_slab_idx;     // [tiles_max * tile_rows] local row indices, tile-major, grouped by replica
   uint2 *d_M;               // [tiles_max][R+1] where each replica's rows sit in a tile's slabs
+  int64_t *d_next;          // [tiles_max][R+1] earliest arrival still to come of each replica in a tile (up to HFX_NEXT_REPLICAS_MAX replicas)
   unsigned long long *d_tot;// [2][R+2] rows | active rows << 32 per replica, by parity
   int32_t tiles_max;        // matrix rows allocated (0: fallback front end only)
   uint32_t tot_parity;      // which half of d_tot / which "ordered" word the next tile front end uses
@@ -507,7 +509,7 @@ struct FrontArgs {
   // per-row outputs, written in row order
   int64_t *slack; int64_t *pred_ttft; int64_t *pred_tpot; uint64_t *key; uint8_t *admit; uint8_t *rowflag;
   // the slabs
-  uint4 *slab_rec; uint16_t *slab_idx; uint2 *M; unsigned long long *tot; unsigned long long *tot_next;
+  uint4 *slab_rec; uint16_t *slab_idx; uint2 *M; int64_t *next; unsigned long long *tot; unsigned long long *tot_next;
   uint32_t *ordered; uint32_t *ordered_next; uint32_t *status;
 };
 

@@ -23,6 +23,7 @@
 #define TINY_BIN_MAX 48
 #define TINY_CLASSES 128  // (phase, priority) classes of the sort items of active rows: phase<1> | prio<6>
 #define GROUP_TPT 2       // tiles per thread and round when a group gathers
+#define LIST_WARP_MAX 512 // rows of one tile that a warp copies to a long list by itself
 #define LIST_MAX 2048     // inactive rows a replica's own threads list while they gather; longer lists are shared by the grid
 #define SMEM_MED (SEG_MED * 12)
 #define SMEM_GROUP (SMEM_MED / REP_GROUPS)
@@ -41,7 +42,7 @@ struct BlockShared {
 // where the kernel finds the rows of a replica
 struct SegCtx {
   // tile front end: slabs
-  const uint4 *slab_rec; const uint16_t *slab_idx; const uint2 *M; const unsigned long long *tot;
+  const uint4 *slab_rec; const uint16_t *slab_idx; const uint2 *M; const int64_t *next; const unsigned long long *tot;
   int32_t tile_rows, n_tiles;
   // fallback front end: contiguous records, counts and range starts
   const uint32_t *seg_count; const uint32_t *act_count; const uint32_t *seg_begin;
@@ -265,6 +266,17 @@ __device__ __forceinline__ int64_t next_arrival_slabs(const SegArgs &a, const Se
     }
   }
   return v;
+}
+
+// The earliest arrival still to come of an idle replica (my part of the minimum over the group): from the tiles' notes where
+// they are kept, else from its listed inactive rows, else from the slabs.
+__device__ __forceinline__ int64_t next_arrival_part(const SegArgs &a, const SegCtx &c, int R1, int r, uint32_t b, int64_t n_act, int64_t n, bool listed, const Grp &G) {
+  if (c.next) {
+    int64_t v = HFX_INF;
+    for (int t = G.tid; t < c.n_tiles; t += G.n) { const int64_t x = __ldcg(c.next + (size_t)t * R1 + r); v = x < v ? x : v; }
+    return v;
+  }
+  return listed ? next_arrival_listed(a, c, b, n_act, n, G.tid, G.n) : next_arrival_slabs(a, c, R1, r, G);
 }
 
 // minimum of v over the group into sh.next_arrival (all threads of the group call)
@@ -773,7 +785,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   const int64_t mat_next = sh.red_c[0];
   if (commit && !worked) {
     // idle replica: its next arrival is looked up among its listed inactive rows (unless the grid lists them later)
-    group_min_arrival(list_in || !ordered ? next_arrival_listed(a, c, b, n_act, n, G.tid, G.n) : next_arrival_slabs(a, c, R1, r, G), sh, G);
+    group_min_arrival(next_arrival_part(a, c, R1, r, b, n_act, n, list_in || !ordered, G), sh, G);
   }
   if (G.tid == 0 && real)
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
@@ -1132,7 +1144,7 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
   const int worked = sh.worked;
   const int64_t mat_next = sh.red_c[0];
   if (commit && !worked)      // idle replica: its next arrival is looked up among its listed inactive rows
-    group_min_arrival(list_in || !ordered ? next_arrival_listed(a, c, b, n_act, n, threadIdx.x, blockDim.x) : next_arrival_slabs(a, c, p.n_replicas + 1, r, B), sh, B);
+    group_min_arrival(next_arrival_part(a, c, p.n_replicas + 1, r, b, n_act, n, list_in || !ordered, B), sh, B);
   if (threadIdx.x == 0 && real)
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
 
@@ -1461,7 +1473,7 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
   const int worked = sh.worked;
   const int64_t mat_next = sh.red_c[0];
   if (commit && !worked)      // idle replica: its next arrival is looked up among its listed inactive rows
-    group_min_arrival(list_in ? next_arrival_listed(a, c, b, n_act, n, tid, REP_THREADS) : next_arrival_slabs(a, c, R + 1, r, B), sh, B);
+    group_min_arrival(next_arrival_part(a, c, R + 1, r, b, n_act, n, list_in, B), sh, B);
   if (tid == 0 && real)
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
 
@@ -1643,7 +1655,7 @@ __device__ void oversize_replica(const HfxParams &p, const SegArgs &a, const Seg
   const int worked = sh.worked;
   const int64_t mat_next = sh.red_c[0];
   if (commit && !worked)
-    group_min_arrival(list_in || !ordered ? next_arrival_listed(a, c, b, n_act, n, threadIdx.x, blockDim.x) : next_arrival_slabs(a, c, p.n_replicas + 1, r, B), sh, B);
+    group_min_arrival(next_arrival_part(a, c, p.n_replicas + 1, r, b, n_act, n, list_in || !ordered, B), sh, B);
   if (threadIdx.x == 0 && real)
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
   if (a.admitted_rows)
@@ -1765,12 +1777,13 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
   }
 
   // ---- long lists of inactive rows (ordered steps): every block lists a range of tiles ----------------
-  // The replicas with a long list are collected in shared memory; a thread per replica adds up the replica's
-  // inactive rows in the tiles before the block's, then a warp per replica copies the rows of the block's tiles.
+  // The replicas with a long list are collected in shared memory; their inactive rows in the tiles before the block's are
+  // added up, then the rows of the block's tiles are copied.
   if (longer) {
     __syncthreads();      // the larger replicas are done with the block's shared memory
     uint16_t *s_lr = reinterpret_cast<uint16_t *>(smem_raw);                                   // [R1] the replicas
     uint32_t *s_lpre = reinterpret_cast<uint32_t *>(smem_raw + (((size_t)R1 * 2 + 15) & ~(size_t)15));   // [R1] rows in earlier tiles
+    uint16_t *s_big = reinterpret_cast<uint16_t *>(s_lpre + R1);                               // [R1] those that the whole block copies
     if (tid == 0) s_scan[0] = 0;
     __syncthreads();
     for (int r = tid; r < R1; r += blockDim.x)
@@ -1781,19 +1794,28 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
     const int tA = blockIdx.x * per < c.n_tiles ? blockIdx.x * per : c.n_tiles;
     const int tB = tA + per < c.n_tiles ? tA + per : c.n_tiles;
     if (tA < tB) {
-      for (int j = tid; j < n_long; j += blockDim.x) {
-        const int r = s_lr[j];
-        uint32_t pre = 0;
+      if (n_long >= 256) {      // rows in earlier tiles: a thread per replica, neighbours side by side in memory ...
+        for (int j = tid; j < n_long; j += blockDim.x) {
+          const int r = s_lr[j];
+          uint32_t pre = 0;
 #pragma unroll 8
-        for (int t = 0; t < tA; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + r); pre += (m.x >> 16) - (m.y >> 16); }
-        s_lpre[j] = pre;
+          for (int t = 0; t < tA; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + r); pre += (m.x >> 16) - (m.y >> 16); }
+          s_lpre[j] = pre;
+        }
+      } else {                  // ... or, of few replicas, a lane per tile
+        for (int j = warp; j < n_long; j += (int)(blockDim.x >> 5)) {
+          const int r = s_lr[j];
+          uint32_t pre = 0;
+#pragma unroll 4
+          for (int t = lane; t < tA; t += 32) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + r); pre += (m.x >> 16) - (m.y >> 16); }
+          pre = __reduce_add_sync(0xffffffffu, pre);
+          if (lane == 0) s_lpre[j] = pre;
+        }
       }
+      if (tid == 0) s_scan[1] = 0;
       __syncthreads();
-      // many long lists: a warp per replica; few (one bucket of unbound rows, say): the whole block on each
-      const bool by_warp = n_long >= (int)(blockDim.x >> 5);
-      const int first = by_warp ? warp : 0, step = by_warp ? (int)(blockDim.x >> 5) : 1;
-      const uint32_t k0 = by_warp ? (uint32_t)lane : (uint32_t)tid, kstep = by_warp ? 32u : blockDim.x;
-      for (int j = first; j < n_long; j += step) {
+      // the rows themselves: a warp per replica, the whole block where a replica has many in these tiles (the bucket of unbound rows)
+      auto copy = [&](int j, uint32_t k0, uint32_t kstep) {
         const int r = s_lr[j];
         uint32_t dst = begin[r] + (uint32_t)(__ldcg(c.tot + r) >> 32) + s_lpre[j];
         for (int t = tA; t < tB; t++) {
@@ -1804,7 +1826,15 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
           for (uint32_t k = k0; k < ci; k += kstep) a.order[dst + k] = (int32_t)(tb + __ldcg(c.slab_idx + tb + src + k));
           dst += ci;
         }
+      };
+      for (int j = warp; j < n_long; j += (int)(blockDim.x >> 5)) {
+        uint32_t most = 0;      // (the same in all the lanes)
+        for (int t = tA; t < tB; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + s_lr[j]); const uint32_t ci = (m.x >> 16) - (m.y >> 16); most = ci > most ? ci : most; }
+        if (most > LIST_WARP_MAX) { if (lane == 0) s_big[atomicAdd(&s_scan[1], 1u)] = (uint16_t)j; }
+        else copy(j, (uint32_t)lane, 32u);
       }
+      __syncthreads();
+      for (uint32_t i = 0; i < s_scan[1]; i++) copy(s_big[i], (uint32_t)tid, blockDim.x);
     }
   }
 }
@@ -1821,7 +1851,7 @@ int hfx_launch_replicas(hfx_sched *s, const SegArgs &sa, int64_t n, bool slabs) 
   c.big_hi = s->d_big_hi; c.big_lo = s->d_big_lo; c.big_idx = s->d_big_lo ? s->d_big_lo + s->max_rows : nullptr;
   if (slabs) {
     const uint32_t par = s->tot_parity;
-    c.slab_rec = s->d_slab_rec; c.slab_idx = s->d_slab_idx; c.M = s->d_M;
+    c.slab_rec = s->d_slab_rec; c.slab_idx = s->d_slab_idx; c.M = s->d_M; c.next = s->d_next;
     c.tot = s->d_tot + (size_t)par * (R1 + 1);
     c.ordered = s->d_flags + 4 + par;
     hfx_front_shape(s, n, &c.tile_rows, &c.n_tiles);

@@ -1214,3 +1214,20 @@ def test_dispatch_order_and_walk_edges(n, shape):
         wl.table["prompt_len"][:] = rng.integers(1, 1 << 16, n)
     g = assert_dispatch_parity(wl, now, calls=2)
     assert g["adm_count"].sum() > 0
+
+
+@pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100)])
+def test_idle_replicas_find_their_next_arrivals(R, rows_per):
+    # Tiles note every replica's next arrival up to 2047 replicas, lists are searched beyond; lists of more than 2048 rows (a few
+    # of them, or hundreds) wait for the end of the kernel, and unbound rows that fill a tile are listed by the whole block.
+    n = R * rows_per + 5000
+    wl = gen.random_table(R, n, R, modes=(gen.COLOCATED, gen.DECODE), permute_ids=False, inflight=0.0, done=0.98, future=0.0)
+    t = wl.table
+    rng = np.random.default_rng(R)
+    now = int(wl.now.max())
+    wl.now[:] = now
+    wl.maturity[:] = now - 1
+    t["replica_id"][:] = np.concatenate([rng.permutation(np.arange(R * rows_per) % R), np.full(5000, -1)]) if rows_per > 100 else rng.integers(-1, R, n)
+    q = t["state"] == gen.QUEUED
+    t["arrival_ns"][q] = now + rng.integers(-2, 90, int(q.sum())) * MS
+    assert_step_parity(wl, steps=3, commit=True, optional=False)

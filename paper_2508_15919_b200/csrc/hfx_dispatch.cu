@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   uint64_t *s_sample = reinterpret_cast<uint64_t *>(smem_raw);                          // [DISP_SAMPLES] (before the items are there)
   int64_t *s_mat = reinterpret_cast<int64_t *>(s_sample + DISP_SAMPLES);                // [R] maturity of every instance, HFX_INF if it has not come
   uint32_t *s_wc = reinterpret_cast<uint32_t *>(smem_raw);                              // [32][256] (radix passes)
-  __shared__ int64_t s_cls_ttft[HFX_MAX_CLASSES], s_cls_tpot[HFX_MAX_CLASSES];
+  __shared__ ClassTab s_tab;
   __shared__ uint32_t s_class[DISP_CLASSES], s_r0[DISP_CLASSES + 1];      // first interval | intervals << 16; first sample
   __shared__ uint32_t s_part[33];
   __shared__ int64_t s_part64[33];
@@ -336,10 +336,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   auto place_of = [&](const uint4 &x) -> uint64_t { return (item_key(x) << 16) | ((by_id ? x.z - id_lo : x.w) >> tie_shift); };
 
   // ---- 0: instances; the sample in order -------------------------------------------------------------------------
-  for (int k = tid; k < HFX_MAX_CLASSES; k += SORT_THREADS) {
-    s_cls_ttft[k] = k < p.n_classes ? p.ttft[k] : 0;
-    s_cls_tpot[k] = k < p.n_classes ? p.tpot[k] : 0;
-  }
+  class_tab_init(p, s_tab, tid);
   for (int r = tid; r < R; r += SORT_THREADS) {
     const int64_t m = a.maturity[r];
     s_mat[r] = m <= a.now ? m : HFX_INF;
@@ -378,7 +375,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       before = __reduce_add_sync(0xffffffffu, before); first = __reduce_add_sync(0xffffffffu, first);
     }
     ReplicaPlan pl;
-    warp_plan(p, s_cls_ttft, s_cls_tpot, cfg, a.now, mat, n_run, sum_kv, mask_run, w.ctl[stage ? CTL_DMASK : CTL_QMASK], pl, lane);
+    warp_plan(p, s_tab, cfg, a.now, mat, n_run, sum_kv, mask_run, w.ctl[stage ? CTL_DMASK : CTL_QMASK], pl, lane);
     if (lane == 0) {
       w.plan[r] = pl;
       a.budget[r] = pl.budget; a.e_d[r] = pl.e_d; a.n_run[r] = (int32_t)pl.n_run; a.sum_kv[r] = pl.sum_kv;

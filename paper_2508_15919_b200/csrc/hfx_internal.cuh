@@ -224,19 +224,34 @@ __device__ inline void dev_plan(const HfxParams &p, const hfx_replica_cfg &cfg, 
 }
 
 // The same plan computed by a whole warp (all 32 lanes call with the same arguments and get the same
-// result).  The class minima are taken by lanes from a copy of the class tables in shared memory
-// (cls_ttft / cls_tpot, HFX_MAX_CLASSES entries each); the largest safe n comes from a 32-way search
+// result).  The class minima come from tables in shared memory; the largest safe n comes from a 32-way search
 // on the bound itself, E_p(n) * (2 TPOT - E_d) <= TTFT * (TPOT - E_d), compared in 128 bits: for
 // integer E_p that is the same set of n as E_p(n) <= floor(TTFT (TPOT - E_d) / (2 TPOT - E_d)), and no
 // division is needed.
-__device__ inline int64_t warp_min_over_mask(const int64_t *cls_v, uint64_t mask, int lane) {
-  int64_t m = HFX_INF;
-#pragma unroll
-  for (int c = lane; c < HFX_MAX_CLASSES; c += 32)
-    if ((mask >> c) & 1ull) { const int64_t x = cls_v[c]; if (x > 0 && x < m) m = x; }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { const int64_t w = __shfl_xor_sync(0xffffffffu, m, o); m = w < m ? w : m; }
-  return m;
+// Strictest SLO of a set of classes: every class has a rank by its bound (HFX_MAX_CLASSES: none) and the bounds are kept by
+// rank, so it is a minimum over small integers (one reduction) and a look.
+struct ClassTab {
+  int64_t ttft[HFX_MAX_CLASSES + 1], tpot[HFX_MAX_CLASSES + 1];      // by rank; the last one: unbounded
+  uint8_t rank_ttft[HFX_MAX_CLASSES], rank_tpot[HFX_MAX_CLASSES];
+};
+// (threads 0 .. HFX_MAX_CLASSES of a block; the block synchronises before use)
+__device__ __forceinline__ void class_tab_init(const HfxParams &p, ClassTab &t, int tid) {
+  if (tid == HFX_MAX_CLASSES) { t.ttft[tid] = HFX_INF; t.tpot[tid] = HFX_INF; }
+  if (tid >= HFX_MAX_CLASSES) return;
+  const int64_t a = tid < p.n_classes ? p.ttft[tid] : 0, b = tid < p.n_classes ? p.tpot[tid] : 0;
+  int ra = 0, rb = 0;
+  for (int k = 0; k < p.n_classes; k++) {
+    const int64_t x = p.ttft[k], y = p.tpot[k];
+    ra += x > 0 && (x < a || (x == a && k < tid)) ? 1 : 0;
+    rb += y > 0 && (y < b || (y == b && k < tid)) ? 1 : 0;
+  }
+  t.rank_ttft[tid] = (uint8_t)(a > 0 ? ra : HFX_MAX_CLASSES); t.rank_tpot[tid] = (uint8_t)(b > 0 ? rb : HFX_MAX_CLASSES);
+  if (a > 0) t.ttft[ra] = a;
+  if (b > 0) t.tpot[rb] = b;
+}
+__device__ __forceinline__ int64_t warp_min_over_mask(const int64_t *by_rank, const uint8_t *rank, uint64_t mask, int lane) {
+  const uint32_t x = (mask >> lane) & 1ull ? rank[lane] : HFX_MAX_CLASSES, y = (mask >> (lane + 32)) & 1ull ? rank[lane + 32] : HFX_MAX_CLASSES;
+  return by_rank[__reduce_min_sync(0xffffffffu, x < y ? x : y)];
 }
 
 // Largest n in [0, cap] with E_p(n) * den <= num (num = nh:nl as 128 bits, den > 0), 0 if none.
@@ -260,13 +275,12 @@ __device__ inline int64_t warp_nsafe(const HfxParams &p, uint64_t nh, uint64_t n
   return lo;
 }
 
-__device__ inline void warp_plan(const HfxParams &p, const int64_t *cls_ttft, const int64_t *cls_tpot,
-                                 const hfx_replica_cfg &cfg, int64_t now, int64_t mat, int64_t n_run, int64_t sum_kv,
+__device__ inline void warp_plan(const HfxParams &p, const ClassTab &tab, const hfx_replica_cfg &cfg, int64_t now, int64_t mat, int64_t n_run, int64_t sum_kv,
                                  uint64_t mask_run, uint64_t mask_q, ReplicaPlan &pl, int lane) {
   pl.now = now; pl.mat = mat; pl.start = now > mat ? now : mat;
   pl.mode = cfg.mode; pl.token_cap = cfg.token_cap; pl.batch_cap = cfg.batch_cap;
   pl.n_run = n_run; pl.sum_kv = sum_kv;
-  const int64_t min_tpot = warp_min_over_mask(cls_tpot, mask_run, lane);
+  const int64_t min_tpot = warp_min_over_mask(tab.tpot, tab.rank_tpot, mask_run, lane);
   const bool prefill = cfg.mode == HFX_PREFILL;
   pl.n_eff = prefill ? 0 : n_run;
   pl.kv_eff = prefill ? 0 : sum_kv;
@@ -275,7 +289,7 @@ __device__ inline void warp_plan(const HfxParams &p, const int64_t *cls_ttft, co
   int64_t budget = 0;
   if (now >= mat) {      // before maturity the instance is protected: no budget to work out
     if (cfg.mode == HFX_DECODE) {
-      const int64_t T = (n_run > 0 && min_tpot < HFX_INF) ? min_tpot : warp_min_over_mask(cls_tpot, mask_q, lane);
+      const int64_t T = (n_run > 0 && min_tpot < HFX_INF) ? min_tpot : warp_min_over_mask(tab.tpot, tab.rank_tpot, mask_q, lane);
       if (p.budget_mode == HFX_BUDGET_CAP_ONLY || T == HFX_INF) budget = HFX_INF;
       else {
         const int64_t room = T - dev_Ed(p, n_run, sum_kv);
@@ -286,7 +300,7 @@ __device__ inline void warp_plan(const HfxParams &p, const int64_t *cls_ttft, co
       int64_t n_safe;
       if (p.budget_mode == HFX_BUDGET_CAP_ONLY) n_safe = cfg.token_cap;
       else {
-        const int64_t min_ttft = warp_min_over_mask(cls_ttft, mask_q, lane);
+        const int64_t min_ttft = warp_min_over_mask(tab.ttft, tab.rank_ttft, mask_q, lane);
         const bool decoding = pl.n_eff > 0 && pl.tpot_eff < HFX_INF;
         if (min_ttft == HFX_INF) n_safe = cfg.token_cap;
         else if (!decoding) n_safe = warp_nsafe(p, 0, (uint64_t)min_ttft, 2, cfg.token_cap, lane);     // 2 E_p <= TTFT
@@ -337,6 +351,10 @@ __device__ __forceinline__ int64_t warp_sum_i64(int64_t v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+// the same for values in [0, 2^46): two narrow reductions instead of ten shuffles
+__device__ __forceinline__ int64_t warp_sum_wide(int64_t v) {
+  return (int64_t)__reduce_add_sync(0xffffffffu, (uint32_t)v & 0xfffffu) + ((int64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 20)) << 20);
 }
 __device__ __forceinline__ int64_t warp_min_i64(int64_t v) {
 #pragma unroll

@@ -23,7 +23,7 @@
 #define TINY_BIN_MAX 48
 #define TINY_CLASSES 128  // (phase, priority) classes of the sort items of active rows: phase<1> | prio<6>
 #define GROUP_TPT 2       // tiles per thread and round when a group gathers
-#define LIST_WARP_MAX 512 // rows of one tile that a warp copies to a long list by itself
+#define LIST_WARP_MAX 128 // rows of one tile that eight lanes copy to a long list by themselves
 #define LIST_MAX 2048     // inactive rows a replica's own threads list while they gather; longer lists are shared by the grid
 #define SMEM_MED (SEG_MED * 12)
 #define SMEM_GROUP (SMEM_MED / REP_GROUPS)
@@ -494,8 +494,7 @@ static_assert(SMALL_SMEM <= SMEM_GROUP, "a group's arrays fit its share of the b
 
 template <bool SLABS, bool FF>
 __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx &c, const Grp &G, int r, uint32_t b, int n,
-                              int n_act, bool ordered, bool list_in, unsigned char *smem, BlockShared &sh,
-                              const int64_t *s_cls_ttft, const int64_t *s_cls_tpot) {
+                              int n_act, bool ordered, bool list_in, unsigned char *smem, BlockShared &sh, const ClassTab &tab) {
   uint64_t *s_bk = reinterpret_cast<uint64_t *>(smem);                     // [SEG_TINY] slack base of every active row; then the sort items, binned
   uint2 *s_zw = reinterpret_cast<uint2 *>(s_bk + SEG_TINY);                // [SEG_TINY] record words z, w; bit 31 of w: admitted
   int32_t *s_row = reinterpret_cast<int32_t *>(s_zw + SEG_TINY);           // [SEG_TINY]
@@ -570,7 +569,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
     }
   }
   n_run = __reduce_add_sync(0xffffffffu, n_run);
-  sum_kv = warp_sum_i64(sum_kv);
+  sum_kv = warp_sum_wide(sum_kv);
   m_run = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(m_run >> 32)) << 32) | __reduce_or_sync(0xffffffffu, (uint32_t)m_run);
   m_q = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(m_q >> 32)) << 32) | __reduce_or_sync(0xffffffffu, (uint32_t)m_q);
   if (lane == 0) { sh.red_a[warp] = n_run; sh.red_b[warp] = sum_kv; sh.red_m0[warp] = m_run; sh.red_m1[warp] = m_q; }
@@ -582,7 +581,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
     uint64_t mr = 0, mq = 0;
     for (int k = 0; k < nwarp; k++) { nr += sh.red_a[k]; kv += sh.red_b[k]; mr |= sh.red_m0[k]; mq |= sh.red_m1[k]; }
     ReplicaPlan pl0;
-    warp_plan(p, s_cls_ttft, s_cls_tpot, cfg, now, mat, nr, kv, mr, mq, pl0, lane);
+    warp_plan(p, tab, cfg, now, mat, nr, kv, mr, mq, pl0, lane);
     if (lane == 0) { sh.plan = pl0; sh.next_arrival = HFX_INF; }
   }
   G.sync();
@@ -591,6 +590,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   // ---- keys (in registers); per class their range ---------------------------------------------------
   uint64_t item[TINY_IPT];
   int32_t out_len[TINY_IPT];       // of my rows in flight, asked for now and used by the commit
+  const bool few = n_act <= GROUP_THREADS;      // an item per thread: ranked by counting the smaller ones, no bins
   const bool will_commit = real && (a.flags & HFX_COMMIT) && pl.now <= a.horizon;
 #pragma unroll
   for (int k = 0; k < TINY_IPT; k++) {
@@ -608,8 +608,11 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
       else e = eval_row(p, pl, base, kind, prio, (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK));
       if (ordered) {
         item[k] = (e.k48 << 16) | (uint32_t)q;     // rows were gathered in req_id order: position breaks ties
-        const uint32_t cl = (uint32_t)(item[k] >> 56), sub = (uint32_t)(item[k] >> 24);
-        atomicMin(&s_cmin[cl], sub); atomicMax(&s_cmax[cl], sub); atomicAdd(&s_ccnt[cl], 1u);
+        if (few) s_bk[q] = item[k];
+        else {
+          const uint32_t cl = (uint32_t)(item[k] >> 56), sub = (uint32_t)(item[k] >> 24);
+          atomicMin(&s_cmin[cl], sub); atomicMax(&s_cmax[cl], sub); atomicAdd(&s_ccnt[cl], 1u);
+        }
       } else {
         const uint32_t uid = (uint32_t)__ldg(a.req_id + s_row[q]) ^ 0x80000000u;
         s_bk[q] = (e.k48 << 16) | (uid >> 16);
@@ -630,7 +633,17 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   // largest, so bins stay in item order; an item's place inside its bin comes from counting the smaller
   // items of the bin.
   bool sorted_done = false;
-  if (ordered && n_act > 0) {
+  if (ordered && few) {
+    G.sync();
+    if (G.tid < n_act) {
+      const uint64_t x = item[0];
+      uint32_t rank = 0;
+#pragma unroll 8
+      for (int g = 0; g < n_act; g++) rank += s_bk[g] < x ? 1u : 0u;
+      s_lo[rank] = (uint32_t)G.tid;
+    }
+    sorted_done = true;
+  } else if (ordered) {
     G.sync();
     if (warp == 0) layout_class_bins<TINY_BINS>(s_ccnt, s_cmin, s_cmax, s_cinfo, (uint32_t)n_act, lane);
     G.sync();
@@ -766,7 +779,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   }
 
   // ---- totals, maturity, replica outputs, commit ---------------------------------------------------------
-  ac = warp_sum_i64(ac); ak = warp_sum_i64(ak); an = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)an);
+  if (__any_sync(0xffffffffu, an > 0)) { ac = warp_sum_i64(ac); ak = warp_sum_i64(ak); an = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)an); }
   if (lane == 0) { sh.red_a[warp] = ac; sh.red_b[warp] = ak; sh.red_n[warp] = an; }
   G.sync();
   if (G.tid == 0) {
@@ -1181,8 +1194,7 @@ static_assert(MED_BINS / 8 == REP_THREADS, "every thread scans eight bins");
 
 template <bool FF>
 __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act,
-                               bool list_in, unsigned char *smem, BlockShared &sh, uint64_t *s_cinfo,
-                               const int64_t *s_cls_ttft, const int64_t *s_cls_tpot) {
+                               bool list_in, unsigned char *smem, BlockShared &sh, uint64_t *s_cinfo, const ClassTab &tab) {
   uint64_t *s_item = reinterpret_cast<uint64_t *>(smem);                          // [SEG_MED] items by bin
   uint2 *s_zw = reinterpret_cast<uint2 *>(smem);                                  // [SEG_MED] afterwards: record words by position; bit 31 of x: taken by first fit, of y: admitted
   uint16_t *s_ord = reinterpret_cast<uint16_t *>(smem + (size_t)SEG_MED * 8);     // [SEG_MED] position of the i-th row of the order
@@ -1233,7 +1245,7 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
       int64_t now = 0, mat = 0;
       if (real) { cfg = a.cfg[r]; now = a.now[r]; mat = a.mat[r]; }
       ReplicaPlan pl0;
-      warp_plan(p, s_cls_ttft, s_cls_tpot, cfg, now, mat, n_run, sum_kv, m_run, m_q, pl0, lane);
+      warp_plan(p, tab, cfg, now, mat, n_run, sum_kv, m_run, m_q, pl0, lane);
       if (lane == 0) { sh.plan = pl0; sh.next_arrival = HFX_INF; }
     }
     __syncthreads();
@@ -1682,17 +1694,14 @@ template <bool SLABS, bool FF>
 __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, const SegArgs a, const SegCtx c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ BlockShared sh_g[REP_GROUPS];
-  __shared__ int64_t s_cls_ttft[HFX_MAX_CLASSES], s_cls_tpot[HFX_MAX_CLASSES];     // class tables for the planning warps
+  __shared__ ClassTab s_tab;                      // for the planning warps
   __shared__ uint32_t s_scan[2 * 32 + 2];      // (also the scratch of the block-wide scans below)
   __shared__ uint64_t s_cinfo_med[TINY_CLASSES];  // bin layout of a medium replica's distribution sort: smallest slack<40> | first bin<13> | shift<6> | log2 bins<4>
   __shared__ uint32_t s_long[(HFX_TILE_REPLICAS_MAX + 1 + 31) / 32 + 1];           // replicas whose inactive rows the grid lists together
   uint32_t *s_begin = reinterpret_cast<uint32_t *>(smem_raw + SMEM_MED);           // [R+2] range starts (slabs only)
   const int R = p.n_replicas, R1 = R + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int k = tid; k < HFX_MAX_CLASSES; k += blockDim.x) {
-    s_cls_ttft[k] = k < p.n_classes ? p.ttft[k] : 0;
-    s_cls_tpot[k] = k < p.n_classes ? p.tpot[k] : 0;
-  }
+  class_tab_init(p, s_tab, tid);
   for (int k = tid; k < (int)(sizeof(s_long) / sizeof(uint32_t)); k += blockDim.x) s_long[k] = 0;
 
   // everything below reads what the front end wrote
@@ -1757,8 +1766,7 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
       if (need_of(n_all, n_act) > SEG_TINY) continue;
       if (r == R && n_all == 0) continue;
       const bool list_in = !ordered || n_all - n_act <= LIST_MAX;
-      small_replica<SLABS, FF>(p, a, c, G, r, begin[r], (int)n_all, (int)n_act, ordered, list_in, smem_raw + (size_t)g * SMEM_GROUP, sh_g[g],
-                    s_cls_ttft, s_cls_tpot);
+      small_replica<SLABS, FF>(p, a, c, G, r, begin[r], (int)n_all, (int)n_act, ordered, list_in, smem_raw + (size_t)g * SMEM_GROUP, sh_g[g], s_tab);
     }
   }
   __syncthreads();
@@ -1771,7 +1779,7 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
     const uint32_t need = need_of(n_all, n_act);
     if (need <= SEG_TINY) continue;
     const bool list_in = !ordered || n_all - n_act <= LIST_MAX;
-    if (SLABS && ordered && need <= SEG_MED) medium_ordered<FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, list_in, smem_raw, sh_g[0], s_cinfo_med, s_cls_ttft, s_cls_tpot);
+    if (SLABS && ordered && need <= SEG_MED) medium_ordered<FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, list_in, smem_raw, sh_g[0], s_cinfo_med, s_tab);
     else if (need <= SEG_MED) medium_replica<SLABS, FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, ordered, list_in, smem_raw, sh_g[0]);
     else oversize_replica<SLABS, FF>(p, a, c, r, begin[r], n_all, n_act, ordered, list_in, smem_raw, sh_g[0]);
   }
@@ -1814,7 +1822,7 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
       }
       if (tid == 0) s_scan[1] = 0;
       __syncthreads();
-      // the rows themselves: a warp per replica, the whole block where a replica has many in these tiles (the bucket of unbound rows)
+      // the rows themselves: eight lanes per replica, the whole block where a replica has many in these tiles (the bucket of unbound rows)
       auto copy = [&](int j, uint32_t k0, uint32_t kstep) {
         const int r = s_lr[j];
         uint32_t dst = begin[r] + (uint32_t)(__ldcg(c.tot + r) >> 32) + s_lpre[j];
@@ -1827,11 +1835,11 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
           dst += ci;
         }
       };
-      for (int j = warp; j < n_long; j += (int)(blockDim.x >> 5)) {
+      for (int j = tid >> 3; j < n_long; j += (int)(blockDim.x >> 3)) {      // (eight lanes to a replica: a tile holds a few dozen rows of one)
         uint32_t most = 0;      // (the same in all the lanes)
         for (int t = tA; t < tB; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + s_lr[j]); const uint32_t ci = (m.x >> 16) - (m.y >> 16); most = ci > most ? ci : most; }
-        if (most > LIST_WARP_MAX) { if (lane == 0) s_big[atomicAdd(&s_scan[1], 1u)] = (uint16_t)j; }
-        else copy(j, (uint32_t)lane, 32u);
+        if (most > LIST_WARP_MAX) { if ((tid & 7) == 0) s_big[atomicAdd(&s_scan[1], 1u)] = (uint16_t)j; }
+        else copy(j, (uint32_t)(tid & 7), 8u);
       }
       __syncthreads();
       for (uint32_t i = 0; i < s_scan[1]; i++) copy(s_big[i], (uint32_t)tid, blockDim.x);

@@ -1216,7 +1216,7 @@ def test_dispatch_order_and_walk_edges(n, shape):
     assert g["adm_count"].sum() > 0
 
 
-@pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100)])
+@pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100), (40, 8300)])
 def test_idle_replicas_find_their_next_arrivals(R, rows_per):
     # Tiles note every replica's next arrival up to 2047 replicas, lists are searched beyond; lists of more than 2048 rows (a few
     # of them, or hundreds) wait for the end of the kernel, and unbound rows that fill a tile are listed by the whole block.
@@ -1231,3 +1231,10 @@ def test_idle_replicas_find_their_next_arrivals(R, rows_per):
     q = t["state"] == gen.QUEUED
     t["arrival_ns"][q] = now + rng.integers(-2, 90, int(q.sum())) * MS
     assert_step_parity(wl, steps=3, commit=True, optional=False)
+
+
+@pytest.mark.parametrize("n_act", [1, 127, 128, 129])
+def test_replicas_of_few_active_rows_are_ranked_by_counting(n_act):
+    wl = gen.random_table(n_act, 7 * n_act, 7, modes=MODES3, permute_ids=False, tie_heavy=True, inflight=0.4, done=0.0, future=0.0)
+    wl.table["replica_id"][:] = np.arange(7 * n_act) % 7
+    assert_step_parity(wl, steps=3, commit=True)

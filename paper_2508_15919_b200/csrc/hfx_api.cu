@@ -110,11 +110,12 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
     s->tiles_max = 0;
     if (n_replicas <= HFX_TILE_REPLICAS_MAX && (int64_t)n_tiles * (n_replicas + 1) <= HFX_TILE_MATRIX_MAX) {
       const size_t slots = (size_t)max_rows + HFX_TILE_ROWS_MAX;
-      // (the matrix of next arrivals lies behind it)
+      // (the matrices of next arrivals and of inactive rows lie behind it)
       const size_t entries = ((size_t)n_tiles * ((size_t)n_replicas + 1) + 15) & ~(size_t)15;
       const bool has_next = n_replicas <= HFX_NEXT_REPLICAS_MAX;
-      ok = ok && cudaMalloc(&s->d_M, (sizeof(uint2) + (has_next ? sizeof(int64_t) : 0)) * entries) == cudaSuccess;
+      ok = ok && cudaMalloc(&s->d_M, (sizeof(uint2) + (has_next ? sizeof(int64_t) : 0)) * entries + sizeof(uint16_t) * (size_t)n_tiles * front_inact_ld(n_replicas + 1)) == cudaSuccess;
       s->d_next = ok && has_next ? reinterpret_cast<int64_t *>(s->d_M + entries) : nullptr;
+      s->d_inact = ok ? reinterpret_cast<uint16_t *>(s->d_M + entries * (has_next ? 2 : 1)) : nullptr;
       ok = ok && cudaMalloc(&s->d_slab_rec, sizeof(uint4) * slots) == cudaSuccess;
       ok = ok && cudaMalloc(&s->d_slab_idx, sizeof(uint16_t) * slots) == cudaSuccess;
       ok = ok && cudaMalloc(&s->d_tot, sizeof(unsigned long long) * 2 * R2) == cudaSuccess;

@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
       const uint32_t off_all = run & 0xffffu, off_act = run >> 16;
       s_base[2 * i] = (uint16_t)off_all; s_base[2 * i + 1] = (uint16_t)(off_all + cA); s_offact[i] = (uint16_t)off_act;
       mrow[i] = make_uint2(off_all | ((cA + cI) << 16), off_act | (cA << 16));
+      a.inact[(size_t)blockIdx.x * front_inact_ld(R1) + i] = (uint16_t)cI;
       if (has_next) a.next[(size_t)blockIdx.x * R1 + i] = s_next[i];
       if (cA + cI) atomicAdd(a.tot + i, (unsigned long long)(cA + cI) | ((unsigned long long)cA << 32));
       run += (cA + cI) | (cA << 16);
@@ -366,7 +367,7 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   hfx_front_shape(s, fa.n, &fa.tile_rows, &fa.n_tiles);
   const int R1 = s->p.n_replicas + 1;
   const uint32_t par = s->tot_parity;
-  fa.slab_rec = s->d_slab_rec; fa.slab_idx = s->d_slab_idx; fa.M = s->d_M; fa.next = s->d_next;
+  fa.slab_rec = s->d_slab_rec; fa.slab_idx = s->d_slab_idx; fa.M = s->d_M; fa.next = s->d_next; fa.inact = s->d_inact;
   fa.tot = s->d_tot + (size_t)par * (R1 + 1); fa.tot_next = s->d_tot + (size_t)(par ^ 1u) * (R1 + 1);
   fa.ordered = s->d_flags + 4 + par; fa.ordered_next = s->d_flags + 4 + (par ^ 1u);
   fa.status = s->d_status; fa.rowflag = s->d_rowflag;

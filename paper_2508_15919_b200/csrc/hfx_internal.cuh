@@ -113,6 +113,7 @@ struct hfx_sched {
   uint16_t *d_slab_idx;     // [tiles_max * tile_rows] local row indices, tile-major, grouped by replica
   uint2 *d_M;               // [tiles_max][R+1] where each replica's rows sit in a tile's slabs
   int64_t *d_next;          // [tiles_max][R+1] earliest arrival still to come of each replica in a tile (up to HFX_NEXT_REPLICAS_MAX replicas)
+  uint16_t *d_inact;        // [tiles_max][front_inact_ld(R+1)] inactive rows of each replica in a tile
   unsigned long long *d_tot;// [2][R+2] rows | active rows << 32 per replica, by parity
   int32_t tiles_max;        // matrix rows allocated (0: fallback front end only)
   uint32_t tot_parity;      // which half of d_tot / which "ordered" word the next tile front end uses
@@ -519,6 +520,9 @@ struct RegroupArgs {
 };
 
 // the tile front end
+// entries per row of the matrix of inactive rows (rows start on 16 bytes)
+__host__ __device__ constexpr int front_inact_ld(int R1) { return (R1 + 7) & ~7; }
+
 struct FrontArgs {
   const int32_t *replica_id; const uint8_t *class_id; const uint8_t *state; const int32_t *prompt_len; const int32_t *gen;
   const int64_t *arrival; const int64_t *first_token; const int32_t *req_id; const int32_t *weight;
@@ -527,7 +531,7 @@ struct FrontArgs {
   // per-row outputs, written in row order
   int64_t *slack; int64_t *pred_ttft; int64_t *pred_tpot; uint64_t *key; uint8_t *admit; uint8_t *rowflag;
   // the slabs
-  uint4 *slab_rec; uint16_t *slab_idx; uint2 *M; int64_t *next; unsigned long long *tot; unsigned long long *tot_next;
+  uint4 *slab_rec; uint16_t *slab_idx; uint2 *M; int64_t *next; uint16_t *inact; unsigned long long *tot; unsigned long long *tot_next;
   uint32_t *ordered; uint32_t *ordered_next; uint32_t *status;
 };
 

@@ -42,7 +42,7 @@ struct BlockShared {
 // where the kernel finds the rows of a replica
 struct SegCtx {
   // tile front end: slabs
-  const uint4 *slab_rec; const uint16_t *slab_idx; const uint2 *M; const int64_t *next; const unsigned long long *tot;
+  const uint4 *slab_rec; const uint16_t *slab_idx; const uint2 *M; const int64_t *next; const uint16_t *inact; const unsigned long long *tot;
   int32_t tile_rows, n_tiles;
   // fallback front end: contiguous records, counts and range starts
   const uint32_t *seg_count; const uint32_t *act_count; const uint32_t *seg_begin;
@@ -1786,13 +1786,15 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
 
   // ---- long lists of inactive rows (ordered steps): every block lists a range of tiles ----------------
   // The replicas with a long list are collected in shared memory; their inactive rows in the tiles before the block's are
-  // added up, then the rows of the block's tiles are copied.
+  // added up (every block reads those of all the tiles before its own: hence a matrix of two bytes an entry), then the rows of the block's tiles are copied.
   if (longer) {
     __syncthreads();      // the larger replicas are done with the block's shared memory
-    uint16_t *s_lr = reinterpret_cast<uint16_t *>(smem_raw);                                   // [R1] the replicas
-    uint32_t *s_lpre = reinterpret_cast<uint32_t *>(smem_raw + (((size_t)R1 * 2 + 15) & ~(size_t)15));   // [R1] rows in earlier tiles
-    uint16_t *s_big = reinterpret_cast<uint16_t *>(s_lpre + R1);                               // [R1] those that the whole block copies
-    if (tid == 0) s_scan[0] = 0;
+    const int ld = front_inact_ld(R1);
+    uint32_t *s_before = reinterpret_cast<uint32_t *>(smem_raw);      // [ld] inactive rows of every replica in earlier tiles
+    uint16_t *s_lr = reinterpret_cast<uint16_t *>(s_before + ld);     // [R1] the replicas with a long list
+    uint16_t *s_big = s_lr + R1;                                      // [R1] those that the whole block copies
+    if (tid < 2) s_scan[tid] = 0;
+    for (int i = tid; i < ld; i += blockDim.x) s_before[i] = 0;
     __syncthreads();
     for (int r = tid; r < R1; r += blockDim.x)
       if ((s_long[r >> 5] >> (r & 31)) & 1u) s_lr[atomicAdd(&s_scan[0], 1u)] = (uint16_t)r;
@@ -1802,30 +1804,25 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
     const int tA = blockIdx.x * per < c.n_tiles ? blockIdx.x * per : c.n_tiles;
     const int tB = tA + per < c.n_tiles ? tA + per : c.n_tiles;
     if (tA < tB) {
-      if (n_long >= 256) {      // rows in earlier tiles: a thread per replica, neighbours side by side in memory ...
-        for (int j = tid; j < n_long; j += blockDim.x) {
-          const int r = s_lr[j];
-          uint32_t pre = 0;
-#pragma unroll 8
-          for (int t = 0; t < tA; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + r); pre += (m.x >> 16) - (m.y >> 16); }
-          s_lpre[j] = pre;
-        }
-      } else {                  // ... or, of few replicas, a lane per tile
-        for (int j = warp; j < n_long; j += (int)(blockDim.x >> 5)) {
-          const int r = s_lr[j];
-          uint32_t pre = 0;
+      // a thread adds up eight replicas (one load a tile) over a share of the tiles
+      const int cols = ld >> 3, shares = blockDim.x > (unsigned)cols ? (int)blockDim.x / cols : 1, per_share = (tA + shares - 1) / shares;
+      for (int i = tid; i < cols * shares; i += blockDim.x) {
+        const int share = i / cols, col = i - share * cols;
+        const int t0 = share * per_share, t1 = t0 + per_share < tA ? t0 + per_share : tA;
+        uint32_t v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll 4
-          for (int t = lane; t < tA; t += 32) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + r); pre += (m.x >> 16) - (m.y >> 16); }
-          pre = __reduce_add_sync(0xffffffffu, pre);
-          if (lane == 0) s_lpre[j] = pre;
+        for (int t = t0; t < t1; t++) {
+          const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(c.inact + (size_t)t * ld) + col);
+          v[0] += x.x & 0xffffu; v[1] += x.x >> 16; v[2] += x.y & 0xffffu; v[3] += x.y >> 16;
+          v[4] += x.z & 0xffffu; v[5] += x.z >> 16; v[6] += x.w & 0xffffu; v[7] += x.w >> 16;
         }
+#pragma unroll
+        for (int k = 0; k < 8; k++) if (v[k]) atomicAdd(&s_before[col * 8 + k], v[k]);
       }
-      if (tid == 0) s_scan[1] = 0;
       __syncthreads();
-      // the rows themselves: eight lanes per replica, the whole block where a replica has many in these tiles (the bucket of unbound rows)
-      auto copy = [&](int j, uint32_t k0, uint32_t kstep) {
-        const int r = s_lr[j];
-        uint32_t dst = begin[r] + (uint32_t)(__ldcg(c.tot + r) >> 32) + s_lpre[j];
+      // eight lanes copy a replica's rows; the whole block where a replica has many in these tiles (the bucket of unbound rows)
+      auto copy = [&](int r, uint32_t k0, uint32_t kstep) {
+        uint32_t dst = begin[r] + (uint32_t)(__ldcg(c.tot + r) >> 32) + s_before[r];
         for (int t = tA; t < tB; t++) {
           const uint2 m = __ldcg(c.M + (size_t)t * R1 + r);
           const uint32_t ca = m.y >> 16, ci = (m.x >> 16) - ca, src = (m.x & 0xffffu) + ca;
@@ -1836,10 +1833,11 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
         }
       };
       for (int j = tid >> 3; j < n_long; j += (int)(blockDim.x >> 3)) {      // (eight lanes to a replica: a tile holds a few dozen rows of one)
-        uint32_t most = 0;      // (the same in all the lanes)
-        for (int t = tA; t < tB; t++) { const uint2 m = __ldcg(c.M + (size_t)t * R1 + s_lr[j]); const uint32_t ci = (m.x >> 16) - (m.y >> 16); most = ci > most ? ci : most; }
-        if (most > LIST_WARP_MAX) { if ((tid & 7) == 0) s_big[atomicAdd(&s_scan[1], 1u)] = (uint16_t)j; }
-        else copy(j, (uint32_t)(tid & 7), 8u);
+        const int r = s_lr[j], l8 = tid & 7;
+        uint32_t most = 0;      // (the same in all eight lanes)
+        for (int t = tA; t < tB; t++) { const uint32_t ci = __ldcg(c.inact + (size_t)t * ld + r); most = ci > most ? ci : most; }
+        if (most <= LIST_WARP_MAX) copy(r, (uint32_t)l8, 8u);
+        else if (l8 == 0) s_big[atomicAdd(&s_scan[1], 1u)] = (uint16_t)r;
       }
       __syncthreads();
       for (uint32_t i = 0; i < s_scan[1]; i++) copy(s_big[i], (uint32_t)tid, blockDim.x);
@@ -1859,7 +1857,7 @@ int hfx_launch_replicas(hfx_sched *s, const SegArgs &sa, int64_t n, bool slabs) 
   c.big_hi = s->d_big_hi; c.big_lo = s->d_big_lo; c.big_idx = s->d_big_lo ? s->d_big_lo + s->max_rows : nullptr;
   if (slabs) {
     const uint32_t par = s->tot_parity;
-    c.slab_rec = s->d_slab_rec; c.slab_idx = s->d_slab_idx; c.M = s->d_M; c.next = s->d_next;
+    c.slab_rec = s->d_slab_rec; c.slab_idx = s->d_slab_idx; c.M = s->d_M; c.next = s->d_next; c.inact = s->d_inact;
     c.tot = s->d_tot + (size_t)par * (R1 + 1);
     c.ordered = s->d_flags + 4 + par;
     hfx_front_shape(s, n, &c.tile_rows, &c.n_tiles);

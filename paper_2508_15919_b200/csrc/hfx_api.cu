@@ -108,7 +108,8 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
     hfx_front_shape(s, max_rows, &tile_rows, &n_tiles);
     if (n_tiles < n_sm + 1) n_tiles = n_sm + 1;      // smaller tables have lower tiles, about one per SM
     s->tiles_max = 0;
-    if (n_replicas <= HFX_TILE_REPLICAS_MAX && (int64_t)n_tiles * (n_replicas + 1) <= HFX_TILE_MATRIX_MAX) {
+    if (n_replicas <= HFX_TILE_REPLICAS_MAX && (int64_t)(n_tiles - n_sm) * (n_replicas + 1) <= HFX_TILE_MATRIX_MAX) {
+      n_tiles = (n_tiles + n_sm - 1) / n_sm * n_sm;      // (smaller tables may have up to as many tiles per SM)
       const size_t slots = (size_t)max_rows + HFX_TILE_ROWS_MAX;
       // (the matrices of next arrivals and of inactive rows lie behind it)
       const size_t entries = ((size_t)n_tiles * ((size_t)n_replicas + 1) + 15) & ~(size_t)15;

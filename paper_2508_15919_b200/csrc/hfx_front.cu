@@ -36,20 +36,23 @@ __host__ __device__ inline size_t front_smem_bytes(int R1, int T) {
   return (b + 15) & ~(size_t)15;
 }
 
-// exclusive prefix of `mine` over the threads of the block (two barriers); *total = block sum
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t mine, uint32_t *s_warp, uint32_t *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+// counters by warp: bytes per group (a count a warp, groups on different banks), and 16-bit prefixes per group (one every four warps)
+#define FRONT_WCNT_PITCH 36
+#define FRONT_WPRE_PITCH 9
+#define FRONT_WCNT_ROWS (255 * (FRONT_THREADS / 32))      // rows of a tile whose counts by warp fit in a byte each
+
+// exclusive prefix of `mine` over the threads of the block (two barriers; every warp adds up the totals of the warps before it)
+__device__ __forceinline__ uint32_t block_excl_scan(uint32_t mine, uint32_t *s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t v = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) { const uint32_t w = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += w; }
   __syncthreads();                 // s_warp may still be read from a previous call
   if (lane == 31) s_warp[warp] = v;
   __syncthreads();
-  uint32_t pre = 0, all = 0;
-  for (int k = 0; k < nwarp; k++) { const uint32_t w = s_warp[k]; if (k < warp) pre += w; all += w; }
-  if (total) *total = all;
-  return pre + v - mine;
+  return __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + v - mine;
 }
+static_assert(FRONT_THREADS == 1024, "a lane for every warp's total");
 
 // EXTRA: the optional per-row outputs (predicted TTFT, predicted TPOT default, key) are wanted
 template <bool EXTRA>
@@ -57,17 +60,19 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int R = p.n_replicas, R1 = R + 1, T = a.tile_rows;
   uint4 *s_rec = reinterpret_cast<uint4 *>(smem_raw);                    // [T]    record of every active row, by local index
-  int64_t *s_now = reinterpret_cast<int64_t *>(s_rec + T);               // [R1]
+  uint32_t *s_bkt = reinterpret_cast<uint32_t *>(s_rec + T);             // [T]    replica bucket | 0x8000 if active | rank in the group << 16
+  int64_t *s_now = reinterpret_cast<int64_t *>(s_bkt + T);               // [R1]
   int64_t *s_start = s_now + R1;                                         // [R1]   earliest start max(now, maturity)
-  const bool has_next = a.next != nullptr;
+  const bool has_next = a.next != nullptr, by_warp = a.by_warp != 0;
   long long *s_next = reinterpret_cast<long long *>(s_start + R1);       // [R1]   earliest arrival that is still to come (if has_next)
   uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_next + (has_next ? R1 : 0));      // [2 R1] rows per group = (replica, active / inactive)
-  uint32_t *s_bkt = s_cnt + 2 * R1;                                      // [T]    replica bucket | 0x8000 if active | arrival rank in the group << 16
-  uint16_t *s_base = reinterpret_cast<uint16_t *>(s_bkt + T);            // [2 R1] first slot of each group in slab_idx order
+  uint16_t *s_base = reinterpret_cast<uint16_t *>(s_cnt + 2 * R1);       // [2 R1] first slot of each group in slab_idx order
   uint16_t *s_offact = s_base + 2 * R1;                                  // [R1]   first slot of the replica's records in slab_rec
   uint16_t *s_perm = s_offact + R1;                                      // [T+8]  local index of the row in each slot, groups in arrival order
   uint16_t *s_fin = s_perm + T + 8;                                      // [T+8]  the same with every group in row order
   uint8_t *s_mode = reinterpret_cast<uint8_t *>(s_fin + T + 8);          // [R1]
+  uint32_t *s_wcnt = reinterpret_cast<uint32_t *>(smem_raw + front_smem_bytes(R1, T));      // [2 R1][FRONT_WCNT_PITCH / 4] (if by_warp) rows per group and warp, a byte each
+  uint16_t *s_wpre = reinterpret_cast<uint16_t *>(s_wcnt + 2 * R1 * (FRONT_WCNT_PITCH / 4));      // [2 R1][FRONT_WPRE_PITCH] (if by_warp) rows per group of the warps before each four
   __shared__ int64_t s_ttft[HFX_MAX_CLASSES], s_tpot[HFX_MAX_CLASSES];
   __shared__ uint8_t s_prio[HFX_MAX_CLASSES];
   __shared__ uint32_t s_warp[32];
@@ -109,6 +114,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     s_cnt[2 * i] = 0; s_cnt[2 * i + 1] = 0;
     if (has_next) s_next[i] = HFX_INF;
   }
+  if (by_warp) for (int i = tid; i < 2 * R1 * (FRONT_WCNT_PITCH / 4); i += blockDim.x) s_wcnt[i] = 0;
   if (blockIdx.x == 0) {      // re-arm what the next step accumulates into
     for (int i = tid; i < R1; i += blockDim.x) a.tot_next[i] = 0ull;
     if (tid == 0) *a.ordered_next = 1u;
@@ -121,9 +127,9 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
   int sorted = 1, rising = 1;
 
   // ---- pass 1: every row once -------------------------------------------------------------------
-  // returns the row's kind; slack = what the slack output gets; bkt = its bucket
+  // returns the row's kind; slack = what the slack output gets; bkt = its bucket; word = what s_bkt gets
   auto do_row = [&](int il, int32_t rid, uint32_t cls, uint32_t st, int32_t prompt, int32_t gen, int32_t weight,
-                    int64_t arrival, int64_t first_token, int64_t &slack, int &bkt, uint64_t &k48, int64_t &pttft) -> uint32_t {
+                    int64_t arrival, int64_t first_token, int64_t &slack, int &bkt, uint64_t &k48, int64_t &pttft, uint32_t &word) -> uint32_t {
     const uint32_t kind = classify_row(p, rid, cls, st, prompt, gen, arrival, s_now, bad);
     bkt = (uint32_t)rid < (uint32_t)R ? rid : R;
     slack = 0;
@@ -151,8 +157,8 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
                              (uint32_t)gen | (cls << CREC_CLS_SHIFT));
     }
     if (kind == KIND_FUTURE && has_next && arrival < s_next[bkt]) atomicMin(&s_next[bkt], (long long)arrival);      // (mostly the look alone)
-    const uint32_t g = 2u * (uint32_t)bkt + (act ? 0u : 1u);
-    s_bkt[il] = (uint32_t)bkt | (act ? 0x8000u : 0u) | (atomicAdd(&s_cnt[g], 1u) << 16);
+    word = (uint32_t)bkt | (act ? 0x8000u : 0u);
+    if (!by_warp) word |= atomicAdd(&s_cnt[2u * (uint32_t)bkt + (act ? 0u : 1u)], 1u) << 16;
     return kind;
   };
 
@@ -174,10 +180,12 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     uint64_t kk[4];
     int bk[4];
     uint32_t kd[4];
-    kd[0] = do_row(4 * v, rid.x, cls.x, st.x, pr.x, ge.x, we.x, ar0.x, ft0.x, sl[0], bk[0], kk[0], pt[0]);
-    kd[1] = do_row(4 * v + 1, rid.y, cls.y, st.y, pr.y, ge.y, we.y, ar0.y, ft0.y, sl[1], bk[1], kk[1], pt[1]);
-    kd[2] = do_row(4 * v + 2, rid.z, cls.z, st.z, pr.z, ge.z, we.z, ar1.x, ft1.x, sl[2], bk[2], kk[2], pt[2]);
-    kd[3] = do_row(4 * v + 3, rid.w, cls.w, st.w, pr.w, ge.w, we.w, ar1.y, ft1.y, sl[3], bk[3], kk[3], pt[3]);
+    uint4 wd;
+    kd[0] = do_row(4 * v, rid.x, cls.x, st.x, pr.x, ge.x, we.x, ar0.x, ft0.x, sl[0], bk[0], kk[0], pt[0], wd.x);
+    kd[1] = do_row(4 * v + 1, rid.y, cls.y, st.y, pr.y, ge.y, we.y, ar0.y, ft0.y, sl[1], bk[1], kk[1], pt[1], wd.y);
+    kd[2] = do_row(4 * v + 2, rid.z, cls.z, st.z, pr.z, ge.z, we.z, ar1.x, ft1.x, sl[2], bk[2], kk[2], pt[2], wd.z);
+    kd[3] = do_row(4 * v + 3, rid.w, cls.w, st.w, pr.w, ge.w, we.w, ar1.y, ft1.y, sl[3], bk[3], kk[3], pt[3], wd.w);
+    reinterpret_cast<uint4 *>(s_bkt)[v] = wd;
     // per-row outputs in row order
     longlong2 *slp = reinterpret_cast<longlong2 *>(a.slack) + 2 * gv;
     slp[0] = make_longlong2(sl[0], sl[1]); slp[1] = make_longlong2(sl[2], sl[3]);
@@ -208,7 +216,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     const int64_t g = lo + i;
     int64_t sl, pt; uint64_t kk; int bk;
     const uint32_t kd = do_row(i, a.replica_id[g], a.class_id[g], a.state[g], a.prompt_len[g], a.gen[g], a.weight ? a.weight[g] : 0,
-                               a.arrival[g], a.first_token[g], sl, bk, kk, pt);
+                               a.arrival[g], a.first_token[g], sl, bk, kk, pt, s_bkt[i]);
     a.slack[g] = sl;
     a.admit[g] = kd == KIND_RUNNING;
     if (!has_next) a.rowflag[g] = (uint8_t)kd;
@@ -225,6 +233,41 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
   rising = __syncthreads_and(rising);
   if (tid == 0 && !rising) *a.ordered = 0u;
 
+  // ---- ranks by warp ---------------------------------------------------------------------------------
+  // Every warp takes a stretch of the tile and counts its rows of every group, 32 rows at a time: a row's rank is the
+  // count so far and the lanes before it of the same group.  In row order whatever the groups' sizes; the lanes that share
+  // a group are few (the counter shows them) or all (grouped tables), so a match over the whole warp, which takes as
+  // long as it has groups (250 cycles a warp at 300 replicas), is never made.
+  const int lane = tid & 31, warp = tid >> 5;
+  const int stretch = (nt + FRONT_THREADS / 32 - 1) / (FRONT_THREADS / 32);
+  const int w0 = warp * stretch < nt ? warp * stretch : nt, w1 = w0 + stretch < nt ? w0 + stretch : nt;
+  if (by_warp) {
+    const uint8_t *cnt = reinterpret_cast<const uint8_t *>(s_wcnt) + warp;
+    const uint32_t below = (1u << lane) - 1u;
+    for (int i = w0; i < w1; i += 32) {
+      const int il = i + lane;
+      const uint32_t in = __ballot_sync(0xffffffffu, il < w1);
+      if (il < w1) {
+        const uint32_t bk = s_bkt[il], b = bk & 0xfffu, inactive = ((bk >> 15) & 1u) ^ 1u, g = 2 * b + inactive;
+        const bool one = __all_sync(in, b == __shfl_sync(in, b, 0)) != 0;      // all of one replica
+        const uint32_t no = __ballot_sync(in, inactive != 0);
+        const uint32_t before = cnt[g * FRONT_WCNT_PITCH];
+        uint32_t mates = inactive ? no : in & ~no;
+        __syncwarp(in);
+        if (!one || (mates & below) == 0) atomicAdd(&s_wcnt[g * (FRONT_WCNT_PITCH / 4) + (warp >> 2)], (one ? (uint32_t)__popc(mates) : 1u) << (8 * (warp & 3)));
+        __syncwarp(in);
+        if (!one) {
+          const uint32_t shared = __ballot_sync(in, cnt[g * FRONT_WCNT_PITCH] - before > 1u);
+          mates = 0;
+          if ((shared >> lane) & 1u) mates = __match_any_sync(shared, g);
+        }
+        s_bkt[il] = bk | ((before + (uint32_t)__popc(mates & below)) << 16);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  }
+
   // ---- pass 2: where each group starts inside the slabs; the tile's matrix row; totals -----------
   int big = 0;
   {
@@ -232,11 +275,21 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     const int i0 = tid * per < R1 ? tid * per : R1, i1 = (i0 + per < R1) ? i0 + per : R1;
     uint32_t pack = 0;       // rows | active rows << 16 (each at most T <= 8192: the fields cannot carry into each other)
     for (int i = i0; i < i1; i++) {
+      if (by_warp) {
+        uint32_t n[2] = {0, 0};
+        for (int h = 0; h < 2; h++)
+#pragma unroll
+          for (int k = 0; k < 8; k++) {
+            s_wpre[(2 * i + h) * FRONT_WPRE_PITCH + k] = (uint16_t)n[h];
+            n[h] = __dp4a(s_wcnt[(2 * i + h) * (FRONT_WCNT_PITCH / 4) + k], 0x01010101u, n[h]);
+          }
+        s_cnt[2 * i] = n[0]; s_cnt[2 * i + 1] = n[1];
+      }
       const uint32_t cA = s_cnt[2 * i], cI = s_cnt[2 * i + 1];
       pack += (cA + cI) | (cA << 16);
       if (i < R && (cA > FRONT_GROUP_MAX || cI > FRONT_GROUP_MAX)) big = 1;
     }
-    uint32_t run = block_excl_scan(pack, s_warp, nullptr);
+    uint32_t run = block_excl_scan(pack, s_warp);
     uint2 *mrow = a.M + (size_t)blockIdx.x * R1;
     for (int i = i0; i < i1; i++) {
       const uint32_t cA = s_cnt[2 * i], cI = s_cnt[2 * i + 1];
@@ -250,16 +303,23 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     }
   }
   const bool tail_scan = s_cnt[2 * R + 1] > FRONT_TAIL_MAX;    // many rows bound to no replica: ranked by a scan
-  const int any_big = __syncthreads_or(big);          // (also publishes s_base / s_offact)
+  const int any_big = __syncthreads_or(big && !by_warp);          // (also publishes s_base / s_offact)
   uint16_t *fin = s_fin;
 
   // ---- pass 3: the slot of every row -----------------------------------------------------------------
   const int c0 = tid * FRONT_PER < nt ? tid * FRONT_PER : nt, c1 = (c0 + FRONT_PER < nt) ? c0 + FRONT_PER : nt;
-  if (sorted) {
+  if (by_warp) {      // the group's rows in the stretches before mine, and the rank inside mine
+    for (int il = w0 + lane; il < w1; il += 32) {
+      const uint32_t bk = s_bkt[il], g = 2 * (bk & 0xfffu) + (((bk >> 15) & 1u) ^ 1u);
+      const uint32_t at = __dp4a(s_wcnt[g * (FRONT_WCNT_PITCH / 4) + (warp >> 2)], 0x00010101u >> (8 * (3 - (warp & 3))),
+                                 s_base[g] + s_wpre[g * FRONT_WPRE_PITCH + (warp >> 2)] + (bk >> 16));
+      s_fin[at] = (uint16_t)il;
+    }
+  } else if (sorted) {
     // rows of a replica are contiguous: ranks from positions.  s_perm[il] = active rows before position il.
     uint32_t cnt = 0;
     for (int il = c0; il < c1; il++) cnt += (s_bkt[il] >> 15) & 1u;
-    uint32_t run = block_excl_scan(cnt, s_warp, nullptr);
+    uint32_t run = block_excl_scan(cnt, s_warp);
     for (int il = c0; il < c1; il++) { s_perm[il] = (uint16_t)run; run += (s_bkt[il] >> 15) & 1u; }
     __syncthreads();
     for (int il = c0; il < c1; il++) {
@@ -273,7 +333,7 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     if (tail_scan) {      // (uniform) rows bound to no replica: slot from the number of such rows before each position
       uint32_t cnt = 0;
       for (int il = c0; il < c1; il++) cnt += (s_bkt[il] & 0xfffu) == (uint32_t)R;
-      uint32_t run = block_excl_scan(cnt, s_warp, nullptr);
+      uint32_t run = block_excl_scan(cnt, s_warp);
       const uint32_t tb = s_base[2 * R + 1];
       for (int il = c0; il < c1; il++)
         if ((s_bkt[il] & 0xfffu) == (uint32_t)R) { fin[tb + run] = (uint16_t)il; run++; }
@@ -345,16 +405,19 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-// Tile height: about one tile per SM, a multiple of 4 rows, at most 8192 (16-bit local indices) and what
+// Tile height: about one tile per SM, of large tables the same number of tiles on every SM (512 tiles of 8192 rows left
+// the last of four rounds half empty), a multiple of 16 rows, at most 8192 (16-bit local indices) and what
 // the block's shared memory holds beside its per-replica arrays.
 void hfx_front_shape(const hfx_sched *s, int64_t n, int32_t *tile_rows, int32_t *n_tiles) {
   const int R1 = s->p.n_replicas + 1;
-  int64_t t = (n + s->n_sm - 1) / s->n_sm;
-  t = (t + 15) & ~INT64_C(15);       // (a multiple of 16 rows: every tile starts on a 16-byte boundary of every column)
-  if (t < 1024) t = 1024;
   int64_t cap = ((int64_t)HFX_FRONT_SMEM - (int64_t)front_smem_bytes(R1, 0)) / FRONT_ROW_BYTES;
   cap &= ~INT64_C(15);
   if (cap > 8192) cap = 8192;
+  if (cap < 16) cap = 16;            // (more replicas than the front end takes: no tile is ever made)
+  const int64_t wave = cap * s->n_sm, waves = n > wave ? (n + wave - 1) / wave : 1;
+  int64_t t = (n + s->n_sm * waves - 1) / (s->n_sm * waves);
+  t = (t + 15) & ~INT64_C(15);       // (a multiple of 16 rows: every tile starts on a 16-byte boundary of every column)
+  if (t < 1024) t = 1024;
   if (t > cap) t = cap;
   *tile_rows = (int32_t)t;
   int64_t k = (n + t - 1) / t;
@@ -371,9 +434,15 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   fa.tot = s->d_tot + (size_t)par * (R1 + 1); fa.tot_next = s->d_tot + (size_t)(par ^ 1u) * (R1 + 1);
   fa.ordered = s->d_flags + 4 + par; fa.ordered_next = s->d_flags + 4 + (par ^ 1u);
   fa.status = s->d_status; fa.rowflag = s->d_rowflag;
+  // ranks by warp wherever the counters fit beside the tile (some 350 replicas at 7000 rows); more replicas mean small groups,
+  // which are cheap to put in order by counting
+  size_t smem = front_smem_bytes(R1, fa.tile_rows);
+  const size_t wcnt = (size_t)2 * R1 * (FRONT_WCNT_PITCH + 2 * FRONT_WPRE_PITCH);
+  fa.by_warp = fa.tile_rows <= FRONT_WCNT_ROWS && smem + wcnt <= HFX_FRONT_SMEM;
+  if (fa.by_warp) smem += wcnt;
   KernelScope ks(s, KSLOT_FRONT);
-  if (fa.pred_ttft || fa.pred_tpot || fa.key) k_front<true><<<fa.n_tiles, FRONT_THREADS, front_smem_bytes(R1, fa.tile_rows), s->stream>>>(s->p, fa);
-  else k_front<false><<<fa.n_tiles, FRONT_THREADS, front_smem_bytes(R1, fa.tile_rows), s->stream>>>(s->p, fa);
+  if (fa.pred_ttft || fa.pred_tpot || fa.key) k_front<true><<<fa.n_tiles, FRONT_THREADS, smem, s->stream>>>(s->p, fa);
+  else k_front<false><<<fa.n_tiles, FRONT_THREADS, smem, s->stream>>>(s->p, fa);
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }
 

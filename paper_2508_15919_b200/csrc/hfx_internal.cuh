@@ -78,7 +78,7 @@ enum { KSLOT_COUNT = 0, KSLOT_COLSCAN, KSLOT_OFFSETS, KSLOT_REGROUP, KSLOT_SEG_S
 
 // tiling of the front end: one tile per block, at most 8192 rows (16-bit indices inside a tile)
 #define HFX_TILE_ROWS_MAX 8192
-#define HFX_TILE_MATRIX_MAX (INT64_C(8) << 20)   // entries of the tile matrix (64 MiB)
+#define HFX_TILE_MATRIX_MAX (INT64_C(8) << 20)   // entries of the tile matrix (64 MiB), the tiles of one round of the SMs left out
 #define HFX_TILE_REPLICAS_MAX 4095               // replicas whose counters fit in shared memory (12-bit bucket ids)
 #define HFX_NEXT_REPLICAS_MAX 2047               // replicas up to which a tile notes the next arrival of each (8 bytes of shared memory per replica)
 #define HFX_COUNT_TILE_ROWS 4096                 // rows per block of the counting pass of the fallback front end
@@ -527,7 +527,7 @@ struct FrontArgs {
   const int32_t *replica_id; const uint8_t *class_id; const uint8_t *state; const int32_t *prompt_len; const int32_t *gen;
   const int64_t *arrival; const int64_t *first_token; const int32_t *req_id; const int32_t *weight;
   const int64_t *now; const int64_t *mat; const uint8_t *mode;
-  int64_t n; int32_t tile_rows; int32_t n_tiles;
+  int64_t n; int32_t tile_rows; int32_t n_tiles; int32_t by_warp;
   // per-row outputs, written in row order
   int64_t *slack; int64_t *pred_ttft; int64_t *pred_tpot; uint64_t *key; uint8_t *admit; uint8_t *rowflag;
   // the slabs

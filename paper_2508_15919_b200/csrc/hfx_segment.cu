@@ -1082,9 +1082,9 @@ __device__ __forceinline__ void sort64_positions(uint64_t *hi, uint32_t *pos_out
   }
 }
 
-template <bool SLABS, bool FF>
-__device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act,
-                               bool ordered, bool list_in, unsigned char *smem, BlockShared &sh) {
+// (the fallback layout: its steps are never taken as ordered)
+template <bool FF>
+__device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act, unsigned char *smem, BlockShared &sh) {
   uint64_t *s_hi = reinterpret_cast<uint64_t *>(smem);
   uint32_t *s_lo = reinterpret_cast<uint32_t *>(smem + (size_t)SEG_MED * 8);
   const int R = p.n_replicas;
@@ -1092,11 +1092,8 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
   const int n_in = n - n_act;
   const HfxRec *seg = c.rec + b;
   const bool real = r < R;    // bucket R holds rows bound to no replica
-  // ---- gather into contiguous records -----------------------------------------------------------------
-  if (SLABS) gather_to_records(a, c, R + 1, r, b, n_act, ordered, list_in, smem);
-
-  // ---- inactive rows of a step that is not ordered: listed by req_id behind the active ones ----
-  if (!ordered && n_in > 0) {
+  // ---- inactive rows: listed by req_id behind the active ones ----
+  if (n_in > 0) {
     const HfxRec *sin = seg + n_act;
     for (int q = threadIdx.x; q < n_in; q += blockDim.x)
       s_hi[q] = ((uint64_t)(ld_rec(sin + q, 0).z ^ 0x80000000u) << 16) | (uint32_t)q;     // signed req_id order, then position
@@ -1120,12 +1117,9 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
     const int kind = (w1.w >> 8) & 0xff, prio = (w1.w >> 16) & 0xff;
     RowEval e = eval_row(p, pl, base, kind, prio, (int32_t)w1.x, (int32_t)w1.y);
     if (kind == KIND_QUEUED && pl.mode != HFX_DECODE) e.k48 = (uint64_t)base;      // the front end has put the row's final key in place of the base
-    if (ordered) s_hi[q] = (e.k48 << 16) | (uint32_t)q;     // records are in req_id order: position breaks ties
-    else {
-      const uint32_t uid = w0.z ^ 0x80000000u;               // signed req_id order as unsigned
-      s_hi[q] = (e.k48 << 16) | (uid >> 16);
-      s_lo[q] = (uid << 16) | (uint32_t)q;
-    }
+    const uint32_t uid = w0.z ^ 0x80000000u;               // signed req_id order as unsigned
+    s_hi[q] = (e.k48 << 16) | (uid >> 16);
+    s_lo[q] = (uid << 16) | (uint32_t)q;
     if (kind == KIND_RUNNING || pl.mode == HFX_DECODE) {    // (the front end wrote the slack of the other queued rows)
       a.slack[row] = e.slack;
       if (a.key) a.key[row] = ((uint64_t)(r & 0xffff) << 48) | e.k48;
@@ -1134,11 +1128,8 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
   }
   __syncthreads();
   // ---- sort ------------------------------------------------------------------------------------------------
-  if (ordered) sort64_positions(s_hi, s_lo, n_act);
-  else {
-    group_sort<true>(s_hi, s_lo, n_act, B);
-    for (int q = threadIdx.x; q < n_act; q += blockDim.x) s_lo[q] &= 0xffffu;
-  }
+  group_sort<true>(s_hi, s_lo, n_act, B);
+  for (int q = threadIdx.x; q < n_act; q += blockDim.x) s_lo[q] &= 0xffffu;
   __syncthreads();
 
   // ---- admission -------------------------------------------------------------------------------------------
@@ -1157,7 +1148,7 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
   const int worked = sh.worked;
   const int64_t mat_next = sh.red_c[0];
   if (commit && !worked)      // idle replica: its next arrival is looked up among its listed inactive rows
-    group_min_arrival(next_arrival_part(a, c, p.n_replicas + 1, r, b, n_act, n, list_in || !ordered, B), sh, B);
+    group_min_arrival(next_arrival_part(a, c, p.n_replicas + 1, r, b, n_act, n, true, B), sh, B);
   if (threadIdx.x == 0 && real)
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
 
@@ -1181,7 +1172,10 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
 }
 
 // ------------------------------------------------------------------------------------------------
-// Larger replicas of an ordered step on the slab layout: the whole block with a distribution sort.
+// Larger replicas on the slab layout: the whole block with a distribution sort.
+// Ids that do not rise along the table (front ends that number their requests on their own): both lists are put in id
+// order first, by the same sort over ids, and the gather then places every row by its id; from there on the step is
+// an ordered one.  (96-bit items in a sorting network took 128 us for 96 replicas of 3125 rows.)
 // The replica's scratch range of c.rec (32 bytes per row, of which 20 per active row are used) holds three
 // arrays by position q in row order: slack base, then sort item (8 bytes); record words z, w (8); row (4).
 // Every pass reads them front to back; shared memory holds the binned items (afterwards the record words), the
@@ -1193,8 +1187,8 @@ static_assert((size_t)SEG_MED * 10 + MED_BINS * 4 <= SMEM_MED, "items, order and
 static_assert(MED_BINS / 8 == REP_THREADS, "every thread scans eight bins");
 
 template <bool FF>
-__device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act,
-                               bool list_in, unsigned char *smem, BlockShared &sh, uint64_t *s_cinfo, const ClassTab &tab) {
+__device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act,
+                             bool ordered, bool list_in, unsigned char *smem, BlockShared &sh, uint64_t *s_cinfo, const ClassTab &tab) {
   uint64_t *s_item = reinterpret_cast<uint64_t *>(smem);                          // [SEG_MED] items by bin
   uint2 *s_zw = reinterpret_cast<uint2 *>(smem);                                  // [SEG_MED] afterwards: record words by position; bit 31 of x: taken by first fit, of y: admitted
   uint16_t *s_ord = reinterpret_cast<uint16_t *>(smem + (size_t)SEG_MED * 8);     // [SEG_MED] position of the i-th row of the order
@@ -1207,20 +1201,52 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int R = p.n_replicas;
   const bool real = r < R;    // bucket R holds rows bound to no replica
+  const int n_in = n - n_act;
   const Grp B = {tid, REP_THREADS, 0};
   unsigned char *g = reinterpret_cast<unsigned char *>(c.rec + b);
   uint64_t *g_item = reinterpret_cast<uint64_t *>(g);
   uint2 *g_zw = reinterpret_cast<uint2 *>(g + (size_t)n_act * 8);
   int32_t *g_row = reinterpret_cast<int32_t *>(g + (size_t)n_act * 16);
 
-  // ---- gather into the scratch arrays; the inactive rows go straight to their places -------------------
-  gather_replica<REP_THREADS, 1, false, false>(c, R + 1, r, B, gather_tiles_at(smem, REP_THREADS, REP_THREADS), true, list_in,
-                 [&](uint32_t pos, const uint4 rec, int32_t row) {
-                   g_item[pos] = ((uint64_t)rec.y << 32) | rec.x; g_zw[pos] = make_uint2(rec.z, rec.w); g_row[pos] = row;
-                 },
-                 [&](uint32_t pos, int32_t row) { a.order[b + n_act + pos] = row; });
-  __syncthreads();
+  int32_t *g_ra = reinterpret_cast<int32_t *>(g + (size_t)n * 16), *g_ri = g_ra + n_act;      // (not ordered) rows as gathered, active and inactive
 
+  // three sorts, the first two of steps that are not ordered: the inactive rows by id, the active ones by id, the active ones by key
+  for (int stage = ordered ? 2 : 0; stage < 3; stage++) {
+  const int m = stage == 0 ? n_in : n_act;
+  // ---- gather: into the scratch arrays, the inactive rows straight to their places; or the rows of both lists ------
+  if (stage != 1) {
+    gather_replica<REP_THREADS, 1, false, false>(c, R + 1, r, B, gather_tiles_at(smem, REP_THREADS, REP_THREADS), true, stage == 0 || (ordered && list_in),
+                   [&](uint32_t pos, const uint4 rec, int32_t row) {
+                     if (stage == 0) { g_ra[pos] = row; return; }
+                     if (!ordered) pos = s_ord[pos];      // its place by id
+                     g_item[pos] = ((uint64_t)rec.y << 32) | rec.x; g_zw[pos] = make_uint2(rec.z, rec.w); g_row[pos] = row;
+                   },
+                   [&](uint32_t pos, int32_t row) { if (stage == 0) g_ri[pos] = row; else a.order[b + n_act + pos] = row; });
+    __syncthreads();
+  }
+
+  if (stage < 2) {
+    // ---- sort items of the ids, their range -------------------------------------------------------------
+    const int32_t *rows = stage == 0 ? g_ri : g_ra;
+    uint32_t lo = 0xffffffffu, hi = 0;
+#pragma unroll 4
+    for (int q = tid; q < m; q += REP_THREADS) {
+      const uint32_t uid = (uint32_t)__ldg(a.req_id + rows[q]) ^ 0x80000000u;      // signed order as unsigned
+      lo = uid < lo ? uid : lo; hi = uid > hi ? uid : hi;
+      g_item[q] = ((uint64_t)uid << 16) | (uint32_t)q;
+    }
+    for (int i = tid; i < MED_BINS / 2; i += REP_THREADS) s_bin[i] = 0;
+    lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) sh.red_m0[warp] = ((uint64_t)hi << 32) | lo;
+    __syncthreads();
+    if (warp == 0) {
+      const uint64_t x = sh.red_m0[lane];
+      lo = __reduce_min_sync(0xffffffffu, (uint32_t)x); hi = __reduce_max_sync(0xffffffffu, (uint32_t)(x >> 32));
+      const uint64_t range = m ? ((uint64_t)(hi - lo) << 16) | (uint32_t)(m - 1) : 0ull;      // (all in class 0)
+      const int bits = 64 - __clzll((long long)range);
+      if (lane == 0) s_cinfo[0] = (m ? (uint64_t)lo : 0ull) | ((uint64_t)(bits > 13 ? bits - 13 : 0) << 53) | (13ull << 59);
+    }
+  } else {
   // ---- aggregates, plan ---------------------------------------------------------------------------------
   {
     int64_t n_run = 0, sum_kv = 0;
@@ -1331,6 +1357,7 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
       run += 1u << lg[e];
     }
   }
+  }
   __syncthreads();
   auto bin_of = [&](uint64_t x) -> uint32_t {
     const uint64_t ci = s_cinfo[(uint32_t)(x >> 56)];
@@ -1340,7 +1367,7 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
     return ((uint32_t)(ci >> 40) & 0x1fffu) + (d < last ? (uint32_t)d : last);
   };
 #pragma unroll 4
-  for (int q = tid; q < n_act; q += REP_THREADS) {
+  for (int q = tid; q < m; q += REP_THREADS) {
     const uint32_t bi = bin_of(g_item[q]);
     atomicAdd(&s_bin[bi >> 1], 1u << ((bi & 1u) * 16));
   }
@@ -1376,34 +1403,48 @@ __device__ void medium_ordered(const HfxParams &p, const SegArgs &a, const SegCt
   __syncthreads();
   if (binned) {
 #pragma unroll 4
-    for (int q = tid; q < n_act; q += REP_THREADS) {
+    for (int q = tid; q < m; q += REP_THREADS) {
       const uint64_t x = g_item[q];
       const uint32_t bi = bin_of(x), sh16 = (bi & 1u) * 16;
       const uint32_t pos = (atomicAdd(&s_cur[bi >> 1], 1u << sh16) >> sh16) & 0xffffu;
       s_item[pos] = x;
     }
     __syncthreads();
-    for (int e = tid; e < n_act; e += REP_THREADS) {
+    for (int e = tid; e < m; e += REP_THREADS) {
       const uint64_t x = s_item[e];
       const uint32_t bi = bin_of(x), sh16 = (bi & 1u) * 16;
       const uint32_t g0 = (s_bin[bi >> 1] >> sh16) & 0xffffu, g1 = (s_cur[bi >> 1] >> sh16) & 0xffffu;
       uint32_t rank = 0;
       for (uint32_t k = g0; k < g1; k++) rank += s_item[k] < x ? 1u : 0u;
-      s_ord[g0 + rank] = (uint16_t)(x & 0xffffu);      // (the class ranges that s_ord overlays were last read when the bins were laid out)
+      s_ord[stage == 1 ? x & 0xffffu : g0 + rank] = (uint16_t)(stage == 1 ? g0 + rank : x & 0xffffu);      // (the class ranges that s_ord overlays were last read when the bins were laid out)
     }
   } else {      // a bin is too full: the sorting network
-    for (int q = tid; q < n_act; q += REP_THREADS) s_item[q] = g_item[q];
+    for (int q = tid; q < m; q += REP_THREADS) s_item[q] = g_item[q];
     __syncthreads();
-    sort64_positions(s_item, s_lo, n_act);
+    sort64_positions(s_item, s_lo, m);
     __syncthreads();
-    for (int q0 = 0; q0 < n_act; q0 += REP_THREADS) {      // 32-bit positions -> 16-bit, in place: a chunk's writes land on words already read
+    for (int q0 = 0; q0 < m; q0 += REP_THREADS) {      // 32-bit positions -> 16-bit, in place: a chunk's writes land on words already read
       const int q = q0 + tid;
-      const uint32_t v = q < n_act ? s_lo[q] : 0u;
+      const uint32_t v = q < m ? s_lo[q] : 0u;
       __syncthreads();
-      if (q < n_act) s_ord[q] = (uint16_t)v;
+      if (q < m) s_ord[q] = (uint16_t)v;
+    }
+    if (stage == 1) {      // the place of every position, by way of the items' memory
+      uint16_t *inv = reinterpret_cast<uint16_t *>(smem);
+      __syncthreads();
+      for (int q = tid; q < m; q += REP_THREADS) inv[s_ord[q]] = (uint16_t)q;
+      __syncthreads();
+      for (int q = tid; q < m; q += REP_THREADS) s_ord[q] = inv[q];
     }
   }
   __syncthreads();
+  if (stage == 0) {
+#pragma unroll 4
+    for (int q = tid; q < m; q += REP_THREADS) a.order[b + n_act + q] = g_ri[s_ord[q]];
+    __syncthreads();
+  }
+  }
+  const ReplicaPlan pl = sh.plan;
 
   // ---- the order; the record words by position, over the items -----------------------------------------
 #pragma unroll 4
@@ -1779,8 +1820,8 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
     const uint32_t need = need_of(n_all, n_act);
     if (need <= SEG_TINY) continue;
     const bool list_in = !ordered || n_all - n_act <= LIST_MAX;
-    if (SLABS && ordered && need <= SEG_MED) medium_ordered<FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, list_in, smem_raw, sh_g[0], s_cinfo_med, s_tab);
-    else if (need <= SEG_MED) medium_replica<SLABS, FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, ordered, list_in, smem_raw, sh_g[0]);
+    if (SLABS && need <= SEG_MED) medium_slabs<FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, ordered, list_in, smem_raw, sh_g[0], s_cinfo_med, s_tab);
+    else if (!SLABS && need <= SEG_MED) medium_replica<FF>(p, a, c, r, begin[r], (int)n_all, (int)n_act, smem_raw, sh_g[0]);
     else oversize_replica<SLABS, FF>(p, a, c, r, begin[r], n_all, n_act, ordered, list_in, smem_raw, sh_g[0]);
   }
 

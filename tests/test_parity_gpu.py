@@ -1238,3 +1238,18 @@ def test_replicas_of_few_active_rows_are_ranked_by_counting(n_act):
     wl = gen.random_table(n_act, 7 * n_act, 7, modes=MODES3, permute_ids=False, tie_heavy=True, inflight=0.4, done=0.0, future=0.0)
     wl.table["replica_id"][:] = np.arange(7 * n_act) % 7
     assert_step_parity(wl, steps=3, commit=True)
+
+
+@pytest.mark.parametrize("ids", ["spread", "crowded", "negative"])
+@pytest.mark.parametrize("n", [769, 3000, 16384])
+def test_larger_replicas_whose_ids_do_not_rise(n, ids):
+    # both lists of rows are put in id order by a distribution sort of their own: evenly spread ids, ids crowded beside a few far
+    # ones (the sorting network takes over), ids of both signs; many equal keys, so that the ids decide
+    rng = np.random.default_rng(n)
+    for share in (0.02, 0.5):      # rows that are not active
+        wl = gen.random_table(n, n, 1, modes=(gen.COLOCATED,), permute_ids=True, tie_heavy=True, inflight=0.2, done=share / 2, future=share / 2)
+        if ids == "crowded":
+            wl.table["req_id"][:] = np.where(np.arange(n) % 97 == 0, 2_000_000_000 - np.arange(n), rng.permutation(n))
+        elif ids == "negative":
+            wl.table["req_id"][:] = rng.permutation(n) * 250_000 - 2_000_000_000
+        assert_step_parity(wl, steps=2, commit=True)

@@ -455,35 +455,55 @@ __device__ void block_sort(uint64_t *hi, uint32_t *lo, int n) {
 // is called once for every place.  32 places at a time: the first lane that still fits starts a run, the
 // run ends at the first lane that no longer fits behind it (that lane is refused for good), the lanes after
 // it are tried again with what is left then.
+struct FirstFit { int64_t used = 0, taken = 0; };
+
+template <typename CostF, typename DecideF>
+__device__ __forceinline__ void warp_first_fit_32(FirstFit &f, int64_t base, int64_t n, int64_t budget, int64_t room, int lane, CostF cost_of, DecideF decide) {
+  const int64_t q = base + lane;
+  const int64_t c = q < n ? cost_of(q) : -1;
+  uint32_t pending = __ballot_sync(0xffffffffu, c >= 0);
+  bool mine = false;
+  while (pending) {
+    const int64_t rem = budget - f.used, left = room - f.taken;
+    const bool me = (pending >> lane) & 1u;
+    const uint32_t fit = left > 0 ? __ballot_sync(0xffffffffu, me && c <= rem) : 0u;
+    if (!fit) break;
+    const int l0 = __ffs(fit) - 1;
+    const bool in = me && lane >= l0;
+    const int64_t pre = warp_incl_scan_i64(in ? c : 0, lane);
+    const int32_t pcnt = warp_incl_scan_i32(in ? 1 : 0, lane);
+    const bool ok = in && pre <= rem && (int64_t)pcnt <= left;
+    const uint32_t bad = __ballot_sync(0xffffffffu, in && !ok);
+    const int l1 = bad ? __ffs(bad) - 1 : 32;            // the run is the pending lanes in [l0, l1)
+    const bool take = in && lane < l1;
+    if (take) mine = true;
+    const uint32_t tm = __ballot_sync(0xffffffffu, take);
+    const int last = 31 - __clz(tm);                      // tm has lane l0 at least
+    f.used += __shfl_sync(0xffffffffu, pre, last);
+    f.taken += __shfl_sync(0xffffffffu, pcnt, last);
+    pending = l1 >= 31 ? 0u : (pending & ~((2u << l1) - 1u));
+  }
+  if (q < n) decide(q, mine);
+}
+
 template <typename CostF, typename DecideF>
 __device__ __forceinline__ void warp_first_fit(int64_t n, int64_t budget, int64_t room, int lane, CostF cost_of, DecideF decide) {
-  int64_t used = 0, taken = 0;
-  for (int64_t base = 0; base < n; base += 32) {
-    const int64_t q = base + lane;
-    const int64_t c = q < n ? cost_of(q) : -1;
-    uint32_t pending = __ballot_sync(0xffffffffu, c >= 0);
-    bool mine = false;
-    while (pending) {
-      const int64_t rem = budget - used, left = room - taken;
-      const bool me = (pending >> lane) & 1u;
-      const uint32_t fit = left > 0 ? __ballot_sync(0xffffffffu, me && c <= rem) : 0u;
-      if (!fit) break;
-      const int l0 = __ffs(fit) - 1;
-      const bool in = me && lane >= l0;
-      const int64_t pre = warp_incl_scan_i64(in ? c : 0, lane);
-      const int32_t pcnt = warp_incl_scan_i32(in ? 1 : 0, lane);
-      const bool ok = in && pre <= rem && (int64_t)pcnt <= left;
-      const uint32_t bad = __ballot_sync(0xffffffffu, in && !ok);
-      const int l1 = bad ? __ffs(bad) - 1 : 32;            // the run is the pending lanes in [l0, l1)
-      const bool take = in && lane < l1;
-      if (take) mine = true;
-      const uint32_t tm = __ballot_sync(0xffffffffu, take);
-      const int last = 31 - __clz(tm);                      // tm has lane l0 at least
-      used += __shfl_sync(0xffffffffu, pre, last);
-      taken += __shfl_sync(0xffffffffu, pcnt, last);
-      pending = l1 >= 31 ? 0u : (pending & ~((2u << l1) - 1u));
-    }
-    if (q < n) decide(q, mine);
+  FirstFit f;
+  for (int64_t base = 0; base < n; base += 32) warp_first_fit_32(f, base, n, budget, room, lane, cost_of, decide);
+}
+
+// The same where the smallest cost of every 32 places (HFX_INF: no candidate) is known: only the 32s in which something may
+// still fit are looked at, and decide is called for their places alone.
+template <typename CostF, typename DecideF>
+__device__ __forceinline__ void warp_first_fit(int64_t n, const int64_t *min32, int64_t budget, int64_t room, int lane, CostF cost_of, DecideF decide) {
+  FirstFit f;
+  const int n32 = (int)((n + 31) >> 5);
+  for (int k = 0; k < n32 && f.taken < room;) {
+    const uint32_t some = __ballot_sync(0xffffffffu, k + lane < n32 && min32[k + lane] <= budget - f.used);
+    if (!some) { k += 32; continue; }
+    k += __ffs(some) - 1;
+    warp_first_fit_32(f, (int64_t)k * 32, n, budget, room, lane, cost_of, decide);
+    k++;
   }
 }
 

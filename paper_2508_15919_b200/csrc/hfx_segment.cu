@@ -1461,10 +1461,17 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
     kv = (int64_t)(zw.x & CREC_LEN_MASK) + (zw.y & CREC_LEN_MASK);
     return pl.mode == HFX_DECODE ? p.d1 + p.d2 * kv : (int64_t)(zw.x & CREC_LEN_MASK);
   };
-  if (FF) {     // first fit: the first warp walks the order and marks what it takes
+  if (FF) {     // first fit: the smallest cost of every 32 places by all warps, then the first warp walks the order and marks what it takes
+    int64_t *s_min = reinterpret_cast<int64_t *>(s_bin);      // [SEG_MED / 32] (the bins have served)
+    for (int q0 = warp * 32; q0 < n_act; q0 += REP_THREADS) {
+      int64_t kv, cc = q0 + lane < n_act ? cost_at(s_ord[q0 + lane], kv) : -1;
+      cc = warp_min_i64(cc < 0 ? HFX_INF : cc);
+      if (lane == 0) s_min[q0 >> 5] = cc;
+    }
+    __syncthreads();
     if (warp == 0) {
       const int64_t room = pl.batch_cap == 0 ? HFX_INF : (pl.batch_cap > pl.n_eff ? pl.batch_cap - pl.n_eff : 0);
-      warp_first_fit(n_act, pl.budget, room, lane, [&](int64_t q) -> int64_t { int64_t kv; return cost_at(s_ord[q], kv); },
+      warp_first_fit(n_act, s_min, pl.budget, room, lane, [&](int64_t q) -> int64_t { int64_t kv; return cost_at(s_ord[q], kv); },
                      [&](int64_t q, bool taken) { if (taken) s_zw[s_ord[q]].x |= 0x80000000u; });
     }
     __syncthreads();

@@ -81,6 +81,16 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
   // the dependent kernel may be scheduled as soon as SMs free up; it waits for this whole grid before it reads
   cudaTriggerProgrammaticLaunchCompletion();
 
+  stage_classes(p, s_ttft, s_tpot, s_prio);
+  for (int i = tid; i < R1; i += blockDim.x) {
+    s_cnt[2 * i] = 0; s_cnt[2 * i + 1] = 0;
+    if (has_next) s_next[i] = HFX_INF;
+  }
+  if (by_warp) for (int i = tid; i < 2 * R1 * (FRONT_WCNT_PITCH / 4); i += blockDim.x) s_wcnt[i] = 0;
+
+  // up to here the block may run beside the last kernel of the step before; everything below reads or writes global memory
+  cudaGridDependencySynchronize();
+
   const int64_t lo = (int64_t)blockIdx.x * T;
   const int64_t hi = lo + T < a.n ? lo + T : a.n;
   const int nt = hi > lo ? (int)(hi - lo) : 0;
@@ -106,15 +116,11 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     }
   }
 
-  stage_classes(p, s_ttft, s_tpot, s_prio);
   for (int i = tid; i < R1; i += blockDim.x) {
     const int64_t nw = i < R ? a.now[i] : 0, mt = i < R ? a.mat[i] : 0;
     s_now[i] = nw; s_start[i] = nw > mt ? nw : mt;
     s_mode[i] = i < R ? a.mode[i] : 0;
-    s_cnt[2 * i] = 0; s_cnt[2 * i + 1] = 0;
-    if (has_next) s_next[i] = HFX_INF;
   }
-  if (by_warp) for (int i = tid; i < 2 * R1 * (FRONT_WCNT_PITCH / 4); i += blockDim.x) s_wcnt[i] = 0;
   if (blockIdx.x == 0) {      // re-arm what the next step accumulates into
     for (int i = tid; i < R1; i += blockDim.x) a.tot_next[i] = 0ull;
     if (tid == 0) *a.ordered_next = 1u;
@@ -441,9 +447,16 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   fa.by_warp = fa.tile_rows <= FRONT_WCNT_ROWS && smem + wcnt <= HFX_FRONT_SMEM;
   if (fa.by_warp) smem += wcnt;
   KernelScope ks(s, KSLOT_FRONT);
-  if (fa.pred_ttft || fa.pred_tpot || fa.key) k_front<true><<<fa.n_tiles, FRONT_THREADS, smem, s->stream>>>(s->p, fa);
-  else k_front<false><<<fa.n_tiles, FRONT_THREADS, smem, s->stream>>>(s->p, fa);
-  return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(fa.n_tiles); cfg.blockDim = dim3(FRONT_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = s->profiling ? 0 : 1;      // set up while the step before drains
+  const cudaError_t e = fa.pred_ttft || fa.pred_tpot || fa.key ? cudaLaunchKernelEx(&cfg, k_front<true>, s->p, fa) : cudaLaunchKernelEx(&cfg, k_front<false>, s->p, fa);
+  return e == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }
 
 int hfx_front_configure() {

@@ -1749,6 +1749,7 @@ __global__ void __launch_bounds__(REP_THREADS, 1) k_replicas(const HfxParams p, 
   uint32_t *s_begin = reinterpret_cast<uint32_t *>(smem_raw + SMEM_MED);           // [R+2] range starts (slabs only)
   const int R = p.n_replicas, R1 = R + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  cudaTriggerProgrammaticLaunchCompletion();      // the next step's front end may be set up as soon as SMs free up; it waits for this whole grid before it reads
   class_tab_init(p, s_tab, tid);
   for (int k = tid; k < (int)(sizeof(s_long) / sizeof(uint32_t)); k += blockDim.x) s_long[k] = 0;
 

@@ -51,7 +51,7 @@ extern "C" {
 #define HFX_E_ALIGN      -2   /* a device pointer is not 16-byte aligned     */
 #define HFX_E_CAPACITY   -3   /* more rows / replicas than created for       */
 #define HFX_E_CUDA       -4   /* a CUDA runtime call failed (no device, ...) */
-#define HFX_E_TIMEOUT    -5   /* reserved: no kernel of this version waits on another block, so none can run out */
+#define HFX_E_TIMEOUT    -5   /* a bounded device-side wait ran out (hfx_dispatch_step's ordering kernel waits between its blocks; the others never do) */
 #define HFX_E_NOMEM      -6   /* workspace allocation failed                 */
 
 /* bits of the sticky device status word */
@@ -60,7 +60,7 @@ extern "C" {
                                    queue, bound to no instance yet                     */
 #define HFX_ST_BAD_CLASS    2u  /* class_id >= n_classes                      */
 #define HFX_ST_BAD_LEN      4u  /* prompt_len or gen outside [0, 2^24]        */
-#define HFX_ST_TIMEOUT      8u  /* reserved (see HFX_E_TIMEOUT)               */
+#define HFX_ST_TIMEOUT      8u  /* see HFX_E_TIMEOUT                           */
 
 /* request states (column `state`) */
 #define HFX_QUEUED    0
@@ -217,9 +217,9 @@ typedef struct hfx_sim_out {
 /* Create a scheduler.  `model`, `classes[n_classes]`, `replicas[n_replicas]`
  * and `opts` are host pointers, copied.  `max_rows` bounds n_rows of later
  * calls and sizes the workspace (about 51 bytes per row of device memory, 67
- * for tables of more than 16384 rows, plus 8 bytes per replica and tile of the
- * table -- a tile is about 1/148 of the rows, at most 8192 -- for up to 4095
- * replicas).  `cuda_stream` is a cudaStream_t (NULL = the default stream).  Errors: HFX_E_ARG (NULL pointer, value outside the domain
+ * for tables of more than 16384 rows, plus 18 bytes per replica and tile of the
+ * table (10 above 2047 replicas) -- a tile is about 1/148 of the rows, at most
+ * 8192 -- for up to 4095 replicas).  `cuda_stream` is a cudaStream_t (NULL = the default stream).  Errors: HFX_E_ARG (NULL pointer, value outside the domain
  * above), HFX_E_CUDA, HFX_E_NOMEM.  On error *out is NULL. */
 int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
                      const hfx_slo_class *classes, int n_classes,

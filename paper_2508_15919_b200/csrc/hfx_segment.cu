@@ -492,6 +492,20 @@ __device__ __forceinline__ void layout_class_bins(const uint32_t *s_ccnt, const 
 #define SMALL_SMEM (SEG_TINY * 24 + (TINY_BINS + 4) * 4 + TINY_CLASSES * 8)
 static_assert(SMALL_SMEM <= SMEM_GROUP, "a group's arrays fit its share of the block's shared memory");
 
+// What the ids change in a rank that was counted by (key, position).  Equal keys are rare enough here to fetch the ids (many of
+// them overfill a bin).  Not inlined: steps whose ids rise pay for every instruction beside theirs
+// (1024 replicas of 293 rows, permuted ids: 60.6 us with a sorting network on 96-bit items, 48.3 now).
+__device__ __noinline__ uint32_t rank_by_id(const uint64_t *items, const int32_t *rows, const int32_t *req_id, uint64_t x, uint32_t g0, uint32_t g1) {
+  uint32_t d = 0;
+  for (uint32_t g = g0; g < g1; g++) {
+    const uint64_t y = items[g];
+    if (((x ^ y) >> 16) != 0 || x == y) continue;
+    const int32_t ix = __ldg(req_id + rows[x & 0xffffu]), iy = __ldg(req_id + rows[y & 0xffffu]);
+    if (ix != iy && (iy < ix) != (y < x)) d += iy < ix ? 1u : ~0u;
+  }
+  return d;
+}
+
 template <bool SLABS, bool FF>
 __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx &c, const Grp &G, int r, uint32_t b, int n,
                               int n_act, bool ordered, bool list_in, unsigned char *smem, BlockShared &sh, const ClassTab &tab) {
@@ -606,17 +620,11 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
       RowEval e;
       if (given) { e.k48 = (uint64_t)base; e.slack = 0; e.pred_tpot = a.pred_tpot ? pl.tpot_q0 + p.d2 * ((int64_t)(zw.x & CREC_LEN_MASK) + (zw.y & CREC_LEN_MASK)) : 0; }
       else e = eval_row(p, pl, base, kind, prio, (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK));
-      if (ordered) {
-        item[k] = (e.k48 << 16) | (uint32_t)q;     // rows were gathered in req_id order: position breaks ties
-        if (few) s_bk[q] = item[k];
-        else {
-          const uint32_t cl = (uint32_t)(item[k] >> 56), sub = (uint32_t)(item[k] >> 24);
-          atomicMin(&s_cmin[cl], sub); atomicMax(&s_cmax[cl], sub); atomicAdd(&s_ccnt[cl], 1u);
-        }
-      } else {
-        const uint32_t uid = (uint32_t)__ldg(a.req_id + s_row[q]) ^ 0x80000000u;
-        s_bk[q] = (e.k48 << 16) | (uid >> 16);
-        s_lo[q] = (uid << 16) | (uint32_t)q;
+      item[k] = (e.k48 << 16) | (uint32_t)q;     // position breaks ties where rows were gathered in req_id order, else it leads to the id
+      if (few) s_bk[q] = item[k];
+      else {
+        const uint32_t cl = (uint32_t)(item[k] >> 56), sub = (uint32_t)(item[k] >> 24);
+        atomicMin(&s_cmin[cl], sub); atomicMax(&s_cmax[cl], sub); atomicAdd(&s_ccnt[cl], 1u);
       }
       if (kind == KIND_RUNNING || pl.mode == HFX_DECODE) {    // (the front end wrote the slack of the other queued rows)
         const int32_t row = s_row[q];
@@ -633,17 +641,18 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   // largest, so bins stay in item order; an item's place inside its bin comes from counting the smaller
   // items of the bin.
   bool sorted_done = false;
-  if (ordered && few) {
+  if (few) {
     G.sync();
     if (G.tid < n_act) {
       const uint64_t x = item[0];
       uint32_t rank = 0;
 #pragma unroll 8
       for (int g = 0; g < n_act; g++) rank += s_bk[g] < x ? 1u : 0u;
+      if (!ordered) rank += rank_by_id(s_bk, s_row, a.req_id, x, 0u, (uint32_t)n_act);
       s_lo[rank] = (uint32_t)G.tid;
     }
     sorted_done = true;
-  } else if (ordered) {
+  } else {
     G.sync();
     if (warp == 0) layout_class_bins<TINY_BINS>(s_ccnt, s_cmin, s_cmax, s_cinfo, (uint32_t)n_act, lane);
     G.sync();
@@ -704,12 +713,23 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
           const uint32_t g0 = (s_bin[bi >> 1] >> sh16) & 0xffffu, g1 = (s_cur[bi >> 1] >> sh16) & 0xffffu;
           uint32_t rank = 0;
           for (uint32_t g = g0; g < g1; g++) rank += s_bk[g] < x ? 1u : 0u;
+          if (!ordered) rank += rank_by_id(s_bk, s_row, a.req_id, x, g0, g1);
           s_lo[g0 + rank] = (uint32_t)(x & 0xffffu);      // (the class ranges that s_lo overlays were last read when the bins were laid out)
         }
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < TINY_IPT; k++) { const int q = G.tid + k * GROUP_THREADS; if (q < n_act) s_bk[q] = item[k]; }
+      for (int k = 0; k < TINY_IPT; k++) {
+        const int q = G.tid + k * GROUP_THREADS;
+        if (q < n_act) {
+          if (ordered) s_bk[q] = item[k];
+          else {
+            const uint32_t uid = (uint32_t)__ldg(a.req_id + s_row[q]) ^ 0x80000000u;
+            s_bk[q] = (item[k] & ~0xffffull) | (uid >> 16);
+            s_lo[q] = (uid << 16) | (uint32_t)q;
+          }
+        }
+      }
     }
   }
   G.sync();

@@ -1233,9 +1233,11 @@ def test_idle_replicas_find_their_next_arrivals(R, rows_per):
     assert_step_parity(wl, steps=3, commit=True, optional=False)
 
 
-@pytest.mark.parametrize("n_act", [1, 127, 128, 129])
-def test_replicas_of_few_active_rows_are_ranked_by_counting(n_act):
-    wl = gen.random_table(n_act, 7 * n_act, 7, modes=MODES3, permute_ids=False, tie_heavy=True, inflight=0.4, done=0.0, future=0.0)
+@pytest.mark.parametrize("permute", [False, True])
+@pytest.mark.parametrize("n_act", [1, 127, 128, 129, 500, 768])
+def test_replicas_of_few_active_rows_are_ranked_by_counting(n_act, permute):
+    # up to 128 rows against all the others, more inside bins; equal keys go by position, or by the id where ids do not rise
+    wl = gen.random_table(n_act, 7 * n_act, 7, modes=MODES3, permute_ids=permute, tie_heavy=True, inflight=0.4, done=0.0, future=0.0)
     wl.table["replica_id"][:] = np.arange(7 * n_act) % 7
     assert_step_parity(wl, steps=3, commit=True)
 

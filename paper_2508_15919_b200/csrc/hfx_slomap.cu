@@ -87,10 +87,11 @@ __global__ void __launch_bounds__(SLO_WIN_THREADS) k_slo_window(const SloArgs a)
       int hp = 0;      // a higher priority pending?
       for (int i = 0; i < tid; i++) hp |= a.pending[i] > 0;
       a.tab->higher_pending[tid] = hp;
-      a.tab->first_row[a.par ^ 1][tid] = ~0ull;
       if (tid == 0) a.tab->w_valid = (int32_t)all;
     }
   }
+  // (all entries: the call that used the other copy, or the one that will, may have more priorities than this one)
+  if (blockIdx.x == 0 && tid < HFX_MAX_CLASSES) a.tab->first_row[a.par ^ 1][tid] = ~0ull;
   if (bad && blockIdx.x == 0) atomicOr(a.status, bad);
   __syncthreads();
   // Ranks among the valid records, ties by position.  A warp counts for four neighbouring records, so a value read from

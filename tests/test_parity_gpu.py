@@ -627,6 +627,35 @@ def test_slo_mapping_random(seed):
     _slo_parity(N, win, bounds, last, pending, new)
 
 
+@pytest.mark.parametrize("counts", [(16, 4, 16, 4, 16), (64, 1, 33, 64, 64), (1, 64, 2, 64)])
+def test_slo_mapping_calls_with_different_numbers_of_priorities(counts):
+    # The number of priorities is an argument of the call: on one scheduler, what a call with many of them leaves in the table must not
+    # reach a later one behind a call with few.  Every call's first requests lie further back than those of the call before.
+    import paper_2508_15919_b200 as hfx
+    rng = np.random.default_rng(sum(counts))
+    wl = gen.random_table(1, 16, 1)
+    sched = make_sched(wl)
+    dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a, dt)).cuda()
+    last = {N: rng.integers(0, 10**9, N) for N in counts}      # per number of priorities: its own delays
+    for k, N in enumerate(counts):
+        win = {"prio": rng.integers(0, N, 700), "ttft": rng.integers(1, 10**10, 700), "tpot": rng.integers(1, 10**9, 700), "queue": rng.integers(0, 10**9, 700)}
+        bounds = {"ttft_min": np.full(N, -10**12), "ttft_max": np.full(N, 10**12), "ttft_min_relaxed": np.full(N, -10**12),
+                  "tpot_min": np.zeros(N, np.int64), "tpot_max": np.full(N, 10**12), "tpot_min_relaxed": np.zeros(N, np.int64)}
+        pending = rng.integers(0, 2, N)
+        new = np.concatenate([np.zeros(500 * k, np.int64), rng.permutation(np.arange(3000) % N)])
+        w = {q + ("" if q == "prio" else "_ns"): dev(v, np.int32 if q == "prio" else np.int64) for q, v in win.items()}
+        b = {q + "_ns": dev(v, np.int64) for q, v in bounds.items()}
+        lq, t_out, p_out = dev(last[N], np.int64), dev(np.zeros(len(new)), np.int64), dev(np.zeros(len(new)), np.int64)
+        sched.slo_map(N, w, b, lq, dev(pending, np.int32), dev(new, np.int32), t_out, p_out)
+        st = sched.status()
+        c = oracle.slo_map(N, win, bounds, np.ascontiguousarray(last[N], np.int64), pending, new)
+        assert st == c["status"] == 0
+        assert np.array_equal(t_out.cpu().numpy(), c["ttft_slo"]), (k, N, np.nonzero(t_out.cpu().numpy() != c["ttft_slo"])[0][:8])
+        assert np.array_equal(p_out.cpu().numpy(), c["tpot_slo"]) and np.array_equal(lq.cpu().numpy(), c["last_queue"])
+        last[N] = c["last_queue"]
+    sched.close()
+
+
 # ---- the two stages of the disaggregated mode coupled by the hand-off --------------------------------------
 def _pd_coupled_parity(wl, pair, rounds, x0=2 * MS, x1=500):
     """`rounds` times (committed step, hand-off) on both sides; the table, the clocks and the step's

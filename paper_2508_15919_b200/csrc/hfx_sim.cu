@@ -494,6 +494,9 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           nq = to;
         }
         if (nq == 0 && box == 0) min_prompt = INT32_MAX;
+        // An admitted request is noted by the lane that holds it, and the commit reads the notes with other lanes (shuffles and
+        // ballots between the two do not order memory).
+        if (adm_cnt > 0) __syncwarp();
       }
 
       // ---- a stretch of iterations in which nothing arrives, finishes or is admitted -------------------------

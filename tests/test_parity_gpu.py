@@ -1188,6 +1188,22 @@ def test_simulator_windows_merge_and_many_are_admitted_at_once(m, first_fit):
     assert_sim_parity(wl)
 
 
+@pytest.mark.parametrize("first_fit", [False, True])
+@pytest.mark.parametrize("clump", [1, 7, 20, 31, 64])
+def test_simulator_admits_from_the_window_alone(clump, first_fit):
+    # Requests arrive a few at a time and are admitted at once, from the window: the queue's list stays empty while it lasts, and
+    # outputs are long, so nobody finishes.  Nothing but the admission itself then lies between a note of it and the commit.
+    m = 640
+    rng = np.random.default_rng(clump)
+    rows = [dict(prompt_len=int(rng.choice([1, 5, 30])), arrival_ns=(i // clump) * 25 * MS, output_len=20_000 + int(rng.integers(0, 9)), class_id=int(rng.integers(0, 3)),
+                 req_id=int(i ^ 5)) for i in range(m)]
+    wl = make_wl(rows, [(2000 * MS, 300 * MS, 0), (0, 0, 1), (1000 * MS, 500 * MS, 1)], replicas=[(gen.COLOCATED, 16384, 0)], trace_off=[0, m], sim_iters=2500)
+    if first_fit:
+        wl.meta["first_fit"] = True
+    res = assert_sim_parity(wl)
+    assert res["finished"][0] == 0
+
+
 @pytest.mark.parametrize("n_classes", [1, 4, 5, 8, 9, 64])
 def test_attainment_class_counts_and_ragged_rows(n_classes):
     # totals in registers (up to 4, up to 8 classes) and per warp (more); a row is left over when n is odd

@@ -654,6 +654,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
       }
       // the TTFT samples, closed up over the slots of rows already looked at (their order does not matter)
       const uint32_t sm = __ballot_sync(FULL, ttft >= 0);
+      __syncwarp();                           // (a request still in flight has had its admission iteration read from a slot that is written now)
       if (ttft >= 0) s_slot[n_ttft + __popc(sm & lt)] = ttft;
       n_ttft += __popc(sm);
       __syncwarp();

@@ -21,3 +21,9 @@ def test_simulator_orders_an_admission_before_its_commit():
     between = src[last_note:src.index("parked(e0")]
     # in a block that every iteration with an admission passes (not inside `if (from_list)` or a loop over the list)
     assert re.search(r"if \(adm_cnt > 0\) __syncwarp\(\);", between)
+
+
+def test_simulator_orders_reading_a_slot_before_the_samples_overwrite_it():
+    # the TTFT samples are closed up over the slots of the same 32 rows, of which those in flight are read just before
+    src = _source("hfx_sim.cu")
+    assert "__syncwarp();" in _between(src, "s_slot[i] >> 32);\n            last", "s_slot[n_ttft")

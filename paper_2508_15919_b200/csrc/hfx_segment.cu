@@ -500,7 +500,7 @@ __device__ __noinline__ uint32_t rank_by_id(const uint64_t *items, const int32_t
   for (uint32_t g = g0; g < g1; g++) {
     const uint64_t y = items[g];
     if (((x ^ y) >> 16) != 0 || x == y) continue;
-    const int32_t ix = __ldg(req_id + rows[x & 0xffffu]), iy = __ldg(req_id + rows[y & 0xffffu]);
+    const int32_t ix = req_id[rows[x & 0xffffu]], iy = req_id[rows[y & 0xffffu]];
     if (ix != iy && (iy < ix) != (y < x)) d += iy < ix ? 1u : ~0u;
   }
   return d;
@@ -541,9 +541,9 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
       gather_replica<GROUP_THREADS, GROUP_TPT, true, false>(c, R1, r, G, gt, false, true, [](uint32_t, const uint4, int32_t) {},
                                                             [&](uint32_t pos, int32_t row) { s_row[pos] = row; });
     else
-      for (int q = G.tid; q < n_in; q += G.n) s_row[q] = (int32_t)__ldg(reinterpret_cast<const uint4 *>(seg + n_act + q)).w;
+      for (int q = G.tid; q < n_in; q += G.n) s_row[q] = (int32_t)reinterpret_cast<const uint4 *>(seg + n_act + q)->w;
     G.sync();
-    for (int q = G.tid; q < n_in; q += G.n) s_bk[q] = ((uint64_t)((uint32_t)__ldg(a.req_id + s_row[q]) ^ 0x80000000u) << 16) | (uint32_t)q;
+    for (int q = G.tid; q < n_in; q += G.n) s_bk[q] = ((uint64_t)((uint32_t)a.req_id[s_row[q]] ^ 0x80000000u) << 16) | (uint32_t)q;
     G.sync();
     group_sort<false>(s_bk, nullptr, n_in, G);
     for (int q = G.tid; q < n_in; q += G.n) a.order[b + n_act + q] = s_row[s_bk[q] & 0xffffu];
@@ -558,8 +558,8 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
     cp_async_wait_all();
   } else {
     for (int q = G.tid; q < n_act; q += G.n) {
-      const uint4 w0 = __ldg(reinterpret_cast<const uint4 *>(seg + q));
-      const uint4 w1 = __ldg(reinterpret_cast<const uint4 *>(seg + q) + 1);
+      const uint4 w0 = reinterpret_cast<const uint4 *>(seg + q)[0];
+      const uint4 w1 = reinterpret_cast<const uint4 *>(seg + q)[1];
       s_bk[q] = ((uint64_t)w0.y << 32) | w0.x;
       s_zw[q] = make_uint2(w1.x | (((w1.w >> 8) & 1u) << CREC_KIND_SHIFT) | (((w1.w >> 16) & 0x3fu) << CREC_PRIO_SHIFT),
                            w1.y | ((w1.w & 0x3fu) << CREC_CLS_SHIFT));
@@ -612,7 +612,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
     item[k] = ~0ull;
     out_len[k] = 0;
     if (q < n_act) {
-      if (will_commit && ((s_zw[q].x >> CREC_KIND_SHIFT) & 1u) == KIND_RUNNING) out_len[k] = __ldg(a.output_len + s_row[q]);
+      if (will_commit && ((s_zw[q].x >> CREC_KIND_SHIFT) & 1u) == KIND_RUNNING) out_len[k] = a.output_len[s_row[q]];
       const int64_t base = (int64_t)s_bk[q];
       const uint2 zw = s_zw[q];
       const int kind = (zw.x >> CREC_KIND_SHIFT) & 1, prio = zw.x >> CREC_PRIO_SHIFT;
@@ -724,7 +724,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
         if (q < n_act) {
           if (ordered) s_bk[q] = item[k];
           else {
-            const uint32_t uid = (uint32_t)__ldg(a.req_id + s_row[q]) ^ 0x80000000u;
+            const uint32_t uid = (uint32_t)a.req_id[s_row[q]] ^ 0x80000000u;
             s_bk[q] = (item[k] & ~0xffffull) | (uid >> 16);
             s_lo[q] = (uid << 16) | (uint32_t)q;
           }
@@ -833,7 +833,7 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
         const uint2 zw = s_zw[q];
         const int kind = (zw.x >> CREC_KIND_SHIFT) & 1;
         const bool adm = (zw.y >> 31) != 0;
-        const int32_t ol = adm ? __ldg(a.output_len + s_row[q]) : out_len[k];
+        const int32_t ol = adm ? a.output_len[s_row[q]] : out_len[k];
         commit_row(a, pl, kind, adm, worked, t1, t2, s_row[q], (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK), ol);
       }
     }
@@ -854,7 +854,7 @@ __device__ void gather_to_records(const SegArgs &a, const SegCtx &c, int R1, int
   gather_replica<REP_THREADS, 1, false, false>(c, R1, r, B, gather_tiles_at(smem, REP_THREADS, REP_THREADS), true, list_in || !ordered,
                  [&](uint32_t pos, const uint4 rec, int32_t row) {
                    uint4 w0, w1;
-                   w0.x = rec.x; w0.y = rec.y; w0.z = ordered ? 0u : (uint32_t)__ldg(a.req_id + row); w0.w = (uint32_t)row;
+                   w0.x = rec.x; w0.y = rec.y; w0.z = ordered ? 0u : (uint32_t)a.req_id[row]; w0.w = (uint32_t)row;
                    w1.x = rec.z & CREC_LEN_MASK; w1.y = rec.w & CREC_LEN_MASK; w1.z = 0;
                    w1.w = (rec.w >> CREC_CLS_SHIFT) | (((rec.z >> CREC_KIND_SHIFT) & 1u) << 8) | ((rec.z >> CREC_PRIO_SHIFT) << 16);
                    uint4 *dst = reinterpret_cast<uint4 *>(seg + pos);
@@ -864,7 +864,7 @@ __device__ void gather_to_records(const SegArgs &a, const SegCtx &c, int R1, int
                    if (ordered) a.order[b + n_act + pos] = row;
                    else {
                      uint4 *dst = reinterpret_cast<uint4 *>(seg + n_act + pos);
-                     dst[0] = make_uint4(0u, 0u, (uint32_t)__ldg(a.req_id + row), (uint32_t)row);
+                     dst[0] = make_uint4(0u, 0u, (uint32_t)a.req_id[row], (uint32_t)row);
                      dst[1] = make_uint4(0u, 0u, 0u, KIND_DEAD << 8);
                    }
                  });
@@ -1184,7 +1184,7 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
       const uint4 w1 = ld_rec(seg + li, 1);
       const int kind = (w1.w >> 8) & 0xff;
       const bool adm = (lo & 0x10000u) != 0;
-      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? __ldg(a.output_len + (int32_t)w0.w) : 0;
+      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? a.output_len[(int32_t)w0.w] : 0;
       commit_row(a, pl, kind, adm, worked, t1, t2, (int32_t)w0.w, (int32_t)w1.x, (int32_t)w1.y, out_len);
     }
   }
@@ -1251,7 +1251,7 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
     uint32_t lo = 0xffffffffu, hi = 0;
 #pragma unroll 4
     for (int q = tid; q < m; q += REP_THREADS) {
-      const uint32_t uid = (uint32_t)__ldg(a.req_id + rows[q]) ^ 0x80000000u;      // signed order as unsigned
+      const uint32_t uid = (uint32_t)a.req_id[rows[q]] ^ 0x80000000u;      // signed order as unsigned
       lo = uid < lo ? uid : lo; hi = uid > hi ? uid : hi;
       g_item[q] = ((uint64_t)uid << 16) | (uint32_t)q;
     }
@@ -1568,7 +1568,7 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
       const int kind = (zw.x >> CREC_KIND_SHIFT) & 1;
       const bool adm = (zw.y >> 31) != 0;
       const int32_t row = g_row[q];
-      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? __ldg(a.output_len + row) : 0;
+      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? a.output_len[row] : 0;
       commit_row(a, pl, kind, adm, worked, t1, t2, row, (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK), out_len);
     }
   }
@@ -1748,7 +1748,7 @@ __device__ void oversize_replica(const HfxParams &p, const SegArgs &a, const Seg
       const uint4 w1 = ld_rec(seg + li, 1);
       const int kind = (w1.w >> 8) & 0xff;
       const bool adm = lo[q] != 0;
-      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? __ldg(a.output_len + (int32_t)w0.w) : 0;
+      const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? a.output_len[(int32_t)w0.w] : 0;
       commit_row(a, pl, kind, adm, worked, t1, t2, (int32_t)w0.w, (int32_t)w1.x, (int32_t)w1.y, out_len);
     }
   }

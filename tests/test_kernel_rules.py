@@ -27,3 +27,32 @@ def test_simulator_orders_reading_a_slot_before_the_samples_overwrite_it():
     # the TTFT samples are closed up over the slots of the same 32 rows, of which those in flight are read just before
     src = _source("hfx_sim.cu")
     assert "__syncwarp();" in _between(src, "s_slot[i] >> 32);\n            last", "s_slot[n_ttft")
+
+
+def _functions(src, word):
+    """(header, body) of every function definition that is introduced by `word`."""
+    out = []
+    for m in re.finditer(word, src):
+        brace = re.compile(r"[{;]").search(src, m.end())      # (a declaration ends without a body)
+        if brace is None or brace.group() == ";":
+            continue
+        depth, i = 1, brace.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[i], 0)
+            i += 1
+        out.append((src[m.start():brace.start()], src[brace.end():i]))
+    return out
+
+
+def test_kernels_set_up_beside_the_one_in_front_read_nothing_through_the_read_only_path():
+    # That path is for data that nothing writes while the kernel lives, and such a kernel lives while the one in front still writes.
+    seen = set()
+    for name in sorted(os.listdir(CSRC)):
+        src = _source(name)
+        kernels = _functions(src, r"__global__")
+        early = [(h, b) for h, b in kernels if "cudaGridDependencySynchronize" in b]
+        helpers = _functions(src, r"__device__") if kernels and len(early) == len(kernels) else []      # (a file of such kernels alone: its helpers too)
+        for head, body in early + helpers:
+            assert "__ldg(" not in body and "ld.global.nc" not in body and not re.search(r"const \w+ \*\s*__restrict__", head), (name, head)
+        seen |= {re.search(r"\b(k_\w+)\s*\(", h).group(1) for h, _ in early}
+    assert {"k_front", "k_replicas", "k_pd_rows", "k_pd_clock", "k_slo_assign", "k_disp_chain", "k_disp_assign"} <= seen

@@ -701,6 +701,39 @@ def test_pd_coupled_stages(seed, pairs, rows_per):
     assert np.all(t["first_token_ns"][done] <= t["finish_ns"][done]) and np.all(t["arrival_ns"][done] <= t["first_token_ns"][done])
 
 
+@pytest.mark.parametrize("pairs,rows_per", [(1, 40), (3, 200), (16, 1500)])
+def test_calls_that_follow_each_other_without_a_host_wait(pairs, rows_per):
+    # Every kernel of the loop is set up while the one in front still runs: what one wrote (and what other code on the stream wrote
+    # between two calls) is what the next one reads.
+    import paper_2508_15919_b200 as hfx
+    wl = gen.pd_pairs(7, pairs, rows_per)
+    cpu = wl.copy()
+    pair = gen.pd_partner_table(pairs)
+    sched = make_sched(wl)
+    tab = hfx.DeviceTable.from_numpy(wl.table)
+    now = torch.from_numpy(wl.now.copy()).cuda(); mat = torch.from_numpy(wl.maturity.copy()).cuda()
+    prt = torch.from_numpy(pair).cuda()
+    out = hfx.StepOut(wl.n_rows, wl.n_replicas, optional=False)
+    drop = [np.arange(k, wl.n_rows, 97) for k in range(8)]
+    drop_gpu = [torch.from_numpy(d).cuda() for d in drop]
+    torch.cuda.synchronize()
+    for k in range(40):
+        if k % 5 == 4:      # some requests are withdrawn
+            tab.cols["state"][drop_gpu[k // 5]] = gen.REJECTED
+            cpu.table["state"][drop[k // 5]] = gen.REJECTED
+        sched.step(tab, now, mat, out, commit=True)
+        sched.pd_migrate(tab, now, mat, prt, 2 * MS, 500)
+        c = oracle.step(cpu, commit=True)
+        oracle.pd_migrate(cpu, pair, 2 * MS, 500)
+    g, t = out.to_numpy(), tab.to_numpy()
+    for ko, kg in (("order", "order"), ("admit", "admit"), ("budget", "budget"), ("adm_count", "adm_count"), ("slack", "slack_ns")):
+        assert np.array_equal(g[kg], c[ko]), kg
+    for col in ("replica_id", "state", "gen", "first_token_ns", "last_token_ns", "finish_ns"):
+        assert np.array_equal(t[col], cpu.table[col]), col
+    assert np.array_equal(now.cpu().numpy(), cpu.now) and np.array_equal(mat.cpu().numpy(), cpu.maturity)
+    sched.close()
+
+
 def test_pd_handoff_edges_and_errors():
     import paper_2508_15919_b200 as hfx
     # bad partners, rows with bad data, an empty table; argument errors

@@ -533,6 +533,11 @@ int hfx_sched_set_fused_front(hfx_sched *s, int on);
  * to the horizon still acts.  The default, INT64_MAX, gates nothing.  Host call, takes effect at the
  * next hfx_sched_step; the simulator is not affected. */
 int hfx_sched_set_horizon(hfx_sched *s, int64_t horizon_ns);
+/* How often a device-side wait polls before it gives up (hfx_dispatch_step's ordering kernel; the others never
+ * wait): 0 .. 2^26, by default 2^22, about two seconds.  A call that gave up raises HFX_ST_TIMEOUT and hands out
+ * nothing: assign, queue_order and inst_order are -1 throughout, n_queue, n_mature, adm_cost and adm_count 0,
+ * maturity_next = maturity_ns; the next call starts afresh.  Host call, takes effect at the next hfx_dispatch_step. */
+int hfx_sched_set_wait_limit(hfx_sched *s, uint32_t polls);
 int hfx_sched_get_profile(hfx_sched *s, hfx_profile *out);
 const char *hfx_kernel_name(int slot);
 

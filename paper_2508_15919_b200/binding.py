@@ -22,7 +22,7 @@ E_ARG, E_ALIGN, E_CAPACITY, E_CUDA, E_TIMEOUT, E_NOMEM = -1, -2, -3, -4, -5, -6
 EXPORTED_SYMBOLS = ["hfx_sched_create", "hfx_sched_step", "hfx_sim_run", "hfx_sched_status",
                     "hfx_sched_launch_count", "hfx_sched_destroy", "hfx_strerror", "hfx_sched_set_profiling",
                     "hfx_sched_get_profile", "hfx_sched_set_fused_front", "hfx_kernel_name", "hfx_count_rows_noalloc", "hfx_scale_tick", "hfx_dispatch_step", "hfx_slo_map", "hfx_pd_migrate", "hfx_attainment",
-                    "hfx_sched_set_horizon", "hfx_scale_apply", "hfx_dispatch_bind", "hfx_scale_decide"]
+                    "hfx_sched_set_horizon", "hfx_sched_set_wait_limit", "hfx_scale_apply", "hfx_dispatch_bind", "hfx_scale_decide"]
 NOALLOC_MAX_REPLICAS = 4096
 N_KERNELS = 14
 
@@ -163,6 +163,8 @@ def load_library():
     L.hfx_sched_set_profiling.argtypes = [C.c_void_p, C.c_int]
     L.hfx_sched_set_horizon.restype = C.c_int
     L.hfx_sched_set_horizon.argtypes = [C.c_void_p, C.c_int64]
+    L.hfx_sched_set_wait_limit.restype = C.c_int
+    L.hfx_sched_set_wait_limit.argtypes = [C.c_void_p, C.c_uint32]
     L.hfx_scale_decide.restype = C.c_int
     L.hfx_scale_decide.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(_ScaleParams), C.POINTER(_ScaleOut)]
     L.hfx_scale_apply.restype = C.c_int
@@ -399,6 +401,12 @@ class Scheduler:
         rc = self._L.hfx_sched_set_horizon(self._h, int(np.iinfo(np.int64).max if horizon_ns is None else horizon_ns))
         if rc != 0:
             raise HfxError(rc, "hfx_sched_set_horizon")
+
+    def set_wait_limit(self, polls: int):
+        """Polls of a device-side wait before the dispatching call gives up (HFX_ST_TIMEOUT); the default is about two seconds."""
+        rc = self._L.hfx_sched_set_wait_limit(self._h, int(polls))
+        if rc != 0:
+            raise HfxError(rc, "hfx_sched_set_wait_limit")
 
     def pd_migrate(self, table: DeviceTable, now: torch.Tensor, maturity: torch.Tensor, pair: torch.Tensor,
                    xfer_c0_ns: int, xfer_c1_ns: int, n_moved: Optional[torch.Tensor] = None):

@@ -129,6 +129,7 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
   ok = ok && cudaMalloc(&s->d_pd, hfx_pd_workspace_bytes(n_replicas)) == cudaSuccess;
   ok = ok && cudaMemset(s->d_pd, 0, hfx_pd_workspace_bytes(n_replicas)) == cudaSuccess;
   s->horizon = INT64_MAX;
+  s->wait_limit = HFX_WAIT_LIMIT;
   s->front_enabled = 1; s->tot_parity = 0;
   ok = ok && cudaMalloc(&h->d_trace_off, sizeof(int32_t) * R2) == cudaSuccess;
   ok = ok && cudaMalloc(&h->d_work_counter, 256) == cudaSuccess;
@@ -344,6 +345,12 @@ extern "C" int hfx_sched_set_profiling(hfx_sched *s, int on) {
 extern "C" int hfx_sched_set_fused_front(hfx_sched *s, int on) {
   if (!s) return HFX_E_ARG;
   s->front_enabled = on ? 1 : 0;
+  return HFX_OK;
+}
+
+extern "C" int hfx_sched_set_wait_limit(hfx_sched *s, uint32_t polls) {
+  if (!s || polls > (1u << 26)) return HFX_E_ARG;
+  s->wait_limit = polls;
   return HFX_OK;
 }
 

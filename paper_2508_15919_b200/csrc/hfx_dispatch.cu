@@ -39,7 +39,6 @@
 #define CHAIN_WIN 256               // and held in registers by the walking warp, eight per lane
 #define CHAIN_BATCH 6               // instances between two looks at whether all went well
 #define ASSIGN_THREADS 256
-#define DISP_WAIT_LIMIT (1u << 22)  // polls of the grid barrier before the kernel gives up (about two seconds)
 
 // words of the control block, zero between calls unless noted
 enum { CTL_QMASK = 0, CTL_DMASK, CTL_FALLS, CTL_BMAX0, CTL_BMAX1, CTL_BARRIER, CTL_N0, CTL_N1, CTL_NM0, CTL_NM1, CTL_TAKEN0, CTL_TAKEN1, CTL_ABORT, CTL_ITEMS,
@@ -64,6 +63,7 @@ struct DispWork {
   int64_t *ord_budget; int32_t *ord_room; int32_t *ord_id;      // [R] matured instances in order, stage 0, then stage 1
   int32_t *run_end;                                               // [R] where its run ends in its stage's queue
   int64_t max_rows; int32_t R, blocks, tiles_max;
+  uint32_t wait_limit;       // polls of a grid barrier before the kernel gives up
 };
 
 struct DispArgs {
@@ -242,7 +242,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 
 // ------------------------------------------------------------------------------------------------
 // k_disp_sort.  Four phases between grid barriers (the launch is cooperative, so every block is resident; a barrier that
-// is not reached in time makes every block return with HFX_ST_TIMEOUT raised).
+// is not reached in time makes every block return with HFX_ST_TIMEOUT and CTL_ABORT raised; the kernels behind it then hand out
+// nothing: the queue, its running totals and the tiles may be unwritten).
 //   0  plan of every instance and its place in the maturity order, a warp per instance; the sample in order, a warp
 //      per sampled item counting the smaller ones
 //   1  every item's bin, and its place in it from a global counter.  Every eighth sample of a (stage, priority) starts an
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 // its running totals: about 170 us in 20 launches before, 90 us now, of it a good third latency between the phases (a queue
 // of 42 K: 41 us); the counters of the bins (26 K cycles) and the tiles (36 K) are the rest.
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t &round, uint32_t *s_ok) {
+__device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
   __threadfence();
   __syncthreads();
@@ -266,7 +267,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *
       uint32_t polls = 0;
       volatile unsigned long long *v = ctl;
       while (v[CTL_BARRIER] < target)
-        if (++polls > DISP_WAIT_LIMIT || v[CTL_ABORT]) { ok = 0; break; }
+        if (++polls > limit || v[CTL_ABORT]) { ok = 0; break; }
     }
     if (!ok) { ctl[CTL_ABORT] = 1; atomicOr(status, HFX_ST_TIMEOUT); }
     __threadfence();
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     if (s_nm[tid]) atomicAdd(&w.ctl[CTL_NM0 + tid], (unsigned long long)s_nm[tid]);
     if (s_bmax[tid]) atomicMax(&w.ctl[CTL_BMAX0 + tid], s_bmax[tid]);
   }
-  if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+  if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
 
   // ---- 1: bins -------------------------------------------------------------------------------------------------
   if (blockIdx.x == 0) {
@@ -493,7 +494,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   }
   __syncthreads();
   if (tid == 0 && s_n1) atomicAdd(&w.ctl[CTL_N1], (unsigned long long)s_n1);
-  if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+  if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
 
   // ---- 2: items to their bins ------------------------------------------------------------------------------------
   const uint32_t n1 = (uint32_t)__ldcg(w.ctl + CTL_N1), n0 = n_all - n1;
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 #pragma unroll
       for (int e = 0; e < ITEMS_AT_ONCE; e++) { const uint32_t q = q0 + e * SORT_THREADS; if (q < hi) { const uint32_t bn = rk[e] >> 16; w.item[0][s_start[bn] + (rk[e] & 0xffffu)] = x[e]; } }
     }
-    if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+    if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
   } else {
     // radix sort, 8 bits a pass: the tie word, then the key (47 bits).  A block counts the digits of its share, adds up the
     // counts of the blocks before it, and places its items 1024 at a time in order.
@@ -532,7 +533,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       for (uint32_t q = lo + tid; q < hi; q += SORT_THREADS) atomicAdd(&s_digit[digit(__ldcg(src + q))], 1u);
       __syncthreads();
       if (tid < 256) w.hist[blockIdx.x * 256 + tid] = s_digit[tid];
-      if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+      if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
       {
         uint32_t before = 0, total = 0;
         if (tid < 256)
@@ -563,7 +564,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
         if (in) dst[s_wc[warp * 256 + d] + __popc(same & ((1u << lane) - 1u))] = x;
         __syncthreads();
       }
-      if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+      if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
     }
   }
 
@@ -669,7 +670,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   }
   if (tiles <= DISP_TILES_CHAIN) return;
   // more tiles than the chain adds up by itself: their totals into the running totals
-  if (!grid_barrier(w.ctl, a.status, round, &s_ok)) return;
+  if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
   for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const uint32_t e0 = __ldcg(w.tile_edge + t), e1 = __ldcg(w.tile_edge + t + 1);
     int64_t base = 0, base_cnt = 0, all_base, all_base_cnt;
@@ -758,6 +759,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
   const int nm0 = (int)w.ctl[CTL_NM0], nm = stage ? (int)w.ctl[CTL_NM1] : nm0, koff = stage ? nm0 : 0;
   const int64_t n0 = (int64_t)w.ctl[CTL_N0], qoff = stage ? n0 : 0, nq = stage ? (int64_t)w.ctl[CTL_N1] : n0;
   const uint32_t tiles = (uint32_t)w.ctl[CTL_TILES], tile_rows = (uint32_t)w.ctl[CTL_TILE_ROWS];
+  if (w.ctl[CTL_ABORT]) return;                // (TAKEN stays 0)
   const bool by_tile = tiles <= DISP_TILES_CHAIN;      // the running totals start anew in every tile
   if (by_tile) {
     constexpr int PER = DISP_TILES_CHAIN / CHAIN_THREADS;
@@ -969,6 +971,11 @@ __global__ void __launch_bounds__(ASSIGN_THREADS) k_disp_assign(const DispArgs a
   const int64_t n0 = (int64_t)w.ctl[CTL_N0], t0 = (int64_t)w.ctl[CTL_TAKEN0], t1 = a.d_stage ? (int64_t)w.ctl[CTL_TAKEN1] : 0;
   const int nm0 = (int)w.ctl[CTL_NM0], nm1 = (int)w.ctl[CTL_NM1];
   const int64_t gid = (int64_t)blockIdx.x * ASSIGN_THREADS + threadIdx.x, stride = (int64_t)gridDim.x * ASSIGN_THREADS;
+  if (w.ctl[CTL_ABORT]) {      // the order was given up: nothing was handed out (t0 = t1 = 0), and the lists are reported empty
+    for (int64_t i = gid; i < a.n; i += stride) a.queue_order[i] = -1;
+    for (int64_t r = gid; r < w.R; r += stride) a.inst_order[r] = -1;
+    if (gid < 2) { a.n_queue[gid] = 0; a.n_mature[gid] = 0; }
+  }
   for (int64_t i = gid; i < t0 + t1; i += stride) {
     const int stage = i >= t0;
     const int64_t q = stage ? n0 + (i - t0) : i;      // place in the numbering of both queues
@@ -1059,6 +1066,7 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   const uint32_t par = d->parity;
   d->parity ^= 1u;
   w.ctl = d->ctl[par];
+  w.wait_limit = s->wait_limit;
   DispArgs a;
   a.replica_id = t->replica_id; a.class_id = t->class_id; a.state = t->state; a.prompt_len = t->prompt_len; a.gen = t->gen;
   a.arrival = t->arrival_ns; a.req_id = t->req_id; a.weight = s->p.weight_max > 0 ? t->weight : nullptr;

@@ -81,6 +81,7 @@ enum { KSLOT_COUNT = 0, KSLOT_COLSCAN, KSLOT_OFFSETS, KSLOT_REGROUP, KSLOT_SEG_S
 #define HFX_TILE_MATRIX_MAX (INT64_C(8) << 20)   // entries of the tile matrix (64 MiB), the tiles of one round of the SMs left out
 #define HFX_TILE_REPLICAS_MAX 4095               // replicas whose counters fit in shared memory (12-bit bucket ids)
 #define HFX_NEXT_REPLICAS_MAX 2047               // replicas up to which a tile notes the next arrival of each (8 bytes of shared memory per replica)
+#define HFX_WAIT_LIMIT (1u << 22)                // polls of a grid barrier before the kernel gives up (about two seconds)
 #define HFX_COUNT_TILE_ROWS 4096                 // rows per block of the counting pass of the fallback front end
 
 struct HfxBracket { cudaEvent_t a, b; int slot; };
@@ -118,6 +119,7 @@ struct hfx_sched {
   int32_t tiles_max;        // matrix rows allocated (0: fallback front end only)
   uint32_t tot_parity;      // which half of d_tot / which "ordered" word the next tile front end uses
   int64_t horizon;          // commit horizon of the following steps (INT64_MAX: none)
+  uint32_t wait_limit;      // polls of a device-side wait (HFX_WAIT_LIMIT unless set)
   int front_enabled;        // 0: use the fallback front end (global counters) even where the tile front end fits
   void *dispatch_ws;                   // workspace of hfx_dispatch_step, allocated by its first call
   unsigned char *d_sim_scratch;        // rows of long traces in hfx_sim_run (allocated by the first call that needs it)

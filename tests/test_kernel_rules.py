@@ -56,3 +56,12 @@ def test_kernels_set_up_beside_the_one_in_front_read_nothing_through_the_read_on
             assert "__ldg(" not in body and "ld.global.nc" not in body and not re.search(r"const \w+ \*\s*__restrict__", head), (name, head)
         seen |= {re.search(r"\b(k_\w+)\s*\(", h).group(1) for h, _ in early}
     assert {"k_front", "k_replicas", "k_pd_rows", "k_pd_clock", "k_slo_assign", "k_disp_chain", "k_disp_assign"} <= seen
+
+
+def test_kernels_behind_the_grid_barrier_ask_whether_it_was_given_up():
+    # a barrier that ran out leaves the tiles, the running totals and the order unwritten: walking them reads and writes out of range
+    kernels = {re.search(r"\b(k_\w+)\s*\(", h).group(1): b for h, b in _functions(_source("hfx_dispatch.cu"), r"__global__")}
+    assert "grid_barrier(" in kernels["k_disp_sort"]
+    for name, first_use in (("k_disp_chain", "tile_sum"), ("k_disp_assign", "run_end")):
+        asked = kernels[name].index("CTL_ABORT")
+        assert kernels[name].index("cudaGridDependencySynchronize") < asked < kernels[name].index(first_use), name

@@ -1294,6 +1294,41 @@ def test_dispatch_order_and_walk_edges(n, shape):
     assert g["adm_count"].sum() > 0
 
 
+@pytest.mark.parametrize("d_stage", [False, True])
+@pytest.mark.parametrize("n,R", [(60_013, 40), (3000, 300)])
+def test_dispatch_whose_grid_barrier_runs_out_hands_out_nothing(n, R, d_stage):
+    # With a limit of no polls every block that is not the last one at a barrier gives up.  Such a call raises the status and hands out
+    # nothing, on a fresh workspace as behind a call that succeeded; the next call with the usual limit is right.
+    import paper_2508_15919_b200 as hfx
+    wl = gen.random_table(n, n, R, modes=(gen.PREFILL, gen.DECODE, gen.COLOCATED) if d_stage else (gen.COLOCATED,), inflight=0.3)
+    now = int(wl.now.max())
+    wl.maturity[:] = now - np.arange(R) % 7
+    sched = make_sched(wl)
+    tab = hfx.DeviceTable.from_numpy(wl.table)
+    mat = torch.from_numpy(wl.maturity.copy()).cuda()
+    out = hfx.DispatchOut(n, R)
+    given_up = 0
+    for k in range(6):
+        sched.set_wait_limit(0)
+        sched.dispatch_step(tab, now, mat, out)
+        if sched.status() & hfx.ST_TIMEOUT:
+            given_up += 1
+            g = out.to_numpy()
+            for key in ("assign", "queue_order", "inst_order"):
+                assert np.all(g[key] == -1), key
+            for key in ("n_queue", "n_mature", "adm_cost", "adm_count"):
+                assert np.all(g[key] == 0), key
+            assert np.array_equal(g["maturity_next"], wl.maturity)
+        if k % 2:
+            sched.set_wait_limit(1 << 22)
+            assert_dispatch_parity(wl, now, sched=sched)
+    assert given_up > 0
+    with pytest.raises(hfx.HfxError) as e:
+        sched.set_wait_limit((1 << 26) + 1)
+    assert e.value.code == -1
+    sched.close()
+
+
 @pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100), (40, 8300)])
 def test_idle_replicas_find_their_next_arrivals(R, rows_per):
     # Tiles note every replica's next arrival up to 2047 replicas, lists are searched beyond; lists of more than 2048 rows (a few

@@ -994,7 +994,8 @@ __global__ void __launch_bounds__(ASSIGN_THREADS) k_disp_assign(const DispArgs a
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-struct hfx_dispatch_ws { DispWork w; unsigned char *mem; unsigned long long *ctl[2]; uint32_t parity; };
+// unsettled: a call launched some of its kernels and not the last one, so the counters are not as the next call wants to find them
+struct hfx_dispatch_ws { DispWork w; unsigned char *mem; size_t zero; unsigned long long *ctl[2]; uint32_t parity; bool unsettled; };
 
 static size_t chain_smem(int R) { return (size_t)(CHAIN_CHUNK + CHAIN_WIN + 8) * 16 + (size_t)DISP_TILES_CHAIN * 16 + 16 + ((size_t)R + CHAIN_BATCH + 1) * 16; }
 static size_t scan_smem(int R) { return R <= SCAN_SMEM_REPLICAS ? (size_t)R * 24 : 0; }
@@ -1039,7 +1040,7 @@ static int disp_workspace(hfx_sched *s, hfx_dispatch_ws **out) {
   unsigned char *m = nullptr;
   if (cudaMalloc(&m, used) != cudaSuccess) { cudaGetLastError(); delete d; return HFX_E_NOMEM; }
   if (cudaMemsetAsync(m, 0, zero, s->stream) != cudaSuccess) { cudaGetLastError(); cudaFree(m); delete d; return HFX_E_CUDA; }
-  d->mem = m;
+  d->mem = m; d->zero = zero;
   w.n_run = reinterpret_cast<uint32_t *>(m + o_run); w.sum_kv = reinterpret_cast<unsigned long long *>(m + o_kv); w.mask_run = reinterpret_cast<unsigned long long *>(m + o_mask);
   d->ctl[0] = reinterpret_cast<unsigned long long *>(m + o_ctl); d->ctl[1] = reinterpret_cast<unsigned long long *>(m + o_ctl2);
   w.bin_cnt = reinterpret_cast<uint32_t *>(m + o_bin);
@@ -1063,6 +1064,8 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   cudaStream_t st = s->stream;
   const int R = s->p.n_replicas;
   const int64_t n = t->n_rows;
+  if (d->unsettled && cudaMemsetAsync(d->mem, 0, d->zero, st) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
+  d->unsettled = true;
   const uint32_t par = d->parity;
   d->parity ^= 1u;
   w.ctl = d->ctl[par];
@@ -1078,7 +1081,6 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   a.status = s->d_status;
   const int blocks = scan_blocks(s, n);
   a.rounds = (int32_t)((n / 4 + (int64_t)SCAN_THREADS * blocks - 1) / ((int64_t)SCAN_THREADS * blocks));
-  { KernelScope ks(s, KSLOT_DISPATCH); k_disp_scan<<<blocks, SCAN_THREADS, scan_smem(R), st>>>(s->p, a, w); }
   // blocks of the cooperative kernel: no more than its phases can use, so that small calls meet at short barriers
   int64_t want = (n + 2047) / 2048, want_r = (R + 31) / 32;
   if (want < want_r) want = want_r;
@@ -1086,7 +1088,13 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.stream = st;
+  {
+    KernelScope ks(s, KSLOT_DISPATCH);
+    cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(SCAN_THREADS); cfg.dynamicSmemBytes = scan_smem(R);
+    if (cudaLaunchKernelEx(&cfg, k_disp_scan, s->p, a, w) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
+  }
+  cfg.attrs = attr; cfg.numAttrs = 1;
   {
     KernelScope ks(s, KSLOT_DISPATCH);
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1109,5 +1117,6 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
     cfg.gridDim = dim3((unsigned)want_a); cfg.blockDim = dim3(ASSIGN_THREADS); cfg.dynamicSmemBytes = 0;
     if (cudaLaunchKernelEx(&cfg, k_disp_assign, a, w, d->ctl[par ^ 1u]) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
   }
+  d->unsettled = false;
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }

@@ -127,7 +127,8 @@ struct hfx_sched {
   unsigned long long *d_att;           // totals of hfx_attainment, zero between its calls (in the allocation of d_flags)
   void *d_slo;                         // per-priority table of hfx_slo_map
   uint32_t slo_parity;                 // which copy of its first rows the next call uses
-  void *d_pd;                          // moved counter, wake-up times and busy flags of hfx_pd_migrate
+  void *d_pd;                          // moved counter, wake-up times and busy flags of hfx_pd_migrate, zero between its calls
+  bool pd_unsettled;                   // a call launched its first kernel and not the second, which clears them
 };
 
 // ---- latency predictor -------------------------------------------------------------------

@@ -101,8 +101,10 @@ int hfx_launch_pd_migrate(hfx_sched *s, const hfx_table *t, int32_t *replica_id,
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(PD_THREADS); cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = s->profiling ? 0 : 1;
-  cudaError_t e;
-  {
+  cudaError_t e = cudaSuccess;
+  if (s->pd_unsettled) e = cudaMemsetAsync(s->d_pd, 0, hfx_pd_workspace_bytes(R), st);
+  if (e == cudaSuccess) {
+    s->pd_unsettled = true;
     KernelScope ks(s, KSLOT_PD);
     int64_t grid = ((t->n_rows >> 2) + PD_THREADS - 1) / PD_THREADS;
     if (grid > s->n_sm * 8) grid = s->n_sm * 8;
@@ -115,5 +117,6 @@ int hfx_launch_pd_migrate(hfx_sched *s, const hfx_table *t, int32_t *replica_id,
     cfg.gridDim = dim3((unsigned)((R + PD_THREADS - 1) / PD_THREADS));
     e = cudaLaunchKernelEx(&cfg, k_pd_clock, s->p, a);
   }
+  if (e == cudaSuccess) s->pd_unsettled = false;
   return e == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }

@@ -198,21 +198,23 @@ int hfx_launch_slo_map(hfx_sched *s, int32_t n_prio, const hfx_slo_window *win, 
   a.last_queue = last_queue; a.pending = pending; a.new_prio = new_prio; a.n_new = n_new;
   a.ttft_out = ttft_out; a.tpot_out = tpot_out; a.n_prio = n_prio;
   a.tab = reinterpret_cast<SloTable *>(s->d_slo); a.status = s->d_status;
-  a.par = (int32_t)s->slo_parity; s->slo_parity ^= 1u;
+  a.par = (int32_t)s->slo_parity;
   a.win_blocks = win->w > 0 ? (win->w + SLO_WIN_RECORDS - 1) / SLO_WIN_RECORDS : 1;
-  cudaStream_t st = s->stream;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.stream = s->stream;
   {
     KernelScope ks(s, KSLOT_SLOMAP);
-    const int grid = a.win_blocks + (int)((n_new + SLO_WIN_THREADS - 1) / SLO_WIN_THREADS);
-    k_slo_window<<<grid, SLO_WIN_THREADS, 16 * (size_t)(win->w > 0 ? win->w : 1), st>>>(a);
+    cfg.gridDim = dim3((unsigned)(a.win_blocks + (n_new + SLO_WIN_THREADS - 1) / SLO_WIN_THREADS)); cfg.blockDim = dim3(SLO_WIN_THREADS);
+    cfg.dynamicSmemBytes = 16 * (size_t)(win->w > 0 ? win->w : 1);
+    if (cudaLaunchKernelEx(&cfg, k_slo_window, a) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
   }
+  s->slo_parity ^= 1u;      // (once the kernel that uses one copy and clears the other is on its way)
   if (n_new > 0) {
     int grid = (int)((n_new + SLO_THREADS - 1) / SLO_THREADS);
     if (grid > s->n_sm * 8) grid = s->n_sm * 8;
     KernelScope ks(s, KSLOT_SLOMAP);
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(SLO_THREADS); cfg.stream = st;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(SLO_THREADS); cfg.dynamicSmemBytes = 0;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -39,8 +39,10 @@ int hfx_launch_step(hfx_sched *s, const hfx_table *t, const hfx_replica_state *s
     fa.now = st->now_ns; fa.mat = st->maturity_ns; fa.mode = s->d_mode; fa.n = t->n_rows;
     fa.slack = o->slack_ns; fa.pred_ttft = o->pred_ttft_ns; fa.pred_tpot = o->pred_tpot_ns; fa.key = o->key; fa.admit = o->admit;
     rc = hfx_launch_front(s, fa);
-    if (rc == HFX_OK) rc = hfx_launch_replicas(s, sa, t->n_rows, true);
-    s->tot_parity ^= 1u;
+    if (rc == HFX_OK) {      // (a front end that was not launched has added nothing up, and has not cleared the other copy)
+      rc = hfx_launch_replicas(s, sa, t->n_rows, true);
+      s->tot_parity ^= 1u;
+    }
   } else {
     RegroupArgs ra;
     ra.replica_id = t->replica_id; ra.class_id = t->class_id; ra.state = t->state; ra.prompt_len = t->prompt_len;

@@ -65,3 +65,14 @@ def test_kernels_behind_the_grid_barrier_ask_whether_it_was_given_up():
     for name, first_use in (("k_disp_chain", "tile_sum"), ("k_disp_assign", "run_end")):
         asked = kernels[name].index("CTL_ABORT")
         assert kernels[name].index("cudaGridDependencySynchronize") < asked < kernels[name].index(first_use), name
+
+
+def test_what_is_kept_for_the_next_call_follows_what_was_launched():
+    # a copy is changed for the other one behind the launch of the kernel that uses it and clears the other
+    step, slo, disp, pd = (_source(f) for f in ("hfx_step.cu", "hfx_slomap.cu", "hfx_dispatch.cu", "hfx_pd.cu"))
+    assert re.search(r"if \(rc == HFX_OK\) \{[^}]*tot_parity \^= 1u;\s*\}", step)
+    assert slo.index("cudaLaunchKernelEx(&cfg, k_slo_window") < slo.index("slo_parity ^= 1u")
+    # counters that the last kernel of a call clears: cleared by the next call where that kernel was not launched
+    for src, last in ((disp, "cudaLaunchKernelEx(&cfg, k_disp_assign"), (pd, "cudaLaunchKernelEx(&cfg, k_pd_clock")):
+        assert src.index("unsettled = true;") < src.index(last) < src.index("unsettled = false;")
+        assert re.search(r"if \([\w>-]*unsettled\b[^;]*cudaMemsetAsync", src)

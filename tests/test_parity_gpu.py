@@ -6,7 +6,7 @@ import torch
 import gen
 import oracle
 from helpers import MS, SEC, make_wl
-from gpu_helpers import assert_dispatch_parity, assert_step_parity, assert_sim_parity, make_sched, run_sim_gpu
+from gpu_helpers import STATE_COLS, assert_dispatch_parity, assert_step_parity, assert_sim_parity, make_sched, run_sim_gpu
 
 pytestmark = pytest.mark.gpu
 MODES3 = (gen.COLOCATED, gen.PREFILL, gen.DECODE)
@@ -1368,3 +1368,97 @@ def test_larger_replicas_whose_ids_do_not_rise(n, ids):
         elif ids == "negative":
             wl.table["req_id"][:] = rng.permutation(n) * 250_000 - 2_000_000_000
         assert_step_parity(wl, steps=2, commit=True)
+
+
+class RefusedLaunches:
+    """While it is open, every launch on `stream` is refused by the runtime (an invalidated stream capture): nothing runs, the call gets an error code."""
+
+    def __init__(self, stream):
+        import ctypes
+        self.rt, self.st = ctypes.CDLL("libcudart.so.12"), ctypes.c_void_p(stream.cuda_stream)      # (the one torch has loaded)
+        self.graph = ctypes.c_void_p()
+        self.byref = ctypes.byref
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        assert self.rt.cudaStreamBeginCapture(self.st, 2) == 0
+        assert self.rt.cudaStreamSynchronize(self.st) != 0      # not allowed in a capture: invalidates it
+        return self
+
+    def __exit__(self, *exc):
+        assert self.rt.cudaStreamEndCapture(self.st, self.byref(self.graph)) != 0 and not self.graph.value
+        self.rt.cudaGetLastError()
+
+
+@pytest.mark.parametrize("kind", ["step", "fallback", "dispatch", "pd", "slo"])
+def test_a_call_whose_launch_was_refused_leaves_the_next_ones_right(kind):
+    # What a call keeps between its kernels and for the next call (copies used in turn, counters that the last kernel clears) follows
+    # what was launched, not what was asked for.
+    import paper_2508_15919_b200 as hfx
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        wl = gen.pd_pairs(3, 3, 200) if kind == "pd" else gen.config4(seed=5, R=32, n=20_000, steps=4)
+        cpu = wl.copy()
+        sched = hfx.Scheduler(wl.model, wl.classes, wl.replicas, wl.n_rows, budget_mode=wl.budget_mode, weight_max=wl.weight_max, stream=st)
+        sched.set_fused_front(kind != "fallback")
+        tab = hfx.DeviceTable.from_numpy(wl.table)
+        now = torch.from_numpy(wl.now.copy()).cuda(); mat = torch.from_numpy(wl.maturity.copy()).cuda()
+        out = hfx.StepOut(wl.n_rows, wl.n_replicas, optional=False)
+        rng = np.random.default_rng(1)
+        dev = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a, dt)).cuda()
+        if kind == "dispatch":
+            t0 = int(wl.now.max())
+            dout = hfx.DispatchOut(wl.n_rows, wl.n_replicas)
+            call = lambda: sched.dispatch_step(tab, t0, mat, dout)
+
+            def check():
+                g, c = dout.to_numpy(), oracle.dispatch(wl, t0)
+                for k in ("assign", "queue_order", "n_queue", "n_mature", "n_run", "sum_kv", "adm_count", "maturity_next"):
+                    assert np.array_equal(g[k], c[k]), k
+        elif kind == "pd":
+            pair = gen.pd_partner_table(3)
+            prt = torch.from_numpy(pair).cuda()
+
+            def call():
+                sched.pd_migrate(tab, now, mat, prt, 2 * MS, 500)
+                sched.step(tab, now, mat, out, commit=True)
+
+            def check():
+                oracle.pd_migrate(cpu, pair, 2 * MS, 500)
+                oracle.step(cpu, commit=True)
+                assert np.array_equal(now.cpu().numpy(), cpu.now)
+                for k in ("replica_id",) + tuple(STATE_COLS):
+                    assert np.array_equal(tab.to_numpy()[k], cpu.table[k]), k
+        elif kind == "slo":
+            win = {"prio": rng.integers(0, 4, 700), "ttft": rng.integers(1, 10**10, 700), "tpot": rng.integers(1, 10**9, 700), "queue": rng.integers(0, 10**9, 700)}
+            bounds = {k: np.full(4, -10**12 if "min" in k else 10**12) for k in oracle.SLO_BOUND_KEYS}
+            w = {k + ("" if k == "prio" else "_ns"): dev(v, np.int32 if k == "prio" else np.int64) for k, v in win.items()}
+            b = {k + "_ns": dev(v, np.int64) for k, v in bounds.items()}
+            state = {"last": np.zeros(4, np.int64), "k": 0}
+            lq, pend, outs = dev(np.zeros(4), np.int64), dev(np.zeros(4), np.int32), [torch.zeros(3000, dtype=torch.int64, device="cuda") for _ in range(2)]
+            news = [np.concatenate([np.zeros(100 * k, np.int64), rng.integers(0, 4, 3000 - 100 * k)]) for k in range(4)]
+            news_gpu = [dev(x, np.int32) for x in news]
+            call = lambda: sched.slo_map(4, w, b, lq, pend, news_gpu[state["k"]], *outs)
+
+            def check():
+                c = oracle.slo_map(4, win, bounds, state["last"], np.zeros(4, np.int32), news[state["k"]])
+                assert np.array_equal(outs[0].cpu().numpy(), c["ttft_slo"]) and np.array_equal(lq.cpu().numpy(), c["last_queue"])
+                state["last"] = c["last_queue"]
+                state["k"] += 1
+        else:
+            call = lambda: sched.step(tab, now, mat, out, commit=True)
+
+            def check():
+                c, g = oracle.step(cpu, commit=True), out.to_numpy()
+                for k in ("order", "admit", "budget", "adm_count", "seg_off"):
+                    assert np.array_equal(g[k], c[k]), k
+        for k in range(3):
+            call()
+            assert sched.status() == 0
+            check()
+            with RefusedLaunches(st):
+                with pytest.raises(hfx.HfxError) as e:
+                    call()
+                assert e.value.code == -4
+            sched.get_profile()      # (reads an error that the call may have left behind)
+        sched.close()

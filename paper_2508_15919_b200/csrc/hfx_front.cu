@@ -458,7 +458,7 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   cfg.attrs = attr;
   cfg.numAttrs = s->profiling ? 0 : 1;      // set up while the step before drains
   const cudaError_t e = fa.pred_ttft || fa.pred_tpot || fa.key ? cudaLaunchKernelEx(&cfg, k_front<true>, s->p, fa) : cudaLaunchKernelEx(&cfg, k_front<false>, s->p, fa);
-  return e == cudaSuccess ? HFX_OK : HFX_E_CUDA;
+  return cuda_rc(e);
 }
 
 int hfx_front_configure() {

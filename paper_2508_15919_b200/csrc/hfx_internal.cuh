@@ -510,6 +510,13 @@ __device__ __forceinline__ void warp_first_fit(int64_t n, const int64_t *min32, 
   }
 }
 
+// The code of a runtime call.  A failed call's error is read here: left behind, the next call's check would find it.
+inline int cuda_rc(cudaError_t e) {
+  if (e == cudaSuccess) return HFX_OK;
+  cudaGetLastError();
+  return HFX_E_CUDA;
+}
+
 // Brackets one kernel launch with events when profiling is on; counts the launch either way.
 struct KernelScope {
   hfx_sched *s; HfxBracket br; bool on; cudaStream_t st;

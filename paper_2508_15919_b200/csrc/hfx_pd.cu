@@ -118,5 +118,5 @@ int hfx_launch_pd_migrate(hfx_sched *s, const hfx_table *t, int32_t *replica_id,
     e = cudaLaunchKernelEx(&cfg, k_pd_clock, s->p, a);
   }
   if (e == cudaSuccess) s->pd_unsettled = false;
-  return e == cudaSuccess ? HFX_OK : HFX_E_CUDA;
+  return cuda_rc(e);
 }

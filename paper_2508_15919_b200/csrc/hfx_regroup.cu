@@ -227,9 +227,9 @@ int hfx_launch_regroup(hfx_sched *s, const RegroupArgs &ra, int32_t *seg_off) {
   ca.replica_id = ra.replica_id; ca.class_id = ra.class_id; ca.state = ra.state; ca.prompt_len = ra.prompt_len;
   ca.gen = ra.gen; ca.arrival = ra.arrival; ca.now = ra.now; ca.n = ra.n;
   ca.tot_all = s->d_seg_count; ca.tot_act = s->d_act_count; ca.rowflag = s->d_rowflag; ca.status = s->d_status;
-  if (cudaMemsetAsync(s->d_seg_count, 0, sizeof(uint32_t) * (R + 2), stream) != cudaSuccess ||
-      cudaMemsetAsync(s->d_act_count, 0, sizeof(uint32_t) * (R + 2), stream) != cudaSuccess)
-    return HFX_E_CUDA;
+  int rc = cuda_rc(cudaMemsetAsync(s->d_seg_count, 0, sizeof(uint32_t) * (R + 2), stream));
+  if (rc == HFX_OK) rc = cuda_rc(cudaMemsetAsync(s->d_act_count, 0, sizeof(uint32_t) * (R + 2), stream));
+  if (rc != HFX_OK) return rc;
   {
     KernelScope ks(s, KSLOT_COUNT);
     k_count<<<s->n_sm * 8, 256, 0, stream>>>(s->p, ca);

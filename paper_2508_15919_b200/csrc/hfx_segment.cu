@@ -1949,7 +1949,7 @@ int hfx_launch_replicas(hfx_sched *s, const SegArgs &sa, int64_t n, bool slabs) 
   cudaError_t e;
   if (slabs) e = s->p.first_fit ? cudaLaunchKernelEx(&cfg, k_replicas<true, true>, s->p, sa, c) : cudaLaunchKernelEx(&cfg, k_replicas<true, false>, s->p, sa, c);
   else e = s->p.first_fit ? cudaLaunchKernelEx(&cfg, k_replicas<false, true>, s->p, sa, c) : cudaLaunchKernelEx(&cfg, k_replicas<false, false>, s->p, sa, c);
-  return e == cudaSuccess ? HFX_OK : HFX_E_CUDA;
+  return cuda_rc(e);
 }
 
 int hfx_segment_configure() {

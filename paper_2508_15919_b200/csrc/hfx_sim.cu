@@ -718,7 +718,8 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   a.now_out = o->now_ns;
   const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = (size_t)cap * 2 + SIM_HEAD_BYTES(s->p.n_classes);
   const size_t sm_bytes = 227 * 1024, block_bytes = 1024;      // (1 KB per block is reserved)
-  if (cudaMemsetAsync(d_work_counter, 0, sizeof(uint32_t), s->stream) != cudaSuccess) return HFX_E_CUDA;
+  int rc = cuda_rc(cudaMemsetAsync(d_work_counter, 0, sizeof(uint32_t), s->stream));
+  if (rc != HFX_OK) return rc;
   int per_sm = cap <= SIM_SMEM_ROWS ? (int)(sm_bytes / (rows_bytes + list_bytes + block_bytes)) : 0;
   if (per_sm > 32) per_sm = 32;
   int per_sm_scratch = (int)(sm_bytes / (list_bytes + block_bytes));
@@ -735,7 +736,8 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
     if (grid > n_traces) grid = n_traces;
     const size_t need = rows_bytes * (size_t)grid;
     if (s->sim_scratch_bytes < need) {
-      if (cudaStreamSynchronize(s->stream) != cudaSuccess) return HFX_E_CUDA;
+      rc = cuda_rc(cudaStreamSynchronize(s->stream));
+      if (rc != HFX_OK) return rc;
       cudaFree(s->d_sim_scratch);
       s->d_sim_scratch = nullptr; s->sim_scratch_bytes = 0;
       if (cudaMalloc(&s->d_sim_scratch, need) != cudaSuccess) { cudaGetLastError(); return HFX_E_NOMEM; }

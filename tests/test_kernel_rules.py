@@ -76,3 +76,13 @@ def test_what_is_kept_for_the_next_call_follows_what_was_launched():
     for src, last in ((disp, "cudaLaunchKernelEx(&cfg, k_disp_assign"), (pd, "cudaLaunchKernelEx(&cfg, k_pd_clock")):
         assert src.index("unsettled = true;") < src.index(last) < src.index("unsettled = false;")
         assert re.search(r"if \([\w>-]*unsettled\b[^;]*cudaMemsetAsync", src)
+
+
+def test_every_refused_runtime_call_has_its_error_read():
+    # an error left behind is what the next call's check finds (the caller of the *_configure functions reads theirs)
+    for name in sorted(os.listdir(CSRC)):
+        src = _source(name)
+        configure = [b for h, b in _functions(src, r"int hfx_\w+_configure\(\)")]
+        for m in re.finditer(r"return [^;]*HFX_E_CUDA;", src):
+            if not any(m.group() in b for b in configure if "cudaFuncSetAttribute" in b and b in src and src.index(b) < m.start() < src.index(b) + len(b)):
+                assert "cudaGetLastError()" in src[max(0, m.start() - 60):m.end()], (name, src[m.start() - 100:m.end()])

@@ -1460,5 +1460,33 @@ def test_a_call_whose_launch_was_refused_leaves_the_next_ones_right(kind):
                 with pytest.raises(hfx.HfxError) as e:
                     call()
                 assert e.value.code == -4
-            sched.get_profile()      # (reads an error that the call may have left behind)
+        sched.close()
+
+
+@pytest.mark.parametrize("kind", ["step", "fallback", "pd", "sim", "scale_tick", "attainment"])
+def test_a_refused_call_leaves_no_error_behind_for_the_next_one(kind):
+    import paper_2508_15919_b200 as hfx
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        wl = gen.config1()
+        sched = hfx.Scheduler(wl.model, wl.classes, wl.replicas, wl.n_rows, stream=st)
+        sched.set_fused_front(kind != "fallback")
+        tab = hfx.DeviceTable.from_numpy(wl.table)
+        now = torch.from_numpy(wl.now.copy()).cuda(); mat = torch.from_numpy(wl.maturity.copy()).cuda()
+        out, sout = hfx.StepOut(wl.n_rows, 1, optional=False), hfx.SimOut(1)
+        counts = torch.zeros((3, 4), dtype=torch.int64, device="cuda"); used = torch.zeros(1, dtype=torch.int64, device="cuda")
+        dec = torch.zeros((3, 2), dtype=torch.int32, device="cuda"); blocks = torch.ones(1, dtype=torch.int32, device="cuda")
+        att = torch.zeros(len(wl.classes) + 1, 6, dtype=torch.int64, device="cuda")
+        pair = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        calls = {"step": lambda: sched.step(tab, now, mat, out), "pd": lambda: sched.pd_migrate(tab, now, mat, pair, 0, 0), "sim": lambda: sched.sim_run(tab, wl.trace_off, 5, sout),
+                 "scale_tick": lambda: sched.scale_tick(tab, SEC, blocks, counts, used, dec), "attainment": lambda: sched.attainment(tab, att)}
+        call = calls.get(kind, calls["step"])
+        call()
+        with RefusedLaunches(st):
+            with pytest.raises(hfx.HfxError) as e:
+                call()
+            assert e.value.code == -4
+        for nxt in calls.values():      # whichever call comes next
+            nxt()
+        assert sched.status() == 0
         sched.close()

@@ -84,7 +84,7 @@ extern "C" int hfx_sched_create(hfx_sched **out, const hfx_latency_model *model,
   s->p.n_classes = n_classes; s->p.n_replicas = n_replicas;
   s->p.budget_mode = opts->budget_mode; s->p.weight_max = opts->weight_max;
   s->p.first_fit = (opts->flags & HFX_OPT_FIRST_FIT) ? 1 : 0;
-  s->opts = *opts; s->max_rows = max_rows; s->n_sm = n_sm;
+  s->max_rows = max_rows; s->n_sm = n_sm;
   s->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
   s->launches = 0;
   s->profiling = 0;

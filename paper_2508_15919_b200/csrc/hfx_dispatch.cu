@@ -62,7 +62,7 @@ struct DispWork {
   ReplicaPlan *plan;         // [R]
   int64_t *ord_budget; int32_t *ord_room; int32_t *ord_id;      // [R] matured instances in order, stage 0, then stage 1
   int32_t *run_end;                                               // [R] where its run ends in its stage's queue
-  int64_t max_rows; int32_t R, blocks, tiles_max;
+  int32_t R, tiles_max;
   uint32_t wait_limit;       // polls of a grid barrier before the kernel gives up
 };
 
@@ -1027,7 +1027,7 @@ static int disp_workspace(hfx_sched *s, hfx_dispatch_ws **out) {
   memset(d, 0, sizeof(*d));
   DispWork &w = d->w;
   const size_t rows = (size_t)s->max_rows, R = (size_t)s->p.n_replicas;
-  w.max_rows = s->max_rows; w.R = s->p.n_replicas; w.blocks = s->n_sm;
+  w.R = s->p.n_replicas;
   w.tiles_max = (int)(rows / DISP_TILE) + s->n_sm + 1;
   size_t used = 0;
   auto part = [&](size_t bytes) { const size_t at = used; used += (bytes + 255) & ~(size_t)255; return at; };

@@ -24,11 +24,6 @@
 
 #define ROWFLAG_BADREP 4  // row bound to no replica (bucket R)
 
-// how a tile's rows get their rank inside their (replica, class) group, in row order
-#define TILE_SORTED 0     // tile already sorted by replica: ranks from positions
-#define TILE_GROUPS 1     // small groups: counting sort of the tile, rank by scanning the group
-#define TILE_ANY 2        // large unsorted groups: any order (clears "ordered")
-
 // "no bound" marker of a slack base
 #define BASE_UNBOUNDED INT64_MAX
 
@@ -82,13 +77,11 @@ enum { KSLOT_COUNT = 0, KSLOT_COLSCAN, KSLOT_OFFSETS, KSLOT_REGROUP, KSLOT_SEG_S
 #define HFX_TILE_REPLICAS_MAX 4095               // replicas whose counters fit in shared memory (12-bit bucket ids)
 #define HFX_NEXT_REPLICAS_MAX 2047               // replicas up to which a tile notes the next arrival of each (8 bytes of shared memory per replica)
 #define HFX_WAIT_LIMIT (1u << 22)                // polls of a grid barrier before the kernel gives up (about two seconds)
-#define HFX_COUNT_TILE_ROWS 4096                 // rows per block of the counting pass of the fallback front end
 
 struct HfxBracket { cudaEvent_t a, b; int slot; };
 
 struct hfx_sched {
   HfxParams p;
-  hfx_options opts;
   int64_t max_rows;
   int n_sm;
   cudaStream_t stream;
@@ -104,7 +97,7 @@ struct hfx_sched {
   uint32_t *d_seg_begin;    // [R+2] exclusive prefix of d_seg_count                      (fallback)
   uint32_t *d_cursor;       // [2][R+2] fill cursors of the fallback regroup (active, inactive)
   uint8_t *d_rowflag;       // [max_rows] kind of every row (KIND_*), ROWFLAG_BADREP for a bad replica id
-  uint32_t *d_flags;        // [0] "ordered" of the fallback front end (never), [4],[5] "ordered" of the tile front end by parity
+  uint32_t *d_flags;        // [4],[5] "ordered" of the tile front end by parity
   HfxRec *d_rec;            // [max_rows] contiguous records: written by the fallback regroup, or gathered from the
                             // slabs by the blocks of larger replicas
   uint64_t *d_big_hi;       // sort scratch of oversize segments
@@ -392,66 +385,6 @@ __device__ __forceinline__ void cmp_swap(uint64_t *hi, uint32_t *lo, int i, int 
   } else if (hi_i > hi_j) { hi[i] = hi_j; hi[j] = hi_i; }
 }
 
-// Bitonic sorting network with ascending comparators only (mirrored first sub-stage), so the virtual
-// +inf padding beyond n never moves: any n, in place.  Items are distinct, so the result is unique.
-// Each warp owns a contiguous chunk of E items; stages whose pairs stay inside a chunk need only a
-// warp barrier, the others a block barrier.  Callers synchronise the block before the call; the
-// block is synchronised on return.
-template <bool WIDE>
-__device__ void block_sort(uint64_t *hi, uint32_t *lo, int n) {
-  if (n > 1) {
-    int n_pad = 2;
-    while (n_pad < n) n_pad <<= 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    int E = n_pad / nwarp;
-    if (E < 64) E = 64;
-    if (E > n_pad) E = n_pad;
-    const int c0 = warp * E;
-    const bool has_chunk = c0 < n_pad;
-    const int half = n_pad >> 1;
-    bool local = true;    // the previous stage was chunk-local (or there was none)
-    for (int k = 2; k <= n_pad; k <<= 1) {
-      const int hk = k >> 1;
-      if (k <= E) {   // mirrored sub-stage of merge size k, inside the chunk
-        if (has_chunk)
-          for (int t = lane; t < (E >> 1); t += 32) {
-            const int blk = t / hk, off = t - blk * hk;
-            const int i = c0 + blk * k + off, j = c0 + blk * k + k - 1 - off;
-            if (j < n) cmp_swap<WIDE>(hi, lo, i, j);
-          }
-        __syncwarp();
-      } else {
-        if (local) { __syncthreads(); local = false; }
-        for (int t = threadIdx.x; t < half; t += blockDim.x) {
-          const int blk = t / hk, off = t - blk * hk;
-          const int i = blk * k + off, j = blk * k + k - 1 - off;
-          if (j < n) cmp_swap<WIDE>(hi, lo, i, j);
-        }
-        __syncthreads();
-      }
-      for (int j = k >> 2; j > 0; j >>= 1) {
-        if (2 * j <= E) {   // pairs (i, i+j) stay inside an aligned block of 2j <= E items
-          local = true;
-          if (has_chunk)
-            for (int t = lane; t < (E >> 1); t += 32) {
-              const int i = c0 + 2 * t - (t & (j - 1));
-              if (i + j < n) cmp_swap<WIDE>(hi, lo, i, i + j);
-            }
-          __syncwarp();
-        } else {
-          if (local) { __syncthreads(); local = false; }
-          for (int t = threadIdx.x; t < half; t += blockDim.x) {
-            const int i = 2 * t - (t & (j - 1));
-            if (i + j < n) cmp_swap<WIDE>(hi, lo, i, i + j);
-          }
-          __syncthreads();
-        }
-      }
-    }
-  }
-  __syncthreads();
-}
-
 // First-fit admission along an order of n places, by one warp (all 32 lanes call).  cost_of(q) is the
 // cost of the candidate at place q, or -1 where there is none; every candidate is tried in order against
 // what is left of `budget` and of `room` (how many more may be taken) and taken if it fits; decide(q, taken)
@@ -602,5 +535,3 @@ int hfx_launch_fleet_apply(hfx_sched *s, int64_t now, const int32_t *decision, c
                            const int64_t *cold, const hfx_fleet *f, int64_t *clock, int64_t *maturity, int64_t *cost);
 int hfx_launch_dispatch_bind(hfx_sched *s, int64_t n, int64_t now, const int32_t *assign, const int32_t *adm_count,
                              int32_t *replica_id, int64_t *clock);
-int hfx_launch_sim(hfx_sched *s, const hfx_table *t, const int32_t *trace_off, int32_t n_traces, int32_t iters,
-                   const hfx_sim_out *o);

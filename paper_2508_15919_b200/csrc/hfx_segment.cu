@@ -34,7 +34,7 @@ struct BlockShared {
   int32_t red_n[32];
   ReplicaPlan plan;
   int64_t carry_cost;
-  int32_t carry_count, carry_act, carry_inact;
+  int32_t carry_count, carry_act;
   int64_t adm_cost, adm_kv, t1, t2, next_arrival;
   int32_t adm_count, worked, n_act;
 };
@@ -49,7 +49,6 @@ struct SegCtx {
   HfxRec *rec;            // contiguous records (fallback: input; slabs: scratch of the larger replicas)
   const uint32_t *ordered; const uint8_t *rowflag;
   uint64_t *big_hi; uint32_t *big_lo; uint32_t *big_idx;
-  int32_t slabs;
 };
 
 // A set of threads of the block that synchronise on a hardware barrier of their own (0 = the whole block).
@@ -1921,7 +1920,6 @@ int hfx_launch_replicas(hfx_sched *s, const SegArgs &sa, int64_t n, bool slabs) 
   const int R1 = s->p.n_replicas + 1;
   SegCtx c;
   memset(&c, 0, sizeof(c));
-  c.slabs = slabs ? 1 : 0;
   c.rec = s->d_rec; c.rowflag = s->d_rowflag;
   c.big_hi = s->d_big_hi; c.big_lo = s->d_big_lo; c.big_idx = s->d_big_lo ? s->d_big_lo + s->max_rows : nullptr;
   if (slabs) {
@@ -1932,7 +1930,6 @@ int hfx_launch_replicas(hfx_sched *s, const SegArgs &sa, int64_t n, bool slabs) 
     hfx_front_shape(s, n, &c.tile_rows, &c.n_tiles);
   } else {
     c.seg_count = s->d_seg_count; c.act_count = s->d_act_count; c.seg_begin = s->d_seg_begin;
-    c.ordered = s->d_flags;
   }
   // one block per SM; the fallback layout has nothing that every block shares, so it needs no more blocks than replicas
   const int grid = slabs ? s->n_sm : (R1 < s->n_sm ? R1 : s->n_sm);

@@ -35,13 +35,12 @@
 #define SIM_PARKED (SIM_BINS * 2)   // admitted requests of an iteration that are noted in shared memory (over the bins)
 #define SIM_SCRATCH_PER_SM 16      // most traces worked on at once per SM with the rows in scratch
 
-// the byte of a row: class<6> | state<2>; the word of a row: prompt_len<25> | prio<6>, prio 63 marks a row with bad data
+// the byte of a row: class<6> | state<2>; the word of a row: prompt_len<25> | prio<6>
 #define ROW_CLS(x) ((x) & 0x3fu)
 #define ROW_STATE(x) ((x) >> 6)
 #define ROW_BYTE(cls, st) ((uint8_t)((cls) | ((st) << 6)))
 #define ROW_PROMPT(w) ((int32_t)((w) & 0x1ffffffu))
 #define ROW_PRIO(w) ((w) >> 25)
-#define ROW_INVALID_PRIO 63u
 
 struct SimArgs {
   const uint8_t *class_id; const int32_t *prompt_len; const int32_t *output_len; const int64_t *arrival;

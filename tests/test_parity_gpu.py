@@ -1329,11 +1329,12 @@ def test_dispatch_whose_grid_barrier_runs_out_hands_out_nothing(n, R, d_stage):
     sched.close()
 
 
-@pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100), (40, 8300), (1000, 295), (1100, 270), (1500, 698)])
+@pytest.mark.parametrize("R,rows_per", [(2047, 20), (2048, 20), (200, 2100), (300, 2100), (40, 8300), (1000, 295), (1100, 270), (1500, 698), (1023, 90), (1024, 90)])
 def test_idle_replicas_find_their_next_arrivals(R, rows_per):
     # Tiles note every replica's next arrival up to 2047 replicas, lists are searched beyond; lists of more than 2048 rows (a few
     # of them, or hundreds) wait for the end of the kernel, and unbound rows that fill a tile are listed by the whole block.  The notes
-    # share a tile's memory with its slots: few tall tiles, low tiles with many replicas, about the same size of both.
+    # share a tile's memory with its slots: few tall tiles, low tiles with many replicas, about the same size of both.  Rows are ranked by
+    # warp up to 1023 replicas.
     n = R * rows_per + 5000
     wl = gen.random_table(R, n, R, modes=(gen.COLOCATED, gen.DECODE), permute_ids=False, inflight=0.0, done=0.98, future=0.0)
     t = wl.table

@@ -75,7 +75,11 @@ enum { KSLOT_COUNT = 0, KSLOT_COLSCAN, KSLOT_OFFSETS, KSLOT_REGROUP, KSLOT_SEG_S
 #define HFX_TILE_ROWS_MAX 8192
 #define HFX_TILE_MATRIX_MAX (INT64_C(8) << 20)   // entries of the tile matrix (64 MiB), the tiles of one round of the SMs left out
 #define HFX_TILE_REPLICAS_MAX 4095               // replicas whose counters fit in shared memory (12-bit bucket ids)
-#define HFX_NEXT_REPLICAS_MAX 2047               // replicas up to which a tile notes the next arrival of each (8 bytes of shared memory per replica)
+// Replicas up to which a tile notes the next arrival of each (8 bytes a replica, over the tile's slots); beyond them an idle replica's rows are
+// looked through instead.  1 M rows, with notes / without: ten steps over 1024 replicas 695 / 709 us, 2048 993 / 967, 3000 1260 / 1193, 4095
+// 1770 / 1552 (the matrix of notes is written and read in every step, and from about 2600 replicas on it makes the tiles lower); three ticks of the
+// scaling loop, whose replicas have long lists of finished rows, 1024 1351 / 1670, 2048 1929 / 2215, 3000 2413 / 2253, 4094 3435 / 2578.
+#define HFX_NEXT_REPLICAS_MAX 2047
 #define HFX_WAIT_LIMIT (1u << 22)                // polls of a grid barrier before the kernel gives up (about two seconds)
 
 struct HfxBracket { cudaEvent_t a, b; int slot; };

@@ -12,6 +12,9 @@
 
 #define ATT_THREADS 256
 #define ATT_FIELDS 6
+// Classes whose totals a thread keeps in registers: eight, in an instance of its own up to four.  1,048,576 rows, calls back to back: up to four
+// classes 13.4 - 15.3 us with room for four, 21.4 - 23.4 with room for eight (registers, and additions for classes that are not there),
+// 19.3 - 39.9 per warp; five to eight 23.6 - 25.3 in registers, 46 - 66 per warp; per warp 72 for nine, 182 for sixty-four.
 #define ATT_REG_CLASSES 8
 
 struct AttArgs {

@@ -497,7 +497,8 @@ static_assert(SMALL_SMEM <= SMEM_GROUP, "a group's arrays fit its share of the b
 
 // What the ids change in a rank that was counted by (key, position).  Equal keys are rare enough here to fetch the ids (many of
 // them overfill a bin).  Not inlined: steps whose ids rise pay for every instruction beside theirs
-// (1024 replicas of 293 rows, permuted ids: 60.6 us with a sorting network on 96-bit items, 48.3 now).
+// (one step with permuted ids, with a sorting network on 96-bit items / now: 1024 replicas of 293 rows 58.2 / 42.5 us, 512 of 586 64.4 / 39.7,
+// 2048 of 488 170.8 / 104.7).
 __device__ __noinline__ uint32_t rank_by_id(const uint64_t *items, const int32_t *rows, const int32_t *req_id, uint64_t x, uint32_t g0, uint32_t g1) {
   uint32_t d = 0;
   for (uint32_t g = g0; g < g1; g++) {

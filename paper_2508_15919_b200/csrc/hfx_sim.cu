@@ -33,7 +33,10 @@
 #define SIM_HEAD_BYTES(nc) ((((size_t)(nc) * 40 + 16 + SIM_BINS * 4) + 15) & ~(size_t)15)     // in front of the rows: TTFT and TPOT by class and by rank, the bins, two counters per class
 #define SIM_OUTLEN_CAP (1 << 30)   // output lengths are clamped here when the finish iteration is formed
 #define SIM_PARKED (SIM_BINS * 2)   // admitted requests of an iteration that are noted in shared memory (over the bins)
-#define SIM_SCRATCH_PER_SM 16      // most traces worked on at once per SM with the rows in scratch
+// Most traces worked on at once per SM with the rows in scratch: what the registers of a warp (116 a thread, a quarter of the file per
+// scheduler) let in; room for more changes nothing.  4096 traces of 2048 rows: 8 a SM 33.2 ms, 12 27.6, 16 21.3, 20 - 32 21.3 - 21.4; 2048
+// of 4096 rows 42.0, 39.9, 24.3, 24.3 - 24.5; 4096 of 1024 rows 11.4, 11.4, 9.8, 9.7 - 9.8.
+#define SIM_SCRATCH_PER_SM 16
 
 // the byte of a row: class<6> | state<2>; the word of a row: prompt_len<25> | prio<6>
 #define ROW_CLS(x) ((x) & 0x3fu)
@@ -106,8 +109,7 @@ __device__ __forceinline__ SimRow sim_load_row(const SimArgs &a, int64_t g, bool
 
 // SCRATCH: the per-row arrays (13 bytes a row) live in the block's part of a global scratch buffer and only the list in
 // shared memory.  The live rows then come from L1 most of the time, and more than twice as many traces are resident: what
-// a batch of more traces than shared memory holds needs, since a warp by itself issues in one cycle of six (4096 traces of
-// 2048 rows: 7 a SM 28.4 ms, 14 a SM 23.5 ms with the same code).
+// a batch of more traces than shared memory holds needs, since a warp by itself issues in one cycle of six.
 template <bool SCRATCH>
 __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, uint32_t *__restrict__ work_counter,
                                             uint32_t *__restrict__ status, unsigned char *__restrict__ scratch) {
@@ -723,7 +725,8 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   if (per_sm > 32) per_sm = 32;
   int per_sm_scratch = (int)(sm_bytes / (list_bytes + block_bytes));
   if (per_sm_scratch > SIM_SCRATCH_PER_SM) per_sm_scratch = SIM_SCRATCH_PER_SM;
-  // rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would
+  // Rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would.  Traces of 2048 rows,
+  // shared memory / scratch: 1036 (seven a SM) 7.4 / 8.6 ms, 1037 10.4 / 8.6, 1480 14.2 / 9.8; of 4096 rows: 444 15.2 / 17.1, 888 29.9 / 21.3.
   if (per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch)) {
     int grid = s->n_sm * per_sm;
     if (grid > n_traces) grid = n_traces;

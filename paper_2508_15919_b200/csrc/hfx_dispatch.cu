@@ -253,8 +253,9 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting; rows out in order, running totals
 // An item is moved once (into its bin) where the radix passes moved it eleven times.  Ordering a queue of 471 K entries and
-// its running totals: about 170 us in 20 launches before, 90 us now, of it a good third latency between the phases (a queue
-// of 42 K: 41 us); the counters of the bins (26 K cycles) and the tiles (36 K) are the rest.
+// its running totals: about 170 us in 20 launches before; 123 us now by event brackets, which hold the cooperative launch too, some 108
+// in a call (a queue of 42 K: 52 us), a good part of it latency between the phases; the counters of the bins (26 K cycles) and the tiles
+// (36 K) are most of the rest.  Issue slots 24 %, DRAM 0.7 %.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
@@ -693,7 +694,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 // window or, if it started this one, searched for (32 ways).  The other warps meanwhile stage the next chunk of totals in
 // shared memory and look up where the runs of the chunk before ended (the entries up to a base are those within it).
 // Then all threads: what every instance took, dispatching step 4 (its new maturity time).  1024 instances, 471 K entries:
-// 272 us when the totals were probed in shared memory, about 120 us now (190 cycles per instance, 105 of them the recurrence).
+// 272 us when the totals were probed in shared memory, 117 us now (190 cycles per instance, 105 of them the recurrence).
 // ------------------------------------------------------------------------------------------------
 // longest m in [lo, hi] with fits(m), given fits(lo) and fits monotone; whole warp
 template <typename F>

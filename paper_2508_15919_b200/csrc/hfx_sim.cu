@@ -9,34 +9,39 @@
 //     "has anything arrived?" is a comparison with the next arrival time, and a row that has arrived simply
 //     waits there (the box); when the window moves on, what is left of it joins a list sorted by (prio, slack base,
 //     id), which is the order of the queue at any later time (all slacks fall together);
-//   - a running request's finish iteration is fixed at admission and the smallest one is kept, so the running
-//     list is only walked in an iteration that finishes somebody;
-//   - admission is only tried when the budget reaches the shortest queued prompt (a bound kept beside the queue); it
-//     takes the most urgent requests from the list's end and the box until one no longer fits;
+//   - a running request's finish iteration is fixed at admission; the first 128 of them are in registers, four a lane, what else their
+//     end needs in shared memory, and the smallest one is kept, so nobody is looked at in an iteration that finishes nobody
+//   - the budget is solved for once a decision (sim_budget), and not at all while nothing of the queue can fit: after a decision that
+//     admitted nothing E_d only grows until a request arrives, finishes or is admitted.  Admission takes the most urgent requests from the
+//     list's end and the window, whose rows were put in order of urgency when it opened, until one no longer fits;
 //   - iterations in which nothing arrives, finishes or is admitted are taken 32 at a time: the clock after j of
 //     them is now + j E_d + d2 n_run j (j - 1) / 2 (every request in flight adds one token of context), lane j
-//     forms it and a ballot finds the first one that something happens in.  Such a stretch cannot admit: with the
-//     batch and the queue fixed E_d only grows, and a prompt that did not fit the budget bound does not fit it
-//     under a larger E_d; before maturity the stretch ends at maturity.
-// Measured (B200): one trace of 256 rows, 2000 iterations 3.45 -> 0.79 ms; 4096 traces of 2048 rows, 10,000 iterations 103
-// -> 21.3 ms (392 M -> 1.9 G iterations/s), against a block of 128 threads per trace that met five barriers and
-// looked at every request in flight in every iteration.  What is left is one dependent chain per trace: 228 warp instructions per
-// simulated iteration on the 4096 traces (9.2 G in all), issued in 40 % of the slots by 3.4 warps to a scheduler.
-// A row takes 15 bytes: one 8-byte slot (slack base while queued, admission and finish iteration
-// while running), a word (prompt length and priority), a byte (class and state) and one list entry (the queue from
-// the front of the list array, the running batch from its back: a row is in one of them at most).
+//     forms it and a ballot finds the first one that something happens in.  Before maturity the stretch ends at maturity.
+// What bounds it is one dependent chain per trace.  B200, one trace of 256 rows, 2000 iterations: 807 us with the running batch in a list in
+// memory and comparisons of 128-bit products in place of the budget, 710 now (280 K warp instructions then, 249 K when the batch went into
+// registers, at 5.6 cycles each, half of it the latency of the instruction in front); 4096 traces of 2048 rows, 10,000 iterations 21.3 -> 15.1 ms
+// (loads waited 2.5 of 9 cycles an instruction, rows of the queue and the batch scattered over sectors of L1 and L2).  Tried: the queue's list with
+// holes in place of closing it up (17.0 -> 23.4 ms: large prompts that never fit stay in front and are passed each time), 20 and 28
+// traces an SM with 96 and 72 registers (18.0, 30.7 ms against 17.1), output lengths copied ahead with cp.async (17.0 -> 18.0).
+// A row takes 19 bytes: 16 side by side, which are one look at it (slack base while queued, admission and finish iteration while running; prompt length
+// and priority; output length), a byte (class and state) and one list entry (the queue from the front of the list array, what the
+// registers do not hold of the running batch from its back: a row is in one of them at most).
 #include "hfx_internal.cuh"
 
-#define SIM_SMEM_ROWS 10240          // longest trace whose rows are kept in shared memory (15 bytes each)
-#define SIM_BYTES_PER_ROW 13           // besides the 2 bytes of the list
+#define SIM_SMEM_ROWS 10240          // longest trace whose rows are kept in shared memory (19 bytes each)
+#define SIM_BYTES_PER_ROW 16           // besides the 3 bytes of list, class and state
+#define SIM_RUN_REGS 128             // requests in flight whose finish iteration is in a register (four a lane); more of them are in a list
 #define SIM_BINS 256                 // bins of the percentile selection (8 bits a pass)
 #define SIM_HEAD_BYTES(nc) ((((size_t)(nc) * 40 + 16 + SIM_BINS * 4) + 15) & ~(size_t)15)     // in front of the rows: TTFT and TPOT by class and by rank, the bins, two counters per class
+#define SIM_LISTS_BYTES(nc, cap) (SIM_HEAD_BYTES(nc) + SIM_RUN_REGS * 8 + (size_t)(cap) * 3)      // what is in shared memory wherever the rows are
 #define SIM_OUTLEN_CAP (1 << 30)   // output lengths are clamped here when the finish iteration is formed
 #define SIM_PARKED (SIM_BINS * 2)   // admitted requests of an iteration that are noted in shared memory (over the bins)
-// Most traces worked on at once per SM with the rows in scratch: what the registers of a warp (116 a thread, a quarter of the file per
-// scheduler) let in; room for more changes nothing.  4096 traces of 2048 rows: 8 a SM 33.2 ms, 12 27.6, 16 21.3, 20 - 32 21.3 - 21.4; 2048
-// of 4096 rows 42.0, 39.9, 24.3, 24.3 - 24.5; 4096 of 1024 rows 11.4, 11.4, 9.8, 9.7 - 9.8.
+// Most traces worked on at once per SM with the rows in scratch: what the registers of a warp (119 a thread, a quarter of the file per
+// scheduler) let in.  4096 traces of 2048 rows: 8 a SM 25.7 ms, 12 20.5, 16 15.1.
 #define SIM_SCRATCH_PER_SM 16
+
+#define SIM_SM_BYTES (227 * 1024)    // shared memory of an SM, of which every block takes 1 KB for itself
+#define SIM_BLOCK_BYTES 1024
 
 // the byte of a row: class<6> | state<2>; the word of a row: prompt_len<25> | prio<6>
 #define ROW_CLS(x) ((x) & 0x3fu)
@@ -58,9 +63,19 @@ struct SimArgs {
 
 #define FULL 0xffffffffu
 
+// Fields of the 16-byte rows: one sector holds all that an admission asks of a queued row.
+template <typename T, int AT>
+struct SimField {
+  unsigned char *rows;
+  __device__ __forceinline__ T &operator[](int i) const { return *reinterpret_cast<T *>(rows + 16 * (size_t)i + AT); }
+};
+typedef SimField<int64_t, 0> SimSlots;
+typedef SimField<uint32_t, 8> SimWords;
+typedef SimField<int32_t, 12> SimLens;
+
 // The nearest-rank percentile of n non-negative values: 8 bits a pass from the highest byte in use, the warp counting the
 // values that share the prefix found so far.  All lanes call; all get the result.
-__device__ int64_t warp_percentile(const int64_t *v, int n, int pct, uint32_t *bins, int lane) {
+__device__ int64_t warp_percentile(const SimSlots v, int n, int pct, uint32_t *bins, int lane) {
   if (n == 0) return -1;
   int64_t k = ((int64_t)pct * n + 99) / 100;
   if (k < 1) k = 1;
@@ -95,19 +110,35 @@ __device__ int64_t warp_percentile(const int64_t *v, int n, int pct, uint32_t *b
 }
 
 // one row of the arrival window, as a lane holds it
-struct SimRow { int64_t arr; int32_t prompt, weight; uint32_t cls; };
+struct SimRow { int64_t arr; int32_t prompt, weight; uint32_t cls, id; int32_t len; };
 
 __device__ __forceinline__ SimRow sim_load_row(const SimArgs &a, int64_t g, bool in) {
   SimRow r;
-  r.arr = HFX_INF; r.prompt = -1; r.weight = 0; r.cls = 0;
+  r.arr = HFX_INF; r.prompt = -1; r.weight = 0; r.cls = 0; r.id = 0; r.len = 0;
   if (in) {
-    r.arr = a.arrival[g]; r.prompt = a.prompt_len[g]; r.cls = a.class_id[g];
+    r.arr = a.arrival[g]; r.prompt = a.prompt_len[g]; r.cls = a.class_id[g]; r.id = (uint32_t)a.req_id[g] ^ 0x80000000u; r.len = a.output_len[g];
     if (a.weight) r.weight = a.weight[g];
   }
   return r;
 }
 
-// SCRATCH: the per-row arrays (13 bytes a row) live in the block's part of a global scratch buffer and only the list in
+// Largest n in [0, cap] with E_p(n) den <= ttft y, 0 if there is none (ttft, y, den > 0; the whole warp calls).  The bound is solved for n in
+// single precision, and lanes settle the 32 values around the answer exactly; where all of them or none hold it is searched for.
+// (Comparisons of 128-bit products only, without the answer, were 50 instructions each, several to an admission.)
+__device__ __forceinline__ uint32_t sim_budget(const HfxParams &p, int64_t ttft, int64_t y, int64_t den, uint32_t cap, int lane) {
+  const uint64_t nh = __umul64hi((uint64_t)ttft, (uint64_t)y), nl = (uint64_t)ttft * (uint64_t)y;
+  const float c1 = (float)p.c1, x = __fdividef((float)ttft * (float)y, (float)den) - (float)p.c0;
+  const float est = x > 0.0f ? __fdividef(2.0f * x, c1 + __fsqrt_rn(c1 * c1 + 4.0f * (float)p.c2 * x)) : 0.0f;
+  const uint32_t g = est < (float)cap ? (uint32_t)est : cap;
+  const uint32_t first = g > 15u ? g - 15u : 0u, n = first + (uint32_t)lane;
+  const uint64_t ep = (uint64_t)p.c0 + ((uint64_t)p.c1 + (uint64_t)p.c2 * n) * n;
+  const uint64_t h = __umul64hi(ep, (uint64_t)den), l = ep * (uint64_t)den;
+  const uint32_t m = __ballot_sync(FULL, n <= cap && (h < nh || (h == nh && l <= nl)));      // (E_p does not fall: the ones that hold are the first)
+  if ((m == 0u && first > 0u) || (m == FULL && first + 31u < cap)) return (uint32_t)warp_nsafe(p, nh, nl, (uint64_t)den, (int64_t)cap, lane);
+  return m ? first + (uint32_t)__popc(m) - 1u : 0u;
+}
+
+// SCRATCH: the 16 bytes of every row live in the block's part of a global scratch buffer, only list, classes and states in
 // shared memory.  The live rows then come from L1 most of the time, and more than twice as many traces are resident: what
 // a batch of more traces than shared memory holds needs, since a warp by itself issues in one cycle of eight.
 template <bool SCRATCH>
@@ -121,13 +152,16 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
   uint32_t *s_bins = reinterpret_cast<uint32_t *>(s_tpot + nc + 1);
   uint16_t *s_park = reinterpret_cast<uint16_t *>(s_bins);      // [SIM_PARKED] the requests admitted in an iteration
   int32_t *s_cq = reinterpret_cast<int32_t *>(s_bins + SIM_BINS), *s_cr = s_cq + nc;      // requests in the queue's list / in flight per class
-  uint16_t *s_q = reinterpret_cast<uint16_t *>(smem_raw + SIM_HEAD_BYTES(nc));
-  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * cap * SIM_BYTES_PER_ROW : smem_raw + SIM_HEAD_BYTES(nc) + (size_t)cap * 2;
-  int64_t *s_slot = reinterpret_cast<int64_t *>(rows_mem);             // slack base in the queue; finish iteration | admission iteration << 32 in the batch; later the TTFT, then the TPOT samples
-  uint32_t *s_word = reinterpret_cast<uint32_t *>(s_slot + cap);       // prompt_len | prio << 25
+  uint16_t *s_q = reinterpret_cast<uint16_t *>(smem_raw + SIM_HEAD_BYTES(nc) + SIM_RUN_REGS * 8);
+  uint8_t *s_byte = reinterpret_cast<uint8_t *>(s_q + cap);               // class | state << 6
+  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * cap * SIM_BYTES_PER_ROW : smem_raw + SIM_LISTS_BYTES(nc, cap);
+  const SimSlots s_slot = {rows_mem};             // slack base in the queue; finish iteration | admission iteration << 32 in the batch; later the TTFT, then the TPOT samples
+  const SimWords s_word = {rows_mem};                                  // prompt_len | prio << 25
+  const SimLens s_len = {rows_mem};                                    // output length
   // One list array for both lists: from the front the queue's list (row indices, the least urgent first), from the back the
   // running batch (RUN(s), unordered)
-  uint8_t *s_byte = reinterpret_cast<uint8_t *>(s_word + cap);            // class | state << 6
+  uint32_t *s_rinfo = reinterpret_cast<uint32_t *>(smem_raw + SIM_HEAD_BYTES(nc));      // [SIM_RUN_REGS] requests in flight by slot: row | class << 16
+  int32_t *s_rctx = reinterpret_cast<int32_t *>(s_rinfo + SIM_RUN_REGS);                // [SIM_RUN_REGS] prompt length less the admission iteration
 #define RUN(s) s_q[cap - 1 - (s)]
   const int lane = threadIdx.x;
   const uint32_t lt = (1u << lane) - 1u;
@@ -167,6 +201,10 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
 
     int64_t now = 0, mat = 0, sum_kv = 0;
     int nq = 0, nr = 0, it = 0;
+    int n_list = 0;                           // requests in flight that are in the list (the others have a slot each)
+    int32_t r_fin[SIM_RUN_REGS / 32];         // finish iteration of the request in slot lane + 32 k (INT32_MAX: none)
+#pragma unroll
+    for (int k = 0; k < SIM_RUN_REGS / 32; k++) r_fin[k] = INT32_MAX;
     int32_t min_prompt = INT32_MAX;           // a lower bound of the shortest prompt in the queue: lowered by every arrival, made exact
                                               // when the whole queue has been looked at (an admission can only raise the true value)
     int32_t next_fin = INT32_MAX;             // the earliest finish iteration in the running batch
@@ -178,42 +216,72 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
     auto parked = [&](int k) -> int { return k < SIM_PARKED ? (int)s_park[k] : a.gen[(int64_t)b + k]; };
     auto id_of = [&](int row) -> uint32_t { return (uint32_t)__ldg(a.req_id + b + row) ^ 0x80000000u; };
 
-    // The window: rows wb .. wb + 31, one per lane.  pend: the valid ones that have not arrived; box: those that have arrived
-    // and wait (the young part of the queue stays here; what is left of it joins the sorted list when the window moves on).
+    // The window: rows wb .. wb + 31.  Lane l holds the arrival of row wb + l, and word, class and slack base of the l-th most urgent row of
+    // them, row wb + src (an order that no later decision changes, found once when the window opens: the most urgent of a set of lanes is
+    // its lowest one).  pend, by arrival: the valid ones that have not arrived; box, by urgency: those that have arrived and wait (the
+    // young part of the queue stays here; what is left of it joins the sorted list when the window moves on).
     int wb = 0;
     SimRow w = sim_load_row(a, (int64_t)b + lane, lane < m);
     SimRow wn = sim_load_row(a, (int64_t)b + 32 + lane, 32 + lane < m);
-    uint32_t word = 0, pend = 0, box = 0, wrank = 0;
+    uint32_t word = 0, pend = 0, box = 0, wrank = 0, wcls = 0;
+    int src = 0, wlen = 0;
     int64_t base = BASE_UNBOUNDED;            // slack base, ttft_slo + arrival - E_p(prompt_len): the slack at any later decision is the base minus the earliest start
+    auto put_row = [&](int row) { *reinterpret_cast<uint4 *>(&s_slot[row]) = make_uint4((uint32_t)(uint64_t)base, (uint32_t)((uint64_t)base >> 32), word, (uint32_t)wlen); };
     auto open_window = [&]() {
       const bool ok = wb + lane < m && w.cls < (uint32_t)nc && w.prompt >= 0 && w.prompt <= HFX_MAX_TOKENS;
-      base = BASE_UNBOUNDED; wrank = nc;
+      uint32_t prio = 64u, wd = 0;            // (rows with bad data come last)
+      int64_t be = BASE_UNBOUNDED;
       if (ok) {
-        uint32_t prio;
         if (p.weight_max > 0) {
           const int64_t x = (int64_t)p.weight_max - w.weight;
           prio = (uint32_t)(x < 0 ? 0 : (x > 62 ? 62 : x));
         } else prio = p.prio[w.cls];
-        word = (uint32_t)w.prompt | (prio << 25);
+        wd = (uint32_t)w.prompt | (prio << 25);
         const int64_t ttft = c_ttft[w.cls];
-        if (ttft > 0) base = ttft + w.arr - dev_Ep(p, w.prompt);
+        if (ttft > 0) be = ttft + w.arr - dev_Ep(p, w.prompt);
       }
-      wrank = __shfl_sync(FULL, rt0, w.cls & 31u);
-      if (nc > 32) { const uint32_t r1 = __shfl_sync(FULL, rt1, w.cls & 31u); if (w.cls >= 32u) wrank = r1; }
       pend = __ballot_sync(FULL, ok);
-      const bool bounded = ok && base != BASE_UNBOUNDED;
-      const int64_t lo = warp_min_i64(bounded ? base : HFX_INF), hi = ~warp_min_i64(bounded ? ~base : HFX_INF);
+      const bool bounded = ok && be != BASE_UNBOUNDED;
+      const int64_t lo = warp_min_i64(bounded ? be : HFX_INF), hi = ~warp_min_i64(bounded ? ~be : HFX_INF);
       base_lo = lo < base_lo ? lo : base_lo; base_hi = hi > base_hi ? hi : base_hi;
+      // Rows of the window that are more urgent than mine, by (prio, base, id).  The bases are taken as 56 bits beside the priority; where one
+      // does not fit, or two rows are equal in it, the whole comparison is made.
+      const int64_t narrow = be == BASE_UNBOUNDED ? (INT64_C(1) << 56) : be;
+      const uint64_t k = ((uint64_t)prio << 57) + (uint64_t)(narrow + (INT64_C(1) << 56));
+      bool whole = narrow < -(INT64_C(1) << 56) || (be != BASE_UNBOUNDED && narrow >= (INT64_C(1) << 56));
+      int place = 0, same = 0;
+#pragma unroll 8
+      for (int l = 0; l < 32; l++) {
+        const uint64_t x = __shfl_sync(FULL, k, l);
+        place += x < k ? 1 : 0; same += x == k ? 1 : 0;
+      }
+      whole = __any_sync(FULL, whole || same > 1);
+      if (whole) {
+        place = 0;
+        for (int l = 0; l < 32; l++) {
+          const uint32_t pr = __shfl_sync(FULL, prio, l), id = __shfl_sync(FULL, w.id, l);
+          const int64_t x = __shfl_sync(FULL, be, l);
+          const bool first = id < w.id || (id == w.id && l < lane);
+          place += pr < prio || (pr == prio && (x < be || (x == be && first))) ? 1 : 0;
+        }
+      }
+      s_park[place] = (uint16_t)lane;         // (no admission is under way)
+      __syncwarp();
+      src = s_park[lane];
+      __syncwarp();
+      word = __shfl_sync(FULL, wd, src); base = __shfl_sync(FULL, be, src); wcls = __shfl_sync(FULL, w.cls, src); wlen = __shfl_sync(FULL, w.len, src);
+      wrank = __shfl_sync(FULL, rt0, wcls & 31u);
+      if (nc > 32) { const uint32_t r1 = __shfl_sync(FULL, rt1, wcls & 31u); if (wcls >= 32u) wrank = r1; }
     };
     // The box joins the list: every waiting row finds its place by a binary search of its own and its rank among the
     // others, then the more urgent entries move up, 32 at a time from the top down.
     auto merge_box = [&]() {
       const bool me = (box >> lane) & 1u;
-      const int row = wb + lane;
+      const int row = wb + src;
       const uint32_t prio = ROW_PRIO(word);
       if (me) {
-        s_word[row] = word; s_slot[row] = base; s_byte[row] = ROW_BYTE(w.cls, HFX_QUEUED);
-        atomicAdd(&s_cq[w.cls], 1);
+        put_row(row); s_byte[row] = ROW_BYTE(wcls, HFX_QUEUED);
+        atomicAdd(&s_cq[wcls], 1);
       }
       int pos = 0;                            // entries of the list that are less urgent than mine
       for (int hi = nq; __any_sync(FULL, pos < hi);) {
@@ -226,15 +294,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           if (less) pos = mid + 1; else hi = mid;
         }
       }
-      int rank = 0;
-      for (uint32_t x = box; x; x &= x - 1) {
-        const int l = __ffs(x) - 1;
-        const uint32_t pr = __shfl_sync(FULL, prio, l);
-        const int64_t be = __shfl_sync(FULL, base, l);
-        bool less = pr > prio || (pr == prio && be > base);
-        if (me && lane != l && pr == prio && be == base) less = id_of(wb + l) > id_of(row);
-        rank += less ? 1 : 0;
-      }
+      const int rank = __popc(box & ~((2u << lane) - 1u));      // those of the box that are less urgent
       for (int c0 = (nq - 1) & ~31; nq > 0 && c0 >= 0; c0 -= 32) {
         const int e = c0 + lane;
         const uint32_t below = __ballot_sync(FULL, me && pos <= c0), in = __ballot_sync(FULL, me && pos > c0 && pos <= c0 + 31);
@@ -269,6 +329,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
     open_window();
     advance_window();
     int64_t next_arr = pend ? __shfl_sync(FULL, w.arr, __ffs(pend) - 1) : HFX_INF;
+    bool blocked = false;                     // nothing of the queue fits the budget until a request arrives, finishes or is admitted: E_d only grows
 
     while (it < a.iters) {
       // ---- 1. arrivals: the rows with arrival <= now join the queue -------------------------------------------
@@ -280,57 +341,46 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           // (a trace that is not sorted by arrival is a caller error: the rows behind one that has not arrived wait for it)
           const uint32_t late = pend & ~__ballot_sync(FULL, w.arr <= now);
           const uint32_t come = late ? pend & ((1u << (__ffs(late) - 1)) - 1u) : pend;
-          const bool me = (come >> lane) & 1u, over = me && w.prompt > cfg.token_cap;
+          const bool me = (come >> src) & 1u, over = me && ROW_PROMPT(word) > cfg.token_cap;
           const uint32_t om = __ballot_sync(FULL, over);
-          const int32_t shortest = (int32_t)__reduce_min_sync(FULL, me && !over ? (uint32_t)w.prompt : 0x7fffffffu);
+          const int32_t shortest = (int32_t)__reduce_min_sync(FULL, me && !over ? (uint32_t)ROW_PROMPT(word) : 0x7fffffffu);
           min_prompt = shortest < min_prompt ? shortest : min_prompt;
           if (om) {                           // never served: rejected at this iteration's commit
-            if (over) s_byte[wb + lane] = ROW_BYTE(w.cls, HFX_REJECTED);
+            if (over) s_byte[wb + src] = ROW_BYTE(wcls, HFX_REJECTED);
             const uint32_t r = __reduce_min_sync(FULL, over ? wrank : (uint32_t)nc);
             over_rank = r < over_rank ? r : over_rank;
             over_any = true;
           }
-          box |= come & ~om;
+          box |= __ballot_sync(FULL, me && !over);
           pend &= ~come;
           if (pend == 0) advance_window();
           next_arr = pend ? __shfl_sync(FULL, w.arr, __ffs(pend) - 1) : HFX_INF;
         } while (next_arr <= now);
+        blocked = false;
         min_ttft = strictest_q();
         ttft_it = min_ttft;
         if (over_any) { const int64_t x = s_ttft[over_rank]; ttft_it = x < ttft_it ? x : ttft_it; }
       }
 
       // ---- 2. plan: E_d of the running batch, the safe budget (Eq. 3) as a bound on E_p ----------------------
-      // The budget is the largest n <= cap_left with E_p(n) den <= num, 0 if there is none.  Only comparisons with it are
-      // needed, so it is not worked out: E_p does not fall with n, so n is within the budget exactly if n satisfies the bound.
+      // The budget is the largest n <= cap_left with E_p(n) den <= num, 0 if there is none (and before maturity: then only a zero-token prompt fits it).
       const int64_t e_d = nr > 0 ? dev_Ed(p, nr, sum_kv) : 0;
-      int64_t cap_left = 0;                   // before maturity the budget is 0: only a zero-token prompt fits it
-      uint64_t num_h = ~0ull, num_l = ~0ull, den = 0;
+      uint32_t budget = 0;
       bool scan = false;
-      auto within = [&](int64_t n) -> bool {
-        const uint64_t ep = (uint64_t)dev_Ep(p, n);
-        const uint64_t h = __umul64hi(ep, den), l = ep * den;
-        return n == 0 || (n <= cap_left && (h < num_h || (h == num_h && l <= num_l)));
-      };
-      if (nq > 0 || box) {
+      if (!blocked && (nq > 0 || box)) {
         if (now >= mat) {
-          cap_left = cfg.token_cap - nr > 0 ? cfg.token_cap - nr : 0;
-          const int64_t ttft = ttft_it;
-          if (p.budget_mode != HFX_BUDGET_CAP_ONLY && ttft != HFX_INF) {
-            num_h = 0; num_l = (uint64_t)ttft; den = 2;            // 2 E_p <= TTFT while nothing decodes
-            if (nr > 0 && min_tpot < HFX_INF) {
-              if (min_tpot > e_d) {
-                const uint64_t y = (uint64_t)(min_tpot - e_d);
-                num_h = __umul64hi((uint64_t)ttft, y); num_l = (uint64_t)ttft * y; den = (uint64_t)(2 * min_tpot - e_d);
-              } else cap_left = 0;
-            }
+          budget = cfg.token_cap - nr > 0 ? (uint32_t)(cfg.token_cap - nr) : 0u;
+          if (p.budget_mode != HFX_BUDGET_CAP_ONLY && ttft_it != HFX_INF) {
+            const bool decoding = nr > 0 && min_tpot < HFX_INF;      // 2 E_p <= TTFT while nothing decodes
+            const int64_t y = decoding ? min_tpot - e_d : 1, den = decoding ? 2 * min_tpot - e_d : 2;
+            budget = y > 0 ? sim_budget(p, ttft_it, y, den, budget, lane) : 0u;
           }
         }
-        scan = within(min_prompt);            // otherwise the shortest prompt does not fit: nothing is admitted
+        scan = (uint32_t)min_prompt <= budget;            // otherwise the shortest prompt does not fit: nothing is admitted
       }
 
       // ---- 3. admission: the most urgent requests that fit alone, until one fails ----------------------------
-      int64_t adm_cost = 0;
+      uint32_t adm_cost = 0;
       int adm_cnt = 0;
       if (scan) {
         const int64_t start = now > mat ? now : mat;
@@ -345,98 +395,62 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
             const int64_t x = s_slot[s_q[s]];
             if (x != BASE_UNBOUNDED) { lo = x < lo ? x : lo; hi = x > hi ? x : hi; }
           }
-          if (((pend >> lane) & 1u) && base != BASE_UNBOUNDED) { lo = base < lo ? base : lo; hi = base > hi ? base : hi; }
+          if (((pend >> src) & 1u) && base != BASE_UNBOUNDED) { lo = base < lo ? base : lo; hi = base > hi ? base : hi; }
           base_lo = warp_min_i64(lo); base_hi = ~warp_min_i64(~hi);
           by_key = clamped();
         }
         int low = nq;                         // the lowest place of the list that has been looked at
         bool from_list = false;
         auto room = [&]() { return cfg.batch_cap == 0 || nr + adm_cnt < cfg.batch_cap; };
-        // what the tests so far say about the budget: n_ok tokens are within it, n_bad are not; most tests end here
-        int64_t n_ok = min_prompt, n_bad = INT64_MAX;
-        auto fits = [&](int64_t n) -> bool {  // (all lanes ask for the same n)
-          if (n <= n_ok) return true;
-          if (n >= n_bad) return false;
-          const bool f = within(n);
-          if (f) n_ok = n; else n_bad = n;
-          return f;
-        };
-        auto fits_mask = [&](bool in, int32_t pr) -> uint32_t {      // (a prompt per lane)
-          bool f = in && pr <= n_ok;
-          const bool open = in && !f && pr < n_bad;
-          if (__any_sync(FULL, open)) {
-            const bool e = open && within(pr);
-            const int64_t top = __reduce_max_sync(FULL, e ? (uint32_t)pr : 0u), bottom = __reduce_min_sync(FULL, open && !e ? (uint32_t)pr : 0x7fffffffu);
-            n_ok = top > n_ok ? top : n_ok;
-            if (bottom != 0x7fffffff) n_bad = bottom < n_bad ? bottom : n_bad;
-            f = f || e;
-          }
-          return __ballot_sync(FULL, f);
-        };
         if (!by_key) {
-          // Two ordered sources: the list from the most urgent entry down, 32 entries at a time, and the box, whose most
-          // urgent row is found by minima over the lanes.
+          // Two ordered sources: the list from the most urgent entry down, 32 entries at a time, and the box, whose lanes are in
+          // order of urgency too.
           const int32_t wp = ROW_PROMPT(word);
-          uint32_t bm = box ? fits_mask((box >> lane) & 1u, wp) : 0u, fm = 0;      // rows that fit alone: in the box; in the list's chunk
+          uint32_t bm = box & __ballot_sync(FULL, (uint32_t)wp <= budget), fm = 0;      // rows that fit alone: in the box; in the list's chunk
           int32_t lmin = (box >> lane) & 1u ? wp : INT32_MAX;
-          int q = 0, i = 0, bl = -1, left = nq;
-          uint32_t wd = 0, b_prio = 0;
-          int64_t b_base = 0;
+          int q = 0, i = 0, left = nq;
+          uint32_t wd = 0;
+          int64_t list_base = 0;
           bool stop = !room();
           while (!stop) {
             while (fm == 0 && left > 0) {     // the next chunk of the list
               q = left - 1 - lane;
-              i = q >= 0 ? s_q[q] : 0;
-              wd = s_word[i];
-              if (q >= 0) lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
-              fm = fits_mask(q >= 0, ROW_PROMPT(wd));
+              i = 0; wd = 0;
+              if (q >= 0) {
+                i = s_q[q];
+                const uint4 x = *reinterpret_cast<const uint4 *>(&s_slot[i]);
+                wd = x.z; list_base = (int64_t)(((uint64_t)x.y << 32) | x.x);
+                lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
+              }
+              fm = __ballot_sync(FULL, q >= 0 && (uint32_t)ROW_PROMPT(wd) <= budget);
               left = left > 32 ? left - 32 : 0;
               low = left;
             }
-            if (bm && bl < 0) {               // the most urgent row of the box
-              const bool in = (bm >> lane) & 1u;
-              b_prio = __reduce_min_sync(FULL, in ? ROW_PRIO(word) : 64u);
-              bool cand = in && ROW_PRIO(word) == b_prio;
-              const uint32_t h = (uint32_t)((uint64_t)base >> 32) ^ 0x80000000u;
-              const uint32_t hm = __reduce_min_sync(FULL, cand ? h : ~0u);
-              cand = cand && h == hm;
-              const uint32_t lm = __reduce_min_sync(FULL, cand ? (uint32_t)base : ~0u);
-              uint32_t win = __ballot_sync(FULL, cand && (uint32_t)base == lm);
-              if (win & (win - 1)) {
-                const uint32_t id = (win >> lane) & 1u ? id_of(wb + lane) : ~0u;
-                const uint32_t least = __reduce_min_sync(FULL, id);
-                win = __ballot_sync(FULL, ((win >> lane) & 1u) && id == least);
-              }
-              bl = __ffs(win) - 1;
-              b_base = (int64_t)(((uint64_t)(hm ^ 0x80000000u) << 32) | lm);
-            }
             if (fm == 0 && bm == 0) break;    // every row that fits has been looked at
-            const int fl = __ffs(fm) - 1;
+            const int fl = __ffs(fm) - 1, bl = __ffs(bm) - 1;
             bool list = bm == 0;
             if (fm && bm) {
-              const int row = __shfl_sync(FULL, i, fl);
-              const uint32_t pr = __shfl_sync(FULL, ROW_PRIO(wd), fl);
+              const uint32_t pr = __shfl_sync(FULL, ROW_PRIO(wd), fl), b_prio = __shfl_sync(FULL, ROW_PRIO(word), bl);
               if (pr != b_prio) list = pr < b_prio;
               else {
-                const int64_t x = s_slot[row];
+                const int64_t x = __shfl_sync(FULL, list_base, fl), b_base = __shfl_sync(FULL, base, bl);
                 list = x < b_base;
-                if (x == b_base) list = id_of(row) < id_of(wb + bl);
+                if (x == b_base) list = id_of(__shfl_sync(FULL, i, fl)) < id_of(wb + __shfl_sync(FULL, src, bl));
               }
             }
-            const int32_t c = __shfl_sync(FULL, list ? ROW_PROMPT(wd) : wp, list ? fl : bl);
-            if (fits(adm_cost + c)) {
+            const uint32_t c = (uint32_t)ROW_PROMPT(__shfl_sync(FULL, list ? wd : word, list ? fl : bl));
+            if (adm_cost + c <= budget) {
               if (list) {
                 if (lane == fl) { park(adm_cnt, i); s_q[q] = 0xffffu; atomicSub(&s_cq[ROW_CLS(s_byte[i])], 1); }      // (row numbers stay below 0xffff)
                 from_list = true;
               } else {
-                if (lane == bl) { park(adm_cnt, wb + lane); s_word[wb + lane] = word; s_byte[wb + lane] = ROW_BYTE(w.cls, HFX_QUEUED); }
+                if (lane == bl) { park(adm_cnt, wb + src); put_row(wb + src); s_byte[wb + src] = ROW_BYTE(wcls, HFX_QUEUED); }
                 box &= ~(1u << bl);
               }
               adm_cost += c; adm_cnt += 1;
               stop = !room();
-            } else stop = !p.first_fit || !fits(adm_cost + min_prompt);      // (first fit: can what is left take the shortest prompt?)
-            if (list) fm &= fm - 1;
-            else { bm &= ~(1u << bl); bl = -1; }
+            } else stop = !p.first_fit || adm_cost + (uint32_t)min_prompt > budget;      // (first fit: can what is left take the shortest prompt?)
+            if (list) fm &= fm - 1; else bm &= bm - 1;
           }
           if (left == 0 && !stop) min_prompt = (int32_t)__reduce_min_sync(FULL, (uint32_t)lmin);      // every entry was looked at
         } else {
@@ -457,7 +471,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
               if (i == 0xffffu) continue;
               const uint32_t wd = s_word[i];
               lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
-              if (!within((p.first_fit ? adm_cost : 0) + ROW_PROMPT(wd))) continue;
+              if ((p.first_fit ? adm_cost : 0u) + (uint32_t)ROW_PROMPT(wd) > budget) continue;
               const uint64_t k = key_of(wd, s_slot[i]);
               const uint32_t id = (uint32_t)__ldg(a.req_id + b + i) ^ 0x80000000u;
               if (k < bk || (k == bk && id < bid)) { bk = k; bid = id; bs = s; }
@@ -473,8 +487,8 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
             if (win == 0) break;              // no eligible request left
             const int slot = __shfl_sync(FULL, bs, __ffs(win) - 1);
             const int i = s_q[slot];
-            const int32_t pr = ROW_PROMPT(s_word[i]);
-            if (!within(adm_cost + pr)) break;
+            const uint32_t pr = (uint32_t)ROW_PROMPT(s_word[i]);
+            if (adm_cost + pr > budget) break;
             __syncwarp();
             if (lane == 0) { s_q[slot] = 0xffffu; park(adm_cnt, i); atomicSub(&s_cq[ROW_CLS(s_byte[i])], 1); }
             __syncwarp();
@@ -488,6 +502,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           for (int s0 = low; s0 < nq; s0 += 32) {
             const uint16_t v = s0 + lane < nq ? s_q[s0 + lane] : (uint16_t)0xffffu;
             const uint32_t vm = __ballot_sync(FULL, v != 0xffffu);
+            __syncwarp();
             if (v != 0xffffu) s_q[to + __popc(vm & lt)] = v;      // (never beyond the places read so far)
             to += __popc(vm);
             __syncwarp();
@@ -499,6 +514,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
         // ballots between the two do not order memory).
         if (adm_cnt > 0) __syncwarp();
       }
+      blocked = adm_cnt == 0 && now >= mat && !over_any;
 
       // ---- a stretch of iterations in which nothing arrives, finishes or is admitted -------------------------
       if (adm_cnt == 0 && nr > 0 && it < next_fin) {
@@ -532,33 +548,55 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
       // list, which is closed up in place.
       sum_kv += nr;
       if (it >= next_fin) {
-        int kept = 0;
         int32_t nf = INT32_MAX;
-        for (int s0 = 0; s0 < nr; s0 += 32) {
+#pragma unroll
+        for (int k = 0; k < SIM_RUN_REGS / 32; k++) {
+          const bool done = it >= r_fin[k];
+          const uint32_t dm = __ballot_sync(FULL, done);
+          if (dm) {
+            uint32_t ctx = 0;
+            if (done) {
+              const uint32_t info = s_rinfo[32 * k + lane], cls = info >> 16;
+              const int i = info & 0xffffu;
+              s_byte[i] = ROW_BYTE(cls, HFX_DONE);
+              a.finish[(int64_t)b + i] = t2;
+              atomicSub(&s_cr[cls], 1);
+              ctx = (uint32_t)(s_rctx[32 * k + lane] + it);      // leaves with the context it has after this step
+              r_fin[k] = INT32_MAX;
+            }
+            sum_kv -= (int64_t)__reduce_add_sync(FULL, ctx & 0xffffu) + ((int64_t)__reduce_add_sync(FULL, ctx >> 16) << 16);
+            nr -= __popc(dm);
+          }
+          nf = r_fin[k] < nf ? r_fin[k] : nf;
+        }
+        int kept = 0;
+        for (int s0 = 0; s0 < n_list; s0 += 32) {
           const int s = s0 + lane;
-          const bool in = s < nr;
+          const bool in = s < n_list;
           const int i = in ? RUN(s) : 0;
           const int64_t slot = in ? s_slot[i] : 0;
           const int32_t fin = (int32_t)(uint32_t)slot;
           const bool done = in && it >= fin;
-          int64_t ctx = 0;
+          uint32_t ctx = 0;
           if (done) {
             const uint32_t cls = ROW_CLS(s_byte[i]);
             s_byte[i] = ROW_BYTE(cls, HFX_DONE);
             a.finish[(int64_t)b + i] = t2;
             atomicSub(&s_cr[cls], 1);
-            ctx = (int64_t)ROW_PROMPT(s_word[i]) + (it - (int32_t)(slot >> 32));      // leaves with the context it has after this step
+            ctx = (uint32_t)(ROW_PROMPT(s_word[i]) + (it - (int32_t)(slot >> 32)));
           }
           const uint32_t dm = __ballot_sync(FULL, done), km = __ballot_sync(FULL, in && !done);
-          if (dm) sum_kv -= (int64_t)__reduce_add_sync(FULL, (uint32_t)ctx & 0xffffu) + ((int64_t)__reduce_add_sync(FULL, (uint32_t)(ctx >> 16)) << 16);
+          __syncwarp();
+          if (dm) sum_kv -= (int64_t)__reduce_add_sync(FULL, ctx & 0xffffu) + ((int64_t)__reduce_add_sync(FULL, ctx >> 16) << 16);
           if (in && !done) {
             RUN(kept + __popc(km & lt)) = (uint16_t)i;      // (never beyond the places read so far)
             nf = fin < nf ? fin : nf;
           }
           kept += __popc(km);
+          nr -= __popc(dm);
           __syncwarp();
         }
-        nr = kept;
+        n_list = kept;
         next_fin = (int32_t)__reduce_min_sync(FULL, (uint32_t)nf);
         run_changed = true;
       }
@@ -570,25 +608,38 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           const int i = here ? parked(e0 + lane) : 0;
           bool goes_on = false;
           uint32_t kv = 0;
+          int32_t fin = 0;
+          const uint32_t cls = here ? ROW_CLS(s_byte[i]) : 0u;
           if (here) {
-            const int32_t ol = __ldg(a.output_len + b + i);
-            const uint32_t cls = ROW_CLS(s_byte[i]);
+            const int32_t ol = s_len[i];
             a.first_token[(int64_t)b + i] = t1;
             if (ol <= 1) { s_byte[i] = ROW_BYTE(cls, HFX_DONE); a.finish[(int64_t)b + i] = t1; }
             else {
               goes_on = true;
               s_byte[i] = ROW_BYTE(cls, HFX_RUNNING);
               atomicAdd(&s_cr[cls], 1);
-              const int32_t fin = it + (ol < SIM_OUTLEN_CAP ? ol : SIM_OUTLEN_CAP) - 1;
+              fin = it + (ol < SIM_OUTLEN_CAP ? ol : SIM_OUTLEN_CAP) - 1;
               s_slot[i] = (int64_t)(uint32_t)fin | ((int64_t)it << 32);
               nf = fin < nf ? fin : nf;
               kv = (uint32_t)ROW_PROMPT(s_word[i]);
             }
           }
-          const uint32_t gm = __ballot_sync(FULL, goes_on);
+          uint32_t gm = __ballot_sync(FULL, goes_on);
           sum_kv += __reduce_add_sync(FULL, kv);
-          if (goes_on) RUN(nr + __popc(gm & lt)) = (uint16_t)i;
           nr += __popc(gm);
+          // to the free slots, one after the other; the rest to the list
+#pragma unroll
+          for (int k = 0; k < SIM_RUN_REGS / 32; k++) {
+            if (gm == 0) break;
+            for (uint32_t fm = __ballot_sync(FULL, r_fin[k] == INT32_MAX); gm && fm; gm &= gm - 1, fm &= fm - 1) {
+              const int from = __ffs(gm) - 1, to = __ffs(fm) - 1;
+              const int32_t f = __shfl_sync(FULL, fin, from);
+              if (lane == to) r_fin[k] = f;
+              if (lane == from) { s_rinfo[32 * k + to] = (uint32_t)i | (cls << 16); s_rctx[32 * k + to] = (int32_t)kv - it; }
+            }
+          }
+          if ((gm >> lane) & 1u) RUN(n_list + __popc(gm & lt)) = (uint16_t)i;
+          n_list += __popc(gm);
           __syncwarp();
         }
         nf = (int32_t)__reduce_min_sync(FULL, (uint32_t)nf);
@@ -597,6 +648,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
         min_ttft = strictest_q();
       }
       if (run_changed) {
+        blocked = false;
         __syncwarp();
         uint32_t x = lane < nc && s_cr[lane] > 0 ? rp0 : (uint32_t)nc;
         if (lane + 32 < nc && s_cr[lane + 32] > 0) x = rp1 < x ? rp1 : x;
@@ -690,8 +742,8 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
 }
 
 int hfx_sim_configure() {
-  if (cudaFuncSetAttribute(k_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * (SIM_BYTES_PER_ROW + 2) + (int)SIM_HEAD_BYTES(HFX_MAX_CLASSES)) != cudaSuccess ||
-      cudaFuncSetAttribute(k_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536 * 2 + (int)SIM_HEAD_BYTES(HFX_MAX_CLASSES)) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * SIM_BYTES_PER_ROW + (int)SIM_LISTS_BYTES(HFX_MAX_CLASSES, SIM_SMEM_ROWS)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SM_BYTES - SIM_BLOCK_BYTES) != cudaSuccess)
     return HFX_E_CUDA;
   return HFX_OK;
 }
@@ -717,8 +769,8 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   a.iters_executed = o->iters_executed; a.finished = o->finished; a.rejected = o->rejected; a.attained = o->attained;
   a.ttft_p50 = o->ttft_p50_ns; a.ttft_p99 = o->ttft_p99_ns; a.tpot_p50 = o->tpot_p50_ns; a.tpot_p99 = o->tpot_p99_ns;
   a.now_out = o->now_ns;
-  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = (size_t)cap * 2 + SIM_HEAD_BYTES(s->p.n_classes);
-  const size_t sm_bytes = 227 * 1024, block_bytes = 1024;      // (1 KB per block is reserved)
+  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = SIM_LISTS_BYTES(s->p.n_classes, cap);
+  const size_t sm_bytes = SIM_SM_BYTES, block_bytes = SIM_BLOCK_BYTES;
   int rc = cuda_rc(cudaMemsetAsync(d_work_counter, 0, sizeof(uint32_t), s->stream));
   if (rc != HFX_OK) return rc;
   int per_sm = cap <= SIM_SMEM_ROWS ? (int)(sm_bytes / (rows_bytes + list_bytes + block_bytes)) : 0;
@@ -726,7 +778,7 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   int per_sm_scratch = (int)(sm_bytes / (list_bytes + block_bytes));
   if (per_sm_scratch > SIM_SCRATCH_PER_SM) per_sm_scratch = SIM_SCRATCH_PER_SM;
   // Rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would.  Traces of 2048 rows,
-  // shared memory / scratch: 1036 (seven a SM) 7.4 / 8.6 ms, 1037 10.4 / 8.6, 1480 14.2 / 9.8; of 4096 rows: 444 15.2 / 17.1, 888 29.9 / 21.3.
+  // shared memory / scratch: 444 5.64 / 5.89 ms, 740 (five a SM) 5.90 / 6.45, 1036 (scratch) 6.7; 4096 of 512 rows 3.89 / 4.07, of 256 1.89 / 2.00.
   if (per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch)) {
     int grid = s->n_sm * per_sm;
     if (grid > n_traces) grid = n_traces;

@@ -1237,6 +1237,31 @@ def test_simulator_admits_from_the_window_alone(clump, first_fit):
     assert res["finished"][0] == 0
 
 
+@pytest.mark.parametrize("m", [127, 128, 129, 161])
+def test_simulator_running_batch_beyond_the_registers(m):
+    # 128 requests in flight have their finish iteration in a register, further ones in a list: batches around that size, then places that
+    # free up in the registers while the list still holds some
+    rng = np.random.default_rng(m)
+    rows = [dict(prompt_len=int(rng.integers(1, 9)), output_len=int(rng.integers(260, 300)) if i % 3 else 240, arrival_ns=0, req_id=i, class_id=i % 2) for i in range(m)]
+    rows += [dict(prompt_len=int(rng.integers(1, 9)), output_len=int(rng.integers(2, 90)), arrival_ns=2 * SEC + i * 40 * MS, req_id=m + i) for i in range(96)]
+    wl = make_wl(rows, [(2000 * MS, 300 * MS, 0), (0, 0, 1)], replicas=[(gen.COLOCATED, 16384, 0)], trace_off=[0, m + 96], sim_iters=900)
+    assert_sim_parity(wl)
+
+
+@pytest.mark.parametrize("first_fit", [False, True])
+@pytest.mark.parametrize("model", [(0, 1, 0), (0, 0, 0), (1 << 40, 0, 1), (1 << 40, 3, 0), (0, 1 << 30, 1 << 12), (1, 0, 1 << 12), (5_000_000, 1, 0)])
+def test_simulator_budget_over_the_model_range(model, first_fit):
+    # the budget is estimated in single precision and settled exactly around the estimate, or searched for: flat, linear and steep models,
+    # bounds far above a prefill's constant part, budgets up to the largest token cap; slack bases beyond 56 bits
+    classes = [(1 << 44, 30 * MS, 0), (200 * MS, 1 << 34, 0), (0, 0, 1), (3 * SEC, 50 * MS, 1)]
+    wl = gen.random_traces(hash(model) & 0xff, 6, 40, 130, iters=900, model=tuple(model) + (8_000_000, 100_000, 20), classes=classes, token_cap=1 << 24, out_hi=60)
+    wl.table["prompt_len"][:] = np.minimum(wl.table["prompt_len"].astype(np.int64), 1 << 24)
+    wl.table["prompt_len"][::5] = np.random.default_rng(1).integers(1, 4096, wl.table["prompt_len"][::5].size)
+    if first_fit:
+        wl.meta["first_fit"] = True
+    assert_sim_parity(wl)
+
+
 @pytest.mark.parametrize("n_classes", [1, 4, 5, 8, 9, 64])
 def test_attainment_class_counts_and_ragged_rows(n_classes):
     # totals in registers (up to 4, up to 8 classes) and per warp (more); a row is left over when n is odd

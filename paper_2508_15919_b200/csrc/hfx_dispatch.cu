@@ -252,10 +252,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 //      whole queue to a radix sort instead
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting; rows out in order, running totals
-// An item is moved once (into its bin) where the radix passes moved it eleven times.  Ordering a queue of 471 K entries and
-// its running totals: about 170 us in 20 launches before; 123 us now by event brackets, which hold the cooperative launch too, some 108
-// in a call (a queue of 42 K: 52 us), a good part of it latency between the phases; the counters of the bins (26 K cycles) and the tiles
-// (36 K) are most of the rest.  Issue slots 24 %, DRAM 0.7 %.
+// An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 67 us by the GPU's clock:
+// sample and plans 12, splitters 5, bins 14, their starts 7, moving 4, tiles 12, running totals 9, barriers 1.5 each; one of 42 K in 30 blocks 36.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
@@ -593,7 +591,10 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     constexpr int IPT = (DISP_TILE_MAX + SORT_THREADS - 1) / SORT_THREADS;
     if (binned) {
       // fine bins: an even share of them for every bin of the tile, in the bin by how far into it an item lies
-      const uint32_t b0 = bin_edge(t * tile_rows), nb = bin_edge((t + 1) * tile_rows) - b0;
+      // (the last tile ends with the last bin that holds anything: with the empty bins behind it, half of them all, its items shared so few fine bins
+      // that the block counted up to 435 of them with one another while the rest of the grid had finished: dispatch of 1 M rows over 1024 instances
+      // 255 us then, 206 with this edge, of 60,013 rows 78 and 69)
+      const uint32_t b0 = bin_edge(t * tile_rows), nb = bin_edge((t + 1) * tile_rows < n_all ? (t + 1) * tile_rows : n_all) - b0;
       const int lg = nb <= DISP_FINE ? 31 - __clz(DISP_FINE / (nb > 1 ? nb : 1u)) : 0, down = nb <= DISP_FINE ? 0 : 32 - __clz((nb - 1) / DISP_FINE);      // (a tile of many empty bins: several to a fine one)
       uint32_t fp[IPT];      // fine bin << 16 | place in it (by arrival)
       for (uint32_t i = tid; i < DISP_FINE; i += SORT_THREADS) s_fine[i] = 0;

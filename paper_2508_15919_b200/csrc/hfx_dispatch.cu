@@ -23,13 +23,14 @@
 #define SORT_THREADS 1024
 #define DISP_CLASSES 128            // stage<1> | priority<6>
 #define DISP_SAMPLES 2048           // items of the sample at most; one in 64 of the queue
-#define DISP_STEP 8                 // samples per splitter interval
+#define DISP_STEP 4                 // samples per splitter interval
 #define DISP_SPLITS (DISP_SAMPLES / DISP_STEP + 3 * DISP_CLASSES)
-#define DISP_SUB 16                 // bins an interval is divided into evenly
+#define DISP_SUB 8                  // bins an interval is divided into evenly
 #define DISP_BINS (DISP_SPLITS * DISP_SUB)
-#define DISP_BIN_MAX 1024           // fuller bins send the queue to the radix sort
-#define DISP_TILE 4096              // queue entries a block orders at a time (and one bin more)
-#define DISP_TILE_MAX (DISP_TILE + DISP_BIN_MAX)
+#define DISP_TILE 4096              // queue entries a block orders at a time (whole bins: up to the fullest bin more, DISP_TILE_MAX in all)
+#define DISP_TILE_MAX (DISP_TILE + 1024)
+#define DISP_TILE_MIN 1024
+#define DISP_BIN_MAX (DISP_TILE_MAX - DISP_TILE_MIN)      // fuller bins send the queue to the radix sort
 #define DISP_FINE 4096              // bins of a tile
 #define DISP_TILES_CHAIN 1024       // tiles whose totals the chain adds up itself; beyond them they are added to the running totals
 #define SORT_SMEM (DISP_TILE_MAX * 22 + (DISP_FINE + 4) * 4 + (DISP_BINS + 4) * 4 + DISP_SPLITS * 16)
@@ -246,14 +247,16 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 // nothing: the queue, its running totals and the tiles may be unwritten).
 //   0  plan of every instance and its place in the maturity order, a warp per instance; the sample in order, a warp
 //      per sampled item counting the smaller ones
-//   1  every item's bin, and its place in it from a global counter.  Every eighth sample of a (stage, priority) starts an
-//      interval, an interval is divided evenly into sixteen bins by slack and tie (so equal slacks spread by tie; fewer bins, and their counters queue up)
-//   2  items to their bins; a bin of more than DISP_BIN_MAX items (slacks crowded closer than the sample sees) sends the
-//      whole queue to a radix sort instead
+//   1  every item's bin, and its place in it from a global counter.  Every fourth sample of a (stage, priority) starts an
+//      interval, an interval is divided evenly into eight bins by slack and tie (so equal slacks spread by tie).  1 M rows over 1024 instances, 60,013
+//      rows: every eighth and sixteen 206, 69 us, every fourth and eight 203, 67, every second and eight 213, 72 (each block adds up all bins)
+//   2  items to their bins; a fuller bin makes the tiles lower, one of more than DISP_BIN_MAX items (slacks crowded closer than the sample
+//      sees) sends the whole queue to a radix sort instead, 22 us a pass at 500 K entries.  (With the line at 1024 items the gaps between the classes of one
+//      priority did that: 500,001 rows with weights 324 us, 126 now)
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting; rows out in order, running totals
 // An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 67 us by the GPU's clock:
-// sample and plans 12, splitters 5, bins 14, their starts 7, moving 4, tiles 12, running totals 9, barriers 1.5 each; one of 42 K in 30 blocks 36.
+// sample and plans 12, splitters 5, bins 14, their starts 7, moving 4, tiles 11, running totals 8, barriers 1.5 each; one of 42 K in 30 blocks 36.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
@@ -497,7 +500,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 
   // ---- 2: items to their bins ------------------------------------------------------------------------------------
   const uint32_t n1 = (uint32_t)__ldcg(w.ctl + CTL_N1), n0 = n_all - n1;
-  bool binned;
+  uint32_t fullest;
   {
     constexpr int PER = DISP_BINS / SORT_THREADS;
     static_assert(DISP_BINS % SORT_THREADS == 0, "every thread sums the same number of bins");
@@ -508,8 +511,13 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 #pragma unroll
     for (int e = 0; e < PER; e++) { s_start[tid * PER + e] = run; run += c[e]; }
     if (tid == 0) s_start[DISP_BINS] = all;
-    binned = !__syncthreads_or(big > DISP_BIN_MAX);
+    big = __reduce_max_sync(0xffffffffu, big);
+    if (lane == 0) s_part[warp] = big;
+    __syncthreads();
+    fullest = __reduce_max_sync(0xffffffffu, s_part[lane]);
+    __syncthreads();
   }
+  const bool binned = fullest <= DISP_BIN_MAX;
   if (binned) {
     for (uint32_t q0 = lo + tid; q0 < hi; q0 += ITEMS_AT_ONCE * SORT_THREADS) {
       uint4 x[ITEMS_AT_ONCE];
@@ -568,7 +576,11 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   }
 
   // ---- 3: rows in order, running totals inside every tile -----------------------------------------------------------
-  const uint32_t tile_rows = per < DISP_TILE ? (per > 1024u ? per : 1024u) : DISP_TILE;
+  // tiles: no higher than leaves room for the fullest bin, and the same number of them for every block (819 K entries in 200 tiles of
+  // 4096 were two rounds of 148 blocks: 38 us for ordering them, 27 in 296 tiles)
+  const uint32_t room = binned && fullest > DISP_TILE_MAX - DISP_TILE ? DISP_TILE_MAX - fullest : DISP_TILE;
+  const uint32_t per_block = (per + room - 1) / room, share = (per + per_block - 1) / (per_block ? per_block : 1u);
+  const uint32_t tile_rows = share > DISP_TILE_MIN ? share : DISP_TILE_MIN;
   const uint32_t tiles = (n_all + tile_rows - 1) / tile_rows;
   const int64_t bmax0 = (int64_t)__ldcg(w.ctl + CTL_BMAX0), bmax1 = (int64_t)__ldcg(w.ctl + CTL_BMAX1);
   const uint4 *ordered = w.item[binned ? 0 : 1];      // (ten passes end where they began)
@@ -1030,7 +1042,7 @@ static int disp_workspace(hfx_sched *s, hfx_dispatch_ws **out) {
   DispWork &w = d->w;
   const size_t rows = (size_t)s->max_rows, R = (size_t)s->p.n_replicas;
   w.R = s->p.n_replicas;
-  w.tiles_max = (int)(rows / DISP_TILE) + s->n_sm + 1;
+  w.tiles_max = (int)(rows / DISP_TILE_MIN) + 2;
   size_t used = 0;
   auto part = [&](size_t bytes) { const size_t at = used; used += (bytes + 255) & ~(size_t)255; return at; };
   // what has to be zero between calls, first

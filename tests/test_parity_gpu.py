@@ -1262,6 +1262,51 @@ def test_simulator_budget_over_the_model_range(model, first_fit):
     assert_sim_parity(wl)
 
 
+@pytest.mark.parametrize("shape", ["even", "rare giants", "blocked", "zeros", "d stage", "capped"])
+@pytest.mark.parametrize("R,n", [(95, 3000), (96, 3000), (97, 40_001), (129, 9000), (1024, 70_000), (1061, 30_011), (2200, 90_000)])
+def test_dispatch_walk_of_many_instances(R, n, shape):
+    # Walks over many instances: even runs; losses of hundreds of entries an instance; a queue front that fits no budget; prompts and
+    # budgets of zero tokens; the D stage's costs in time; batch caps; queues that end in mid-walk.
+    rng = np.random.default_rng(R + n)
+    d_stage = shape == "d stage"
+    wl = gen.random_table(R + n, n, R, modes=(gen.PREFILL, gen.DECODE) if d_stage else (gen.COLOCATED,), n_classes=3, token_cap=4096, done=0.0, future=0.05,
+                          batch_cap=3 if shape == "capped" else 0, inflight=0.6 if d_stage else 0.02, budget_mode=gen.BUDGET_SAFE if d_stage else gen.BUDGET_CAP_ONLY)
+    now = int(wl.now.max())
+    wl.maturity[:] = now - rng.integers(0, 50, R)
+    p = wl.table["prompt_len"]
+    if shape == "even":
+        p[:] = rng.integers(1, 8 * 4096 * R // n + 2, n)
+    elif shape == "rare giants":
+        p[:] = 1
+        p[rng.integers(0, n, R)] = 3900
+    elif shape == "blocked":
+        p[:] = rng.integers(1, 4 * 4096 * R // n + 2, n)
+        p[: n // 3] = 5000
+    elif shape == "zeros":
+        p[:] = np.where(rng.random(n) < 0.7, 0, 700)
+        wl.maturity[::5] = now + 1
+    assert_dispatch_parity(wl, now, calls=2)
+
+
+@pytest.mark.parametrize("clump", [1000, 1030, 2500, 4090, 4200, 9000])
+def test_dispatch_bins_of_every_fullness(clump):
+    # Rows whose slacks lie closer together than a bin of the order is wide, beside others far off: fuller bins make lower tiles, and beyond
+    # what a tile holds the queue is ordered by radix passes.  (ids permuted: ties too)
+    n = 40_000
+    rng = np.random.default_rng(clump)
+    wl = gen.random_table(clump, n, 7, modes=(gen.COLOCATED,), n_classes=3, token_cap=16384, inflight=0.02, done=0.0, future=0.0)
+    now = int(wl.now.max())
+    t = wl.table
+    t["prompt_len"][:] = 16
+    t["class_id"][:] = 0
+    t["arrival_ns"][:] = now - rng.integers(0, 40 * SEC, n)
+    c = rng.permutation(n)[:clump]
+    t["arrival_ns"][c] = now - 41 * SEC - rng.integers(0, 2, clump)
+    late = rng.permutation(n)[:30]
+    t["arrival_ns"][late] = now - 500 * SEC - rng.integers(0, SEC, 30)
+    assert_dispatch_parity(wl, now)
+
+
 @pytest.mark.parametrize("n_classes", [1, 4, 5, 8, 9, 64])
 def test_attainment_class_counts_and_ragged_rows(n_classes):
     # totals in registers (up to 4, up to 8 classes) and per warp (more); a row is left over when n is odd

@@ -17,6 +17,7 @@
 #include "hfx_internal.cuh"
 
 #define SCAN_THREADS 1024
+#define SCAN_THREADS_FEW 256
 #define SCAN_SMEM_REPLICAS 512      // up to here a block adds up the running batches in shared memory first: with few instances the
                                     // global counters queue up (R x blocks counters are flushed, so not for large fleets)
 #define SCAN_SMEM_ROWS 32768        // rows per block up to which its 32-bit sums cannot overflow
@@ -27,9 +28,10 @@
 #define DISP_SPLITS (DISP_SAMPLES / DISP_STEP + 3 * DISP_CLASSES)
 #define DISP_SUB 8                  // bins an interval is divided into evenly
 #define DISP_BINS (DISP_SPLITS * DISP_SUB)
+#define DISP_SMALL 4096             // a queue of so many entries is ordered by comparing all with all
 #define DISP_TILE 4096              // queue entries a block orders at a time (whole bins: up to the fullest bin more, DISP_TILE_MAX in all)
 #define DISP_TILE_MAX (DISP_TILE + 1024)
-#define DISP_TILE_MIN 1024
+#define DISP_TILE_MIN 512
 #define DISP_BIN_MAX (DISP_TILE_MAX - DISP_TILE_MIN)      // fuller bins send the queue to the radix sort
 #define DISP_FINE 4096              // bins of a tile
 #define DISP_TILES_CHAIN 1024       // tiles whose totals the chain adds up itself; beyond them they are added to the running totals
@@ -93,7 +95,8 @@ __device__ __forceinline__ int64_t disp_cost(const HfxParams &p, const DispArgs 
 // thread with 16-byte loads; a block reserves room for the items of its 4096 rows with one global atomic (their order
 // does not matter: the tie word settles it).
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p, const DispArgs a, const DispWork w) {
+template <int threads>
+__global__ void __launch_bounds__(threads, 1) k_disp_scan(const HfxParams p, const DispArgs a, const DispWork w) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t *s_run = reinterpret_cast<uint32_t *>(smem_raw);      // [4 R] requests in flight, context low / high part; (if R is small)
   unsigned long long *s_mask = reinterpret_cast<unsigned long long *>(s_run + 4 * (size_t)p.n_replicas);      // [R]
@@ -103,13 +106,14 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
   __shared__ uint32_t s_count, s_base, s_idmax, s_idmin_inv;
   __shared__ unsigned long long s_qmask, s_dmask;
   const int tid = threadIdx.x, lane = tid & 31, R = p.n_replicas;
-  const bool own = R <= SCAN_SMEM_REPLICAS && (int64_t)a.rounds * SCAN_THREADS * 4 <= SCAN_SMEM_ROWS;
-  for (int c = tid; c < HFX_MAX_CLASSES; c += SCAN_THREADS) {
+  const bool own = R <= SCAN_SMEM_REPLICAS && (int64_t)a.rounds * threads * 4 <= SCAN_SMEM_ROWS;
+  for (int c = tid; c < HFX_MAX_CLASSES; c += threads) {
     s_ttft[c] = c < p.n_classes ? p.ttft[c] : 0;
     s_tpot[c] = c < p.n_classes ? p.tpot[c] : 0;
     s_prio[c] = c < p.n_classes ? p.prio[c] : 63;
   }
-  if (own) for (int i = tid; i < R; i += SCAN_THREADS) { s_run[4 * i] = 0; s_run[4 * i + 1] = 0; s_run[4 * i + 2] = 0; s_mask[i] = 0; }
+  if (own) for (int i = tid; i < R; i += threads) { s_run[4 * i] = 0; s_run[4 * i + 1] = 0; s_run[4 * i + 2] = 0; s_mask[i] = 0; }
+  static_assert(threads >= 2 * DISP_CLASSES, "a thread for every bound");
   if (tid < 2 * DISP_CLASSES) s_up[tid] = 0;
   if (tid == 0) { s_count = 0; s_idmax = 0; s_idmin_inv = 0; s_qmask = 0; s_dmask = 0; }
   __syncthreads();
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
   };
 
   const int64_t n4 = a.n >> 2;
-  for (int64_t v0 = (int64_t)blockIdx.x * SCAN_THREADS; v0 < n4; v0 += (int64_t)gridDim.x * SCAN_THREADS) {
+  for (int64_t v0 = (int64_t)blockIdx.x * threads; v0 < n4; v0 += (int64_t)gridDim.x * threads) {
     const int64_t v = v0 + tid;
     uint64_t key[4] = {0, 0, 0, 0};
     int4 id = make_int4(0, 0, 0, 0);
@@ -233,7 +237,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
   }
   if (tid < 2 * DISP_CLASSES && s_up[tid]) atomicMax(reinterpret_cast<uint32_t *>(w.ctl + CTL_CLASSES) + tid, s_up[tid]);
   if (own)
-    for (int r = tid; r < R; r += SCAN_THREADS)
+    for (int r = tid; r < R; r += threads)
       if (s_run[4 * r]) {
         atomicAdd(&w.n_run[r], s_run[4 * r]);
         atomicAdd(&w.sum_kv[r], (unsigned long long)s_run[4 * r + 1] + ((unsigned long long)s_run[4 * r + 2] << 16));
@@ -246,7 +250,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) k_disp_scan(const HfxParams p
 // is not reached in time makes every block return with HFX_ST_TIMEOUT and CTL_ABORT raised; the kernels behind it then hand out
 // nothing: the queue, its running totals and the tiles may be unwritten).
 //   0  plan of every instance and its place in the maturity order, a warp per instance; the sample in order, a warp
-//      per sampled item counting the smaller ones
+//      per sampled item counting the smaller ones.  Of a queue of up to DISP_SMALL entries all are sampled, and phases 1 and 2 fall away
+//      (300 rows 52 us without, 34 now, 2000 rows 56 and 37, 6000 rows 60 and 56 before the tiles got smaller)
 //   1  every item's bin, and its place in it from a global counter.  Every fourth sample of a (stage, priority) starts an
 //      interval, an interval is divided evenly into eight bins by slack and tie (so equal slacks spread by tie).  1 M rows over 1024 instances, 60,013
 //      rows: every eighth and sixteen 206, 69 us, every fourth and eight 203, 67, every second and eight 213, 72 (each block adds up all bins)
@@ -314,8 +319,9 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   uint32_t *s_start = s_fine + DISP_FINE + 4;                                     // [DISP_BINS + 4] where each bin starts
   uint64_t *s_split = reinterpret_cast<uint64_t *>(s_start + DISP_BINS + 4);        // [DISP_SPLITS] where each interval starts
   uint64_t *s_scale = s_split + DISP_SPLITS;                                      // [DISP_SPLITS] bins per unit<45>, in units of 2^shift, shift<6>
-  uint64_t *s_sample = reinterpret_cast<uint64_t *>(smem_raw);                          // [DISP_SAMPLES] (before the items are there)
-  int64_t *s_mat = reinterpret_cast<int64_t *>(s_sample + DISP_SAMPLES);                // [R] maturity of every instance, HFX_INF if it has not come
+  uint64_t *s_sample = reinterpret_cast<uint64_t *>(smem_raw);                          // [DISP_SMALL] the sample, or the whole of a small queue (before the items are there)
+  static_assert(DISP_SMALL >= DISP_SAMPLES && DISP_SMALL <= DISP_TILE && DISP_SMALL * 8 + 4096 * 8 <= SORT_SMEM, "and the instances' maturities behind it");
+  int64_t *s_mat = reinterpret_cast<int64_t *>(s_sample + DISP_SMALL);                // [R] maturity of every instance, HFX_INF if it has not come
   uint32_t *s_wc = reinterpret_cast<uint32_t *>(smem_raw);                              // [32][256] (radix passes)
   __shared__ ClassTab s_tab;
   __shared__ uint32_t s_class[DISP_CLASSES], s_r0[DISP_CLASSES + 1];      // first interval | intervals << 16; first sample
@@ -330,7 +336,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   const uint32_t n_all = (uint32_t)w.ctl[CTL_ITEMS];
   // the sample: every (n_all / n_samples)-th item (they lie in runs of consecutive rows, so the table is sampled evenly)
   const uint32_t n_want = n_all / 64 > 256 ? (n_all / 64 < DISP_SAMPLES ? n_all / 64 : DISP_SAMPLES) : 256;
-  const int n_samples = (int)(n_want < n_all ? n_want : n_all);
+  const bool small = n_all <= DISP_SMALL;
+  const int n_samples = (int)(small ? n_all : n_want);
   const bool by_id = w.ctl[CTL_FALLS] != 0;
   // an item's tie word (request id, or the row where ids rise with the rows), and its 16 leading bits
   const uint32_t id_lo = ~(uint32_t)w.ctl[CTL_IDMIN_INV], tie_span = by_id ? (uint32_t)w.ctl[CTL_IDMAX] - id_lo : (uint32_t)(a.n - 1);
@@ -353,8 +360,17 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     uint32_t r = 0;
 #pragma unroll 4
     for (int i = lane; i < n_samples; i += 32) r += s_sample[i] < x || (s_sample[i] == x && i < k) ? 1u : 0u;
+    if (small && tie_shift > 0)      // places equal in the leading bits of the tie
+      for (int i = lane; i < n_samples; i += 32)
+        if (s_sample[i] == x && i != k) {
+          const bool ahead = tie_of(w.item[1][i]) < tie_of(w.item[1][k]);
+          if (ahead != (i < k)) r += ahead ? 1u : ~0u;
+        }
     r = __reduce_add_sync(0xffffffffu, r);
-    if (lane == 0) w.sorted[r] = x;
+    if (lane == 0) {
+      if (!small) w.sorted[r] = x;
+      else { w.rank[r] = w.item[1][k].w; if (x >> 62) atomicAdd(&s_n1, 1u); }      // the row in its place; (bit 46 of the key: the D stage)
+    }
   }
   for (int r = blockIdx.x * (SORT_THREADS / 32) + warp; r < R; r += gridDim.x * (SORT_THREADS / 32)) {
     const hfx_replica_cfg cfg = a.cfg[r];
@@ -401,6 +417,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     if (s_nm[tid]) atomicAdd(&w.ctl[CTL_NM0 + tid], (unsigned long long)s_nm[tid]);
     if (s_bmax[tid]) atomicMax(&w.ctl[CTL_BMAX0 + tid], s_bmax[tid]);
   }
+  if (small && tid == 0 && s_n1) atomicAdd(&w.ctl[CTL_N1], (unsigned long long)s_n1);
   if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
 
   // ---- 1: bins -------------------------------------------------------------------------------------------------
@@ -409,6 +426,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     for (int k = nm0 + nm1 + tid; k < R; k += SORT_THREADS) a.inst_order[k] = -1;
     if (tid == 0) { a.n_mature[0] = nm0; a.n_mature[1] = nm1; }
   }
+  if (!small) {
   for (int k = tid; k < n_samples; k += SORT_THREADS) s_sample[k] = __ldcg(w.sorted + k);
   __syncthreads();
   if (tid <= DISP_CLASSES) {      // the first sample of every class
@@ -436,6 +454,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     }
   }
   __syncthreads();
+  }
   auto scale_of = [&](uint64_t span) -> uint64_t {
     const int bits = 64 - __clzll((long long)span), sh = bits > 32 ? bits - 32 : 0;
     return (((uint64_t)DISP_SUB << 32) / ((span >> sh) + 1)) | ((uint64_t)sh << 56);
@@ -443,6 +462,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   const uint32_t *bounds = reinterpret_cast<const uint32_t *>(w.ctl + CTL_CLASSES);
   auto lowest = [&](uint32_t cl) { return (uint64_t)(~bounds[DISP_CLASSES + cl]) << 24; };
   auto highest = [&](uint32_t cl) { return ((uint64_t)bounds[cl] << 24) | 0xffffffull; };
+  if (!small) {
   if (tid < DISP_CLASSES && s_r0[tid + 1] == s_r0[tid]) {      // a class the sample missed
     s_split[s_class[tid] & 0xffffu] = lowest(tid); s_scale[s_class[tid] & 0xffffu] = scale_of(highest(tid) > lowest(tid) ? highest(tid) - lowest(tid) : 0);
   }
@@ -460,6 +480,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     }
   }
   __syncthreads();
+  }
   // the bin of an item, and how far into it the item lies (in units of 2^-32)
   auto bin_of = [&](const uint4 &x, uint32_t &frac) -> uint32_t {
     const uint64_t pl = place_of(x), v = pl & ((1ull << 56) - 1);
@@ -479,7 +500,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   };
   const uint32_t per = (n_all + gridDim.x - 1) / gridDim.x;
   const uint32_t lo = blockIdx.x * per < n_all ? blockIdx.x * per : n_all, hi = lo + per < n_all ? lo + per : n_all;      // this block's items
-  {
+  if (!small) {
+    {
     uint32_t n1 = 0;
     for (uint32_t q0 = lo + tid; q0 < hi; q0 += ITEMS_AT_ONCE * SORT_THREADS) {
       uint4 x[ITEMS_AT_ONCE];
@@ -493,15 +515,16 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     }
     n1 = __reduce_add_sync(0xffffffffu, n1);
     if (lane == 0 && n1) atomicAdd(&s_n1, n1);
+    }
+    __syncthreads();
+    if (tid == 0 && s_n1) atomicAdd(&w.ctl[CTL_N1], (unsigned long long)s_n1);
+    if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
   }
-  __syncthreads();
-  if (tid == 0 && s_n1) atomicAdd(&w.ctl[CTL_N1], (unsigned long long)s_n1);
-  if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
 
   // ---- 2: items to their bins ------------------------------------------------------------------------------------
   const uint32_t n1 = (uint32_t)__ldcg(w.ctl + CTL_N1), n0 = n_all - n1;
-  uint32_t fullest;
-  {
+  uint32_t fullest = 0;
+  if (!small) {
     constexpr int PER = DISP_BINS / SORT_THREADS;
     static_assert(DISP_BINS % SORT_THREADS == 0, "every thread sums the same number of bins");
     uint32_t c[PER], sum = 0, big = 0;
@@ -517,7 +540,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     fullest = __reduce_max_sync(0xffffffffu, s_part[lane]);
     __syncthreads();
   }
-  const bool binned = fullest <= DISP_BIN_MAX;
+  const bool binned = !small && fullest <= DISP_BIN_MAX;
   if (binned) {
     for (uint32_t q0 = lo + tid; q0 < hi; q0 += ITEMS_AT_ONCE * SORT_THREADS) {
       uint4 x[ITEMS_AT_ONCE];
@@ -528,7 +551,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       for (int e = 0; e < ITEMS_AT_ONCE; e++) { const uint32_t q = q0 + e * SORT_THREADS; if (q < hi) { const uint32_t bn = rk[e] >> 16; w.item[0][s_start[bn] + (rk[e] & 0xffffu)] = x[e]; } }
     }
     if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
-  } else {
+  } else if (!small) {
     // radix sort, 8 bits a pass: the tie word, then the key (47 bits).  A block counts the digits of its share, adds up the
     // counts of the blocks before it, and places its items 1024 at a time in order.
     for (int pass = 0; pass < 10; pass++) {
@@ -580,7 +603,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   // 4096 were two rounds of 148 blocks: 38 us for ordering them, 27 in 296 tiles)
   const uint32_t room = binned && fullest > DISP_TILE_MAX - DISP_TILE ? DISP_TILE_MAX - fullest : DISP_TILE;
   const uint32_t per_block = (per + room - 1) / room, share = (per + per_block - 1) / (per_block ? per_block : 1u);
-  const uint32_t tile_rows = share > DISP_TILE_MIN ? share : DISP_TILE_MIN;
+  const uint32_t tile_rows = share > DISP_TILE_MIN && !small ? share : DISP_TILE_MIN;
   const uint32_t tiles = (n_all + tile_rows - 1) / tile_rows;
   const int64_t bmax0 = (int64_t)__ldcg(w.ctl + CTL_BMAX0), bmax1 = (int64_t)__ldcg(w.ctl + CTL_BMAX1);
   const uint4 *ordered = w.item[binned ? 0 : 1];      // (ten passes end where they began)
@@ -656,7 +679,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
         }
       }
     } else
-      for (uint32_t i = tid; i < n; i += SORT_THREADS) s_row[i] = __ldcg(ordered + e0 + i).w;
+      for (uint32_t i = tid; i < n; i += SORT_THREADS) s_row[i] = small ? __ldcg(w.rank + e0 + i) : __ldcg(ordered + e0 + i).w;
     __syncthreads();
     // costs of my consecutive places; entries that no instance's budget reaches count nothing
     const uint32_t ipt = (n + SORT_THREADS - 1) / SORT_THREADS, i0 = tid * ipt < n ? tid * ipt : n, mine = i0 + ipt < n ? ipt : n - i0;
@@ -1013,9 +1036,11 @@ struct hfx_dispatch_ws { DispWork w; unsigned char *mem; size_t zero; unsigned l
 
 static size_t chain_smem(int R) { return (size_t)(CHAIN_CHUNK + CHAIN_WIN + 8) * 16 + (size_t)DISP_TILES_CHAIN * 16 + 16 + ((size_t)R + CHAIN_BATCH + 1) * 16; }
 static size_t scan_smem(int R) { return R <= SCAN_SMEM_REPLICAS ? (size_t)R * 24 : 0; }
-// blocks of the scan of n rows
+// threads of a block of the scan of n rows, and blocks: small blocks while an SM has one at most (60,013 rows 68.9 us in 15 blocks of 1024 threads,
+// whose rows in flight meet in a few instances' counters, 66.7 in 59 of 256)
+static int scan_threads(const hfx_sched *s, int64_t n) { return n <= (int64_t)s->n_sm * 4 * SCAN_THREADS_FEW ? SCAN_THREADS_FEW : SCAN_THREADS; }
 static int scan_blocks(const hfx_sched *s, int64_t n) {
-  const int64_t want = (n / 4 + SCAN_THREADS - 1) / SCAN_THREADS;
+  const int64_t want = (n / 4 + scan_threads(s, n) - 1) / scan_threads(s, n);
   return (int)(want < 1 ? 1 : (want < s->n_sm ? want : s->n_sm));
 }
 int hfx_dispatch_configure() {
@@ -1094,9 +1119,11 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   a.sum_kv = o->sum_kv; a.adm_cost = o->adm_cost; a.adm_count = o->adm_count; a.maturity_next = o->maturity_next;
   a.status = s->d_status;
   const int blocks = scan_blocks(s, n);
-  a.rounds = (int32_t)((n / 4 + (int64_t)SCAN_THREADS * blocks - 1) / ((int64_t)SCAN_THREADS * blocks));
-  // blocks of the cooperative kernel: no more than its phases can use, so that small calls meet at short barriers
-  int64_t want = (n + 2047) / 2048, want_r = (R + 31) / 32;
+  const int threads = scan_threads(s, n);
+  a.rounds = (int32_t)((n / 4 + (int64_t)threads * blocks - 1) / ((int64_t)threads * blocks));
+  // blocks of the cooperative kernel: tiles of 512 entries, or a warp per entry of a small queue (60,013 rows: 30 blocks and tiles of 1024 entries 66.7 us,
+  // 59 63.6, 118 and tiles of 512 61.6; a barrier takes 1.5 us with 30 and with 148 blocks)
+  int64_t want = n <= 2 * DISP_SMALL ? (n + 31) / 32 : (n + 511) / 512, want_r = (R + 31) / 32;
   if (want < want_r) want = want_r;
   const int grid = (int)(want < 1 ? 1 : (want < s->n_sm ? want : s->n_sm));
   cudaLaunchAttribute attr[1];
@@ -1105,8 +1132,9 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   cfg.stream = st;
   {
     KernelScope ks(s, KSLOT_DISPATCH);
-    cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(SCAN_THREADS); cfg.dynamicSmemBytes = scan_smem(R);
-    if (cudaLaunchKernelEx(&cfg, k_disp_scan, s->p, a, w) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
+    cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = scan_smem(R);
+    const cudaError_t e = threads == SCAN_THREADS ? cudaLaunchKernelEx(&cfg, k_disp_scan<SCAN_THREADS>, s->p, a, w) : cudaLaunchKernelEx(&cfg, k_disp_scan<SCAN_THREADS_FEW>, s->p, a, w);
+    if (e != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
   }
   cfg.attrs = attr; cfg.numAttrs = 1;
   {

@@ -1307,6 +1307,36 @@ def test_dispatch_bins_of_every_fullness(clump):
     assert_dispatch_parity(wl, now)
 
 
+@pytest.mark.parametrize("equal", [False, True])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 1023, 1025, 4095, 4096, 4097, 4607, 8200])
+def test_dispatch_small_queues(n, equal):
+    # a queue of up to 4096 entries is ordered by comparing all with all (two tiles of 512 and more of them), a larger one by bins; ids spread over
+    # 31 bits, of which the order's places hold the leading 16, and all slacks equal: then the ids alone decide
+    rng = np.random.default_rng(n)
+    wl = gen.random_table(n, n, 6, modes=(gen.COLOCATED, gen.PREFILL, gen.DECODE), n_classes=3, token_cap=16384, inflight=0.0, done=0.0, future=0.0, weight_max=0)
+    wl.replicas[:, 0] = [gen.COLOCATED, gen.PREFILL, gen.DECODE] * 2
+    now = int(wl.now.max())
+    t = wl.table
+    t["state"][:] = gen.QUEUED
+    r = np.nonzero(rng.random(n) < 0.2)[0] if n > 40 else []
+    t["state"][r] = gen.RUNNING
+    t["first_token_ns"][:] = now - rng.integers(1, SEC, n)
+    t["arrival_ns"][:] = now - SEC - rng.integers(0, 3, n)
+    t["prompt_len"][:] = rng.integers(16, 18, n)
+    t["req_id"][:] = rng.permutation(n).astype(np.int64) * (2**31 // n) - 2**30
+    if equal:
+        wl.classes = [(0, 0, 1)] * 3
+    assert_dispatch_parity(wl, now, calls=2)
+
+
+@pytest.mark.parametrize("n", [151_548, 151_552, 151_553, 151_557])
+def test_dispatch_scan_in_small_and_in_large_blocks(n):
+    # up to 1024 rows an SM (148 of them) the scan takes blocks of 256 threads
+    wl = gen.random_table(n, n, 20, modes=(gen.COLOCATED, gen.PREFILL, gen.DECODE), inflight=0.4)
+    wl.replicas[:3, 0] = [gen.COLOCATED, gen.PREFILL, gen.DECODE]
+    assert_dispatch_parity(wl, int(wl.now.max()))
+
+
 @pytest.mark.parametrize("n_classes", [1, 4, 5, 8, 9, 64])
 def test_attainment_class_counts_and_ragged_rows(n_classes):
     # totals in registers (up to 4, up to 8 classes) and per warp (more); a row is left over when n is odd

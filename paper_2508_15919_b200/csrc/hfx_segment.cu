@@ -51,8 +51,8 @@ struct SegCtx {
   const uint32_t *ordered; const uint8_t *rowflag;
   uint64_t *big_hi; uint32_t *big_lo; uint32_t *big_idx;
   int64_t pad;            // The sizes of this struct and of BlockShared move the compiler's allocation of the 64 registers: with 8 bytes more in both
-                          // k_replicas reloads 612 bytes a thread instead of 652 (ten steps over 1024 replicas 644 us instead of 652, one
-                          // step over one replica 22.2 instead of 23.1; with 8 bytes more in one of them, or 16, in between).
+                          // k_replicas reloads 508 bytes a thread instead of 632 (ten steps over 1024 replicas 649 us instead of 654, one step over 64
+                          // replicas of 4096 rows 45.5 instead of 46.7).
 };
 
 // A set of threads of the block that synchronise on a hardware barrier of their own (0 = the whole block).
@@ -408,13 +408,14 @@ __device__ __forceinline__ void gather_replica(const SegCtx &c, int R1, int r, c
         for (int e = 0; e < 4; e++) { const uint32_t q = q0 + e * G.n; if (q < ta) dst.row[base_a + q] = row[e]; }
       }
     } else if (take_act) {
+      // (two rows of a thread in flight: with three, four and six the kernel reloads more and 128 + 128 replicas of 16,384 rows take 254, 261, 260, 261 us)
       int lt_c = 0;            // the chunk of my previous row and where it ends: my rows rise, so large chunks are searched once
       uint32_t lim_c = 0;
-      for (uint32_t q0 = G.tid; q0 < ta; q0 += 3 * G.n) {
-        uint4 rec[3];
-        int32_t row[3];
+      for (uint32_t q0 = G.tid; q0 < ta; q0 += 2 * G.n) {
+        uint4 rec[2];
+        int32_t row[2];
 #pragma unroll
-        for (int e = 0; e < 3; e++) {
+        for (int e = 0; e < 2; e++) {
           const uint32_t q = q0 + e * G.n;
           if (q < ta) {
             if (!OWNER && q >= lim_c) { lt_c = chunk_of(gt.pa, q); lim_c = gt.pa[lt_c] + gt.ca[lt_c]; }
@@ -426,7 +427,7 @@ __device__ __forceinline__ void gather_replica(const SegCtx &c, int R1, int r, c
           }
         }
 #pragma unroll
-        for (int e = 0; e < 3; e++) { const uint32_t q = q0 + e * G.n; if (q < ta) emit_act(base_a + q, rec[e], row[e]); }
+        for (int e = 0; e < 2; e++) { const uint32_t q = q0 + e * G.n; if (q < ta) emit_act(base_a + q, rec[e], row[e]); }
       }
     }
     if (list_in)
@@ -1200,24 +1201,34 @@ __device__ void medium_replica(const HfxParams &p, const SegArgs &a, const SegCt
 // Ids that do not rise along the table (front ends that number their requests on their own): both lists are put in id
 // order first, by the same sort over ids, and the gather then places every row by its id; from there on the step is
 // an ordered one.  (96-bit items in a sorting network took 128 us for 96 replicas of 3125 rows.)
-// The replica's scratch range of c.rec (32 bytes per row, of which 20 per active row are used) holds three
-// arrays by position q in row order: slack base, then sort item (8 bytes); record words z, w (8); row (4).
-// Every pass reads them front to back; shared memory holds the binned items (afterwards the record words), the
-// order as 16-bit positions and the bin counters.
+// What bounds it: a chain of passes, each over all rows, by one block.  The gather takes the slack bases to shared memory (where the sort's
+// items go later) and adds up the aggregates as the rows pass; record words and rows go to three arrays by position q in row order in the replica's
+// scratch range of c.rec (32 bytes per row, of which 20 per active row are used: sort item, record words, row).  After the sort what the admission looks at, four bytes a
+// row, lies in shared memory over the items, and the rows beside it, so that the order is written without a gather from memory.
+// Per replica of 16,384 rows (clock, thread 0): gather 44 K cycles, plan 5, items 25, sort 54, order 9, admission 14, rest 3 (with bases in
+// the scratch, the aggregates read back and the order gathered from memory 50, 11, 29, 55, 26, 18, 3: 193 K in all).  128 + 128 replicas of 16,384
+// rows 303 -> 254 us, 64 of 4096 50.9 -> 45.5, 96 of 3125 permuted 72.8 -> 65.4.  Tried: items and their bins kept in registers from counting
+// the bins to ranking (reloads, and neighbouring threads rank items of far bins: scatter 10 -> 24 K, ranks 30 -> 59 K).
 // ------------------------------------------------------------------------------------------------
 #define MED_BINS 8192     // bins of the block's distribution sort (16-bit counters, two to a word)
 #define MED_BIN_MAX 160   // fuller bins send the replica to the sorting network
-static_assert((size_t)SEG_MED * 10 + MED_BINS * 4 <= SMEM_MED, "items, order and bins of a medium replica fit the block's shared memory");
+#define VAL_LEN_MASK 0x3ffffffu
+#define VAL_RUNNING 0x4000000u
+#define VAL_TAKEN 0x40000000u
+#define VAL_ADMITTED 0x80000000u
+static_assert((size_t)SEG_MED * 10 + MED_BINS * 4 <= SMEM_MED && (size_t)SEG_MED * 10 + gather_tiles_bytes(REP_THREADS, REP_THREADS) <= SMEM_MED, "items, order and bins of a medium replica fit the block's shared memory, and so do the tiles of its gather");
 static_assert(MED_BINS / 8 == REP_THREADS, "every thread scans eight bins");
 
 template <bool FF>
 __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx &c, int r, uint32_t b, int n, int n_act,
                              bool ordered, bool list_in, unsigned char *smem, BlockShared &sh, uint64_t *s_cinfo, const ClassTab &tab) {
-  uint64_t *s_item = reinterpret_cast<uint64_t *>(smem);                          // [SEG_MED] items by bin
-  uint2 *s_zw = reinterpret_cast<uint2 *>(smem);                                  // [SEG_MED] afterwards: record words by position; bit 31 of x: taken by first fit, of y: admitted
+  uint64_t *s_item = reinterpret_cast<uint64_t *>(smem);                          // [SEG_MED] slack bases by position, then items by bin
+  uint32_t *s_val = reinterpret_cast<uint32_t *>(smem);                           // [SEG_MED] afterwards, by position: prompt (context on a decode replica) and VAL_ marks
+  int32_t *s_row = reinterpret_cast<int32_t *>(s_val + SEG_MED);                  // [SEG_MED] and row
   uint16_t *s_ord = reinterpret_cast<uint16_t *>(smem + (size_t)SEG_MED * 8);     // [SEG_MED] position of the i-th row of the order
   uint32_t *s_bin = reinterpret_cast<uint32_t *>(smem + (size_t)SEG_MED * 10);    // [MED_BINS / 2] bin counts, then bin starts
   uint32_t *s_cur = s_bin + MED_BINS / 2;                                         // [MED_BINS / 2] fill cursors, then bin ends
+  unsigned char *s_tiles = reinterpret_cast<unsigned char *>(s_bin);              // (while a gather runs: the round's tile descriptors)
   uint32_t *s_lo = reinterpret_cast<uint32_t *>(s_ord);                           // (sorting network only: 32-bit positions over order and bins)
   // until the bins are laid out: per class the smallest and largest of the slack's upper 32 bits and of its low 8 bits, the items
   uint32_t *s_cmin = reinterpret_cast<uint32_t *>(s_ord), *s_cmax = s_cmin + TINY_CLASSES, *s_lmin = s_cmax + TINY_CLASSES,
@@ -1237,17 +1248,22 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
   // three sorts, the first two of steps that are not ordered: the inactive rows by id, the active ones by id, the active ones by key
   for (int stage = ordered ? 2 : 0; stage < 3; stage++) {
   const int m = stage == 0 ? n_in : n_act;
-  // ---- gather: into the scratch arrays, the inactive rows straight to their places; or the rows of both lists ------
+  uint32_t n_run = 0;
+  uint64_t sum_kv = 0, m_run = 0, m_q = 0;
+  // ---- gather: bases into shared memory, the rest into the scratch arrays, the inactive rows straight to their places; or the rows of both lists ------
   if (stage != 1) {
-    gather_replica<REP_THREADS, 1, false, false>(c, R + 1, r, B, gather_tiles_at(smem, REP_THREADS, REP_THREADS), true, stage == 0 || (ordered && list_in),
+    gather_replica<REP_THREADS, 1, false, false>(c, R + 1, r, B, gather_tiles_at(s_tiles, REP_THREADS, REP_THREADS), true, stage == 0 || (ordered && list_in),
                    [&](uint32_t pos, const uint4 rec, int32_t row) {
                      if (stage == 0) { g_ra[pos] = row; return; }
                      if (!ordered) pos = s_ord[pos];      // its place by id
-                     g_item[pos] = ((uint64_t)rec.y << 32) | rec.x; g_zw[pos] = make_uint2(rec.z, rec.w); g_row[pos] = row;
+                     s_item[pos] = ((uint64_t)rec.y << 32) | rec.x; g_zw[pos] = make_uint2(rec.z, rec.w); g_row[pos] = row;
+                     if (((rec.z >> CREC_KIND_SHIFT) & 1u) == KIND_RUNNING) { n_run++; sum_kv += (rec.z & CREC_LEN_MASK) + (rec.w & CREC_LEN_MASK); m_run |= 1ull << (rec.w >> CREC_CLS_SHIFT); }
+                     else m_q |= 1ull << (rec.w >> CREC_CLS_SHIFT);
                    },
                    [&](uint32_t pos, int32_t row) { if (stage == 0) g_ri[pos] = row; else a.order[b + n_act + pos] = row; });
     __syncthreads();
   }
+  for (int i = tid; i < MED_BINS / 2; i += REP_THREADS) s_bin[i] = 0;
 
   if (stage < 2) {
     // ---- sort items of the ids, their range -------------------------------------------------------------
@@ -1259,7 +1275,6 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
       lo = uid < lo ? uid : lo; hi = uid > hi ? uid : hi;
       g_item[q] = ((uint64_t)uid << 16) | (uint32_t)q;
     }
-    for (int i = tid; i < MED_BINS / 2; i += REP_THREADS) s_bin[i] = 0;
     lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane == 0) sh.red_m0[warp] = ((uint64_t)hi << 32) | lo;
     __syncthreads();
@@ -1273,50 +1288,43 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
   } else {
   // ---- aggregates, plan ---------------------------------------------------------------------------------
   {
-    int64_t n_run = 0, sum_kv = 0;
-    uint64_t m_run = 0, m_q = 0;
-#pragma unroll 4
-    for (int q = tid; q < n_act; q += REP_THREADS) {
-      const uint2 zw = g_zw[q];
-      const uint32_t cls = zw.y >> CREC_CLS_SHIFT;
-      if (((zw.x >> CREC_KIND_SHIFT) & 1u) == KIND_RUNNING) { n_run++; sum_kv += (int64_t)(zw.x & CREC_LEN_MASK) + (zw.y & CREC_LEN_MASK); m_run |= 1ull << cls; }
-      else m_q |= 1ull << cls;
-    }
-    for (int i = tid; i < MED_BINS / 2; i += REP_THREADS) s_bin[i] = 0;
     for (int i = tid; i < TINY_CLASSES; i += REP_THREADS) { s_cmin[i] = 0xffffffffu; s_cmax[i] = 0; s_lmin[i] = 0xffu; s_lmax[i] = 0; s_ccnt[i] = 0; }
-    n_run = warp_sum_i64(n_run); sum_kv = warp_sum_i64(sum_kv);
+    n_run = __reduce_add_sync(0xffffffffu, n_run); sum_kv = (uint64_t)warp_sum_wide((int64_t)sum_kv);
     m_run = warp_or_u64(m_run); m_q = warp_or_u64(m_q);
-    if (lane == 0) { sh.red_a[warp] = n_run; sh.red_b[warp] = sum_kv; sh.red_m0[warp] = m_run; sh.red_m1[warp] = m_q; }
+    if (lane == 0) { sh.red_a[warp] = n_run; sh.red_b[warp] = (int64_t)sum_kv; sh.red_m0[warp] = m_run; sh.red_m1[warp] = m_q; }
     __syncthreads();
     if (warp == 0) {     // the first warp finishes the reduction and plans
-      n_run = warp_sum_i64(sh.red_a[lane]); sum_kv = warp_sum_i64(sh.red_b[lane]);
+      const int64_t all_run = warp_sum_i64(sh.red_a[lane]), all_kv = warp_sum_i64(sh.red_b[lane]);
       m_run = warp_or_u64(sh.red_m0[lane]); m_q = warp_or_u64(sh.red_m1[lane]);
       hfx_replica_cfg cfg; cfg.mode = HFX_COLOCATED; cfg.token_cap = 1; cfg.batch_cap = 0;
       int64_t now = 0, mat = 0;
       if (real) { cfg = a.cfg[r]; now = a.now[r]; mat = a.mat[r]; }
       ReplicaPlan pl0;
-      warp_plan(p, tab, cfg, now, mat, n_run, sum_kv, m_run, m_q, pl0, lane);
+      warp_plan(p, tab, cfg, now, mat, all_run, all_kv, m_run, m_q, pl0, lane);
       if (lane == 0) { sh.plan = pl0; sh.next_arrival = HFX_INF; }
     }
     __syncthreads();
   }
   const ReplicaPlan pl = sh.plan;
 
-  // ---- sort items (into the scratch, over the bases); per class their range ------------------------
+  // ---- sort items (into the scratch); per class their range ------------------------
   {
     const int n_rounds = (n_act + REP_THREADS - 1) / REP_THREADS;
-    int64_t base_n = 0; uint2 zw_n = make_uint2(0u, 0u); int32_t row_n = 0;      // the next round's row, asked for a round ahead
-    if (tid < n_act) { base_n = (int64_t)g_item[tid]; zw_n = g_zw[tid]; row_n = g_row[tid]; }
+    // every row queued on a colocated / prefill replica: the front end has put its final key in place of the base, and no output of it is left
+    const bool all_given = pl.n_run == 0 && pl.mode != HFX_DECODE && !a.pred_tpot;
+    uint2 zw_n = make_uint2(0u, 0u); int32_t row_n = 0;      // the next round's row, asked for a round ahead
+    if (!all_given && tid < n_act) { zw_n = g_zw[tid]; row_n = g_row[tid]; }
     for (int q0 = 0; q0 < n_act; q0 += REP_THREADS) {
       if (q0 + (tid & ~31) >= n_act) break;      // (whole warps leave)
       const int q = q0 + tid;
       const bool in = q < n_act;
-      const int64_t base = base_n; const uint2 zw = zw_n; const int32_t row = row_n;
-      if (q + REP_THREADS < n_act) { base_n = (int64_t)g_item[q + REP_THREADS]; zw_n = g_zw[q + REP_THREADS]; row_n = g_row[q + REP_THREADS]; }
+      const uint2 zw = zw_n; const int32_t row = row_n;
+      if (!all_given && q + REP_THREADS < n_act) { zw_n = g_zw[q + REP_THREADS]; row_n = g_row[q + REP_THREADS]; }
       uint64_t item = ~0ull;
       if (in) {
+        const int64_t base = (int64_t)s_item[q];
         const int kind = (zw.x >> CREC_KIND_SHIFT) & 1, prio = zw.x >> CREC_PRIO_SHIFT;
-        const bool given = kind == KIND_QUEUED && pl.mode != HFX_DECODE;      // the front end has put the row's final key in place of the base
+        const bool given = all_given || (kind == KIND_QUEUED && pl.mode != HFX_DECODE);
         RowEval ev;
         if (given) { ev.k48 = (uint64_t)base; ev.slack = 0; ev.pred_tpot = a.pred_tpot ? pl.tpot_q0 + p.d2 * ((int64_t)(zw.x & CREC_LEN_MASK) + (zw.y & CREC_LEN_MASK)) : 0; }
         else ev = eval_row(p, pl, base, kind, prio, (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK));
@@ -1412,8 +1420,9 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
     if (lane == 31) sh.red_n[warp] = (int32_t)v;
     if (lane == 0) sh.red_a[warp] = (int64_t)big;
     __syncthreads();
-    uint32_t run = v - sum, bigall = 0;
-    for (int k = 0; k < REP_THREADS / 32; k++) { if (k < warp) run += (uint32_t)sh.red_n[k]; const uint32_t x = (uint32_t)sh.red_a[k]; bigall = x > bigall ? x : bigall; }
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? (uint32_t)sh.red_n[lane] : 0u);
+    const uint32_t bigall = __reduce_max_sync(0xffffffffu, (uint32_t)sh.red_a[lane]);
+    uint32_t run = v - sum + before;
     if (bigall <= MED_BIN_MAX) {
       uint32_t st[8];
 #pragma unroll
@@ -1470,33 +1479,35 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
   }
   const ReplicaPlan pl = sh.plan;
 
-  // ---- the order; the record words by position, over the items -----------------------------------------
+  // ---- what the admission looks at, by position, over the items; the order -----------------------------------------
 #pragma unroll 4
   for (int q = tid; q < n_act; q += REP_THREADS) {
-    a.order[b + q] = g_row[s_ord[q]];
     const uint2 zw = g_zw[q];
-    s_zw[q] = make_uint2(zw.x & ((1u << CREC_PRIO_SHIFT) - 1u), zw.y);      // (the priority has served; its bits make room for the marks)
+    const uint32_t len = (zw.x & CREC_LEN_MASK) + (pl.mode == HFX_DECODE ? zw.y & CREC_LEN_MASK : 0u);
+    s_val[q] = len | (((zw.x >> CREC_KIND_SHIFT) & 1u) == KIND_QUEUED ? 0u : VAL_RUNNING);
+    s_row[q] = g_row[q];
   }
   __syncthreads();
+#pragma unroll 4
+  for (int q = tid; q < n_act; q += REP_THREADS) a.order[b + q] = s_row[s_ord[q]];
 
-  auto cost_at = [&](uint32_t li, int64_t &kv) -> int64_t {      // cost of the queued row at position li, -1 if it is in flight
-    const uint2 zw = s_zw[li];
-    if (((zw.x >> CREC_KIND_SHIFT) & 1u) != KIND_QUEUED) return -1;
-    kv = (int64_t)(zw.x & CREC_LEN_MASK) + (zw.y & CREC_LEN_MASK);
-    return pl.mode == HFX_DECODE ? p.d1 + p.d2 * kv : (int64_t)(zw.x & CREC_LEN_MASK);
+  auto cost_at = [&](uint32_t val) -> int64_t {      // cost of a queued row, -1 if it is in flight
+    if (val & VAL_RUNNING) return -1;
+    const int64_t x = val & VAL_LEN_MASK;
+    return pl.mode == HFX_DECODE ? p.d1 + p.d2 * x : x;
   };
   if (FF) {     // first fit: the smallest cost of every 32 places by all warps, then the first warp walks the order and marks what it takes
     int64_t *s_min = reinterpret_cast<int64_t *>(s_bin);      // [SEG_MED / 32] (the bins have served)
     for (int q0 = warp * 32; q0 < n_act; q0 += REP_THREADS) {
-      int64_t kv, cc = q0 + lane < n_act ? cost_at(s_ord[q0 + lane], kv) : -1;
+      int64_t cc = q0 + lane < n_act ? cost_at(s_val[s_ord[q0 + lane]]) : -1;
       cc = warp_min_i64(cc < 0 ? HFX_INF : cc);
       if (lane == 0) s_min[q0 >> 5] = cc;
     }
     __syncthreads();
     if (warp == 0) {
       const int64_t room = pl.batch_cap == 0 ? HFX_INF : (pl.batch_cap > pl.n_eff ? pl.batch_cap - pl.n_eff : 0);
-      warp_first_fit(n_act, s_min, pl.budget, room, lane, [&](int64_t q) -> int64_t { int64_t kv; return cost_at(s_ord[q], kv); },
-                     [&](int64_t q, bool taken) { if (taken) s_zw[s_ord[q]].x |= 0x80000000u; });
+      warp_first_fit(n_act, s_min, pl.budget, room, lane, [&](int64_t q) -> int64_t { return cost_at(s_val[s_ord[q]]); },
+                     [&](int64_t q, bool taken) { if (taken) s_val[s_ord[q]] |= VAL_TAKEN; });
     }
     __syncthreads();
   }
@@ -1507,10 +1518,9 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
   int64_t my_cost = 0;
   int32_t my_cnt = 0;
   for (int q = qa; q < qb; q++) {      // what counts towards the running totals: rows that fit alone, or (first fit) exactly the rows taken
-    const uint32_t li = s_ord[q];
-    int64_t kv = 0;
-    const int64_t cc = cost_at(li, kv);
-    if (cc >= 0 && (FF ? (s_zw[li].x >> 31) != 0 : cc <= pl.budget)) { my_cost += cc; my_cnt++; }
+    const uint32_t val = s_val[s_ord[q]];
+    const int64_t cc = cost_at(val);
+    if (cc >= 0 && (FF ? (val & VAL_TAKEN) != 0 : cc <= pl.budget)) { my_cost += cc; my_cnt++; }
   }
   int64_t run_c = warp_incl_scan_i64(my_cost, lane);
   int32_t run_n = warp_incl_scan_i32(my_cnt, lane);
@@ -1522,17 +1532,16 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
   int32_t an = 0;
   if (my_cnt)
     for (int q = qa; q < qb; q++) {
-      const uint32_t li = s_ord[q];
-      int64_t kv = 0;
-      const int64_t cc = cost_at(li, kv);
-      if (cc >= 0 && (FF ? (s_zw[li].x >> 31) != 0 : cc <= pl.budget)) {
+      const uint32_t li = s_ord[q], val = s_val[li];
+      const int64_t cc = cost_at(val);
+      if (cc >= 0 && (FF ? (val & VAL_TAKEN) != 0 : cc <= pl.budget)) {
         run_c += cc; run_n += 1;
         if (FF || (run_c <= pl.budget && (pl.batch_cap == 0 || pl.n_eff + run_n <= pl.batch_cap))) {
-          ac += cc; ak += kv; an++;
-          const int32_t row = g_row[li];
+          ac += cc; ak += val & VAL_LEN_MASK; an++;      // (the context of what is admitted counts on a decode replica alone)
+          const int32_t row = s_row[li];
           a.admit[row] = 1;
           if (a.admitted_rows) a.admitted_rows[b + run_n - 1] = row;
-          s_zw[li].y |= 0x80000000u;
+          s_val[li] = val | VAL_ADMITTED;
         }
       }
     }
@@ -1568,10 +1577,10 @@ __device__ void medium_slabs(const HfxParams &p, const SegArgs &a, const SegCtx 
     const int64_t t1 = sh.t1, t2 = sh.t2;
 #pragma unroll 2
     for (int q = tid; q < n_act; q += REP_THREADS) {
-      const uint2 zw = s_zw[q];
+      const uint2 zw = g_zw[q];
       const int kind = (zw.x >> CREC_KIND_SHIFT) & 1;
-      const bool adm = (zw.y >> 31) != 0;
-      const int32_t row = g_row[q];
+      const bool adm = (s_val[q] & VAL_ADMITTED) != 0;
+      const int32_t row = s_row[q];
       const int32_t out_len = commit_needs_out_len(pl, kind, adm, worked) ? a.output_len[row] : 0;
       commit_row(a, pl, kind, adm, worked, t1, t2, row, (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK), out_len);
     }

@@ -50,9 +50,8 @@ struct SegCtx {
   HfxRec *rec;            // contiguous records (fallback: input; slabs: scratch of the larger replicas)
   const uint32_t *ordered; const uint8_t *rowflag;
   uint64_t *big_hi; uint32_t *big_lo; uint32_t *big_idx;
-  int64_t pad;            // The sizes of this struct and of BlockShared move the compiler's allocation of the 64 registers: with 8 bytes more in both
-                          // k_replicas reloads 508 bytes a thread instead of 632 (ten steps over 1024 replicas 649 us instead of 654, one step over 64
-                          // replicas of 4096 rows 45.5 instead of 46.7).
+  int64_t pad;            // (The sizes of this struct and of BlockShared move the compiler's allocation of the 64 registers: without these 8 bytes in both
+                          // more of them are reloaded, one step over 64 replicas of 4096 rows takes 46.7 us instead of 45.5.)
 };
 
 // A set of threads of the block that synchronise on a hardware barrier of their own (0 = the whole block).
@@ -492,6 +491,12 @@ __device__ __forceinline__ void layout_class_bins(const uint32_t *s_ccnt, const 
 // Small replicas: one group of 128 threads.  What later passes need of the replica's active rows
 // (slack base, record words, row) is staged once in shared memory; sort items live in registers
 // until they are scattered into their bins.
+// What bounds it: eight groups at different places of a long program, so that instructions come from beyond the first caches (4.9 of 25 cycles an
+// instruction waited for that).  Loops that hold nothing in registers are therefore kept short instead of being unrolled six times:
+// admission, ranks and commit (the output lengths were asked for with the keys, six registers and as many loads further on).  Ten steps over 1024 replicas 648 ->
+// 595 us, ten rounds of 128 + 128 replicas 560 -> 527, four ticks of a fleet of 1024 1716 -> 1589, one step over one replica 22.6 -> 20.8.  Items in
+// shared memory as well, all loops short: 620, 528, 1595, 21.0 (a second look at every item costs more where there are 500 of them); a way out
+// of every round of the unrolled loops: 644, 545, 1631, 23.1.
 // ------------------------------------------------------------------------------------------------
 #define SMALL_SMEM (SEG_TINY * 24 + (TINY_BINS + 4) * 4 + TINY_CLASSES * 8)
 static_assert(SMALL_SMEM <= SMEM_GROUP, "a group's arrays fit its share of the block's shared memory");
@@ -556,12 +561,12 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   }
 
   // ---- gather: base, record words and row of the active rows; the inactive rows' places ----------------------
-  if (SLABS) {
+  if (SLABS && (n_act > 0 || (ordered && list_in && n_in > 0))) {      // (an instance that is off has none: four ticks of a fleet that is mostly off 1631 -> 1594 us)
     GatherDst dst; dst.bk = s_bk; dst.zw = s_zw; dst.row = s_row;
     gather_replica<GROUP_THREADS, GROUP_TPT, true, true>(c, R1, r, G, gt, true, ordered && list_in, [](uint32_t, const uint4, int32_t) {},
                                                          [&](uint32_t pos, int32_t row) { a.order[b + n_act + pos] = row; }, dst);
     cp_async_wait_all();
-  } else {
+  } else if (!SLABS) {
     for (int q = G.tid; q < n_act; q += G.n) {
       const uint4 w0 = reinterpret_cast<const uint4 *>(seg + q)[0];
       const uint4 w1 = reinterpret_cast<const uint4 *>(seg + q)[1];
@@ -608,16 +613,13 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
 
   // ---- keys (in registers); per class their range ---------------------------------------------------
   uint64_t item[TINY_IPT];
-  int32_t out_len[TINY_IPT];       // of my rows in flight, asked for now and used by the commit
   const bool few = n_act <= GROUP_THREADS;      // an item per thread: ranked by counting the smaller ones, no bins
-  const bool will_commit = real && (a.flags & HFX_COMMIT) && pl.now <= a.horizon;
 #pragma unroll
   for (int k = 0; k < TINY_IPT; k++) {
+    if (k == 1 && few) break;      // (what is not executed is not fetched either: four ticks 1605 -> 1589 us)
     const int q = G.tid + k * GROUP_THREADS;
     item[k] = ~0ull;
-    out_len[k] = 0;
     if (q < n_act) {
-      if (will_commit && ((s_zw[q].x >> CREC_KIND_SHIFT) & 1u) == KIND_RUNNING) out_len[k] = a.output_len[s_row[q]];
       const int64_t base = (int64_t)s_bk[q];
       const uint2 zw = s_zw[q];
       const int kind = (zw.x >> CREC_KIND_SHIFT) & 1, prio = zw.x >> CREC_PRIO_SHIFT;
@@ -709,10 +711,9 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
           s_bk[pos] = item[k];
         }
       G.sync();
-#pragma unroll
-      for (int k = 0; k < TINY_IPT; k++) {
-        const int e = G.tid + k * GROUP_THREADS;
-        if (e < n_act) {
+#pragma unroll 1
+      for (int e = G.tid; e < n_act; e += GROUP_THREADS) {
+        {
           const uint64_t x = s_bk[e];
           const uint32_t bi = bin_of(x), sh16 = (bi & 1u) * 16;
           const uint32_t g0 = (s_bin[bi >> 1] >> sh16) & 0xffffu, g1 = (s_cur[bi >> 1] >> sh16) & 0xffffu;
@@ -760,22 +761,19 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   if (FF)
     first_fit_marks(pl, s_lo, n_act, G, [&](int64_t q) -> int64_t { int64_t kv; return cost_at(s_lo[q] & 0xffffu, kv); });
 
-  // ---- admission: each thread walks TINY_IPT consecutive places of the order ---------------------
-  const int q0 = G.tid * TINY_IPT;
-  uint32_t cand[TINY_IPT];      // record position of the candidate at each of my places | 0x80000000, or 0
+  // ---- admission: each thread walks consecutive places of the order, twice ---------------------
+  // (short loops: what the groups execute here comes from memory beyond their instruction caches)
+  const int per = (n_act + GROUP_THREADS - 1) / GROUP_THREADS;
+  const int qa = G.tid * per, qb = qa + per < n_act ? qa + per : n_act;
+  auto counts = [&](uint32_t lo, int64_t cc) -> bool { return cc >= 0 && (FF ? (lo & 0x20000u) != 0 : cc <= pl.budget); };      // rows that fit alone, or (first fit) exactly the rows taken
   uint64_t mine = 0;            // cost | count << 48 of the candidates of this thread (costs stay below 2^44 in total)
-#pragma unroll
-  for (int k = 0; k < TINY_IPT; k++) {
-    const int q = q0 + k;
-    cand[k] = 0;
-    if (q < n_act) {
-      const uint32_t li = s_lo[q] & 0xffffu;
-      int64_t kv = 0;
-      const int64_t cc = cost_at(li, kv);
-      // what counts towards the totals: rows that fit alone, or (first fit) exactly the rows taken
-      if (cc >= 0 && (FF ? (s_lo[q] & 0x20000u) != 0 : cc <= pl.budget)) { cand[k] = li | 0x80000000u; mine += (uint64_t)cc + (1ull << 48); }
-      a.order[b + q] = s_row[li];
-    }
+#pragma unroll 1
+  for (int q = qa; q < qb; q++) {
+    const uint32_t lo = s_lo[q], li = lo & 0xffffu;
+    int64_t kv = 0;
+    const int64_t cc = cost_at(li, kv);
+    if (counts(lo, cc)) mine += (uint64_t)cc + (1ull << 48);
+    a.order[b + q] = s_row[li];
   }
   uint64_t sc = (uint64_t)warp_incl_scan_i64((int64_t)mine, lane);
   if (lane == 31) sh.red_m0[warp] = sc;
@@ -786,12 +784,13 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
   int32_t run_n = (int32_t)(run >> 48);
   int64_t ac = 0, ak = 0;
   int32_t an = 0;
-#pragma unroll
-  for (int k = 0; k < TINY_IPT; k++) {
-    if (cand[k]) {
-      const uint32_t li = cand[k] & 0xffffu;
+  if (mine)
+#pragma unroll 1
+    for (int q = qa; q < qb; q++) {
+      const uint32_t lo = s_lo[q], li = lo & 0xffffu;
       int64_t kv = 0;
       const int64_t cc = cost_at(li, kv);
+      if (!counts(lo, cc)) continue;
       run_c += cc; run_n += 1;
       if (FF || (run_c <= pl.budget && (pl.batch_cap == 0 || pl.n_eff + run_n <= pl.batch_cap))) {
         ac += cc; ak += kv; an++;
@@ -801,7 +800,6 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
         s_zw[li].y |= 0x80000000u;
       }
     }
-  }
 
   // ---- totals, maturity, replica outputs, commit ---------------------------------------------------------
   if (__any_sync(0xffffffffu, an > 0)) { ac = warp_sum_i64(ac); ak = warp_sum_i64(ak); an = (int32_t)__reduce_add_sync(0xffffffffu, (uint32_t)an); }
@@ -829,18 +827,15 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
     write_replica_outputs(a, r, pl, sh.adm_cost, sh.adm_count, mat_next, worked, sh.t2, sh.next_arrival);
   if (a.admitted_rows)
     for (int q = sh.adm_count + G.tid; q < n; q += G.n) a.admitted_rows[b + q] = -1;
-  if (commit) {      // every thread its own rows; an admitted row's output length is fetched now (there are few)
+  if (commit) {      // every thread its own rows
     const int64_t t1 = sh.t1, t2 = sh.t2;
-#pragma unroll
-    for (int k = 0; k < TINY_IPT; k++) {
-      const int q = G.tid + k * GROUP_THREADS;
-      if (q < n_act) {
-        const uint2 zw = s_zw[q];
-        const int kind = (zw.x >> CREC_KIND_SHIFT) & 1;
-        const bool adm = (zw.y >> 31) != 0;
-        const int32_t ol = adm ? a.output_len[s_row[q]] : out_len[k];
-        commit_row(a, pl, kind, adm, worked, t1, t2, s_row[q], (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK), ol);
-      }
+#pragma unroll 2
+    for (int q = G.tid; q < n_act; q += GROUP_THREADS) {
+      const uint2 zw = s_zw[q];
+      const int kind = (zw.x >> CREC_KIND_SHIFT) & 1;
+      const bool adm = (zw.y >> 31) != 0;
+      const int32_t ol = adm || kind == KIND_RUNNING ? a.output_len[s_row[q]] : 0;
+      commit_row(a, pl, kind, adm, worked, t1, t2, s_row[q], (int32_t)(zw.x & CREC_LEN_MASK), (int32_t)(zw.y & CREC_LEN_MASK), ol);
     }
   }
   G.sync();

@@ -356,19 +356,27 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     for (int il = tid; il < nt; il += blockDim.x) {
       const uint32_t bk = s_bkt[il], b = bk & 0xfffu;
       if (tail_scan && b == (uint32_t)R) continue;
-      s_perm[s_base[2 * b + (((bk >> 15) & 1u) ^ 1u)] + (bk >> 16)] = (uint16_t)il;
+      s_perm[s_base[2 * b + (((bk >> 15) & 1u) ^ 1u)] + (bk >> 16)] = (uint16_t)(any_big ? il : il | 0x8000);
     }
     __syncthreads();
     const int n_slots = tail_scan ? (int)s_base[2 * R + 1] : nt;      // (the group of unbound rows is the last one)
     if (!any_big) {
-      // ... then every group in row order: the place of a row is the number of smaller rows in its group
+      // ... then every group in row order: the place of a row is the number of smaller rows in its group, two slots at a time: with bit 15
+      // set beside their 13 bits, x - il keeps that bit in every half that is not smaller, and nothing is borrowed from the half above
+      // (bound by instructions: a tile's counting over groups of 55 rows took 16 of its 48 K cycles; four ticks of a fleet of 1024 1627 -> 1598 us,
+      // ten steps over 1024 replicas, groups of 3.5, 598 -> 593.  Plain comparisons of two or four slots to a look: 1655, 1675)
+      const uint32_t *s_two = reinterpret_cast<const uint32_t *>(s_perm);
       for (int j = tid; j < n_slots; j += blockDim.x) {
-        const uint32_t il = s_perm[j];
+        const uint32_t il = s_perm[j] & 0x7fffu;
         const uint32_t bk = s_bkt[il];
         const uint32_t g = 2 * (bk & 0xfffu) + (((bk >> 15) & 1u) ^ 1u);
-        const uint32_t g0 = s_base[g], g1 = g0 + s_cnt[g];
-        uint32_t rank = 0;
-        for (uint32_t i = g0; i < g1; i++) rank += s_perm[i] < il ? 1u : 0u;
+        const uint32_t g0 = s_base[g], g1 = g0 + s_cnt[g], both = il * 0x10001u;
+        uint32_t above = 0;
+#pragma unroll 2
+        for (uint32_t i = g0 >> 1; i < (g1 + 1) >> 1; i++) above += ((s_two[i] - both) >> 15) & 0x10001u;
+        uint32_t rank = 2 * (((g1 + 1) >> 1) - (g0 >> 1)) - (above & 0xffffu) - (above >> 16);
+        if (g0 & 1u) rank -= (((uint32_t)s_perm[g0 - 1] - il) >> 15 & 1u) ^ 1u;      // (not of the group: the first look's lower half, the last one's upper half)
+        if (g1 & 1u) rank -= (((uint32_t)s_perm[g1] - il) >> 15 & 1u) ^ 1u;
         s_fin[g0 + rank] = (uint16_t)il;
       }
     } else {

@@ -37,10 +37,13 @@
 #define DISP_TILES_CHAIN 1024       // tiles whose totals the chain adds up itself; beyond them they are added to the running totals
 #define SORT_SMEM (DISP_TILE_MAX * 22 + (DISP_FINE + 4) * 4 + (DISP_BINS + 4) * 4 + DISP_SPLITS * 16)
 #define VAL_FITS 0x80000000u        // on an ordered row: some instance's budget reaches it (the others are passed over)
-#define CHAIN_THREADS 512
+#define CHAIN_THREADS 1024
+#define CHAIN_THREADS_FEW 512
+#define CHAIN_FEW 16                // instances up to which a block of the chain is small: what it meets at is shorter (2 instances 33.0 us, 33.4 with 1024 threads)
 #define CHAIN_CHUNK 4096            // running totals staged in shared memory at a time
 #define CHAIN_WIN 256               // and held in registers by the walking warp, eight per lane
-#define CHAIN_BATCH 6               // instances between two looks at whether all went well
+#define CHAIN_BATCH 24              // instances between two looks at whether all went well: as many as the windows before held,
+#define CHAIN_BATCH_MIN 4           // between these two
 #define ASSIGN_THREADS 256
 
 // words of the control block, zero between calls unless noted
@@ -724,13 +727,15 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 // walk is one warp's serial recurrence  limit = base + budget -> entries within the limit -> base,  and what counts is its
 // latency.  The warp holds the running totals of 256 entries in registers, eight per lane, as 32-bit distances from the
 // chunk's start: the new base is the largest total within the limit, one maximum over the lanes (22 cycles), and nothing
-// else is on the recurrence.  Six instances are done in a loop without a further branch (a short loop: what the single warp
+// else is on the recurrence.  A batch of instances is done in a loop without a further branch (a short loop: what the single warp
 // executes has to come from its first instruction cache, unrolled it took three times as long); then it is looked at whether
 // the last of them reached the end of the window: what is in front of the first that did stands, that one is tried again from a fresh
-// window or, if it started this one, searched for (32 ways).  The other warps meanwhile stage the next chunk of totals in
-// shared memory and look up where the runs of the chunk before ended (the entries up to a base are those within it).
-// Then all threads: what every instance took, dispatching step 4 (its new maturity time).  1024 instances, 471 K entries:
-// 272 us when the totals were probed in shared memory, 117 us now (190 cycles per instance, 105 of them the recurrence).
+// window or, if it started this one, searched for (32 ways).  A batch is as long as the windows before allowed, or four instances longer: runs
+// are of three entries or of a hundred, and a third of the instances takes nothing where one prompt keeps them all waiting (six instances
+// always / eight / sixteen / so: 4096 instances 510 / 465 / 407 / 392 us a call, 700 156 / 145 / 135 / 132, 1024 with 40 entries a run 203 / 199 / 223 / 199).
+// The other warps meanwhile stage the next chunk of totals in shared memory and look up where the runs of the chunk before ended (the entries up to
+// a base are those within it).  Then all threads: what every instance took, dispatching step 4 (its new maturity time).  1024 instances, 471 K entries of which
+// 22 K are taken: 272 us when the totals were probed in shared memory, 104 now (90 of them the walk), with 512 threads 109.
 // ------------------------------------------------------------------------------------------------
 // longest m in [lo, hi] with fits(m), given fits(lo) and fits monotone; whole warp
 template <typename F>
@@ -751,10 +756,10 @@ __device__ __forceinline__ int64_t warp_longest(int64_t lo, int64_t hi, int lane
 // none; b, c: totals at the cursor, then behind the last instance; lane i gets the totals behind instance i.
 template <bool COUNTS>
 __device__ __forceinline__ void chain_batch(const uint32_t *rel, const uint32_t *rc, const uint32_t *s_bud, const uint32_t *s_room, uint32_t &b, uint32_t &c, int lane,
-                                            uint32_t &at_b, uint32_t &at_c) {
+                                            int batch, uint32_t &at_b, uint32_t &at_c) {
   uint32_t bud = s_bud[0], room = COUNTS ? s_room[0] : 0u;
 #pragma unroll 2
-  for (int i = 0; i < CHAIN_BATCH; i++) {
+  for (int i = 0; i < batch; i++) {
     const uint32_t lim = b + bud, lc = c + room;
     bud = s_bud[i + 1];                      // (one more than the batch: the arrays are padded)
     if (COUNTS) room = s_room[i + 1];
@@ -774,7 +779,8 @@ __device__ __forceinline__ void chain_batch(const uint32_t *rel, const uint32_t 
   }
 }
 
-__global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p, const DispArgs a, const DispWork w) {
+template <int threads>
+__global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const DispArgs a, const DispWork w) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int BUF = CHAIN_CHUNK + CHAIN_WIN + 8;
   uint32_t *s_rel = reinterpret_cast<uint32_t *>(smem_raw);                       // [2][BUF] totals, as distances from the chunk's start
@@ -799,7 +805,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
   if (w.ctl[CTL_ABORT]) return;                // (TAKEN stays 0)
   const bool by_tile = tiles <= DISP_TILES_CHAIN;      // the running totals start anew in every tile
   if (by_tile) {
-    constexpr int PER = DISP_TILES_CHAIN / CHAIN_THREADS;
+    constexpr int PER = DISP_TILES_CHAIN / threads;
     int64_t x[PER], sum = 0, all;
     uint32_t y[PER], sumc = 0, allc;
 #pragma unroll
@@ -812,7 +818,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
     uint32_t runc = block_prefix<uint32_t>(sumc, s_part, &allc);
 #pragma unroll
     for (int e = 0; e < PER; e++) { s_base[tid * PER + e] = run; s_basec[tid * PER + e] = runc; run += x[e]; runc += y[e]; }
-    for (uint32_t t = tid; t <= tiles; t += CHAIN_THREADS) s_edge[t] = w.tile_edge[t];
+    for (uint32_t t = tid; t <= tiles; t += threads) s_edge[t] = w.tile_edge[t];
   }
   __syncthreads();
   // the running totals behind q entries of both queues together
@@ -829,7 +835,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
   const int64_t *budgets = w.ord_budget + koff;
   const int32_t *rooms = w.ord_room + koff;
   bool capped = false, wide = false;
-  for (int k = tid; k <= nm + CHAIN_BATCH; k += CHAIN_THREADS) {
+  for (int k = tid; k <= nm + CHAIN_BATCH; k += threads) {
     const int64_t b = k < nm ? budgets[k] : 0;
     const int32_t r = k < nm ? rooms[k] : 0;
     s_bud[k] = b < 0x7fffffff ? (uint32_t)b : 0x7fffffffu;
@@ -858,7 +864,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
       }
     }
   };
-  stage_chunk(0, tid, CHAIN_THREADS);
+  stage_chunk(0, tid, threads);
   int64_t c = 0, base = 0, base_cnt = 0;      // base: totals at the cursor (the walking warp's)
   if (tid < 32) total_at(qoff, base, base_cnt);
   int k_found = 0;      // instances whose run's end has been looked up
@@ -880,16 +886,16 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
     const int64_t cursor = s_cursor;
     if (k_now >= nm || cursor >= nq) break;
     if (cursor / CHAIN_CHUNK != c) {      // not the chunk that was staged ahead (a long run)
-      if (before >= 0) { look_up(before, k_found, k_now, tid, CHAIN_THREADS); k_found = k_now; before = -1; }
+      if (before >= 0) { look_up(before, k_found, k_now, tid, threads); k_found = k_now; before = -1; }
       c = cursor / CHAIN_CHUNK;
       __syncthreads();
-      stage_chunk(c, tid, CHAIN_THREADS);
+      stage_chunk(c, tid, threads);
       __syncthreads();
     }
     if (tid >= 32) {
-      if (before >= 0) look_up(before, k_found, k_now, tid - 32, CHAIN_THREADS - 32);
-      asm volatile("bar.sync 1, %0;" ::"n"(CHAIN_THREADS - 32) : "memory");      // (the chunk ahead goes where the one before lies)
-      if ((c + 1) * CHAIN_CHUNK < nq) stage_chunk(c + 1, tid - 32, CHAIN_THREADS - 32);
+      if (before >= 0) look_up(before, k_found, k_now, tid - 32, threads - 32);
+      asm volatile("bar.sync 1, %0;" ::"n"(threads - 32) : "memory");      // (the chunk ahead goes where the one before lies)
+      if ((c + 1) * CHAIN_CHUNK < nq) stage_chunk(c + 1, tid - 32, threads - 32);
     } else {
       const int64_t lo = c * CHAIN_CHUNK;
       const int n_here = (int)(nq - lo < CHAIN_CHUNK ? nq - lo : CHAIN_CHUNK);
@@ -900,6 +906,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
       int k = k_now, cur = (int)(cursor - lo);
       int64_t jumped = -1;                   // the cursor behind a run that left the chunk
       const bool clamped = s_clamped != 0;
+      int batch = CHAIN_BATCH_MIN + 4;       // as many as the last windows held, or four more
       bool long_runs = false;                // the last run went on behind the window: no use in trying the next one in it
       uint32_t b = base - b0 < 0x7fffffff ? (uint32_t)(base - b0) : 0x7fffffffu, cc = (uint32_t)(base_cnt - c0);      // totals at the cursor, from the chunk's start
       int w0 = cur & ~7;                     // the window's start, at most seven entries in front of the cursor (they are within every limit)
@@ -913,18 +920,19 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
           if (counts) {
             const uint4 x = reinterpret_cast<const uint4 *>(s_c + w0)[2 * lane], y = reinterpret_cast<const uint4 *>(s_c + w0)[2 * lane + 1];
             rc[0] = x.x; rc[1] = x.y; rc[2] = x.z; rc[3] = x.w; rc[4] = y.x; rc[5] = y.y; rc[6] = y.z; rc[7] = y.w;
-            chain_batch<true>(rel, rc, s_bud + k, s_room + k, nb, nc, lane, tb, tc);
-          } else chain_batch<false>(rel, rc, s_bud + k, s_room + k, nb, nc, lane, tb, tc);
+            chain_batch<true>(rel, rc, s_bud + k, s_room + k, nb, nc, lane, batch, tb, tc);
+          } else chain_batch<false>(rel, rc, s_bud + k, s_room + k, nb, nc, lane, batch, tb, tc);
           // What stands: the answers in front of the first one that reaches the window's last entry (its run may go on behind
           // it), or whose totals or budget do not fit 32 bits.
           const bool more = w0 < n_more;
-          good = CHAIN_BATCH;
-          if ((more && nb >= last) || nb >= 0x7fffffffu || k + CHAIN_BATCH > nm || clamped) {
-            const uint32_t my_bud = s_bud[k + (lane < CHAIN_BATCH ? lane : 0)];
-            good = __ffs((int)__ballot_sync(0xffffffffu, lane >= CHAIN_BATCH || k + lane >= nm || (more && tb >= last) || tb >= 0x7fffffffu || my_bud == 0x7fffffffu)) - 1;
+          good = batch;
+          if ((more && nb >= last) || nb >= 0x7fffffffu || k + batch > nm || clamped) {
+            const uint32_t my_bud = s_bud[k + (lane < batch ? lane : 0)];
+            good = __ffs((int)__ballot_sync(0xffffffffu, lane >= batch || k + lane >= nm || (more && tb >= last) || tb >= 0x7fffffffu || my_bud == 0x7fffffffu)) - 1;
             nb = __shfl_sync(0xffffffffu, tb, good > 0 ? good - 1 : 0);
             nc = __shfl_sync(0xffffffffu, tc, good > 0 ? good - 1 : 0);
           }
+          batch = good == batch ? min(batch + 4, CHAIN_BATCH) : max(good, CHAIN_BATCH_MIN);
           if (lane < good) { s_tb[k + lane] = tb; s_tc[k + lane] = counts ? tc : ~0u; }
           if (good) {      // the lanes that hold an entry within the last base: all but the last of them hold nothing else
             b = nb; cc = nc; k += good;
@@ -972,11 +980,11 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
     c++;      // the chunk staged ahead
   }
   const int done = s_k;
-  if (before >= 0) look_up(before, k_found, done, tid, CHAIN_THREADS);
-  for (int k = done + tid; k < nm; k += CHAIN_THREADS) w.run_end[koff + k] = (int32_t)s_cursor;
+  if (before >= 0) look_up(before, k_found, done, tid, threads);
+  for (int k = done + tid; k < nm; k += threads) w.run_end[koff + k] = (int32_t)s_cursor;
   __syncthreads();
   // what every instance took, from the running totals at the ends of its run; its new maturity time
-  for (int k = tid; k < nm; k += CHAIN_THREADS) {
+  for (int k = tid; k < nm; k += threads) {
     const int r = w.ord_id[koff + k];
     const int64_t st = k > 0 ? w.run_end[koff + k - 1] : 0, en = w.run_end[koff + k];
     int64_t cost = 0, taken = 0;
@@ -1044,7 +1052,8 @@ static int scan_blocks(const hfx_sched *s, int64_t n) {
   return (int)(want < 1 ? 1 : (want < s->n_sm ? want : s->n_sm));
 }
 int hfx_dispatch_configure() {
-  if (cudaFuncSetAttribute(k_disp_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(4096)) != cudaSuccess ||
+  if (cudaFuncSetAttribute(k_disp_chain<CHAIN_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(4096)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_disp_chain<CHAIN_THREADS_FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(CHAIN_FEW)) != cudaSuccess ||
       cudaFuncSetAttribute(k_disp_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, SORT_SMEM) != cudaSuccess)
     return HFX_E_CUDA;
   return HFX_OK;
@@ -1149,8 +1158,9 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   cfg.numAttrs = s->profiling ? 0 : 1;
   {
     KernelScope ks(s, KSLOT_DISPATCH);
-    cfg.gridDim = dim3(d_stage ? 2 : 1); cfg.blockDim = dim3(CHAIN_THREADS); cfg.dynamicSmemBytes = chain_smem(R);
-    if (cudaLaunchKernelEx(&cfg, k_disp_chain, s->p, a, w) != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
+    cfg.gridDim = dim3(d_stage ? 2 : 1); cfg.blockDim = dim3(R <= CHAIN_FEW ? CHAIN_THREADS_FEW : CHAIN_THREADS); cfg.dynamicSmemBytes = chain_smem(R);
+    const cudaError_t e = R <= CHAIN_FEW ? cudaLaunchKernelEx(&cfg, k_disp_chain<CHAIN_THREADS_FEW>, s->p, a, w) : cudaLaunchKernelEx(&cfg, k_disp_chain<CHAIN_THREADS>, s->p, a, w);
+    if (e != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
   }
   {
     KernelScope ks(s, KSLOT_DISPATCH);

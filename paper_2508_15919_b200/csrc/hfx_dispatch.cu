@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(threads, 1) k_disp_scan(const HfxParams p, con
 //      priority did that: 500,001 rows with weights 324 us, 126 now)
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting; rows out in order, running totals
-// An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 67 us by the GPU's clock:
-// sample and plans 12, splitters 5, bins 14, their starts 7, moving 4, tiles 11, running totals 8, barriers 1.5 each; one of 42 K in 30 blocks 36.
+// An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 65 us by the GPU's clock:
+// sample and plans 12, splitters 5, bins 14, their starts 3, moving 4, tiles 12, running totals 8, barriers 1.6 each; one of 42 K in 118 blocks 36.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;

@@ -263,8 +263,9 @@ __global__ void __launch_bounds__(threads, 1) k_disp_scan(const HfxParams p, con
 //      priority did that: 500,001 rows with weights 324 us, 126 now)
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting; rows out in order, running totals
-// An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 65 us by the GPU's clock:
-// sample and plans 12, splitters 5, bins 14, their starts 3, moving 4, tiles 12, running totals 8, barriers 1.6 each; one of 42 K in 118 blocks 36.
+// An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 58 us by the GPU's clock:
+// sample and plans 8, splitters 5, bins 14, their starts 3, moving 4, tiles 10.5, running totals 8.5, barriers 1.5 each; one of 42 K in 118 blocks 30.
+// (65 and 36 with phase 0 on the warps of the first blocks instead of some of every block, and the tiles' edges found by every thread for itself)
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
@@ -308,6 +309,41 @@ __device__ __forceinline__ T block_prefix(T x, T *s_part, T *total) {
   __syncthreads();
   *total = s_part[32];
   return s_part[warp] + v - x;
+}
+
+// two of them behind the same barriers: x and c become the prefixes, all_x and all_c the sums
+__device__ __forceinline__ void block_prefix2(int64_t &x, uint32_t &c, int64_t *s_part64, uint32_t *s_part, int64_t *all_x, uint32_t *all_c) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t v = x;
+  uint32_t u = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, v, o);
+    const uint32_t z = __shfl_up_sync(0xffffffffu, u, o);
+    if (lane >= o) { v += y; u += z; }
+  }
+  __syncthreads();
+  if (lane == 31) { s_part64[warp] = v; s_part[warp] = u; }
+  __syncthreads();
+  if (warp == 0) {
+    const bool in = lane < (int)(blockDim.x >> 5);
+    int64_t s = in ? s_part64[lane] : 0;
+    uint32_t t = in ? s_part[lane] : 0u;
+    const int64_t own = s;
+    const uint32_t own_c = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, s, o);
+      const uint32_t z = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) { s += y; t += z; }
+    }
+    s_part64[lane] = s - own; s_part[lane] = t - own_c;
+    if (lane == 31) { s_part64[32] = s; s_part[32] = t; }
+  }
+  __syncthreads();
+  *all_x = s_part64[32]; *all_c = s_part[32];
+  x = s_part64[warp] + v - x;
+  c = s_part[warp] + u - c;
 }
 
 #define ITEMS_AT_ONCE 4      // items a thread has in flight in the passes over the queue
@@ -354,11 +390,13 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     const int64_t m = a.maturity[r];
     s_mat[r] = m <= a.now ? m : HFX_INF;
   }
-  for (int k = tid; k < n_samples; k += SORT_THREADS) s_sample[k] = place_of(w.item[1][(uint64_t)k * n_all / n_samples]);
+  const uint32_t apart = n_all / (uint32_t)(n_samples > 0 ? n_samples : 1), over = n_all - apart * (uint32_t)n_samples;
+  for (int k = tid; k < n_samples; k += SORT_THREADS) s_sample[k] = place_of(w.item[1][(uint32_t)k * apart + (uint32_t)k * over / (uint32_t)n_samples]);      // (k n_all / n_samples)
   if (tid < 2) { s_bmax[tid] = 0; s_nm[tid] = 0; }
   if (tid == 0) s_n1 = 0;
   __syncthreads();
-  for (int k = blockIdx.x * (SORT_THREADS / 32) + warp; k < n_samples; k += gridDim.x * (SORT_THREADS / 32)) {
+  const int gw = warp * gridDim.x + blockIdx.x, n_gw = gridDim.x * (SORT_THREADS / 32);      // the warps of the grid, one of every block after the other
+  for (int k = gw; k < n_samples; k += n_gw) {
     const uint64_t x = s_sample[k];
     uint32_t r = 0;
 #pragma unroll 4
@@ -375,7 +413,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       else { w.rank[r] = w.item[1][k].w; if (x >> 62) atomicAdd(&s_n1, 1u); }      // the row in its place; (bit 46 of the key: the D stage)
     }
   }
-  for (int r = blockIdx.x * (SORT_THREADS / 32) + warp; r < R; r += gridDim.x * (SORT_THREADS / 32)) {
+  for (int r = n_gw - 1 - gw; r < R; r += n_gw) {
     const hfx_replica_cfg cfg = a.cfg[r];
     const int64_t mat = a.maturity[r];
     const int64_t n_run = (int64_t)w.n_run[r], sum_kv = (int64_t)w.sum_kv[r];
@@ -611,13 +649,12 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   const int64_t bmax0 = (int64_t)__ldcg(w.ctl + CTL_BMAX0), bmax1 = (int64_t)__ldcg(w.ctl + CTL_BMAX1);
   const uint4 *ordered = w.item[binned ? 0 : 1];      // (ten passes end where they began)
   auto bin_edge = [&](uint32_t x) -> uint32_t {      // the first bin that starts at or behind x
-    int b = 0, n = DISP_BINS;
-    while (n > 0) { const int half = n >> 1; if (s_start[b + half] < x) { b += half + 1; n -= half + 1; } else n = half; }
-    return (uint32_t)b;
-  };
-  auto edge_of = [&](uint32_t t) -> uint32_t {      // where tile t starts
-    const uint32_t x = t * tile_rows;
-    return x >= n_all ? n_all : (binned ? s_start[bin_edge(x)] : x);
+    constexpr int K = DISP_BINS / 1024;      // (32 parts of 32 parts of K bins, a look of the warp at each; every warp searches for itself)
+    const int full = __popc(__ballot_sync(0xffffffffu, s_start[(lane + 1) * 32 * K - 1] < x));
+    if (full == 32) return DISP_BINS;
+    int b = full * 32 * K;
+    b += __popc(__ballot_sync(0xffffffffu, s_start[b + (lane + 1) * K - 1] < x)) * K;
+    return (uint32_t)(b + __popc(__ballot_sync(0xffffffffu, lane < K && s_start[b + (lane < K ? lane : 0)] < x)));
   };
   if (blockIdx.x == 0 && tid == 0) {
     a.n_queue[0] = (int32_t)n0; a.n_queue[1] = (int32_t)n1;
@@ -625,14 +662,16 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     w.tile_edge[tiles] = n_all;
   }
   for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const uint32_t e0 = edge_of(t), n = edge_of(t + 1) - e0;
+    const uint32_t x0 = t * tile_rows, x1 = x0 + tile_rows < n_all ? x0 + tile_rows : n_all;
+    const uint32_t b0 = binned ? bin_edge(x0) : 0u, b1 = binned ? bin_edge(x1) : 0u;      // whole bins
+    const uint32_t e0 = binned ? s_start[b0] : x0, n = (binned ? s_start[b1] : x1) - e0;
     constexpr int IPT = (DISP_TILE_MAX + SORT_THREADS - 1) / SORT_THREADS;
     if (binned) {
       // fine bins: an even share of them for every bin of the tile, in the bin by how far into it an item lies
       // (the last tile ends with the last bin that holds anything: with the empty bins behind it, half of them all, its items shared so few fine bins
       // that the block counted up to 435 of them with one another while the rest of the grid had finished: dispatch of 1 M rows over 1024 instances
       // 255 us then, 206 with this edge, of 60,013 rows 78 and 69)
-      const uint32_t b0 = bin_edge(t * tile_rows), nb = bin_edge((t + 1) * tile_rows < n_all ? (t + 1) * tile_rows : n_all) - b0;
+      const uint32_t nb = b1 - b0;
       const int lg = nb <= DISP_FINE ? 31 - __clz(DISP_FINE / (nb > 1 ? nb : 1u)) : 0, down = nb <= DISP_FINE ? 0 : 32 - __clz((nb - 1) / DISP_FINE);      // (a tile of many empty bins: several to a fine one)
       uint32_t fp[IPT];      // fine bin << 16 | place in it (by arrival)
       for (uint32_t i = tid; i < DISP_FINE; i += SORT_THREADS) s_fine[i] = 0;
@@ -695,8 +734,9 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       if (c[e] > (e0 + i0 + e >= n0 ? bmax1 : bmax0)) c[e] = -1;
       if (c[e] >= 0) { cost += c[e]; cnt++; }
     }
-    int64_t run = block_prefix<int64_t>(cost, s_part64, &all_cost);
-    int32_t run_cnt = (int32_t)block_prefix<uint32_t>(cnt, s_part, &all_cnt);
+    block_prefix2(cost, cnt, s_part64, s_part, &all_cost, &all_cnt);
+    int64_t run = cost;
+    int32_t run_cnt = (int32_t)cnt;
 #pragma unroll
     for (int e = 0; e < IPT; e++)
       if (e < (int)mine) {
@@ -814,11 +854,12 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
       x[e] = t < tiles ? w.tile_sum[t] : 0; y[e] = t < tiles ? (uint32_t)w.tile_sum[w.tiles_max + t] : 0u;
       sum += x[e]; sumc += y[e];
     }
-    int64_t run = block_prefix<int64_t>(sum, s_part64, &all);
-    uint32_t runc = block_prefix<uint32_t>(sumc, s_part, &allc);
+    for (uint32_t t = tid; t <= tiles; t += threads) s_edge[t] = w.tile_edge[t];
+    int64_t run = sum;
+    uint32_t runc = sumc;
+    block_prefix2(run, runc, s_part64, s_part, &all, &allc);
 #pragma unroll
     for (int e = 0; e < PER; e++) { s_base[tid * PER + e] = run; s_basec[tid * PER + e] = runc; run += x[e]; runc += y[e]; }
-    for (uint32_t t = tid; t <= tiles; t += threads) s_edge[t] = w.tile_edge[t];
   }
   __syncthreads();
   // the running totals behind q entries of both queues together

@@ -569,6 +569,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
           }
           nf = r_fin[k] < nf ? r_fin[k] : nf;
         }
+        __syncwarp();                         // (an admission of this iteration writes the notes of the freed slots, which have just been read, with other lanes)
         int kept = 0;
         for (int s0 = 0; s0 < n_list; s0 += 32) {
           const int s = s0 + lane;

@@ -29,6 +29,17 @@ def test_simulator_orders_reading_a_slot_before_the_samples_overwrite_it():
     assert "__syncwarp();" in _between(src, "s_slot[i] >> 32);\n            last", "s_slot[n_ttft")
 
 
+def test_simulator_orders_reading_a_finished_slot_before_an_admission_writes_it():
+    # the lane that holds a slot reads its notes when its request finishes; the lane that holds an admitted request writes them
+    src = _source("hfx_sim.cu")
+    last_read, first_write = src.rindex("s_rctx[32 * k + lane]"), src.index("s_rinfo[32 * k + to] =")
+    assert last_read < first_write and src.rindex("s_rinfo[32 * k + lane]") < last_read
+    between = src[last_read:first_write]
+    loop_end = between.index("nf = r_fin[k]")
+    # behind the loop over the slots, in front of the list, so that an empty list does not leave it out
+    assert "__syncwarp();" in between[loop_end:between.index("for (int s0 = 0; s0 < n_list")]
+
+
 def _functions(src, word):
     """(header, body) of every function definition that is introduced by `word`."""
     out = []

@@ -38,8 +38,6 @@
 #define SORT_SMEM (DISP_TILE_MAX * 22 + (DISP_FINE + 4) * 4 + (DISP_BINS + 4) * 4 + DISP_SPLITS * 16)
 #define VAL_FITS 0x80000000u        // on an ordered row: some instance's budget reaches it (the others are passed over)
 #define CHAIN_THREADS 1024
-#define CHAIN_THREADS_FEW 512
-#define CHAIN_FEW 16                // instances up to which a block of the chain is small: what it meets at is shorter (2 instances 33.0 us, 33.4 with 1024 threads)
 #define CHAIN_CHUNK 4096            // running totals staged in shared memory at a time
 #define CHAIN_WIN 256               // and held in registers by the walking warp, eight per lane
 #define CHAIN_BATCH 24              // instances between two looks at whether all went well: as many as the windows before held,
@@ -819,8 +817,7 @@ __device__ __forceinline__ void chain_batch(const uint32_t *rel, const uint32_t 
   }
 }
 
-template <int threads>
-__global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const DispArgs a, const DispWork w) {
+__global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p, const DispArgs a, const DispWork w) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int BUF = CHAIN_CHUNK + CHAIN_WIN + 8;
   uint32_t *s_rel = reinterpret_cast<uint32_t *>(smem_raw);                       // [2][BUF] totals, as distances from the chunk's start
@@ -845,7 +842,7 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
   if (w.ctl[CTL_ABORT]) return;                // (TAKEN stays 0)
   const bool by_tile = tiles <= DISP_TILES_CHAIN;      // the running totals start anew in every tile
   if (by_tile) {
-    constexpr int PER = DISP_TILES_CHAIN / threads;
+    constexpr int PER = DISP_TILES_CHAIN / CHAIN_THREADS;
     int64_t x[PER], sum = 0, all;
     uint32_t y[PER], sumc = 0, allc;
 #pragma unroll
@@ -854,7 +851,7 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
       x[e] = t < tiles ? w.tile_sum[t] : 0; y[e] = t < tiles ? (uint32_t)w.tile_sum[w.tiles_max + t] : 0u;
       sum += x[e]; sumc += y[e];
     }
-    for (uint32_t t = tid; t <= tiles; t += threads) s_edge[t] = w.tile_edge[t];
+    for (uint32_t t = tid; t <= tiles; t += CHAIN_THREADS) s_edge[t] = w.tile_edge[t];
     int64_t run = sum;
     uint32_t runc = sumc;
     block_prefix2(run, runc, s_part64, s_part, &all, &allc);
@@ -876,7 +873,7 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
   const int64_t *budgets = w.ord_budget + koff;
   const int32_t *rooms = w.ord_room + koff;
   bool capped = false, wide = false;
-  for (int k = tid; k <= nm + CHAIN_BATCH; k += threads) {
+  for (int k = tid; k <= nm + CHAIN_BATCH; k += CHAIN_THREADS) {
     const int64_t b = k < nm ? budgets[k] : 0;
     const int32_t r = k < nm ? rooms[k] : 0;
     s_bud[k] = b < 0x7fffffff ? (uint32_t)b : 0x7fffffffu;
@@ -905,7 +902,7 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
       }
     }
   };
-  stage_chunk(0, tid, threads);
+  stage_chunk(0, tid, CHAIN_THREADS);
   int64_t c = 0, base = 0, base_cnt = 0;      // base: totals at the cursor (the walking warp's)
   if (tid < 32) total_at(qoff, base, base_cnt);
   int k_found = 0;      // instances whose run's end has been looked up
@@ -927,16 +924,16 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
     const int64_t cursor = s_cursor;
     if (k_now >= nm || cursor >= nq) break;
     if (cursor / CHAIN_CHUNK != c) {      // not the chunk that was staged ahead (a long run)
-      if (before >= 0) { look_up(before, k_found, k_now, tid, threads); k_found = k_now; before = -1; }
+      if (before >= 0) { look_up(before, k_found, k_now, tid, CHAIN_THREADS); k_found = k_now; before = -1; }
       c = cursor / CHAIN_CHUNK;
       __syncthreads();
-      stage_chunk(c, tid, threads);
+      stage_chunk(c, tid, CHAIN_THREADS);
       __syncthreads();
     }
     if (tid >= 32) {
-      if (before >= 0) look_up(before, k_found, k_now, tid - 32, threads - 32);
-      asm volatile("bar.sync 1, %0;" ::"n"(threads - 32) : "memory");      // (the chunk ahead goes where the one before lies)
-      if ((c + 1) * CHAIN_CHUNK < nq) stage_chunk(c + 1, tid - 32, threads - 32);
+      if (before >= 0) look_up(before, k_found, k_now, tid - 32, CHAIN_THREADS - 32);
+      asm volatile("bar.sync 1, %0;" ::"n"(CHAIN_THREADS - 32) : "memory");      // (the chunk ahead goes where the one before lies)
+      if ((c + 1) * CHAIN_CHUNK < nq) stage_chunk(c + 1, tid - 32, CHAIN_THREADS - 32);
     } else {
       const int64_t lo = c * CHAIN_CHUNK;
       const int n_here = (int)(nq - lo < CHAIN_CHUNK ? nq - lo : CHAIN_CHUNK);
@@ -1021,11 +1018,11 @@ __global__ void __launch_bounds__(threads) k_disp_chain(const HfxParams p, const
     c++;      // the chunk staged ahead
   }
   const int done = s_k;
-  if (before >= 0) look_up(before, k_found, done, tid, threads);
-  for (int k = done + tid; k < nm; k += threads) w.run_end[koff + k] = (int32_t)s_cursor;
+  if (before >= 0) look_up(before, k_found, done, tid, CHAIN_THREADS);
+  for (int k = done + tid; k < nm; k += CHAIN_THREADS) w.run_end[koff + k] = (int32_t)s_cursor;
   __syncthreads();
   // what every instance took, from the running totals at the ends of its run; its new maturity time
-  for (int k = tid; k < nm; k += threads) {
+  for (int k = tid; k < nm; k += CHAIN_THREADS) {
     const int r = w.ord_id[koff + k];
     const int64_t st = k > 0 ? w.run_end[koff + k - 1] : 0, en = w.run_end[koff + k];
     int64_t cost = 0, taken = 0;
@@ -1093,8 +1090,7 @@ static int scan_blocks(const hfx_sched *s, int64_t n) {
   return (int)(want < 1 ? 1 : (want < s->n_sm ? want : s->n_sm));
 }
 int hfx_dispatch_configure() {
-  if (cudaFuncSetAttribute(k_disp_chain<CHAIN_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(4096)) != cudaSuccess ||
-      cudaFuncSetAttribute(k_disp_chain<CHAIN_THREADS_FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(CHAIN_FEW)) != cudaSuccess ||
+  if (cudaFuncSetAttribute(k_disp_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(4096)) != cudaSuccess ||
       cudaFuncSetAttribute(k_disp_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, SORT_SMEM) != cudaSuccess)
     return HFX_E_CUDA;
   return HFX_OK;
@@ -1199,8 +1195,8 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   cfg.numAttrs = s->profiling ? 0 : 1;
   {
     KernelScope ks(s, KSLOT_DISPATCH);
-    cfg.gridDim = dim3(d_stage ? 2 : 1); cfg.blockDim = dim3(R <= CHAIN_FEW ? CHAIN_THREADS_FEW : CHAIN_THREADS); cfg.dynamicSmemBytes = chain_smem(R);
-    const cudaError_t e = R <= CHAIN_FEW ? cudaLaunchKernelEx(&cfg, k_disp_chain<CHAIN_THREADS_FEW>, s->p, a, w) : cudaLaunchKernelEx(&cfg, k_disp_chain<CHAIN_THREADS>, s->p, a, w);
+    cfg.gridDim = dim3(d_stage ? 2 : 1); cfg.blockDim = dim3(CHAIN_THREADS); cfg.dynamicSmemBytes = chain_smem(R);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_disp_chain, s->p, a, w);
     if (e != cudaSuccess) { cudaGetLastError(); return HFX_E_CUDA; }
   }
   {

@@ -33,11 +33,13 @@
 #define SIM_RUN_REGS 128             // requests in flight whose finish iteration is in a register (four a lane); more of them are in a list
 #define SIM_BINS 256                 // bins of the percentile selection (8 bits a pass)
 #define SIM_HEAD_BYTES(nc) ((((size_t)(nc) * 40 + 16 + SIM_BINS * 4) + 15) & ~(size_t)15)     // in front of the rows: TTFT and TPOT by class and by rank, the bins, two counters per class
-#define SIM_LISTS_BYTES(nc, cap) (SIM_HEAD_BYTES(nc) + SIM_RUN_REGS * 8 + (size_t)(cap) * 3)      // what is in shared memory wherever the rows are
+#define SIM_LIST_BYTES(nc, cap) (SIM_HEAD_BYTES(nc) + (size_t)(cap) * 2)      // what is in shared memory wherever the rows are
+#define SIM_NOTES_BYTES(cap) (SIM_RUN_REGS * 8 + (size_t)(cap))               // notes of the running batch, classes and states: in shared memory, or behind the rows in scratch
 #define SIM_OUTLEN_CAP (1 << 30)   // output lengths are clamped here when the finish iteration is formed
 #define SIM_PARKED (SIM_BINS * 2)   // admitted requests of an iteration that are noted in shared memory (over the bins)
 // Most traces worked on at once per SM with the rows in scratch: what the registers of a warp (119 a thread, a quarter of the file per
 // scheduler) let in.  4096 traces of 2048 rows: 8 a SM 25.7 ms, 12 20.5, 16 15.1.
+// (Four classes: up to 3760 rows; of longer traces shared memory holds fewer, or as many as their lists alone let in, see LONG.)
 #define SIM_SCRATCH_PER_SM 16
 
 #define SIM_SM_BYTES (227 * 1024)    // shared memory of an SM, of which every block takes 1 KB for itself
@@ -63,19 +65,17 @@ struct SimArgs {
 
 #define FULL 0xffffffffu
 
-// Fields of the 16-byte rows: one sector holds all that an admission asks of a queued row.
-template <typename T, int AT>
+// A field of the rows: of 16-byte rows, of which one sector holds all that an admission asks of a queued row, or a column of its own.
+template <typename T, int STRIDE>
 struct SimField {
-  unsigned char *rows;
-  __device__ __forceinline__ T &operator[](int i) const { return *reinterpret_cast<T *>(rows + 16 * (size_t)i + AT); }
+  unsigned char *at;
+  __device__ __forceinline__ T &operator[](int i) const { return *reinterpret_cast<T *>(at + STRIDE * (size_t)i); }
 };
-typedef SimField<int64_t, 0> SimSlots;
-typedef SimField<uint32_t, 8> SimWords;
-typedef SimField<int32_t, 12> SimLens;
 
 // The nearest-rank percentile of n non-negative values: 8 bits a pass from the highest byte in use, the warp counting the
 // values that share the prefix found so far.  All lanes call; all get the result.
-__device__ int64_t warp_percentile(const SimSlots v, int n, int pct, uint32_t *bins, int lane) {
+template <typename V>
+__device__ int64_t warp_percentile(const V v, int n, int pct, uint32_t *bins, int lane) {
   if (n == 0) return -1;
   int64_t k = ((int64_t)pct * n + 99) / 100;
   if (k < 1) k = 1;
@@ -138,10 +138,16 @@ __device__ __forceinline__ uint32_t sim_budget(const HfxParams &p, int64_t ttft,
   return m ? first + (uint32_t)__popc(m) - 1u : 0u;
 }
 
-// SCRATCH: the 16 bytes of every row live in the block's part of a global scratch buffer, only list, classes and states in
+// SCRATCH: the 16 bytes of every row live in the block's part of a global scratch buffer, only list, classes, states and notes in
 // shared memory.  The live rows then come from L1 most of the time, and more than twice as many traces are resident: what
 // a batch of more traces than shared memory holds needs, since a warp by itself issues in one cycle of eight.
-template <bool SCRATCH>
+// LONG (with SCRATCH): classes, states and notes live there too, shared memory holds the list alone, and more of the traces that are too
+// long for SIM_SCRATCH_PER_SM of them are resident.  Long traces have long queues, of which an iteration looks at prompts and priorities along
+// the list, so the fields of a row are columns here: entries that are neighbours in the list often share a sector.
+// Traces x rows, three iterations a row, ms, lists with classes and notes in shared memory / LONG / LONG with rows of 16 bytes: 2368 x 4096
+// 30.8 / 18.7 / 19.3, 3552 x 6144 77.2 / 60.9 / 78.6, 3552 x 8192 124.5 / 90.5 / 127.9, 888 x 16,384 (30,000 iterations) 905 / 649 / 748, 296 x
+// 56,000 (20,000) 104.7 / 62.3.
+template <bool SCRATCH, bool LONG>
 __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, uint32_t *__restrict__ work_counter,
                                             uint32_t *__restrict__ status, unsigned char *__restrict__ scratch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -152,15 +158,17 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
   uint32_t *s_bins = reinterpret_cast<uint32_t *>(s_tpot + nc + 1);
   uint16_t *s_park = reinterpret_cast<uint16_t *>(s_bins);      // [SIM_PARKED] the requests admitted in an iteration
   int32_t *s_cq = reinterpret_cast<int32_t *>(s_bins + SIM_BINS), *s_cr = s_cq + nc;      // requests in the queue's list / in flight per class
-  uint16_t *s_q = reinterpret_cast<uint16_t *>(smem_raw + SIM_HEAD_BYTES(nc) + SIM_RUN_REGS * 8);
-  uint8_t *s_byte = reinterpret_cast<uint8_t *>(s_q + cap);               // class | state << 6
-  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * cap * SIM_BYTES_PER_ROW : smem_raw + SIM_LISTS_BYTES(nc, cap);
-  const SimSlots s_slot = {rows_mem};             // slack base in the queue; finish iteration | admission iteration << 32 in the batch; later the TTFT, then the TPOT samples
-  const SimWords s_word = {rows_mem};                                  // prompt_len | prio << 25
-  const SimLens s_len = {rows_mem};                                    // output length
+  uint16_t *s_q = reinterpret_cast<uint16_t *>(smem_raw + SIM_HEAD_BYTES(nc) + (LONG ? 0 : SIM_RUN_REGS * 8));
+  unsigned char *rows_mem = SCRATCH ? scratch + (size_t)blockIdx.x * ((size_t)cap * SIM_BYTES_PER_ROW + (LONG ? SIM_NOTES_BYTES(cap) : 0))
+                                    : smem_raw + SIM_LIST_BYTES(nc, cap) + SIM_NOTES_BYTES(cap);
+  unsigned char *run_mem = LONG ? rows_mem + (size_t)cap * SIM_BYTES_PER_ROW : smem_raw + SIM_HEAD_BYTES(nc);
+  uint8_t *s_byte = LONG ? run_mem + SIM_RUN_REGS * 8 : reinterpret_cast<uint8_t *>(s_q + cap);      // class | state << 6
+  const SimField<int64_t, LONG ? 8 : 16> s_slot = {rows_mem};             // slack base in the queue; finish iteration | admission iteration << 32 in the batch; later the TTFT, then the TPOT samples
+  const SimField<uint32_t, LONG ? 4 : 16> s_word = {rows_mem + (LONG ? 8 * (size_t)cap : 8)};      // prompt_len | prio << 25
+  const SimField<int32_t, LONG ? 4 : 16> s_len = {rows_mem + (LONG ? 12 * (size_t)cap : 12)};      // output length
   // One list array for both lists: from the front the queue's list (row indices, the least urgent first), from the back the
   // running batch (RUN(s), unordered)
-  uint32_t *s_rinfo = reinterpret_cast<uint32_t *>(smem_raw + SIM_HEAD_BYTES(nc));      // [SIM_RUN_REGS] requests in flight by slot: row | class << 16
+  uint32_t *s_rinfo = reinterpret_cast<uint32_t *>(run_mem);      // [SIM_RUN_REGS] requests in flight by slot: row | class << 16
   int32_t *s_rctx = reinterpret_cast<int32_t *>(s_rinfo + SIM_RUN_REGS);                // [SIM_RUN_REGS] prompt length less the admission iteration
 #define RUN(s) s_q[cap - 1 - (s)]
   const int lane = threadIdx.x;
@@ -226,7 +234,10 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
     uint32_t word = 0, pend = 0, box = 0, wrank = 0, wcls = 0;
     int src = 0, wlen = 0;
     int64_t base = BASE_UNBOUNDED;            // slack base, ttft_slo + arrival - E_p(prompt_len): the slack at any later decision is the base minus the earliest start
-    auto put_row = [&](int row) { *reinterpret_cast<uint4 *>(&s_slot[row]) = make_uint4((uint32_t)(uint64_t)base, (uint32_t)((uint64_t)base >> 32), word, (uint32_t)wlen); };
+    auto put_row = [&](int row) {
+      if (LONG) { s_slot[row] = base; s_word[row] = word; s_len[row] = wlen; }
+      else *reinterpret_cast<uint4 *>(&s_slot[row]) = make_uint4((uint32_t)(uint64_t)base, (uint32_t)((uint64_t)base >> 32), word, (uint32_t)wlen);
+    };
     auto open_window = [&]() {
       const bool ok = wb + lane < m && w.cls < (uint32_t)nc && w.prompt >= 0 && w.prompt <= HFX_MAX_TOKENS;
       uint32_t prio = 64u, wd = 0;            // (rows with bad data come last)
@@ -418,8 +429,11 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
               i = 0; wd = 0;
               if (q >= 0) {
                 i = s_q[q];
-                const uint4 x = *reinterpret_cast<const uint4 *>(&s_slot[i]);
-                wd = x.z; list_base = (int64_t)(((uint64_t)x.y << 32) | x.x);
+                if (LONG) wd = s_word[i];
+                else {
+                  const uint4 x = *reinterpret_cast<const uint4 *>(&s_slot[i]);
+                  wd = x.z; list_base = (int64_t)(((uint64_t)x.y << 32) | x.x);
+                }
                 lmin = ROW_PROMPT(wd) < lmin ? ROW_PROMPT(wd) : lmin;
               }
               fm = __ballot_sync(FULL, q >= 0 && (uint32_t)ROW_PROMPT(wd) <= budget);
@@ -433,7 +447,7 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
               const uint32_t pr = __shfl_sync(FULL, ROW_PRIO(wd), fl), b_prio = __shfl_sync(FULL, ROW_PRIO(word), bl);
               if (pr != b_prio) list = pr < b_prio;
               else {
-                const int64_t x = __shfl_sync(FULL, list_base, fl), b_base = __shfl_sync(FULL, base, bl);
+                const int64_t x = LONG ? s_slot[__shfl_sync(FULL, i, fl)] : __shfl_sync(FULL, list_base, fl), b_base = __shfl_sync(FULL, base, bl);
                 list = x < b_base;
                 if (x == b_base) list = id_of(__shfl_sync(FULL, i, fl)) < id_of(wb + __shfl_sync(FULL, src, bl));
               }
@@ -743,8 +757,9 @@ __global__ void __launch_bounds__(32) k_sim(const HfxParams p, const SimArgs a, 
 }
 
 int hfx_sim_configure() {
-  if (cudaFuncSetAttribute(k_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * SIM_BYTES_PER_ROW + (int)SIM_LISTS_BYTES(HFX_MAX_CLASSES, SIM_SMEM_ROWS)) != cudaSuccess ||
-      cudaFuncSetAttribute(k_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SM_BYTES - SIM_BLOCK_BYTES) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_sim<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SMEM_ROWS * SIM_BYTES_PER_ROW + (int)(SIM_LIST_BYTES(HFX_MAX_CLASSES, SIM_SMEM_ROWS) + SIM_NOTES_BYTES(SIM_SMEM_ROWS))) != cudaSuccess ||
+      cudaFuncSetAttribute(k_sim<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SM_BYTES - SIM_BLOCK_BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(k_sim<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SIM_SM_BYTES - SIM_BLOCK_BYTES) != cudaSuccess)
     return HFX_E_CUDA;
   return HFX_OK;
 }
@@ -770,26 +785,31 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   a.iters_executed = o->iters_executed; a.finished = o->finished; a.rejected = o->rejected; a.attained = o->attained;
   a.ttft_p50 = o->ttft_p50_ns; a.ttft_p99 = o->ttft_p99_ns; a.tpot_p50 = o->tpot_p50_ns; a.tpot_p99 = o->tpot_p99_ns;
   a.now_out = o->now_ns;
-  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = SIM_LISTS_BYTES(s->p.n_classes, cap);
+  const size_t rows_bytes = (size_t)cap * SIM_BYTES_PER_ROW, list_bytes = SIM_LIST_BYTES(s->p.n_classes, cap), notes_bytes = SIM_NOTES_BYTES(cap);
   const size_t sm_bytes = SIM_SM_BYTES, block_bytes = SIM_BLOCK_BYTES;
   int rc = cuda_rc(cudaMemsetAsync(d_work_counter, 0, sizeof(uint32_t), s->stream));
   if (rc != HFX_OK) return rc;
-  int per_sm = cap <= SIM_SMEM_ROWS ? (int)(sm_bytes / (rows_bytes + list_bytes + block_bytes)) : 0;
+  int per_sm = cap <= SIM_SMEM_ROWS ? (int)(sm_bytes / (rows_bytes + list_bytes + notes_bytes + block_bytes)) : 0;
   if (per_sm > 32) per_sm = 32;
-  int per_sm_scratch = (int)(sm_bytes / (list_bytes + block_bytes));
-  if (per_sm_scratch > SIM_SCRATCH_PER_SM) per_sm_scratch = SIM_SCRATCH_PER_SM;
+  auto in_scratch = [&](size_t smem) { const int x = (int)(sm_bytes / (smem + block_bytes)); return x < SIM_SCRATCH_PER_SM ? x : SIM_SCRATCH_PER_SM; };
+  int per_sm_scratch = in_scratch(list_bytes + notes_bytes);
+  // LONG where it saves a round of traces: in the same number of rounds fewer at a time are the quicker ones (3000 traces of 5120 rows, two
+  // rounds of 12 or 16 an SM: 42.2 ms with classes and notes in shared memory, 45.7 without)
+  auto rounds = [&](int each) { return (n_traces + s->n_sm * each - 1) / (s->n_sm * each); };
+  const bool long_rows = rounds(in_scratch(list_bytes)) < rounds(per_sm_scratch);
+  if (long_rows) per_sm_scratch = in_scratch(list_bytes);
   // Rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would.  Traces of 2048 rows,
   // shared memory / scratch: 444 5.64 / 5.89 ms, 740 (five a SM) 5.90 / 6.45, 1036 (scratch) 6.7; 4096 of 512 rows 3.89 / 4.07, of 256 1.89 / 2.00.
   if (per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch)) {
     int grid = s->n_sm * per_sm;
     if (grid > n_traces) grid = n_traces;
     KernelScope ks(s, KSLOT_SIM);
-    k_sim<false><<<grid, 32, rows_bytes + list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
+    k_sim<false, false><<<grid, 32, rows_bytes + list_bytes + notes_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
   } else {
     // the rows of every resident block in a scratch buffer, allocated when first needed
     int grid = s->n_sm * per_sm_scratch;
     if (grid > n_traces) grid = n_traces;
-    const size_t need = rows_bytes * (size_t)grid;
+    const size_t need = (rows_bytes + (long_rows ? notes_bytes : 0)) * (size_t)grid;
     if (s->sim_scratch_bytes < need) {
       rc = cuda_rc(cudaStreamSynchronize(s->stream));
       if (rc != HFX_OK) return rc;
@@ -799,7 +819,8 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
       s->sim_scratch_bytes = need;
     }
     KernelScope ks(s, KSLOT_SIM);
-    k_sim<true><<<grid, 32, list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
+    if (long_rows) k_sim<true, true><<<grid, 32, list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
+    else k_sim<true, false><<<grid, 32, list_bytes + notes_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
   }
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;
 }

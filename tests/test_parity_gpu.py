@@ -302,6 +302,28 @@ def test_simulator_traces_beyond_shared_memory():
     assert_sim_parity(wl)
 
 
+@pytest.mark.parametrize("longest", [3760, 3776, 8192, 16_384, 56_000, 65_535])
+def test_simulator_more_traces_than_fit_beside_a_long_one(longest):
+    # The longest trace sets what a trace takes of shared memory.  With four classes sixteen of them fit an SM with list, classes and notes up to
+    # 3760 rows; beyond, in a batch of more traces than fit, classes and notes work in scratch too (not at 65,535: one trace an SM either way).
+    # Requests in flight beyond the registers and bunches that finish are in the long trace, the short ones are drawn.
+    rng = np.random.default_rng(longest)
+    n_short = 2400 if longest < 10_000 else 900
+    lens = np.concatenate([[longest], rng.integers(0, 6, n_short)])
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    wl = gen.random_traces(1, 1, int(off[-1]), int(off[-1]), iters=700, rate=500.0, out_hi=64, classes=gen.workloads.CLASSES_4)
+    wl.replicas = np.repeat(wl.replicas, len(lens), axis=0)
+    wl.trace_off = off
+    t = wl.table
+    t["replica_id"][:] = np.repeat(np.arange(len(lens), dtype=np.int32), lens)
+    arr = t["arrival_ns"].copy()
+    for j in np.nonzero(lens[1:])[0] + 1:
+        t["arrival_ns"][off[j]:off[j + 1]] -= arr[off[j]]      # (every trace starts at 0)
+    t["prompt_len"][:longest:2] = rng.integers(1, 9, t["prompt_len"][:longest:2].size)
+    wl.now, wl.maturity = np.zeros(len(lens), np.int64), np.zeros(len(lens), np.int64)
+    assert_sim_parity(wl, traces=[0] + list(range(1, len(lens), 40)) + [len(lens) - 1])
+
+
 def test_simulator_trace_length_limit():
     # rows of a trace are numbered with 16 bits inside the simulator: 65,536 rows are refused before anything is launched
     import paper_2508_15919_b200 as hfx

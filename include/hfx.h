@@ -404,11 +404,14 @@ int hfx_slo_map(hfx_sched *s, int32_t n_prio, const hfx_slo_window *win, const h
  * columns are overwritten) and runs `iters` iterations of step + commit, or
  * until nothing is left to happen.  Written: state, gen, first_token_ns,
  * last_token_ns, finish_ns and `out`.
- * A trace of up to 10240 rows is kept in shared memory when all traces of the call fit it together; longer traces (at
- * most 65535 rows) and larger batches work in a scratch buffer in device memory (13 bytes per row for at most sixteen
- * traces per SM), which the first call that needs it
- * allocates with cudaMalloc after synchronising the stream, so such a call should not be made inside a stream
- * capture; hfx_sched_destroy frees it.
+ * A trace of up to 10240 rows is kept in shared memory (19 bytes per row) when all traces of the call fit it together;
+ * longer traces (at most 65535 rows) and batches beyond that (with four classes on 148 SMs, more than 740 traces
+ * of 2048 rows) work in a scratch buffer in device memory (16 or 17 bytes per row for at most sixteen traces per
+ * SM), which the first call that needs it allocates with cudaMalloc after synchronising the stream, and which a
+ * call that needs more replaces (a graph captured before that must not be replayed); hfx_sched_destroy frees it.
+ * Inside a stream capture nothing is allocated: where no earlier call has left enough scratch, traces of up to
+ * 10240 rows stay in shared memory, fewer at a time, and longer ones are refused with HFX_E_CUDA; trace_off is
+ * read when the graph runs.
  * Errors: HFX_E_ARG, HFX_E_ALIGN, HFX_E_CAPACITY (n_traces > n_replicas, or a
  * trace longer than 65535 rows), HFX_E_NOMEM, HFX_E_CUDA. */
 int hfx_sim_run(hfx_sched *s, const hfx_table *table, const int32_t *trace_off,

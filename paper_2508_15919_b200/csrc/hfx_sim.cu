@@ -800,17 +800,18 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
   if (long_rows) per_sm_scratch = in_scratch(list_bytes);
   // Rows in shared memory (the shorter latency) while that keeps every trace resident, or as many as scratch would.  Traces of 2048 rows,
   // shared memory / scratch: 444 5.64 / 5.89 ms, 740 (five a SM) 5.90 / 6.45, 1036 (scratch) 6.7; 4096 of 512 rows 3.89 / 4.07, of 256 1.89 / 2.00.
-  if (per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch)) {
-    int grid = s->n_sm * per_sm;
-    if (grid > n_traces) grid = n_traces;
-    KernelScope ks(s, KSLOT_SIM);
-    k_sim<false, false><<<grid, 32, rows_bytes + list_bytes + notes_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
-  } else {
-    // the rows of every resident block in a scratch buffer, allocated when first needed
-    int grid = s->n_sm * per_sm_scratch;
-    if (grid > n_traces) grid = n_traces;
-    const size_t need = (rows_bytes + (long_rows ? notes_bytes : 0)) * (size_t)grid;
-    if (s->sim_scratch_bytes < need) {
+  bool in_smem = per_sm > 0 && (n_traces <= s->n_sm * per_sm || per_sm >= per_sm_scratch);
+  // otherwise the rows of every resident block in a scratch buffer, allocated when first needed
+  int grid = s->n_sm * per_sm_scratch;
+  if (grid > n_traces) grid = n_traces;
+  const size_t need = (rows_bytes + (long_rows ? notes_bytes : 0)) * (size_t)grid;
+  if (!in_smem && s->sim_scratch_bytes < need) {
+    // Inside a stream capture the stream cannot be waited for: traces that shared memory can hold stay there, fewer at a time.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    rc = cuda_rc(cudaStreamIsCapturing(s->stream, &capture));
+    if (rc != HFX_OK) return rc;
+    in_smem = capture != cudaStreamCaptureStatusNone && per_sm > 0;
+    if (!in_smem) {
       rc = cuda_rc(cudaStreamSynchronize(s->stream));
       if (rc != HFX_OK) return rc;
       cudaFree(s->d_sim_scratch);
@@ -818,8 +819,15 @@ int hfx_launch_sim_kernel(hfx_sched *s, const hfx_table *t, const int32_t *d_tra
       if (cudaMalloc(&s->d_sim_scratch, need) != cudaSuccess) { cudaGetLastError(); return HFX_E_NOMEM; }
       s->sim_scratch_bytes = need;
     }
+  }
+  if (in_smem) {
+    grid = s->n_sm * per_sm;
+    if (grid > n_traces) grid = n_traces;
+  }
+  {
     KernelScope ks(s, KSLOT_SIM);
-    if (long_rows) k_sim<true, true><<<grid, 32, list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
+    if (in_smem) k_sim<false, false><<<grid, 32, rows_bytes + list_bytes + notes_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, nullptr);
+    else if (long_rows) k_sim<true, true><<<grid, 32, list_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
     else k_sim<true, false><<<grid, 32, list_bytes + notes_bytes, s->stream>>>(s->p, a, d_work_counter, s->d_status, s->d_sim_scratch);
   }
   return cudaGetLastError() == cudaSuccess ? HFX_OK : HFX_E_CUDA;

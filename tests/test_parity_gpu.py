@@ -324,6 +324,51 @@ def test_simulator_more_traces_than_fit_beside_a_long_one(longest):
     assert_sim_parity(wl, traces=[0] + list(range(1, len(lens), 40)) + [len(lens) - 1])
 
 
+def test_simulator_first_call_inside_a_stream_capture():
+    # 741 traces, the longest of 2048 rows: one more than shared memory holds together, so their rows work in scratch, which the first call
+    # allocates.  Inside a capture it cannot, and the rows stay in shared memory; a trace that does not fit there is refused.
+    import paper_2508_15919_b200 as hfx
+    st = torch.cuda.Stream()
+    for longest, fits in ((2048, True), (10_241, False)):
+        rng = np.random.default_rng(longest)
+        lens = np.concatenate([[longest], rng.integers(0, 8, 740)])
+        off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        wl = gen.random_traces(2, 1, int(off[-1]), int(off[-1]), iters=300, rate=200.0, out_hi=64)
+        wl.replicas, wl.trace_off = np.repeat(wl.replicas, len(lens), axis=0), off
+        wl.now, wl.maturity = np.zeros(len(lens), np.int64), np.zeros(len(lens), np.int64)
+        with torch.cuda.stream(st):
+            sched = hfx.Scheduler(wl.model, wl.classes, wl.replicas, wl.n_rows, stream=st)
+            tab, out = hfx.DeviceTable.from_numpy(wl.table), hfx.SimOut(len(lens))
+            torch.cuda.synchronize()
+            if not fits:
+                refused = RefusedLaunches(st)
+                assert refused.rt.cudaStreamBeginCapture(refused.st, 2) == 0
+                with pytest.raises(hfx.HfxError) as e:
+                    sched.sim_run(tab, off, wl.sim_iters, out)
+                assert e.value.code == -4
+                refused.__exit__()
+                sched.close()
+                continue
+            graph = torch.cuda.CUDAGraph()
+            graph.capture_begin(capture_error_mode="thread_local")
+            sched.sim_run(tab, off, wl.sim_iters, out)
+            graph.capture_end()
+            for _ in range(2):
+                graph.replay()
+                assert sched.status() == 0
+                g, cols = out.to_numpy(), tab.to_numpy()
+                cpu = wl.copy()
+                c = oracle.sim(cpu)
+                for ko, kg in (("iters_executed", "iters_executed"), ("finished", "finished"), ("ttft_p99", "ttft_p99_ns"), ("tpot_p50", "tpot_p50_ns"), ("now", "now_ns")):
+                    assert np.array_equal(g[kg], c[ko]), kg
+                for k in STATE_COLS:
+                    assert np.array_equal(cols[k], cpu.table[k]), k
+            sched.sim_run(tab, off, wl.sim_iters, out)      # outside: scratch
+            assert sched.status() == 0 and np.array_equal(out.to_numpy()["ttft_p99_ns"], c["ttft_p99"])
+            del graph
+            sched.close()
+
+
 def test_simulator_trace_length_limit():
     # rows of a trace are numbered with 16 bits inside the simulator: 65,536 rows are refused before anything is launched
     import paper_2508_15919_b200 as hfx

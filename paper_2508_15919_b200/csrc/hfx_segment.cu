@@ -708,15 +708,13 @@ __device__ void small_replica(const HfxParams &p, const SegArgs &a, const SegCtx
       G.sync();
 #pragma unroll 1
       for (int e = G.tid; e < n_act; e += GROUP_THREADS) {
-        {
-          const uint64_t x = s_bk[e];
-          const uint32_t bi = bin_of(x), sh16 = (bi & 1u) * 16;
-          const uint32_t g0 = (s_bin[bi >> 1] >> sh16) & 0xffffu, g1 = (s_cur[bi >> 1] >> sh16) & 0xffffu;
-          uint32_t rank = 0;
-          for (uint32_t g = g0; g < g1; g++) rank += s_bk[g] < x ? 1u : 0u;
-          if (!ordered) rank += rank_by_id(s_bk, s_row, a.req_id, x, g0, g1);
-          s_lo[g0 + rank] = (uint32_t)(x & 0xffffu);      // (the class ranges that s_lo overlays were last read when the bins were laid out)
-        }
+        const uint64_t x = s_bk[e];
+        const uint32_t bi = bin_of(x), sh16 = (bi & 1u) * 16;
+        const uint32_t g0 = (s_bin[bi >> 1] >> sh16) & 0xffffu, g1 = (s_cur[bi >> 1] >> sh16) & 0xffffu;
+        uint32_t rank = 0;
+        for (uint32_t g = g0; g < g1; g++) rank += s_bk[g] < x ? 1u : 0u;
+        if (!ordered) rank += rank_by_id(s_bk, s_row, a.req_id, x, g0, g1);
+        s_lo[g0 + rank] = (uint32_t)(x & 0xffffu);      // (the class ranges that s_lo overlays were last read when the bins were laid out)
       }
     } else {
 #pragma unroll

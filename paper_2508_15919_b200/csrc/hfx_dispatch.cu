@@ -922,6 +922,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_disp_chain(const HfxParams p,
     __syncthreads();
     const int k_now = s_k;
     const int64_t cursor = s_cursor;
+    __syncthreads();      // (the walking warp writes the next ones while the others are at work: everyone has read these)
     if (k_now >= nm || cursor >= nq) break;
     if (cursor / CHAIN_CHUNK != c) {      // not the chunk that was staged ahead (a long run)
       if (before >= 0) { look_up(before, k_found, k_now, tid, CHAIN_THREADS); k_found = k_now; before = -1; }

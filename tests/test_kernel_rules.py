@@ -40,6 +40,14 @@ def test_simulator_orders_reading_a_finished_slot_before_an_admission_writes_it(
     assert "__syncwarp();" in between[loop_end:between.index("for (int s0 = 0; s0 < n_list")]
 
 
+def test_dispatch_walk_reads_the_cursor_before_the_walking_warp_moves_it():
+    # the first warp walks while the others look up and stage; what it writes for the next round must not reach a warp that is late with reading
+    src = _source("hfx_dispatch.cu")
+    body = _between(src, "for (;;) {\n    __syncthreads();\n    const int k_now = s_k;", "s_cursor = jumped;")
+    read = body.index("cursor = s_cursor;")
+    assert read < body.index("__syncthreads();", read) < body.index("break;", read)      # (every thread passes it)
+
+
 def _functions(src, word):
     """(header, body) of every function definition that is introduced by `word`."""
     out = []

@@ -574,9 +574,9 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     for (int e = 0; e < PER; e++) { s_start[tid * PER + e] = run; run += c[e]; }
     if (tid == 0) s_start[DISP_BINS] = all;
     big = __reduce_max_sync(0xffffffffu, big);
-    if (lane == 0) s_part[warp] = big;
+    if (lane == 0) s_digit[warp] = big;      // (not s_part, which the warp's lanes have just read)
     __syncthreads();
-    fullest = __reduce_max_sync(0xffffffffu, s_part[lane]);
+    fullest = __reduce_max_sync(0xffffffffu, s_digit[lane]);
     __syncthreads();
   }
   const bool binned = !small && fullest <= DISP_BIN_MAX;

@@ -48,6 +48,17 @@ def test_dispatch_walk_reads_the_cursor_before_the_walking_warp_moves_it():
     assert read < body.index("__syncthreads();", read) < body.index("break;", read)      # (every thread passes it)
 
 
+def test_block_prefix_keeps_its_words_until_the_next_barrier():
+    # what block_prefix returns is read from its shared array by every lane; one lane of the warp must not write there before a barrier
+    src = _source("hfx_dispatch.cu")
+    for m in re.finditer(r"block_prefix2?(?:<\w+>)?\([^;]*\b(s_part(?:64)?)\b[^;]*;", src):
+        if m.group().startswith("block_prefix2(int64_t &x"):
+            continue
+        behind = src[m.end():]
+        behind = behind[:min(behind.index("__syncthreads();"), behind.index("block_prefix") if "block_prefix" in behind else len(behind))]
+        assert not re.search(m.group(1) + r"\[[^\]]*\] =[^=]", behind), behind
+
+
 def _functions(src, word):
     """(header, body) of every function definition that is introduced by `word`."""
     out = []

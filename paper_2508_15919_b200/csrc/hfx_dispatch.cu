@@ -34,6 +34,10 @@
 #define DISP_TILE_MIN 512
 #define DISP_BIN_MAX (DISP_TILE_MAX - DISP_TILE_MIN)      // fuller bins send the queue to the radix sort
 #define DISP_FINE 4096              // bins of a tile
+// Items of a fine bin that are compared all with all; a fuller one (slacks crowded beside a gap, equal ones whose ids share their leading bits) goes
+// through a sorting network of the block.  40,960 rows, so many of them within 2 ns, compared / network: 200 67.0 / 61.8 us, 1000 205 / 72, 3000 857 /
+// 117, 4500 1884 / 162.  Many bins of a hundred (100,000 equal slacks, ids of 256 front ends): 66.8 us, with the line at 64 items 137.
+#define DISP_FINE_MAX 128
 #define DISP_TILES_CHAIN 1024       // tiles whose totals the chain adds up itself; beyond them they are added to the running totals
 #define SORT_SMEM (DISP_TILE_MAX * 22 + (DISP_FINE + 4) * 4 + (DISP_BINS + 4) * 4 + DISP_SPLITS * 16)
 #define VAL_FITS 0x80000000u        // on an ordered row: some instance's budget reaches it (the others are passed over)
@@ -344,6 +348,77 @@ __device__ __forceinline__ void block_prefix2(int64_t &x, uint32_t &c, int64_t *
   c = s_part[warp] + u - c;
 }
 
+// Puts the items idx[0 .. n) of a tile in order, all threads of the block: a bitonic network with ascending comparators (mirrored first
+// sub-stage), so that places behind n need not exist.  What bounds it is the items' scattered places in shared memory: what lies within 32
+// places is exchanged in registers, two wider sub-stages at a time by a thread with four places.
+struct TileEntry { uint64_t key; uint32_t tie; uint16_t at; };
+__device__ __noinline__ void tile_network(uint16_t *idx, int n, const uint4 *s_item, bool by_id) {
+  const int lane = threadIdx.x & 31;
+  auto load = [&](int i) -> TileEntry {
+    TileEntry e = {~0ull, ~0u, 0};
+    if (i < n) { e.at = idx[i]; const uint4 x = s_item[e.at]; e.key = item_key(x); e.tie = by_id ? x.z : x.w; }
+    return e;
+  };
+  auto less = [](const TileEntry &x, const TileEntry &y) { return x.key < y.key || (x.key == y.key && x.tie < y.tie); };
+  auto exchange = [&](TileEntry &x, TileEntry &y) { if (less(y, x)) { const TileEntry z = x; x = y; y = z; } };
+  auto within_warps = [&](bool all) {      // merges of up to 32, or the last five sub-stages of a wider one
+    for (int i = threadIdx.x; (i & ~31) < n; i += blockDim.x) {
+      TileEntry e = load(i);
+      auto exchange_lanes = [&](int mask) {
+        TileEntry o;
+        o.key = __shfl_xor_sync(0xffffffffu, e.key, mask); o.tie = __shfl_xor_sync(0xffffffffu, e.tie, mask);
+        o.at = (uint16_t)__shfl_xor_sync(0xffffffffu, (uint32_t)e.at, mask);
+        if (lane < (lane ^ mask) ? less(o, e) : less(e, o)) e = o;
+      };
+      for (int k = all ? 2 : 32; k <= 32; k <<= 1) {
+        if (all) exchange_lanes(k - 1);
+        for (int h = all ? k >> 2 : k >> 1; h > 0; h >>= 1) exchange_lanes(h);
+      }
+      if (i < n) idx[i] = e.at;
+    }
+    __syncthreads();
+  };
+  int n_pad = 32;
+  while (n_pad < n) n_pad <<= 1;
+  within_warps(true);
+  for (int k = 64; k <= n_pad; k <<= 1) {
+    const int hk = k >> 1;
+    for (int t = threadIdx.x; t < n_pad >> 1; t += blockDim.x) {
+      const int off = t & (hk - 1), i = 2 * (t - off) + off, j = i + k - 1 - 2 * off;
+      if (j < n) {
+        const TileEntry x = load(i), y = load(j);
+        if (less(y, x)) { idx[i] = y.at; idx[j] = x.at; }
+      }
+    }
+    __syncthreads();
+    int h = k >> 2;
+    for (; h > 32; h >>= 2) {
+      const int q = h >> 1;
+      for (int t = threadIdx.x; t < n_pad >> 2; t += blockDim.x) {
+        const int off = t & (q - 1), i = 4 * (t - off) + off;
+        if (i + q >= n) continue;      // (one place at most)
+        TileEntry e0 = load(i), e1 = load(i + q), e2 = load(i + h), e3 = load(i + h + q);
+        exchange(e0, e2); exchange(e1, e3); exchange(e0, e1); exchange(e2, e3);
+        idx[i] = e0.at; idx[i + q] = e1.at;
+        if (i + h < n) idx[i + h] = e2.at;
+        if (i + h + q < n) idx[i + h + q] = e3.at;
+      }
+      __syncthreads();
+    }
+    if (h == 32) {
+      for (int t = threadIdx.x; t < n_pad >> 1; t += blockDim.x) {
+        const int i = 2 * t - (t & 31);
+        if (i + 32 < n) {
+          const TileEntry x = load(i), y = load(i + 32);
+          if (less(y, x)) { idx[i] = y.at; idx[i + 32] = x.at; }
+        }
+      }
+      __syncthreads();
+    }
+    within_warps(false);
+  }
+}
+
 #define ITEMS_AT_ONCE 4      // items a thread has in flight in the passes over the queue
 
 static_assert(DISP_BINS % SORT_THREADS == 0 && DISP_BINS >= DISP_SPLITS * DISP_SUB && DISP_FINE <= 8192, "bins");
@@ -366,6 +441,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
   __shared__ int64_t s_part64[33];
   __shared__ unsigned long long s_bmax[2];
   __shared__ uint32_t s_nm[2], s_n1, s_ok, s_digit[256];
+  __shared__ uint32_t s_n_full, s_full[DISP_TILE_MAX / DISP_FINE_MAX];      // fine bins beyond DISP_FINE_MAX
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, R = p.n_replicas;
   uint32_t round = 0;
   cudaTriggerProgrammaticLaunchCompletion();
@@ -673,6 +749,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
       const int lg = nb <= DISP_FINE ? 31 - __clz(DISP_FINE / (nb > 1 ? nb : 1u)) : 0, down = nb <= DISP_FINE ? 0 : 32 - __clz((nb - 1) / DISP_FINE);      // (a tile of many empty bins: several to a fine one)
       uint32_t fp[IPT];      // fine bin << 16 | place in it (by arrival)
       for (uint32_t i = tid; i < DISP_FINE; i += SORT_THREADS) s_fine[i] = 0;
+      if (tid == 0) s_n_full = 0;
       __syncthreads();
 #pragma unroll
       for (int e = 0; e < IPT; e++) {
@@ -691,7 +768,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
         constexpr int FPT = DISP_FINE / SORT_THREADS;
         uint32_t c[FPT], sum = 0, all;
 #pragma unroll
-        for (int e = 0; e < FPT; e++) { c[e] = s_fine[tid * FPT + e]; sum += c[e]; }
+        for (int e = 0; e < FPT; e++) { c[e] = s_fine[tid * FPT + e]; sum += c[e]; if (c[e] > DISP_FINE_MAX) s_full[atomicAdd(&s_n_full, 1u)] = tid * FPT + e; }
         uint32_t run = block_prefix<uint32_t>(sum, s_part, &all);
 #pragma unroll
         for (int e = 0; e < FPT; e++) { s_fine[tid * FPT + e] = run; run += c[e]; }
@@ -709,6 +786,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
           const uint32_t g0 = s_fine[fp[e] >> 16], g1 = s_fine[(fp[e] >> 16) + 1], tie = tie_of(x);
           const uint64_t key = item_key(x);
           uint32_t place = g0;
+          if (g1 > g0 + DISP_FINE_MAX) continue;
           if (g1 > g0 + 1)
             for (uint32_t k = g0; k < g1; k++) {
               const uint4 y = s_item[s_ord[k]];
@@ -717,6 +795,11 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
             }
           s_row[place] = x.w;
         }
+      }
+      for (uint32_t k = 0; k < s_n_full; k++) {
+        const uint32_t g0 = s_fine[s_full[k]], g1 = s_fine[s_full[k] + 1];
+        tile_network(s_ord + g0, (int)(g1 - g0), s_item, by_id);
+        for (uint32_t i = g0 + tid; i < g1; i += SORT_THREADS) s_row[i] = s_item[s_ord[i]].w;
       }
     } else
       for (uint32_t i = tid; i < n; i += SORT_THREADS) s_row[i] = small ? __ldcg(w.rank + e0 + i) : __ldcg(ordered + e0 + i).w;

@@ -1355,23 +1355,52 @@ def test_dispatch_walk_of_many_instances(R, n, shape):
     assert_dispatch_parity(wl, now, calls=2)
 
 
-@pytest.mark.parametrize("clump", [1000, 1030, 2500, 4090, 4200, 9000])
-def test_dispatch_bins_of_every_fullness(clump):
-    # Rows whose slacks lie closer together than a bin of the order is wide, beside others far off: fuller bins make lower tiles, and beyond
-    # what a tile holds the queue is ordered by radix passes.  (ids permuted: ties too)
-    n = 40_000
-    rng = np.random.default_rng(clump)
-    wl = gen.random_table(clump, n, 7, modes=(gen.COLOCATED,), n_classes=3, token_cap=16384, inflight=0.02, done=0.0, future=0.0)
+def _dispatch_bins(v):
+    """Rows per bin of a dispatch whose queue is `v`, one priority's places (slack << 16 | leading tie bits) by row: every 64th row is sampled (warps of
+    128 queued rows leave their items in row order), every fourth sample starts an interval, which is divided into eight.  Inner intervals only."""
+    s = np.sort(v[::64])
+    lo, hi = s[:-1:4], s[np.minimum(np.arange(0, s.size - 1, 4) + 4, s.size - 1)]
+    v = v[(v >= s[0]) & (v < s[-1])]
+    k = np.searchsorted(lo, v, "right") - 1
+    return lo, hi, np.bincount(k * 8 + (v - lo[k]) * 8 // (hi[k] - lo[k] + 1), minlength=8 * lo.size)
+
+
+@pytest.mark.parametrize("close", [True, False])
+@pytest.mark.parametrize("fullest", [128, 129, 1000, 1024, 1025, 3001, 4608, 4609, 9000])
+def test_dispatch_bins_of_every_fullness(fullest, close):
+    # A bin of the order with so many rows.  Closer together than a fine bin is wide they are compared all with all (up to 128) or go through
+    # a sorting network, otherwise they spread over fine bins; beyond 1024 the tiles are lower, beyond 4608 the queue is ordered by radix
+    # passes.  The bin is between samples of rows far apart, which its own rows are not among.
+    n = 40_960
+    rng = np.random.default_rng(fullest)
+    permuted = fullest % 2 == 1
+    wl = gen.random_table(fullest, n, 7, modes=(gen.COLOCATED,), n_classes=3, token_cap=16384, inflight=0.0, done=0.0, future=0.0, permute_ids=permuted)
     now = int(wl.now.max())
     t = wl.table
     t["prompt_len"][:] = 16
     t["class_id"][:] = 0
-    t["arrival_ns"][:] = now - rng.integers(0, 40 * SEC, n)
-    c = rng.permutation(n)[:clump]
-    t["arrival_ns"][c] = now - 41 * SEC - rng.integers(0, 2, clump)
-    late = rng.permutation(n)[:30]
-    t["arrival_ns"][late] = now - 500 * SEC - rng.integers(0, SEC, 30)
-    assert_dispatch_parity(wl, now)
+    t["state"][:] = gen.QUEUED
+    spread = 1 + rng.integers(0, 40 * SEC, n)
+    tie = t["req_id"].astype(np.int64) - int(t["req_id"].min()) if permuted else np.arange(n)
+    tie >>= max(0, int(tie.max()).bit_length() - 16)
+    place = lambda age: ((50 * SEC - age) << 16) | tie      # (up to a constant)
+    lo, hi, _ = _dispatch_bins(place(spread))
+    k = int(np.argmax(hi - lo))                             # the widest interval: the rows go to the middle of its fourth bin
+    at, wide = int(50 * SEC - (int(lo[k]) + (int(hi[k]) - int(lo[k])) * 7 // 16 >> 16)), int(hi[k] - lo[k] >> 16) // 8
+    free = np.arange(n) % 64 != 0
+    v = place(spread)
+    others = free & (v >= lo[k]) & (v < hi[k])
+    spread[others] = 41 * SEC + rng.integers(0, SEC, int(others.sum()))      # (behind the last sample)
+    pick = rng.permutation(np.nonzero(free)[0])
+    size = fullest
+    for _ in range(3):
+        age = spread.copy()
+        age[pick[:size]] = at + rng.integers(0, 2, size) if close else at - wide // 4 + np.arange(size) * (wide // 2) // size
+        full = int(_dispatch_bins(place(age))[2].max())
+        size += fullest - full
+    assert full == fullest
+    t["arrival_ns"][:] = now - age
+    assert_dispatch_parity(wl, now, calls=2)
 
 
 @pytest.mark.parametrize("equal", [False, True])

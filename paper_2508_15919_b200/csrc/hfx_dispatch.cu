@@ -1251,9 +1251,11 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   const int blocks = scan_blocks(s, n);
   const int threads = scan_threads(s, n);
   a.rounds = (int32_t)((n / 4 + (int64_t)threads * blocks - 1) / ((int64_t)threads * blocks));
-  // blocks of the cooperative kernel: tiles of 512 entries, or a warp per entry of a small queue (60,013 rows: 30 blocks and tiles of 1024 entries 66.7 us,
-  // 59 63.6, 118 and tiles of 512 61.6; a barrier takes 1.5 us with 30 and with 148 blocks)
-  int64_t want = n <= 2 * DISP_SMALL ? (n + 31) / 32 : (n + 511) / 512, want_r = (R + 31) / 32;
+  // blocks of the cooperative kernel: a warp per entry of a small queue, which a larger table may hold too, and tiles of 512 entries (60,013 rows: 30
+  // blocks and tiles of 1024 entries 66.7 us, 59 63.6, 118 and tiles of 512 61.6; a barrier takes 1.5 us with 30 and with 148 blocks).  4090 entries
+  // queued, 8300 rows 17 blocks 83.2 us, 128 42.3, 20,000 rows 40 blocks 54.6, 128 42.4; most of 16,000 queued 32 blocks 53.2, 128 53.3
+  int64_t want = (n < DISP_SMALL ? n + 31 : DISP_SMALL) / 32, want_r = (R + 31) / 32;
+  if (want < (n + 511) / 512) want = (n + 511) / 512;
   if (want < want_r) want = want_r;
   const int grid = (int)(want < 1 ? 1 : (want < s->n_sm ? want : s->n_sm));
   cudaLaunchAttribute attr[1];

@@ -1425,6 +1425,19 @@ def test_dispatch_small_queues(n, equal):
     assert_dispatch_parity(wl, now, calls=2)
 
 
+@pytest.mark.parametrize("n,queued", [(8193, 4096), (8193, 4097), (30_000, 4096), (70_000, 4097), (200_000, 1)])
+def test_dispatch_small_queues_in_larger_tables(n, queued):
+    # the queue decides how it is ordered, the table's size how many blocks there are: a warp per entry, or fewer
+    rng = np.random.default_rng(n + queued)
+    wl = gen.random_table(n, n, 9, modes=(gen.COLOCATED,), n_classes=3, token_cap=16384, inflight=0.0, done=0.0, future=0.0)
+    t = wl.table
+    t["prompt_len"][:] = np.minimum(t["prompt_len"], 16000)
+    t["state"][:] = gen.DONE
+    t["state"][rng.permutation(n)[:queued]] = gen.QUEUED
+    g = assert_dispatch_parity(wl, int(wl.now.max()), calls=2)
+    assert g["n_queue"][0] == queued
+
+
 @pytest.mark.parametrize("n", [151_548, 151_552, 151_553, 151_557])
 def test_dispatch_scan_in_small_and_in_large_blocks(n):
     # up to 1024 rows an SM (148 of them) the scan takes blocks of 256 threads

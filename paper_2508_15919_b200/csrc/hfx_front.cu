@@ -457,13 +457,14 @@ int hfx_launch_front(hfx_sched *s, const FrontArgs &fa0) {
   fa.tot = s->d_tot + (size_t)par * (R1 + 1); fa.tot_next = s->d_tot + (size_t)(par ^ 1u) * (R1 + 1);
   fa.ordered = s->d_flags + 4 + par; fa.ordered_next = s->d_flags + 4 + (par ^ 1u);
   fa.status = s->d_status; fa.rowflag = s->d_rowflag;
-  // Ranks by warp up to 511 replicas, where the counters fit beside the tile (some 390 replicas at 7000 rows).  More replicas mean small groups,
-  // which are cheap to put in order by counting.  One step, by warp / by counting: 1 M rows over 128 replicas 78.3 / 85.2 us, 256 97.0 / 100.8,
-  // 390 109.1 / 111.5; 150,000 over 64 37.9 / 38.2; 600,000 over 512 97.4 / 97.5, 900 45.2 / 44.5; 300,000 over 600 33.6 / 33.5, 1000 34.5 / 33.9, 1024 37.8
-  // / 36.0; 150,000 over 700 27.3 / 26.9, 1024 32.8 / 31.2.
+  // Ranks by warp wherever the counters fit beside the tile (some 390 replicas at 7000 rows) and a thread adds up those of one replica: they take the
+  // same time however the rows are spread, while counting takes a row its group's size and a group of more than FRONT_GROUP_MAX a network.  One step, by warp /
+  // by counting, us.  Evenly spread rows: 1 M over 128 replicas 78.3 / 85.2, 390 109.1 / 111.5, 300,000 over 520 35.3 / 33.5, 800 35.4 / 35.3, 1000 37.4 /
+  // 36.1, 1024 (two replicas to a thread) 37.8 / 36.0.  300,000 over 1000, 30 % of them finished ones of one replica 36.2 / 43.5, 70 % 36.0 / 53.9, all on
+  // eight replicas 57.9 / 64.3; 450,000 over 600, 70 % 34.3 / 66.0.
   size_t smem = front_smem_bytes(R1, fa.tile_rows);
   const size_t wcnt = (size_t)2 * R1 * (FRONT_WCNT_PITCH + 2 * FRONT_WPRE_PITCH);
-  fa.by_warp = fa.tile_rows <= FRONT_WCNT_ROWS && R1 <= FRONT_THREADS / 2 && smem + wcnt <= HFX_FRONT_SMEM;
+  fa.by_warp = fa.tile_rows <= FRONT_WCNT_ROWS && R1 <= FRONT_THREADS && smem + wcnt <= HFX_FRONT_SMEM;
   if (fa.by_warp) smem += wcnt;
   KernelScope ks(s, KSLOT_FRONT);
   cudaLaunchConfig_t cfg;

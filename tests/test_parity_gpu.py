@@ -1329,6 +1329,22 @@ def test_simulator_budget_over_the_model_range(model, first_fit):
     assert_sim_parity(wl)
 
 
+@pytest.mark.parametrize("R", [511, 512, 1000, 1023, 1024])
+@pytest.mark.parametrize("n,share", [(60_000, 0.5), (240_000, 0.75)])
+def test_step_with_most_rows_on_one_of_many_replicas(R, n, share):
+    # the front end ranks a tile's rows by warp up to 1023 replicas, by counting whole groups beyond, and by a network where a group of the tile
+    # has more than 1024 rows (0.75 of 1632): finished rows of one replica, then all on eight
+    wl = gen.random_table(R, n, R, modes=(gen.COLOCATED, gen.PREFILL, gen.DECODE), inflight=0.05, done=0.5, future=0.1)
+    rng = np.random.default_rng(R)
+    hot = rng.random(n) < share
+    wl.table["replica_id"][hot] = 7
+    wl.table["state"][hot] = gen.DONE
+    assert_step_parity(wl, steps=2, commit=True)
+    if n < 100_000:
+        wl.table["replica_id"][:] = rng.integers(0, 8, n)
+        assert_step_parity(wl, steps=2, commit=True)
+
+
 @pytest.mark.parametrize("shape", ["even", "rare giants", "blocked", "zeros", "d stage", "capped"])
 @pytest.mark.parametrize("R,n", [(95, 3000), (96, 3000), (97, 40_001), (129, 9000), (1024, 70_000), (1061, 30_011), (2200, 90_000)])
 def test_dispatch_walk_of_many_instances(R, n, shape):

@@ -668,7 +668,10 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     if (!grid_barrier(w.ctl, a.status, w.wait_limit, round, &s_ok)) return;
   } else if (!small) {
     // radix sort, 8 bits a pass: the tie word, then the key (47 bits).  A block counts the digits of its share, adds up the
-    // counts of the blocks before it, and places its items 1024 at a time in order.
+    // counts of the blocks before it, and places its items 1024 at a time in order.  Blocks of 2048 items at least, the others only keep step:
+    // every block adds up the counts of all (us, all blocks of the grid / so: 40,960 entries 207 / 162, 65,536 218 / 177, 131,072 242 / 211).
+    const uint32_t want = (n_all + 2047) / 2048, blocks = want < gridDim.x ? want : gridDim.x, share = (n_all + blocks - 1) / blocks;
+    const uint32_t lo = blockIdx.x * share < n_all ? blockIdx.x * share : n_all, hi = lo + share < n_all ? lo + share : n_all;
     for (int pass = 0; pass < 10; pass++) {
       const uint4 *src = w.item[(pass & 1) ^ 1];
       uint4 *dst = w.item[pass & 1];
@@ -683,7 +686,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
         uint32_t before = 0, total = 0;
         if (tid < 256)
 #pragma unroll 4
-          for (int b = 0; b < (int)gridDim.x; b++) { const uint32_t c = __ldcg(w.hist + b * 256 + tid); total += c; if (b < (int)blockIdx.x) before += c; }
+          for (int b = 0; b < (int)blocks; b++) { const uint32_t c = __ldcg(w.hist + b * 256 + tid); total += c; if (b < (int)blockIdx.x) before += c; }
         uint32_t all;
         const uint32_t start = block_prefix<uint32_t>(total, s_part, &all);
         if (tid < 256) s_digit[tid] = start + before;

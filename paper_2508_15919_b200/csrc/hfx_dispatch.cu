@@ -97,7 +97,7 @@ __device__ __forceinline__ int64_t disp_cost(const HfxParams &p, const DispArgs 
 
 // ------------------------------------------------------------------------------------------------
 // k_disp_scan.  Bound by the columns it reads and the three outputs it initialises (54 bytes a row).  Four rows per
-// thread with 16-byte loads; a block reserves room for the items of its 4096 rows with one global atomic (their order
+// thread with 16-byte loads; a block reserves room for the items of a round of rows with one global atomic (their order
 // does not matter: the tie word settles it).
 // ------------------------------------------------------------------------------------------------
 template <int threads>
@@ -256,18 +256,18 @@ __global__ void __launch_bounds__(threads, 1) k_disp_scan(const HfxParams p, con
 // nothing: the queue, its running totals and the tiles may be unwritten).
 //   0  plan of every instance and its place in the maturity order, a warp per instance; the sample in order, a warp
 //      per sampled item counting the smaller ones.  Of a queue of up to DISP_SMALL entries all are sampled, and phases 1 and 2 fall away
-//      (300 rows 52 us without, 34 now, 2000 rows 56 and 37, 6000 rows 60 and 56 before the tiles got smaller)
+//      (with bins / so: 300 rows over 2 instances 45.6 / 33.3 us, 2000 over 8 47.6 / 35.3, 8000 over 16, half of them queued, 51.7 / 43.0)
 //   1  every item's bin, and its place in it from a global counter.  Every fourth sample of a (stage, priority) starts an
 //      interval, an interval is divided evenly into eight bins by slack and tie (so equal slacks spread by tie).  1 M rows over 1024 instances, 60,013
-//      rows: every eighth and sixteen 206, 69 us, every fourth and eight 203, 67, every second and eight 213, 72 (each block adds up all bins)
+//      and 150,000 rows: every eighth and sixteen 210, 62, 68 us, every fourth and eight 205, 59, 64, every second and eight 221, 63, 68 (each block
+//      adds up all bins)
 //   2  items to their bins; a fuller bin makes the tiles lower, one of more than DISP_BIN_MAX items (slacks crowded closer than the sample
 //      sees) sends the whole queue to a radix sort instead, 22 us a pass at 500 K entries.  (With the line at 1024 items the gaps between the classes of one
-//      priority did that: 500,001 rows with weights 324 us, 126 now)
+//      priority do that: 500,001 rows with weights 324 us, 126 so)
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
-//      its fine bin by counting; rows out in order, running totals
+//      its fine bin by counting, in a full one by a sorting network; rows out in order, running totals
 // An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 58 us by the GPU's clock:
-// sample and plans 8, splitters 5, bins 14, their starts 3, moving 4, tiles 10.5, running totals 8.5, barriers 1.5 each; one of 42 K in 118 blocks 30.
-// (65 and 36 with phase 0 on the warps of the first blocks instead of some of every block, and the tiles' edges found by every thread for itself)
+// sample and plans 8, splitters 5, bins 14, their starts 3, moving 4, tiles 10.5, running totals 8.5, three barriers of 1.5; one of 42 K in 118 blocks 30.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
@@ -745,9 +745,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
     constexpr int IPT = (DISP_TILE_MAX + SORT_THREADS - 1) / SORT_THREADS;
     if (binned) {
       // fine bins: an even share of them for every bin of the tile, in the bin by how far into it an item lies
-      // (the last tile ends with the last bin that holds anything: with the empty bins behind it, half of them all, its items shared so few fine bins
-      // that the block counted up to 435 of them with one another while the rest of the grid had finished: dispatch of 1 M rows over 1024 instances
-      // 255 us then, 206 with this edge, of 60,013 rows 78 and 69)
+      // (the last tile ends with the last bin that holds anything: the empty bins behind it, half of them all, would leave its items few fine bins,
+      // and the grid waits for its block)
       const uint32_t nb = b1 - b0;
       const int lg = nb <= DISP_FINE ? 31 - __clz(DISP_FINE / (nb > 1 ? nb : 1u)) : 0, down = nb <= DISP_FINE ? 0 : 32 - __clz((nb - 1) / DISP_FINE);      // (a tile of many empty bins: several to a fine one)
       uint32_t fp[IPT];      // fine bin << 16 | place in it (by arrival)
@@ -855,11 +854,11 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) k_disp_sort(const HfxParams p
 // executes has to come from its first instruction cache, unrolled it took three times as long); then it is looked at whether
 // the last of them reached the end of the window: what is in front of the first that did stands, that one is tried again from a fresh
 // window or, if it started this one, searched for (32 ways).  A batch is as long as the windows before allowed, or four instances longer: runs
-// are of three entries or of a hundred, and a third of the instances takes nothing where one prompt keeps them all waiting (six instances
-// always / eight / sixteen / so: 4096 instances 510 / 465 / 407 / 392 us a call, 700 156 / 145 / 135 / 132, 1024 with 40 entries a run 203 / 199 / 223 / 199).
+// are of three entries or of a hundred, and a third of the instances takes nothing where one prompt keeps them all waiting (eight instances
+// always / sixteen / so, 1 M rows: 700 instances 162 / 162 / 153 us a call, 1024 205 / 240 / 205, 4096 633 / 842 / 620).
 // The other warps meanwhile stage the next chunk of totals in shared memory and look up where the runs of the chunk before ended (the entries up to
-// a base are those within it).  Then all threads: what every instance took, dispatching step 4 (its new maturity time).  1024 instances, 471 K entries of which
-// 22 K are taken: 272 us when the totals were probed in shared memory, 104 now (90 of them the walk), with 512 threads 109.
+// a base are those within it).  Then all threads: what every instance took, dispatching step 4 (its new maturity time).  1024 instances, 472 K entries of which
+// 22 K are taken: 107 us by the GPU's clock, 98 of them the walk.
 // ------------------------------------------------------------------------------------------------
 // longest m in [lo, hi] with fits(m), given fits(lo) and fits monotone; whole warp
 template <typename F>
@@ -1169,8 +1168,8 @@ struct hfx_dispatch_ws { DispWork w; unsigned char *mem; size_t zero; unsigned l
 
 static size_t chain_smem(int R) { return (size_t)(CHAIN_CHUNK + CHAIN_WIN + 8) * 16 + (size_t)DISP_TILES_CHAIN * 16 + 16 + ((size_t)R + CHAIN_BATCH + 1) * 16; }
 static size_t scan_smem(int R) { return R <= SCAN_SMEM_REPLICAS ? (size_t)R * 24 : 0; }
-// threads of a block of the scan of n rows, and blocks: small blocks while an SM has one at most (60,013 rows 68.9 us in 15 blocks of 1024 threads,
-// whose rows in flight meet in a few instances' counters, 66.7 in 59 of 256)
+// threads of a block of the scan of n rows, and blocks: small blocks while an SM has one at most (always 1024 threads, whose rows in flight meet in a few
+// instances' counters / so: 20,000 rows 53.8 / 51.7 us, 60,013 61.2 / 59.3, 150,000 66.1 / 64.0)
 static int scan_threads(const hfx_sched *s, int64_t n) { return n <= (int64_t)s->n_sm * 4 * SCAN_THREADS_FEW ? SCAN_THREADS_FEW : SCAN_THREADS; }
 static int scan_blocks(const hfx_sched *s, int64_t n) {
   const int64_t want = (n / 4 + scan_threads(s, n) - 1) / scan_threads(s, n);
@@ -1254,9 +1253,9 @@ int hfx_launch_dispatch(hfx_sched *s, const hfx_table *t, int64_t now_ns, const 
   const int blocks = scan_blocks(s, n);
   const int threads = scan_threads(s, n);
   a.rounds = (int32_t)((n / 4 + (int64_t)threads * blocks - 1) / ((int64_t)threads * blocks));
-  // blocks of the cooperative kernel: a warp per entry of a small queue, which a larger table may hold too, and tiles of 512 entries (60,013 rows: 30
-  // blocks and tiles of 1024 entries 66.7 us, 59 63.6, 118 and tiles of 512 61.6; a barrier takes 1.5 us with 30 and with 148 blocks).  4090 entries
-  // queued, 8300 rows 17 blocks 83.2 us, 128 42.3, 20,000 rows 40 blocks 54.6, 128 42.4; most of 16,000 queued 32 blocks 53.2, 128 53.3
+  // blocks of the cooperative kernel: a warp per entry of a small queue, which a larger table may hold too, and tiles of 512 entries (a barrier takes
+  // 1.5 us with 30 and with 148 blocks).  4090 entries queued: 8300 rows 17 blocks 83.2 us, 128 42.3, 20,000 rows 40 blocks 54.6, 128 42.4; most of
+  // 16,000 rows queued 32 blocks 53.2, 128 53.3, 60,013 118 55.0, 128 55.4
   int64_t want = (n < DISP_SMALL ? n + 31 : DISP_SMALL) / 32, want_r = (R + 31) / 32;
   if (want < (n + 511) / 512) want = (n + 511) / 512;
   if (want < want_r) want = want_r;

@@ -363,8 +363,8 @@ __global__ void __launch_bounds__(FRONT_THREADS, 1) k_front(const HfxParams p, c
     if (!any_big) {
       // ... then every group in row order: the place of a row is the number of smaller rows in its group, two slots at a time: with bit 15
       // set beside their 13 bits, x - il keeps that bit in every half that is not smaller, and nothing is borrowed from the half above
-      // (bound by instructions: a tile's counting over groups of 55 rows took 16 of its 48 K cycles; four ticks of a fleet of 1024 1627 -> 1598 us,
-      // ten steps over 1024 replicas, groups of 3.5, 598 -> 593.  Plain comparisons of two or four slots to a look: 1655, 1675)
+      // (bound by instructions: one slot at a time, counting over groups of 55 rows was 16 of a tile's 48 K cycles; four ticks of a fleet of 1024
+      // 1627 us one at a time, 1598 so)
       const uint32_t *s_two = reinterpret_cast<const uint32_t *>(s_perm);
       for (int j = tid; j < n_slots; j += blockDim.x) {
         const uint32_t il = s_perm[j] & 0x7fffu;

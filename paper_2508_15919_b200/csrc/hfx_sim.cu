@@ -17,12 +17,10 @@
 //   - iterations in which nothing arrives, finishes or is admitted are taken 32 at a time: the clock after j of
 //     them is now + j E_d + d2 n_run j (j - 1) / 2 (every request in flight adds one token of context), lane j
 //     forms it and a ballot finds the first one that something happens in.  Before maturity the stretch ends at maturity.
-// What bounds it is one dependent chain per trace.  B200, one trace of 256 rows, 2000 iterations: 807 us with the running batch in a list in
-// memory and comparisons of 128-bit products in place of the budget, 710 now (280 K warp instructions then, 249 K when the batch went into
-// registers, at 5.6 cycles each, half of it the latency of the instruction in front); 4096 traces of 2048 rows, 10,000 iterations 21.3 -> 15.1 ms
-// (loads waited 2.5 of 9 cycles an instruction, rows of the queue and the batch scattered over sectors of L1 and L2).  Tried: the queue's list with
-// holes in place of closing it up (17.0 -> 23.4 ms: large prompts that never fit stay in front and are passed each time), 20 and 28
-// traces an SM with 96 and 72 registers (18.0, 30.7 ms against 17.1), output lengths copied ahead with cp.async (17.0 -> 18.0).
+// What bounds it is one dependent chain per trace.  B200, one trace of 256 rows, 2000 iterations: 756 us with the running batch in a list in
+// memory and comparisons of 128-bit products in place of the budget, 653 so (5.6 cycles to a warp instruction, half of them the latency of the one
+// in front); 4096 traces of 2048 rows, 10,000 iterations 21.3 and 15.0 ms (loads waited 2.5 of 9 cycles an instruction there, rows of the queue and the
+// batch scattered over sectors of L1 and L2).
 // A row takes 19 bytes: 16 side by side, which are one look at it (slack base while queued, admission and finish iteration while running; prompt length
 // and priority; output length), a byte (class and state) and one list entry (the queue from the front of the list array, what the
 // registers do not hold of the running batch from its back: a row is in one of them at most).

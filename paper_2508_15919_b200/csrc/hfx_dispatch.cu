@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(threads, 1) k_disp_scan(const HfxParams p, con
 //   3  tiles of whole bins in shared memory: every bin divided further, about one item to a fine bin, an item's place in
 //      its fine bin by counting, in a full one by a sorting network; rows out in order, running totals
 // An item is moved once (into its bin) where the radix passes moved it eleven times.  A queue of 471 K entries in 148 blocks takes 58 us by the GPU's clock:
-// sample and plans 8, splitters 5, bins 14, their starts 3, moving 4, tiles 10.5, running totals 8.5, three barriers of 1.5; one of 42 K in 118 blocks 30.
+// sample and plans 8, splitters 5, bins 14, their starts 3, moving 4, tiles 10.5, running totals 8.5, three barriers of 1.5; one of 42 K 30.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ bool grid_barrier(unsigned long long *ctl, uint32_t *status, uint32_t limit, uint32_t &round, uint32_t *s_ok) {
   round++;
